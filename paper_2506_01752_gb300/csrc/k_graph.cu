@@ -8,6 +8,11 @@
 //   edge listed once, at its endpoint of lower (degree, id). A warp per node
 //   counts the neighbours above it, one block scans the counts into row
 //   pointers, and a warp per node writes the entries in row order.
+// * the mutation's adjacency: the rows in processing order (degree
+//   descending), padded to groups of four entries with the id n, so that a
+//   thread reads four neighbours with one 16-byte load; and a record per node
+//   (id, first group, degree) in the same order, one load instead of the
+//   chain order -> row pointers.
 //
 // Every index these kernels form is in range because the host checks ran
 // first; the oriented entries are also bounded by their buffer, so a graph
@@ -124,6 +129,37 @@ orient_fill_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__
     }
 }
 
+// nodes[k] = (v, first group of four of its adjacency, deg v, 0) of the node
+// at position k of the order; its place follows from its degree because the
+// order is by degree.
+__global__ void __launch_bounds__(kBlock)
+node_records_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ order,
+                    const int2 *__restrict__ by_degree, int4 *__restrict__ nodes)
+{
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int v = order[k];
+        const int d = row_ptr[v + 1] - row_ptr[v];
+        const int2 at = by_degree[d];
+        nodes[k] = make_int4(v, at.y + (k - at.x) * ((d + 3) / 4), d, 0);
+    }
+}
+
+// The rows of the mutation's adjacency, a warp each, padded with n.
+__global__ void __launch_bounds__(kBlock)
+mutation_rows_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
+                     const int4 *__restrict__ nodes, int4 *__restrict__ adj)
+{
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int k = warp; k < n; k += nwarps) {
+        const int4 rec = nodes[k];
+        const int beg = __ldg(row_ptr + rec.x);
+        int32_t *row = reinterpret_cast<int32_t *>(adj + rec.y);
+        for (int e = lane; e < ((rec.z + 3) & ~3); e += 32) row[e] = e < rec.z ? __ldg(col_idx + beg + e) : n;
+    }
+}
+
 int warp_grid(const void *kernel, int n, int sms)
 {
     int per_sm = 0;
@@ -144,6 +180,17 @@ cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx,
     scan_kernel<<<1, 1024, 0, s>>>(eptr, n + 1);
     orient_fill_kernel<<<warp_grid((const void *)orient_fill_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr, col_idx,
                                                                                               eptr, eidx, cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mutation_adjacency(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
+                                      const int2 *by_degree, int4 *nodes, int4 *adj, int sms, cudaStream_t s)
+{
+    long long blocks = ((long long)n + kBlock - 1) / kBlock;
+    if (blocks > 16ll * sms) blocks = 16ll * sms;
+    node_records_kernel<<<(int)blocks, kBlock, 0, s>>>(n, row_ptr, order, by_degree, nodes);
+    mutation_rows_kernel<<<warp_grid((const void *)mutation_rows_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr, col_idx,
+                                                                                                  nodes, adj);
     return cudaGetLastError();
 }
 

@@ -164,8 +164,14 @@ __device__ __forceinline__ void crossover_body(const GenParams gp, const int32_t
                                                const uint32_t *__restrict__ gen_ptr, int *__restrict__ dcount,
                                                int vblock, int vgrid)
 {
-    // The mutation kernel that follows appends deferred pairs from zero.
-    if (vblock == 0 && threadIdx.x < 3) dcount[threadIdx.x] = 0;
+    // The mutation kernel that follows appends deferred pairs from zero, and
+    // counts the own label first if that settled at least half of the last
+    // generation's sampled pairs.
+    if (vblock == 0 && threadIdx.x == 0) {
+        const int pairs = dcount[kDcountPairs], ok = dcount[kDcountOk];
+        dcount[kDcountFast] = pairs > 0 && 2 * ok >= pairs ? 1 : 0;
+        for (int k = 0; k <= kDcountOk; ++k) dcount[k] = 0;
+    }
     extern __shared__ int smem[];
     const int W = gp.W, np = gp.np, E = gp.es;
     const int nq = W >> 2;
@@ -372,107 +378,53 @@ crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__res
 // below thr_m and deg(v) > 0; it then takes the most frequent label among its
 // neighbours in the post-crossover child (synchronous: all reads come from
 // `child`), the tie among the t most frequent labels broken by the MTIE word
-// (the pick(u, t)-th smallest). A warp takes a node; its lanes take the
-// node's selected children, whose neighbour labels are staged into a
-// per-warp tile (a column per pair). Degree <= 32: when many pairs are
-// selected, each lane sorts its own pair's labels in registers with a
-// merge-exchange network of 8, 12, .., 28 or 32 entries (the smallest that
-// holds the degree) and reads the tied labels off the runs, all pairs at
-// once; when few are, the whole warp votes on two pairs at a time (one
-// neighbour per lane grouped by __match_any_sync, the pick(u, t)-th tied
-// label by removing minima or, for deep ranks, by sorting the tied labels
-// across the warp). Degree > 32: when the node's history says it pays, a
-// Misra-Gries summary with K counters (K = 1 up to degree 64, 3 above) and an
-// exact recount of its survivors settle every pair whose best count c has
-// (K + 1) c > deg (every label reaching c is then a candidate); the other
-// pairs of degree 33..kDeferMax are listed for mutation_vote_kernel (one pair
-// per thread, labels sorted in registers), those of degree kDeferMax + 1 ..
-// kSharedTableMax take a count table in shared memory, one pair at a time,
-// and those above are listed for mutation_hub_kernel (a warp per pair, its
-// count table in global scratch).
+// (the pick(u, t)-th smallest).
+//
+// A pair is a (node, selected child). A warp takes a batch of nodes, copies
+// their rows to Q, and lists the batch's pairs; then every lane works on a
+// pair of its own, so that the lanes stay full whatever number of children a
+// node has selected (about 20 of 100 at M_P 0.2). In a settled population the
+// result is nearly always the label the node already has, and counting the
+// neighbours that hold it proves that: when it is on more than half of them
+// it is the unique mode. The pairs this leaves open take the exact vote, by
+// degree:
+//   up to 32     in the same warp, a pair per lane: the labels are gathered
+//                into registers, sorted by a merge-exchange network of 8, 12,
+//                .., 28 or 32 entries (the smallest that holds the degree) and
+//                the tied labels read off the runs
+//   33..128      listed for mutation_vote_kernel, a pair per thread
+//   129..512     a warp per pair: count table in shared memory (the node's
+//                pairs are split over kWideParts warps)
+//   above 512    listed for mutation_hub_kernel, a block per pair
+// Whether the count of the own label is worth its pass over the neighbours is
+// read from the last generation: the share of the pairs it settled (or would
+// have settled), for degree <= 32 over a sample of all pairs, above per node.
+//
+// The neighbours come from the mutation's own adjacency: rows in processing
+// order (degree descending), padded to four entries with the id n, whose
+// child row holds a value above every label, so that four neighbours are one
+// 16-byte load and padding needs no test.
 // ---------------------------------------------------------------------------
 
-// The ka-th and kb-th smallest of the distinct labels held by the lanes of
-// two candidate sets ca and cb, by removing the minimum k times; the two
-// chains run side by side so that their reductions overlap. la / lb receive
-// the lanes (-1 for an empty set). Labels are non-negative.
-__device__ __forceinline__ void select_kth_lane2(unsigned ca, int xa, unsigned ka, unsigned cb, int xb, unsigned kb,
-                                                 int &la, int &lb)
+// MTIE word of child i at node v.
+__device__ __forceinline__ uint32_t tie_word(const GenParams &gp, int v, int i, uint32_t g)
 {
-    const int lane = threadIdx.x & 31;
-    unsigned acta = ca, actb = cb;
-    const unsigned kmax = ka > kb ? ka : kb;
-    for (unsigned s = 0; s < kmax; ++s) {
-        const unsigned mna = __reduce_min_sync(kFull, ((acta >> lane) & 1u) ? (unsigned)xa : 0xffffffffu);
-        const unsigned mnb = __reduce_min_sync(kFull, ((actb >> lane) & 1u) ? (unsigned)xb : 0xffffffffu);
-        const unsigned ra = __ballot_sync(kFull, ((acta >> lane) & 1u) && (unsigned)xa == mna);
-        const unsigned rb = __ballot_sync(kFull, ((actb >> lane) & 1u) && (unsigned)xb == mnb);
-        if (s < ka) acta &= ~ra;
-        if (s < kb) actb &= ~rb;
-    }
-    const unsigned mna = __reduce_min_sync(kFull, ((acta >> lane) & 1u) ? (unsigned)xa : 0xffffffffu);
-    const unsigned mnb = __reduce_min_sync(kFull, ((actb >> lane) & 1u) ? (unsigned)xb : 0xffffffffu);
-    la = __ffs(__ballot_sync(kFull, ((acta >> lane) & 1u) && (unsigned)xa == mna)) - 1;
-    lb = __ffs(__ballot_sync(kFull, ((actb >> lane) & 1u) && (unsigned)xb == mnb)) - 1;
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)(i >> 2), g, kStageMutTie), gp.key0, gp.key1);
+    return word_of(r, i & 3);
 }
 
-// Two ascending bitonic sorts across the warp (one value per lane each),
-// run as independent chains.
-__device__ __forceinline__ void warp_sort32x2(unsigned &a, unsigned &b)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const unsigned pa = __shfl_xor_sync(kFull, a, j);
-            const unsigned pb = __shfl_xor_sync(kFull, b, j);
-            const bool keep_min = ((lane & j) == 0) == ((lane & k) == 0);
-            a = keep_min ? min(a, pa) : max(a, pa);
-            b = keep_min ? min(b, pb) : max(b, pb);
-        }
-    }
-}
-
-// Above this tie rank the k-th tied label comes from sorting the tied labels
-// rather than from removing the minimum k times.
-constexpr unsigned kRemovalMax = 4;
-
-// MTIE words of the lane's four children at node v (computed by every lane
-// together, the first time a tie occurs at v).
-__device__ __forceinline__ uint4 tie_words(const GenParams &gp, int v, int lane, uint32_t g)
-{
-    return philox4x32_10(make_uint4((uint32_t)v, (uint32_t)lane, g, kStageMutTie), gp.key0, gp.key1);
-}
-
-// A neighbour id read from the CSR; in the debug build an id outside [0, n)
-// is recorded and replaced by 0, so that the access it feeds stays in bounds.
+// A neighbour id read from the adjacency; in the debug build an id outside
+// [0, n] is recorded and replaced by n (the padding row), so that the access
+// it feeds stays in bounds.
 __device__ __forceinline__ int checked_node(int u, int n)
 {
-    return MOCD_CHECK(u >= 0 && u < n, kCheckNode, u) ? u : 0;
+    return MOCD_CHECK(u >= 0 && u <= n, kCheckNode, u) ? u : n;
 }
 
 __device__ __forceinline__ uint32_t hash_slot(int x, int hbits)
 {
     return ((uint32_t)x * 2654435761u) >> (32 - hbits);
 }
-
-// Asynchronous 4-byte global -> shared copy (no register staging) and the
-// wait for all of this thread's outstanding copies.
-__device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem_src) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
-constexpr int kTileStride = 33;  // padded row of the per-warp label tile
-constexpr int kTileRows = 32;    // neighbours whose labels the tile keeps
-static_assert(kDeferMax == 4 * kTileRows, "deferred classes: degrees 33..64 and 65..128");
 
 // Start of deferred-vote class c in the list: the classes are stored one
 // after the other (written with selects: indexing the kernel parameter array
@@ -485,7 +437,10 @@ __device__ __forceinline__ int defer_capacity(const GenParams &gp, int c)
 {
     return c == 0 ? gp.defer_cap[0] : c == 1 ? gp.defer_cap[1] : gp.defer_cap[2];
 }
-constexpr int kMutBlock = 128;   // mutation threads per block (shared memory bound)
+constexpr int kLaneMax = 32;     // largest degree of the per-lane vote
+constexpr int kMutBlock = 128;   // mutation threads per block
+constexpr int kHubBlock = 256;   // threads per block of the hub kernel
+constexpr int kBatch = 8;        // most nodes of a warp's batch
 
 // Sorting networks for any N: Batcher's merge exchange in the form of
 // Knuth, TAOCP vol. 3, Sec. 5.2.2, Algorithm M (for a power of two it is
@@ -583,28 +538,27 @@ __device__ __forceinline__ int select_at(const int (&x)[N], int pos)
     return y[0];
 }
 
-// Exact neighbour-majority of one pair by its own lane: the pair's deg <= N
-// labels (1 <= deg <= N <= 32) are sorted in registers; equal labels then
-// form runs, the longest runs are the tied labels in ascending order, and the
-// pick(u, t)-th of them is the result. Bit j of e is set when entries j and
-// j + 1 are equal, so a run of L labels is L - 1 consecutive set bits; each
-// step m &= m >> 1 shortens every run of set bits by one, and the last
-// non-zero m has one bit per longest run, at its first entry (all entries
-// when no two labels are equal).
-template <int N>
-__device__ __forceinline__ int lane_pick(int (&x)[N], int deg, uint32_t u)
+// The first entries of the longest runs of equal values among the deg sorted
+// entries behind e (bit j of e: entries j and j + 1 are equal, both < deg):
+// a run of L values is L - 1 consecutive set bits; each step m &= m >> 1
+// shortens every run of set bits by one, and the last non-zero m has one bit
+// per longest run, at its first entry (all entries when no two are equal).
+// best: the length of those runs.
+__device__ __forceinline__ unsigned longest_runs(unsigned e, int deg, int &best)
 {
-    sort_network<N>(x);
-    unsigned e = 0;
-#pragma unroll
-    for (int j = 0; j + 1 < N; ++j) e |= (x[j] == x[j + 1] ? 1u : 0u) << j;
     e &= deg >= 2 ? 0xffffffffu >> (33 - deg) : 0u;  // pairs (j, j + 1) with j + 1 < deg
     unsigned starts = deg >= 32 ? 0xffffffffu : (1u << deg) - 1u;
-    for (unsigned m = e; m != 0u; m &= m >> 1) starts = m;
-    const int t = __popc(starts);
-    const unsigned kk = t > 1 ? pick_index(u, (uint32_t)t) : 0u;
-    // Position of the kk-th set bit of `starts`, halving the window each step.
-    unsigned m = starts, k = kk;
+    best = 1;
+    for (unsigned m = e; m != 0u; m &= m >> 1) {
+        starts = m;
+        ++best;
+    }
+    return starts;
+}
+
+// Position of the k-th set bit of m (k < popc(m)), halving the window.
+__device__ __forceinline__ int kth_bit(unsigned m, unsigned k)
+{
     int pos = 0;
 #pragma unroll
     for (int w = 16; w >= 1; w >>= 1) {
@@ -618,61 +572,59 @@ __device__ __forceinline__ int lane_pick(int (&x)[N], int deg, uint32_t u)
             m = low;
         }
     }
-    return select_at<N>(x, pos);
+    return pos;
 }
 
-// Lane-parallel exact vote of every selected pair of a node with
-// deg <= kTileRows (N >= deg): each lane sorts its pair's deg labels (its
-// column of the staged tile) in registers and writes its result.
+// Exact neighbour-majority of one pair by its own lane (deg <= N <= 32; 0
+// for a lane without a pair): the labels are gathered into registers (the
+// padding and the entries past it sort last), sorted, and the tied labels are
+// the longest runs in ascending order. All lanes of the warp call together.
 template <int N>
-__device__ __forceinline__ void lane_votes(const int *tile, int deg, bool mine, int i, uint4 tw, int *s_res)
+__device__ __forceinline__ int lane_vote(const GenParams &gp, const int4 *__restrict__ adj,
+                                         const int32_t *__restrict__ child, int v, int i, int beg, int deg, uint32_t g,
+                                         int &best)
 {
-    const int src = i >> 2;
-    const uint32_t w0 = __shfl_sync(0xffffffffu, tw.x, src);
-    const uint32_t w1 = __shfl_sync(0xffffffffu, tw.y, src);
-    const uint32_t w2 = __shfl_sync(0xffffffffu, tw.z, src);
-    const uint32_t w3 = __shfl_sync(0xffffffffu, tw.w, src);
-    const int k = i & 3;
-    const uint32_t u = k == 0 ? w0 : (k == 1 ? w1 : (k == 2 ? w2 : w3));
-    const int *col = tile + (threadIdx.x & 31);
+    const int32_t *col = child + i;
     int x[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) x[j] = j < deg ? col[j * kTileStride] : INT_MAX;
-    const int res = lane_pick<N>(x, deg, u);
-    if (mine) s_res[i] = res;
+    for (int j = 0; j < N; j += 4) {
+        const bool in = j < deg;
+        const int4 u = in ? __ldg(adj + beg + j / 4) : make_int4(0, 0, 0, 0);
+        x[j + 0] = in ? col[(size_t)checked_node(u.x, gp.n) * gp.W] : INT_MAX;
+        x[j + 1] = in ? col[(size_t)checked_node(u.y, gp.n) * gp.W] : INT_MAX;
+        x[j + 2] = in ? col[(size_t)checked_node(u.z, gp.n) * gp.W] : INT_MAX;
+        x[j + 3] = in ? col[(size_t)checked_node(u.w, gp.n) * gp.W] : INT_MAX;
+    }
+    sort_network<N>(x);
+    unsigned e = 0;
+#pragma unroll
+    for (int j = 0; j + 1 < N; ++j) e |= (x[j] == x[j + 1] ? 1u : 0u) << j;
+    const unsigned starts = longest_runs(e, deg, best);
+    const int t = __popc(starts);
+    unsigned kk = 0;
+    if (__any_sync(kFull, t > 1)) kk = t > 1 ? pick_index(tie_word(gp, v, i, g), (uint32_t)t) : 0u;
+    return select_at<N>(x, kth_bit(starts, kk));
 }
 
-// The smallest network size of the per-lane vote that holds deg labels, and
-// the fewest pairs (lanes) for which the per-lane vote beats the warp vote.
-__device__ __forceinline__ int lane_vote_min_pairs(int deg)
-{
-    return deg <= 8 ? 2 : deg <= 16 ? 5 : 10;
-}
-
-// Exact neighbour-majority of one pair of a node with degree > kDeferMax by
-// the whole warp: a per-warp open-addressing count table (in shared memory,
-// or for the hubs above kSharedTableMax in global scratch), sized to the
-// node (the
-// smallest power of two with at least 2 deg slots), filled with one insert
-// per distinct label of each 32-neighbour chunk (__match_any_sync gives the
-// multiplicity). The labels reaching the largest count are then compacted
-// (one slot per distinct label) and the pick(u, t)-th smallest of them is
-// found either by stepping up through the minima (shallow ranks) or bit by
-// bit from the top (deep ranks).
+// Exact neighbour-majority of one pair of a node with degree kDeferMax + 1 ..
+// kSharedTableMax by the whole warp: an open-addressing count table in shared
+// memory, sized to the node (the smallest power of two with at least 2 deg
+// slots), filled with one insert per distinct label of each 32-neighbour chunk
+// (__match_any_sync gives the multiplicity). The labels reaching the largest
+// count are then compacted (one slot per distinct label) and the pick(u, t)-th
+// smallest of them is found either by stepping up through the minima (shallow
+// ranks) or bit by bit from the top (deep ranks).
 __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_t *__restrict__ child,
-                                            const int32_t *__restrict__ col_idx, int beg, int deg,
-                                            const int *tile_col, int i, int *hkey, int *hcnt, uint32_t tie_u,
-                                            unsigned &best_count)
+                                               const int *__restrict__ nbr, int deg, int v, int i, int *hkey,
+                                               int *hcnt, uint32_t g, unsigned &best_count)
 {
-    // tile_col: the staged labels of the first kTileRows neighbours, or NULL
-    // (all are gathered from `child`).
     const int lane = threadIdx.x & 31;
     const int W = gp.W;
-    // 2 deg <= 2 dmax <= the per-warp capacity, so the table fits.
-    int hbits = 7;
+    // 2 deg <= the per-warp capacity (gp.hash_size), so the table fits.
+    int hbits = 8;
     while ((1 << hbits) < 2 * deg) ++hbits;
     const int HS = 1 << hbits;
-    const int per_lane = HS >> 5;
+    const int per_lane = HS >> 5;  // 8 .. 32
     for (int e = lane; e < HS; e += 32) {
         hkey[e] = -1;
         hcnt[e] = 0;
@@ -681,9 +633,7 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
     for (int e0 = 0; e0 < deg; e0 += 32) {
         const bool in = e0 + lane < deg;
         int x = (int)(0x80000000u | lane);
-        if (in)
-            x = (tile_col && e0 + lane < kTileRows) ? tile_col[(e0 + lane) * kTileStride]
-                                                    : child[(size_t)checked_node(__ldg(col_idx + beg + e0 + lane), gp.n) * W + i];
+        if (in) x = child[(size_t)checked_node(__ldg(nbr + e0 + lane), gp.n) * W + i];
         // One insert per distinct label of the chunk, with its multiplicity.
         const unsigned peers = __match_any_sync(kFull, x);
         if (in && (peers & ((1u << lane) - 1u)) == 0) {
@@ -705,45 +655,24 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
     for (int s = 0; s < per_lane; ++s) mx_l = max(mx_l, (unsigned)hcnt[lane + 32 * s]);
     const unsigned mx = __reduce_max_sync(kFull, mx_l);
     best_count = mx;
-    // The tied labels: compacted into hcnt[0, t) when each lane has at most
-    // 32 slots (a bit mask per lane); in larger (hub) tables the keys of the
-    // slots below the top count are cleared instead, and the tied labels are
-    // the keys still set, scanned over the whole table.
-    int t;
-    const int *tied;
-    int span;
-    if (per_lane <= 32) {
-        unsigned act = 0;
-        for (int s = 0; s < per_lane; ++s)
-            if ((unsigned)hcnt[lane + 32 * s] == mx) act |= 1u << s;
-        // Compact the tied labels into hcnt[0, t) (the counts are no longer needed).
-        const unsigned mine = (unsigned)__popc(act);
-        unsigned incl = mine;
+    unsigned act = 0;
+    for (int s = 0; s < per_lane; ++s)
+        if ((unsigned)hcnt[lane + 32 * s] == mx) act |= 1u << s;
+    // Compact the tied labels into hcnt[0, t) (the counts are no longer needed).
+    const unsigned mine = (unsigned)__popc(act);
+    unsigned incl = mine;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned y = __shfl_up_sync(kFull, incl, d);
-            if (lane >= d) incl += y;
-        }
-        t = (int)__shfl_sync(kFull, incl, 31);
-        int at = (int)(incl - mine);
-        __syncwarp();
-        for (int s = 0; s < per_lane; ++s)
-            if ((act >> s) & 1u) hcnt[at++] = hkey[lane + 32 * s];
-        tied = hcnt;
-        span = t;
-    } else {
-        unsigned mine = 0;
-        for (int s = 0; s < per_lane; ++s) {
-            const int e = lane + 32 * s;
-            if ((unsigned)hcnt[e] == mx) ++mine;
-            else hkey[e] = -1;
-        }
-        t = (int)__reduce_add_sync(kFull, mine);
-        tied = hkey;
-        span = HS;
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += y;
     }
+    const int t = (int)__shfl_sync(kFull, incl, 31);
+    int at = (int)(incl - mine);
     __syncwarp();
-    const unsigned kk = t > 1 ? pick_index(tie_u, (uint32_t)t) : 0u;
+    for (int s = 0; s < per_lane; ++s)
+        if ((act >> s) & 1u) hcnt[at++] = hkey[lane + 32 * s];
+    __syncwarp();
+    const unsigned kk = t > 1 ? pick_index(tie_word(gp, v, i, g), (uint32_t)t) : 0u;
     int res;
     if (kk > (unsigned)gp.label_bits) {
         // Deep rank: at bit b (from the top), count the tied labels that agree
@@ -754,10 +683,9 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
         for (int b = gp.label_bits - 1; b >= 0; --b) {
             const unsigned above = ~((2u << b) - 1u);  // the bits above b
             unsigned c = 0;
-            for (int e = lane; e < span; e += 32) {
-                const int key = tied[e];
-                if (key < 0) continue;  // a cleared slot of a hub table
-                c += (((unsigned)key & above) == prefix && (((unsigned)key >> b) & 1u) == 0u) ? 1u : 0u;
+            for (int e = lane; e < t; e += 32) {
+                const unsigned key = (unsigned)hcnt[e];
+                c += ((key & above) == prefix && ((key >> b) & 1u) == 0u) ? 1u : 0u;
             }
             const unsigned cnt = __reduce_add_sync(kFull, c);
             if (rank >= cnt) {
@@ -772,8 +700,8 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
         int last = -1;
         for (unsigned s = 0; s <= kk; ++s) {
             unsigned my = 0xffffffffu;
-            for (int e = lane; e < span; e += 32) {
-                const int key = tied[e];
+            for (int e = lane; e < t; e += 32) {
+                const int key = hcnt[e];
                 if (key > last) my = min(my, (unsigned)key);
             }
             last = (int)__reduce_min_sync(kFull, my);
@@ -784,28 +712,162 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
     return res;
 }
 
-__global__ void __launch_bounds__(kMutBlock, 6)
-mutation_kernel(GenParams gp, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                const int32_t *__restrict__ order, const int32_t *__restrict__ child, int32_t *__restrict__ q,
-                const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist,
-                unsigned long long *__restrict__ acc, uint32_t *__restrict__ hint, int2 *__restrict__ dlist,
-                int *__restrict__ dcount)
+// D of the evaluation's degree histogram: child i's final label of a node of
+// degree d (label-major cell label * W + i). The old value is not needed, so
+// this is a reduction that does not stall.
+__device__ __forceinline__ void add_degree(const GenParams &gp, uint32_t *__restrict__ hist, int label, int i, int d)
 {
-    extern __shared__ int smem[];
-    const int W = gp.W, np = gp.np;
+    if (MOCD_CHECK(label >= 0 && label < gp.n, kCheckLabel, label))
+        atomicAdd(hist + (size_t)label * gp.W + i, (unsigned)d);
+}
+
+// Bit k set: child 4 * lane + k of node v mutates.
+__device__ __forceinline__ unsigned selected(const GenParams &gp, int v, int lane, uint32_t g)
+{
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)lane, g, kStageMutCoin), gp.key0, gp.key1);
+    const int i0 = 4 * lane;
+    return ((i0 + 0 < gp.np && (unsigned long long)r.x < gp.thr_m) ? 1u : 0u) |
+           ((i0 + 1 < gp.np && (unsigned long long)r.y < gp.thr_m) ? 2u : 0u) |
+           ((i0 + 2 < gp.np && (unsigned long long)r.z < gp.thr_m) ? 4u : 0u) |
+           ((i0 + 3 < gp.np && (unsigned long long)r.w < gp.thr_m) ? 8u : 0u);
+}
+
+// Node row of a warp: Q gets the children's own labels, the histogram the
+// unselected ones (mutating pairs add theirs once decided), and the selected
+// children go to list[total ..] tagged with `tag`. Returns their number.
+__device__ __forceinline__ int take_row(const GenParams &gp, int v, int deg, bool active, const int4 &out, int lane,
+                                        uint32_t g, int4 *__restrict__ Q4, uint32_t *__restrict__ hist,
+                                        unsigned short *list, int total, int tag)
+{
+    unsigned sel = 0;
+    if (active && deg > 0) sel = selected(gp, v, lane, g);
+    if (active) {
+        Q4[(size_t)v * (gp.W >> 2) + lane] = out;
+        if (deg > 0) {
+            const int i0 = 4 * lane;
+            if (i0 + 0 < gp.np && !(sel & 1u)) add_degree(gp, hist, out.x, i0 + 0, deg);
+            if (i0 + 1 < gp.np && !(sel & 2u)) add_degree(gp, hist, out.y, i0 + 1, deg);
+            if (i0 + 2 < gp.np && !(sel & 4u)) add_degree(gp, hist, out.z, i0 + 2, deg);
+            if (i0 + 3 < gp.np && !(sel & 8u)) add_degree(gp, hist, out.w, i0 + 3, deg);
+        }
+    }
+    // Place of the lane's selected children: its count (0 .. 4) by bits.
+    const unsigned lt = (1u << lane) - 1u;
+    const int mine = __popc(sel);
+    const unsigned b0 = __ballot_sync(kFull, mine & 1), b1 = __ballot_sync(kFull, mine & 2),
+                   b2 = __ballot_sync(kFull, mine & 4);
+    int at = total + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if ((sel >> k) & 1u) list[at++] = (unsigned short)(tag | (4 * lane + k));
+    return __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+}
+
+// Deferred pairs of one class, appended by the lanes of `who` (warp-uniform).
+// The capacity is the class's nodes x N_p, every pair a generation can defer:
+// the check only keeps a corrupted count in bounds.
+__device__ __forceinline__ void defer_pairs(const GenParams &gp, int cls, unsigned who, int node, int i, int lane,
+                                            int2 *__restrict__ dlist, int *__restrict__ dcount)
+{
+    int first = 0;
+    if (lane == 0) first = atomicAdd(dcount + cls, __popc(who));
+    first = __shfl_sync(kFull, first, 0);
+    if ((who >> lane) & 1u) {
+        const int at = first + __popc(who & ((1u << lane) - 1u));
+        if (at < defer_capacity(gp, cls)) dlist[defer_offset(gp, cls) + at] = make_int2(node, i);
+    }
+}
+
+// hint of a node (or part): (pairs << 16) | pairs whose own label was on more
+// than half of the neighbours, last generation; 0: no history.
+__device__ __forceinline__ bool own_label_pays(uint32_t h)
+{
+    return h != 0u && 2u * (h & 0xffffu) >= (h >> 16);
+}
+
+// One item of the nodes above kDeferMax: a hub (idx < gp.n_hub), whose pairs
+// are all listed for mutation_hub_kernel, or part `part` of a node of degree
+// kDeferMax + 1 .. kSharedTableMax: the quads q with q % kWideParts == part.
+__device__ __noinline__ void wide_item(const GenParams &gp, int item, const int4 *__restrict__ nodes,
+                                       const int4 *__restrict__ adj, const int32_t *__restrict__ child,
+                                       int32_t *__restrict__ q, uint32_t *__restrict__ hist,
+                                       uint32_t *__restrict__ hint, int2 *__restrict__ dlist, int *__restrict__ dcount,
+                                       unsigned short *list, int *hkey, int *hcnt, uint32_t g)
+{
+    const int lane = threadIdx.x & 31;
+    const int nq = gp.W >> 2;
+    const bool hub = item < gp.n_hub;
+    const int idx = hub ? item : gp.n_hub + (item - gp.n_hub) / kWideParts;
+    const int part = hub ? 0 : (item - gp.n_hub) % kWideParts;
+    const int4 rec = __ldg(nodes + idx);
+    const int v = rec.x, deg = rec.z;
+    const bool active = lane < nq && (hub || lane % kWideParts == part);
+    const int4 out = active ? reinterpret_cast<const int4 *>(child)[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
+    const int total = take_row(gp, v, deg, active, out, lane, g, reinterpret_cast<int4 *>(q), hist, list, 0, 0);
+    uint32_t *h = hint + (hub ? idx : gp.n + (idx - gp.n_hub) * kWideParts + part);
+    const bool fast = own_label_pays(*h);
+    __syncwarp();
+    if (hub) {
+        // The flag travels with the pair: the hub kernel rewrites the hint.
+        for (int base = 0; base < total; base += 32) {
+            const bool has = base + lane < total;
+            defer_pairs(gp, 2, __ballot_sync(kFull, has), idx | (fast ? kHubFast : 0), has ? list[base + lane] : 0, lane,
+                        dlist, dcount);
+        }
+        if (lane == 0) *h = (uint32_t)total << 16;
+        return;
+    }
+    int ok = 0;
+    const int *nbr = reinterpret_cast<const int *>(adj + rec.y);
+    for (int k = 0; k < total; ++k) {
+        const int i = list[k];
+        const int own = child[(size_t)v * gp.W + i];
+        bool settled = false;
+        if (fast) {
+            int c = 0;
+#pragma unroll 4
+            for (int e = lane; e < deg; e += 32) c += child[(size_t)checked_node(__ldg(nbr + e), gp.n) * gp.W + i] == own;
+            settled = 2 * __reduce_add_sync(kFull, c) > deg;
+        }
+        int lab = own;
+        if (!settled) {
+            unsigned mx = 0;
+            lab = warp_mode_table(gp, child, nbr, deg, v, i, hkey, hcnt, g, mx);
+            settled = !fast && lab == own && 2 * (int)mx > deg;
+            if (lane == 0 && lab != own) q[(size_t)v * gp.W + i] = lab;
+        }
+        ok += settled ? 1 : 0;
+        if (lane == 0) add_degree(gp, hist, lab, i, deg);
+    }
+    if (lane == 0) *h = ((uint32_t)total << 16) | (uint32_t)ok;
+}
+
+// WIDE: the graph has degrees above kDeferMax. batch: nodes a warp takes at a
+// time (<= kBatch).
+template <bool WIDE>
+__global__ void __launch_bounds__(kMutBlock, 6)
+mutation_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict__ nodes, const int4 *__restrict__ adj,
+                const int32_t *__restrict__ child, int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr,
+                uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc, uint32_t *__restrict__ hint,
+                int2 *__restrict__ dlist, int *__restrict__ dcount, int batch)
+{
+    __shared__ unsigned short s_list[kMutBlock / 32][kBatch * kMaxPop];
+    __shared__ int4 s_rec[kMutBlock / 32][kBatch];
+    __shared__ int s_ok[kMutBlock / 32][kBatch];
+    extern __shared__ int s_table[];  // WIDE: per warp, keys and counts
+    const int W = gp.W;
     const int nq = W >> 2;
     const uint32_t g = *gen_ptr;
+    const bool lane_fast = dcount[kDcountFast] != 0;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    const int HS = gp.hash_size;
-    int *s_list = smem + wib * (2 * kMaxPop + kTileRows * kTileStride + 2 * HS);  // selected children
-    int *s_res = s_list + kMaxPop;              // by child index: v's own label, then the result
-    int *tile = s_res + kMaxPop;                // [kTileRows][kTileStride]: label of neighbour j, pair lane
-    int *hkey = tile + kTileRows * kTileStride;
-    int *hcnt = hkey + HS;
+    unsigned short *list = s_list[wib];
+    int4 *recs = s_rec[wib];
+    int *oks = s_ok[wib];
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const bool active = lane < nq;
+    const unsigned lt = (1u << lane) - 1u;
     const int4 *__restrict__ C4 = reinterpret_cast<const int4 *>(child);
     int4 *__restrict__ Q4 = reinterpret_cast<int4 *>(q);
 
@@ -816,337 +878,145 @@ mutation_kernel(GenParams gp, const int32_t *__restrict__ row_ptr, const int32_t
         for (int t = threadIdx.x; t < 2 * kMaxPop; t += blockDim.x) acc[t] = 0;
 
     // Nodes in degree-descending order: every warp starts with one of the
-    // costliest nodes, which balances the grid-stride loop.
-    for (int idx = warp; idx < gp.n; idx += nwarps) {
-        const int v = __ldg(order + idx);
-        const int beg = __ldg(row_ptr + v);
-        const int end = __ldg(row_ptr + v + 1);
-        const int deg = MOCD_CHECK(end >= beg, kCheckRowPtr, v) ? end - beg : 0;
-        int4 out = active ? C4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
-        unsigned sel = 0;  // bit k: child 4 * lane + k mutates
-        if (active && deg > 0) {
-            const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)lane, g, kStageMutCoin),
-                                          gp.key0, gp.key1);
-            const int i0 = 4 * lane;
-            sel = ((i0 + 0 < np && (unsigned long long)r.x < gp.thr_m) ? 1u : 0u) |
-                  ((i0 + 1 < np && (unsigned long long)r.y < gp.thr_m) ? 2u : 0u) |
-                  ((i0 + 2 < np && (unsigned long long)r.z < gp.thr_m) ? 4u : 0u) |
-                  ((i0 + 3 < np && (unsigned long long)r.w < gp.thr_m) ? 8u : 0u);
-        }
-        // Compact the selected children of v into s_list (warp prefix sum).
-        const int mine = __popc(sel);
-        int incl = mine;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(kFull, incl, d);
-            if (lane >= d) incl += y;
-        }
-        const int nsel = __shfl_sync(kFull, incl, 31);
-        if (nsel > 0) {
-            int at = incl - mine;
-            for (int k = 0; k < 4; ++k)
-                if ((sel >> k) & 1u) s_list[at++] = 4 * lane + k;
-            if (active) reinterpret_cast<int4 *>(s_res)[lane] = out;
+    // costliest batches, which balances the grid-stride loop.
+    const int wide = WIDE ? gp.n_hub + gp.n_wide * kWideParts : 0;
+    const int first = WIDE ? gp.n_hub + gp.n_wide : 0;
+    const int items = wide + (gp.n - first + batch - 1) / batch;
+    for (int item = warp; item < items; item += nwarps) {
+        if (WIDE && item < wide) {
+            wide_item(gp, item, nodes, adj, child, q, hist, hint, dlist, dcount, list,
+                      s_table + wib * 2 * gp.hash_size, s_table + wib * 2 * gp.hash_size + gp.hash_size, g);
             __syncwarp();
-            const int my_u0 = lane < deg ? checked_node(__ldg(col_idx + beg + lane), gp.n) : 0;
-            // Degree <= kTileRows: the exact per-lane votes below settle all
-            // pairs at once and cost less than the Misra-Gries pass, even once
-            // the population has settled. Above: the pass runs when the last
-            // generation's exact results (whichever path produced them) say
-            // that most of v's pairs had a label above deg / (K + 1), the pairs
-            // the pass settles. hint = (pairs << 16) | such pairs; 0: no
-            // history.
-            const uint32_t h = deg > kTileRows ? hint[v] : 0u;
-            const bool use_mg = deg > kTileRows && (h == 0u || 2u * (h & 0xffffu) >= (h >> 16));
-            const bool deferred_class = (deg > kTileRows && deg <= kDeferMax) || deg > kSharedTableMax;
-            int nsettle = 0;  // pairs of v with 4 (best count) > deg, settled here
-            bool have_tw = false;
-            uint4 tw = make_uint4(0, 0, 0, 0);
-            for (int base = 0; base < nsel; base += 32) {
-                // Lane = pair (selected child i of node v).
-                const bool has = base + lane < nsel;
-                const int i = has ? s_list[base + lane] : 0;
-                // The tile is read by the pass and by the votes of degree <= 32
-                // and > kDeferMax; pairs of the deferred degrees need it only
-                // for the pass. Degree <= kTileRows with enough selected pairs
-                // takes the per-lane vote, else the warp vote.
-                const bool lane_path =
-                    deg <= kTileRows && __popc(__ballot_sync(kFull, has)) >= lane_vote_min_pairs(deg);
-                const int dt = (use_mg || !deferred_class) ? min(deg, kTileRows) : 0;
-                for (int j = 0; j < dt; ++j) {
-                    const int u = __shfl_sync(kFull, my_u0, j);
-                    if (has) cp_async4(tile + j * kTileStride + lane, child + (size_t)u * W + i);
-                }
-                cp_async_wait_all();
-                __syncwarp();
-                // Pass 1: a Misra-Gries summary with K counters keeps every
-                // label occurring more than deg / (K + 1) times; pass 2 counts
-                // the survivors exactly. K = 1 (Boyer-Moore) up to degree
-                // 2 kTileRows, whose unsettled pairs take the cheap deferred
-                // vote; K = 3 above, where the fallback costs more and settling
-                // more pairs pays. The labels of the first kTileRows
-                // neighbours are read from the tile, the rest from global
-                // memory (eight loads in flight). Empty counters keep distinct
-                // negative labels until first filled; an empty counter that
-                // still holds x takes it back (the same summary as filling a
-                // free one, since no label is ever held by two counters).
-                const int kc = deg <= 2 * kTileRows ? 1 : 3;
-                int s0 = -2, s1 = -3, s2 = -4;  // candidates (labels no neighbour has when empty)
-                int h0 = 0, h1 = 0, h2 = 0;     // their exact counts
-                auto pass = [&](auto kconst) {
-                    constexpr int K = decltype(kconst)::value;
-                    int c0 = -1, c1 = -2, c2 = -3, n0 = 0, n1 = 0, n2 = 0;
-                    auto mg = [&](int x, bool ok) {
-                        if (K == 1) {
-                            const bool e0 = n0 == 0;
-                            n0 = !ok ? n0 : (x == c0 || e0) ? n0 + 1 : n0 - 1;
-                            c0 = ok && e0 ? x : c0;
-                            return;
-                        }
-                        const bool m0 = x == c0, m1 = x == c1, m2 = x == c2;
-                        const bool hit = m0 || m1 || m2;
-                        const bool e0 = n0 == 0, e1 = n1 == 0, e2 = n2 == 0;
-                        const bool f0 = !hit && e0, f1 = !hit && !e0 && e1, f2 = !hit && !e0 && !e1 && e2;
-                        const int dec = (ok && !hit && !e0 && !e1 && !e2) ? 1 : 0;
-                        n0 = ok && (m0 || f0) ? n0 + 1 : n0 - dec;
-                        n1 = ok && (m1 || f1) ? n1 + 1 : n1 - dec;
-                        n2 = ok && (m2 || f2) ? n2 + 1 : n2 - dec;
-                        c0 = ok && f0 ? x : c0;
-                        c1 = ok && f1 ? x : c1;
-                        c2 = ok && f2 ? x : c2;
-                    };
-                    if (has) {
-#pragma unroll 4
-                        for (int j = 0; j < dt; ++j) mg(tile[j * kTileStride + lane], true);
-                    }
-                    for (int e0 = kTileRows; e0 < deg; e0 += 32) {
-                        const int my_u = e0 + lane < deg ? checked_node(__ldg(col_idx + beg + e0 + lane), gp.n) : 0;
-                        const int cnt = min(32, deg - e0);
-                        for (int j0 = 0; j0 < cnt; j0 += 8) {
-                            int xs[8];
-#pragma unroll
-                            for (int t = 0; t < 8; ++t) {
-                                const int u = __shfl_sync(kFull, my_u, min(j0 + t, cnt - 1));
-                                xs[t] = (has && j0 + t < cnt) ? child[(size_t)u * W + i] : 0;
-                            }
-#pragma unroll
-                            for (int t = 0; t < 8; ++t) mg(xs[t], has && j0 + t < cnt);
-                        }
-                    }
-                    s0 = n0 > 0 ? c0 : -2;
-                    if (K > 1) {
-                        s1 = n1 > 0 ? c1 : -3;
-                        s2 = n2 > 0 ? c2 : -4;
-                    }
-                    auto tally = [&](int x) {
-                        h0 += x == s0;
-                        if (K > 1) {
-                            h1 += x == s1;
-                            h2 += x == s2;
-                        }
-                    };
-                    // The first kTileRows labels are still in the tile.
-                    if (has) {
-#pragma unroll 4
-                        for (int j = 0; j < kTileRows; ++j) tally(tile[j * kTileStride + lane]);
-                    }
-                    for (int e0 = kTileRows; e0 < deg; e0 += 32) {
-                        const int my_u = e0 + lane < deg ? checked_node(__ldg(col_idx + beg + e0 + lane), gp.n) : 0;
-                        const int cnt = min(32, deg - e0);
-                        for (int j0 = 0; j0 < cnt; j0 += 8) {
-                            int xs[8];
-#pragma unroll
-                            for (int t = 0; t < 8; ++t) {
-                                const int u = __shfl_sync(kFull, my_u, min(j0 + t, cnt - 1));
-                                xs[t] = (has && j0 + t < cnt) ? child[(size_t)u * W + i] : -1;
-                            }
-#pragma unroll
-                            for (int t = 0; t < 8; ++t) tally(xs[t]);
-                        }
-                    }
-                };
-                if (use_mg) {
-                    if (kc == 1)
-                        pass(std::integral_constant<int, 1>{});
-                    else
-                        pass(std::integral_constant<int, 3>{});
-                }
-                // If the best candidate count c satisfies (K + 1) c > deg, every
-                // label reaching c is a candidate: the tied set is complete and
-                // exact.
-                const int best = max(h0, max(h1, h2));
-                const bool done = has && use_mg && (kc + 1) * best > deg;
-                if (done) {
-                    // Tied candidates in ascending order, then the MTIE pick.
-                    int a = h0 == best ? s0 : INT_MAX;
-                    int b = h1 == best ? s1 : INT_MAX;
-                    int c = h2 == best ? s2 : INT_MAX;
-                    int lo = min(a, b), hi = max(a, b);
-                    a = lo; b = hi;
-                    lo = min(b, c); hi = max(b, c);
-                    b = lo; c = hi;
-                    lo = min(a, b); hi = max(a, b);
-                    a = lo; b = hi;
-                    const int t = 1 + (b != INT_MAX) + (c != INT_MAX);
-                    int lab = a;
-                    if (t > 1) {
-                        const uint4 r = tie_words(gp, v, i >> 2, g);
-                        const uint32_t kk = pick_index(word_of(r, i & 3), (uint32_t)t);
-                        lab = kk == 0 ? a : (kk == 1 ? b : c);
-                    }
-                    s_res[i] = lab;
-                }
-                __syncwarp();
-                unsigned rest = __ballot_sync(kFull, has && !done);
-                nsettle += __popc(__ballot_sync(kFull, done));
-                if (rest && deferred_class) {
-                    // Degrees kTileRows + 1 .. kDeferMax: the exact vote of every
-                    // remaining pair runs in mutation_vote_kernel, one pair per
-                    // thread with its labels sorted in registers; hubs above
-                    // kSharedTableMax: in mutation_hub_kernel, a warp per pair.
-                    // The pair's slot of the row holds -1 until then.
-                    const int cls = deg > kDeferMax ? 2 : deg <= 2 * kTileRows ? 0 : 1;
-                    int first = 0;
-                    if (lane == 0) first = atomicAdd(dcount + cls, __popc(rest));
-                    first = __shfl_sync(kFull, first, 0);
-                    if ((rest >> lane) & 1u) {
-                        const int at_list = first + __popc(rest & ((1u << lane) - 1u));
-                        // The capacity is the class's nodes x N_p, every pair
-                        // a generation can defer: the check only keeps a
-                        // corrupted count in bounds.
-                        if (at_list < defer_capacity(gp, cls)) dlist[defer_offset(gp, cls) + at_list] = make_int2(v, i);
-                        s_res[i] = -1;
-                    }
-                    rest = 0;
-                }
-                if (rest && !have_tw) {
-                    tw = tie_words(gp, v, lane, g);
-                    have_tw = true;
-                }
-                if (lane_path) {
-                    // Many selected pairs: every lane settles its own pair with
-                    // a sorting network of the smallest size that holds deg
-                    // labels (all pairs at once).
-                    const bool mine = (rest >> lane) & 1u;
-                    if (deg <= 8) lane_votes<8>(tile, deg, mine, i, tw, s_res);
-                    else if (deg <= 12) lane_votes<12>(tile, deg, mine, i, tw, s_res);
-                    else if (deg <= 16) lane_votes<16>(tile, deg, mine, i, tw, s_res);
-                    else if (deg <= 20) lane_votes<20>(tile, deg, mine, i, tw, s_res);
-                    else if (deg <= 24) lane_votes<24>(tile, deg, mine, i, tw, s_res);
-                    else if (deg <= 28) lane_votes<28>(tile, deg, mine, i, tw, s_res);
-                    else lane_votes<32>(tile, deg, mine, i, tw, s_res);
-                    rest = 0;
-                }
-                if (deg <= kTileRows) {
-                    // Exact vote by the whole warp (lane = neighbour), two
-                    // unresolved pairs at a time as independent chains.
-                    const unsigned lt = (1u << lane) - 1u;
-                    const bool nb = lane < deg;
-                    const int pad = (int)(0x80000000u | (unsigned)lane);  // distinct, never a label
-                    while (rest) {
-                        const int la = __ffs(rest) - 1;
-                        rest &= rest - 1;
-                        const bool two = rest != 0u;
-                        const int lb = two ? __ffs(rest) - 1 : la;
-                        if (two) rest &= rest - 1;
-                        const int ia = __shfl_sync(kFull, i, la);
-                        const int ib = __shfl_sync(kFull, i, lb);
-                        const int xa = nb ? tile[lane * kTileStride + la] : pad;
-                        const int xb = (nb && two) ? tile[lane * kTileStride + lb] : pad;
-                        const unsigned pa = __match_any_sync(kFull, xa);
-                        const unsigned pb = __match_any_sync(kFull, xb);
-                        const unsigned ca = nb ? (unsigned)__popc(pa) : 0u;
-                        const unsigned cb = nb ? (unsigned)__popc(pb) : 0u;
-                        const unsigned ma = __reduce_max_sync(kFull, ca);
-                        const unsigned mb = __reduce_max_sync(kFull, cb);
-                        const unsigned da = __ballot_sync(kFull, ca == ma && (pa & lt) == 0u);
-                        const unsigned db = __ballot_sync(kFull, cb == mb && (pb & lt) == 0u);
-                        const uint32_t ua = __shfl_sync(kFull, word_of(tw, ia & 3), ia >> 2);
-                        const uint32_t ub = __shfl_sync(kFull, word_of(tw, ib & 3), ib >> 2);
-                        const int ta = __popc(da), tb = __popc(db);
-                        const unsigned ka = ta > 1 ? pick_index(ua, (uint32_t)ta) : 0u;
-                        const unsigned kb = (two && tb > 1) ? pick_index(ub, (uint32_t)tb) : 0u;
-                        int ra, rb;
-                        if (ka > kRemovalMax || kb > kRemovalMax) {
-                            // The tied labels are distinct (one leader per label):
-                            // sorted ascending, with the other lanes last, the
-                            // k-th tied label sits in lane k.
-                            unsigned va = ((da >> lane) & 1u) ? (unsigned)xa : 0xffffffffu;
-                            unsigned vb = (two && ((db >> lane) & 1u)) ? (unsigned)xb : 0xffffffffu;
-                            warp_sort32x2(va, vb);
-                            ra = (int)__shfl_sync(kFull, va, (int)ka);
-                            rb = (int)__shfl_sync(kFull, vb, (int)kb);
-                        } else {
-                            int sa = __ffs(da) - 1, sb = __ffs(db) - 1;
-                            if (ta > 1 || (two && tb > 1)) select_kth_lane2(da, xa, ka, two ? db : 0u, xb, kb, sa, sb);
-                            if (!two) sb = 0;
-                            ra = __shfl_sync(kFull, xa, sa);
-                            rb = __shfl_sync(kFull, xb, sb);
-                        }
-                        if (lane == 0) {
-                            s_res[ia] = ra;
-                            if (two) s_res[ib] = rb;
-                        }
-                    }
-                }
-                // Degree > kDeferMax: a shared count table, one pair at a time.
-                while (rest) {
-                    const int l = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    const int ic = __shfl_sync(kFull, i, l);
-                    const uint32_t u = __shfl_sync(kFull, word_of(tw, ic & 3), ic >> 2);
-                    unsigned mx = 0;
-                    const int lab = warp_mode_table(gp, child, col_idx, beg, deg, tile + l, ic, hkey, hcnt, u, mx);
-                    if (lane == 0) s_res[ic] = lab;
-                    nsettle += 4 * (int)mx > deg ? 1 : 0;
-                }
-                __syncwarp();
+            continue;
+        }
+        const int idx0 = first + (item - wide) * batch;
+        const int nb = min(batch, gp.n - idx0);
+        int4 rec = make_int4(0, 0, 0, 0);
+        if (lane < nb) {
+            rec = __ldg(nodes + idx0 + lane);
+            const bool fast = rec.z <= kLaneMax ? lane_fast : own_label_pays(hint[idx0 + lane]);
+            recs[lane] = make_int4(rec.x, rec.y, rec.z, fast ? rec.z : 0);  // .w: degree if the count pays
+            oks[lane] = 0;
+        }
+        int total = 0, nsel = 0;
+        int v = __shfl_sync(kFull, rec.x, 0);
+        int4 nxt = active ? C4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
+        for (int k = 0; k < nb; ++k) {
+            const int deg = __shfl_sync(kFull, rec.z, k);
+            const int4 out = nxt;
+            const int cur = v;
+            if (k + 1 < nb) {  // the next row is requested before this one is processed
+                v = __shfl_sync(kFull, rec.x, k + 1);
+                if (active) nxt = C4[(size_t)v * nq + lane];
             }
-            __syncwarp();
-            // The deferred pairs add theirs in mutation_vote_kernel.
-            if (lane == 0 && deg > kTileRows) hint[v] = ((uint32_t)nsel << 16) | (uint32_t)nsettle;
-            // s_res holds the unselected children's labels and the results.
-            if (active) out = reinterpret_cast<const int4 *>(s_res)[lane];
-            __syncwarp();
+            const int c = take_row(gp, cur, deg, active, out, lane, g, Q4, hist, list, total, k << 7);
+            nsel = lane == k ? c : nsel;
+            total += c;
         }
-        if (active) {
-            Q4[(size_t)v * nq + lane] = out;
-            // D of the evaluation's degree histogram: every child's final label
-            // of v gets deg(v) (label-major cell label * W + child). The old
-            // value is not needed, so these are reductions that do not stall.
-            // A deferred pair (-1) gets its label and its addition from
-            // mutation_vote_kernel.
-            if (deg > 0) {
-                const int i0 = 4 * lane;
-                const unsigned d = (unsigned)deg;
-                if (i0 + 0 < np && out.x >= 0 && MOCD_CHECK(out.x < gp.n, kCheckLabel, v))
-                    atomicAdd(hist + (size_t)out.x * W + i0 + 0, d);
-                if (i0 + 1 < np && out.y >= 0 && MOCD_CHECK(out.y < gp.n, kCheckLabel, v))
-                    atomicAdd(hist + (size_t)out.y * W + i0 + 1, d);
-                if (i0 + 2 < np && out.z >= 0 && MOCD_CHECK(out.z < gp.n, kCheckLabel, v))
-                    atomicAdd(hist + (size_t)out.z * W + i0 + 2, d);
-                if (i0 + 3 < np && out.w >= 0 && MOCD_CHECK(out.w < gp.n, kCheckLabel, v))
-                    atomicAdd(hist + (size_t)out.w * W + i0 + 3, d);
+        __syncwarp();
+
+        // The own label's count; open pairs are compacted to the list's front.
+        int open = 0, settled32 = 0;
+        const bool any_fast = __any_sync(kFull, lane < nb && recs[lane < nb ? lane : 0].w != 0);
+        if (!any_fast) open = total;
+        for (int base = 0; any_fast && base < total; base += 32) {
+            const bool has = base + lane < total;
+            const int e = has ? list[base + lane] : 0;
+            const int i = e & 127;
+            const int4 r = recs[e >> 7];
+            const int32_t *col = child + i;
+            const int own = has ? col[(size_t)r.x * W] : 0;
+            const int n4 = has ? (r.w + 3) >> 2 : 0;  // groups of four neighbours to count
+            const int n4_max = __reduce_max_sync(kFull, n4);
+            int c = 0;
+            for (int j = 0; j < n4_max; j += 2) {
+                const bool p0 = j < n4, p1 = j + 1 < n4;
+                const int4 u0 = p0 ? __ldg(adj + r.y + j) : make_int4(0, 0, 0, 0);
+                const int4 u1 = p1 ? __ldg(adj + r.y + j + 1) : make_int4(0, 0, 0, 0);
+                int x[8];
+                x[0] = p0 ? col[(size_t)checked_node(u0.x, gp.n) * W] : -1;
+                x[1] = p0 ? col[(size_t)checked_node(u0.y, gp.n) * W] : -1;
+                x[2] = p0 ? col[(size_t)checked_node(u0.z, gp.n) * W] : -1;
+                x[3] = p0 ? col[(size_t)checked_node(u0.w, gp.n) * W] : -1;
+                x[4] = p1 ? col[(size_t)checked_node(u1.x, gp.n) * W] : -1;
+                x[5] = p1 ? col[(size_t)checked_node(u1.y, gp.n) * W] : -1;
+                x[6] = p1 ? col[(size_t)checked_node(u1.z, gp.n) * W] : -1;
+                x[7] = p1 ? col[(size_t)checked_node(u1.w, gp.n) * W] : -1;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) c += x[t] == own;
             }
+            const bool ok = has && 2 * c > r.z;
+            if (ok) {
+                add_degree(gp, hist, own, i, r.z);
+                if (r.z > kLaneMax) atomicAdd(oks + (e >> 7), 1);
+            }
+            settled32 += __popc(__ballot_sync(kFull, ok && r.z <= kLaneMax));
+            const unsigned rest = __ballot_sync(kFull, has && !ok);
+            __syncwarp();
+            if (has && !ok) list[open + __popc(rest & lt)] = (unsigned short)e;
+            open += __popc(rest);
         }
+        __syncwarp();
+
+        // The exact votes of the open pairs (degrees still descending).
+        int pairs32 = settled32;
+        for (int base = 0; base < open; base += 32) {
+            const bool has = base + lane < open;
+            const int e = has ? list[base + lane] : 0;
+            const int i = e & 127;
+            int4 r = recs[e >> 7];
+            const unsigned big = __ballot_sync(kFull, has && r.z > kLaneMax);
+            if (big) {
+                const unsigned far = __ballot_sync(kFull, has && r.z > 2 * kLaneMax);
+                if (far) defer_pairs(gp, 1, far, idx0 + (e >> 7), i, lane, dlist, dcount);
+                if (big & ~far) defer_pairs(gp, 0, big & ~far, idx0 + (e >> 7), i, lane, dlist, dcount);
+            }
+            const bool mine = has && r.z <= kLaneMax;
+            const int deg = mine ? r.z : 0;
+            const int top = __reduce_max_sync(kFull, deg);
+            if (top == 0) continue;
+            int res, best;
+            if (top <= 8) res = lane_vote<8>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else if (top <= 12) res = lane_vote<12>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else if (top <= 16) res = lane_vote<16>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else if (top <= 20) res = lane_vote<20>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else if (top <= 24) res = lane_vote<24>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else if (top <= 28) res = lane_vote<28>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            else res = lane_vote<32>(gp, adj, child, r.x, i, r.y, deg, g, best);
+            bool same = false;
+            if (mine) {
+                const size_t cell = (size_t)r.x * W + i;
+                same = res == child[cell];
+                if (!same) q[cell] = res;
+                add_degree(gp, hist, res, i, deg);
+            }
+            pairs32 += __popc(__ballot_sync(kFull, mine));
+            settled32 += __popc(__ballot_sync(kFull, mine && same && r.w == 0 && 2 * best > deg));
+        }
+        // The history: per node above kLaneMax, a sample of the batches below
+        // (the deferred pairs add theirs in mutation_vote_kernel).
+        if (lane < nb && rec.z > kLaneMax) hint[idx0 + lane] = ((uint32_t)nsel << 16) | (uint32_t)oks[lane];
+        if (((item - wide) & 7) == 0 && lane == 0 && pairs32 > 0) {
+            atomicAdd(dcount + kDcountPairs, pairs32);
+            atomicAdd(dcount + kDcountOk, settled32);
+        }
+        __syncwarp();
     }
 }
 
 // The exact neighbour-majority of one deferred pair (node of degree
-// kTileRows + 1 .. N) per thread: the pair's labels are gathered into
-// registers (INT_MAX beyond the degree), sorted by the odd-even merge
-// network, and the pick(u, t)-th of the t longest runs is the result, u the
-// MTIE word. The thread writes the label into Q, adds deg(v) to the degree
-// histogram (as the mutation kernel does for the other pairs) and, when the
-// best count c has (K + 1) c > deg (K the counters of the node's Misra-Gries
-// pass: 1 for degree <= 64, else 3), counts the pair in v's hint.
+// kLaneMax + 1 .. N) per thread: the pair's labels are gathered into
+// registers, sorted by the merge-exchange network, and the pick(u, t)-th of
+// the t longest runs is the result, u the MTIE word. The thread writes the
+// label into Q, adds deg(v) to the degree histogram and, when the own label is
+// on more than half of the neighbours, counts the pair in the node's hint.
 template <int N>
-__device__ __forceinline__ void mutation_vote_body(const GenParams gp, int cls, const int32_t *__restrict__ row_ptr,
-                                                   const int32_t *__restrict__ col_idx,
-                                                   const int32_t *__restrict__ child, int32_t *__restrict__ q,
-                                                   const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist,
-                                                   uint32_t *__restrict__ hint, const int2 *__restrict__ dlist,
-                                                   const int *__restrict__ dcount, int vblock, int vgrid)
+__device__ __forceinline__ void mutation_vote_body(const GenParams &gp, int cls, const int4 *__restrict__ nodes,
+                                                   const int4 *__restrict__ adj, const int32_t *__restrict__ child,
+                                                   int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr,
+                                                   uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
+                                                   const int2 *__restrict__ dlist, const int *__restrict__ dcount,
+                                                   int vblock, int vgrid)
 {
     constexpr int NW = (N + 63) / 64;
     const uint32_t g = *gen_ptr;
@@ -1155,16 +1025,23 @@ __device__ __forceinline__ void mutation_vote_body(const GenParams gp, int cls, 
     const int2 *list = dlist + defer_offset(gp, cls);
     for (int t = vblock * blockDim.x + threadIdx.x; t < total; t += vgrid * blockDim.x) {
         const int2 e = list[t];
-        const int v = e.x, i = e.y;
-        if (!MOCD_CHECK(v >= 0 && v < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;
-        const int beg = __ldg(row_ptr + v);
-        const int deg = min(__ldg(row_ptr + v + 1) - beg, N);
+        const int i = e.y;
+        if (!MOCD_CHECK(e.x >= 0 && e.x < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;
+        const int4 rec = __ldg(nodes + e.x);
+        const int v = rec.x, deg = min(rec.z, N);
+        const int32_t *col = child + i;
         int x[N];
 #pragma unroll
-        for (int j = 0; j < N; ++j)
-            x[j] = j < deg ? child[(size_t)checked_node(__ldg(col_idx + beg + j), gp.n) * W + i] : INT_MAX;
+        for (int j = 0; j < N; j += 4) {
+            const bool in = j < deg;
+            const int4 u = in ? __ldg(adj + rec.y + j / 4) : make_int4(0, 0, 0, 0);
+            x[j + 0] = in ? col[(size_t)checked_node(u.x, gp.n) * W] : INT_MAX;
+            x[j + 1] = in ? col[(size_t)checked_node(u.y, gp.n) * W] : INT_MAX;
+            x[j + 2] = in ? col[(size_t)checked_node(u.z, gp.n) * W] : INT_MAX;
+            x[j + 3] = in ? col[(size_t)checked_node(u.w, gp.n) * W] : INT_MAX;
+        }
         sort_network<N>(x);
-        // Runs of equal labels as in lane_pick, over NW 64-bit words: bit j
+        // Runs of equal labels as in longest_runs, over NW 64-bit words: bit j
         // of eq is set when entries j and j + 1 (< deg) are equal; each step
         // m &= m >> 1 (across words) shortens every run of set bits by one,
         // and the last non-zero m marks the first entry of each longest run.
@@ -1199,11 +1076,7 @@ __device__ __forceinline__ void mutation_vote_body(const GenParams gp, int cls, 
 #pragma unroll
         for (int w = 0; w < NW; ++w) tcount += __popcll(starts[w]);
         unsigned kk = 0;
-        if (tcount > 1) {
-            const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)(i >> 2), g, kStageMutTie), gp.key0,
-                                          gp.key1);
-            kk = pick_index(word_of(r, i & 3), (uint32_t)tcount);
-        }
+        if (tcount > 1) kk = pick_index(tie_word(gp, v, i, g), (uint32_t)tcount);
         // Position of the kk-th set bit of the starts mask.
         int pos = 0;
         unsigned k = kk;
@@ -1232,21 +1105,21 @@ __device__ __forceinline__ void mutation_vote_body(const GenParams gp, int cls, 
             break;
         }
         const int res = select_at<N>(x, pos);
-        q[(size_t)v * W + i] = res;
-        if (MOCD_CHECK(res >= 0 && res < gp.n, kCheckLabel, v)) atomicAdd(hist + (size_t)res * W + i, (unsigned)deg);
-        if ((N <= 2 * kTileRows ? 2 : 4) * best > deg) atomicAdd(hint + v, 1u);
+        const size_t cell = (size_t)v * W + i;
+        q[cell] = res;
+        add_degree(gp, hist, res, i, deg);
+        if (2 * best > deg && res == child[cell]) atomicAdd(hint + e.x, 1u);
     }
 }
 
 template <int N>
 __global__ void __launch_bounds__(kMutBlock)
-mutation_vote_kernel(GenParams gp, int cls, const int32_t *__restrict__ row_ptr,
-                     const int32_t *__restrict__ col_idx, const int32_t *__restrict__ child,
-                     int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist,
-                     uint32_t *__restrict__ hint, const int2 *__restrict__ dlist, const int *__restrict__ dcount)
+mutation_vote_kernel(const __grid_constant__ GenParams gp, int cls, const int4 *__restrict__ nodes,
+                     const int4 *__restrict__ adj, const int32_t *__restrict__ child, int32_t *__restrict__ q,
+                     const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
+                     const int2 *__restrict__ dlist, const int *__restrict__ dcount)
 {
-    mutation_vote_body<N>(gp, cls, row_ptr, col_idx, child, q, gen_ptr, hist, hint, dlist, dcount, blockIdx.x,
-                          gridDim.x);
+    mutation_vote_body<N>(gp, cls, nodes, adj, child, q, gen_ptr, hist, hint, dlist, dcount, blockIdx.x, gridDim.x);
 }
 
 // The deferred votes of one degree class of every member of a batch.
@@ -1260,43 +1133,148 @@ mutation_vote_multi_kernel(const BatchMember *__restrict__ members, const int *_
     const int k = member_of_block(starts, count);
     const BatchMember &mb = members[k];
     const PopState &ps = mb.ps;
+    const GenParams gp = mb.gp;
     const int b0 = __ldg(starts + k);
-    mutation_vote_body<N>(mb.gp, cls, mb.row_ptr, mb.col_idx, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist,
-                          ps.dcount, (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
+    mutation_vote_body<N>(gp, cls, mb.nodes, mb.adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist, ps.dcount,
+                          (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
 }
 
-// The listed votes of hubs above kSharedTableMax: a warp per pair, its count
-// table in the warp's slice of the global scratch (2 gp.hub_hs ints). Writes
-// the label into Q, adds deg(v) to the histogram and counts the pair in v's
-// hint when its best count c has 4 c > deg.
-__global__ void __launch_bounds__(kMutBlock)
-mutation_hub_kernel(GenParams gp, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                    const int32_t *__restrict__ child, int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr,
-                    uint32_t *__restrict__ hist, uint32_t *__restrict__ hint, const int2 *__restrict__ dlist,
-                    const int *__restrict__ dcount, int *__restrict__ hub_table)
+// Sum (or maximum) over the hub block; every thread gets it. s_red holds one
+// word per warp; the trailing barrier frees it for the next call.
+template <bool MAX>
+__device__ __forceinline__ unsigned hub_reduce(unsigned x, unsigned *s_red)
 {
+    x = MAX ? __reduce_max_sync(kFull, x) : __reduce_add_sync(kFull, x);
+    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = x;
+    __syncthreads();
+    unsigned r = 0;
+#pragma unroll
+    for (int w = 0; w < kHubBlock / 32; ++w) r = MAX ? max(r, s_red[w]) : r + s_red[w];
+    __syncthreads();
+    return r;
+}
+
+// The listed pairs of hubs above kSharedTableMax, a block each: the own
+// label's count if the node's history says it pays, else (or if it leaves the
+// pair open) the exact vote with a count table of the smallest power of two
+// >= 2 deg slots, in shared memory if it fits there (gp.hub_smem_hs), else in
+// the block's slice of global scratch (2 gp.hub_hs ints). Writes the label
+// into Q, adds deg(v) to the histogram and counts the pair in the hub's hint
+// when its own label is on more than half of the neighbours. A block per pair
+// keeps a hub of thousands of neighbours off the critical path: one warp per
+// pair is a chain of deg / 32 dependent table inserts.
+__global__ void __launch_bounds__(kHubBlock)
+mutation_hub_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict__ nodes,
+                    const int4 *__restrict__ adj, const int32_t *__restrict__ child, int32_t *__restrict__ q,
+                    const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
+                    const int2 *__restrict__ dlist, const int *__restrict__ dcount, int *__restrict__ hub_table)
+{
+    extern __shared__ int s_table[];  // [2 gp.hub_smem_hs]
+    __shared__ unsigned s_red[kHubBlock / 32];
+    __shared__ int s_tied, s_res;
     const uint32_t g = *gen_ptr;
     const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    int *hkey = hub_table + (size_t)warp * 2 * gp.hub_hs;
-    int *hcnt = hkey + gp.hub_hs;
     const int total = min(dcount[2], defer_capacity(gp, 2));
     const int2 *list = dlist + defer_offset(gp, 2);
-    for (int t = warp; t < total; t += nwarps) {
+    for (int t = blockIdx.x; t < total; t += gridDim.x) {
         const int2 e = list[t];
-        const int v = e.x, i = e.y;
-        if (!MOCD_CHECK(v >= 0 && v < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;  // (warp-uniform)
-        const int beg = __ldg(row_ptr + v);
-        const int deg = min(__ldg(row_ptr + v + 1) - beg, gp.hub_hs / 2);
-        const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)(i >> 2), g, kStageMutTie), gp.key0, gp.key1);
-        unsigned mx = 0;
-        const int lab = warp_mode_table(gp, child, col_idx, beg, deg, nullptr, i, hkey, hcnt, word_of(r, i & 3), mx);
-        if (lane == 0) {
-            q[(size_t)v * gp.W + i] = lab;
-            if (MOCD_CHECK(lab >= 0 && lab < gp.n, kCheckLabel, v)) atomicAdd(hist + (size_t)lab * gp.W + i, (unsigned)deg);
-            if (4 * (int)mx > deg) atomicAdd(hint + v, 1u);
+        const int idx = e.x & ~kHubFast, i = e.y;
+        if (!MOCD_CHECK(idx >= 0 && idx < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;  // (block-uniform)
+        const int4 rec = __ldg(nodes + idx);
+        const int v = rec.x, deg = min(rec.z, gp.hub_hs / 2);
+        const int *nbr = reinterpret_cast<const int *>(adj + rec.y);
+        const int32_t *col = child + i;
+        const size_t cell = (size_t)v * gp.W + i;
+        const int own = child[cell];
+        if (e.x & kHubFast) {
+            unsigned c = 0;
+#pragma unroll 4
+            for (int j = threadIdx.x; j < deg; j += kHubBlock)
+                c += col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] == own ? 1u : 0u;
+            if (2 * (int)hub_reduce<false>(c, s_red) > deg) {  // (Q holds the own label already)
+                if (threadIdx.x == 0) {
+                    add_degree(gp, hist, own, i, deg);
+                    atomicAdd(hint + idx, 1u);
+                }
+                continue;
+            }
         }
+        int hbits = 11;
+        while ((1 << hbits) < 2 * deg) ++hbits;
+        const int HS = 1 << hbits;
+        int *hkey = HS <= gp.hub_smem_hs ? s_table : hub_table + (size_t)blockIdx.x * 2 * gp.hub_hs;
+        int *hcnt = hkey + HS;
+        for (int s = threadIdx.x; s < HS; s += kHubBlock) {
+            hkey[s] = -1;
+            hcnt[s] = 0;
+        }
+        if (threadIdx.x == 0) s_tied = 0;
+        __syncthreads();
+        for (int j0 = 0; j0 < deg; j0 += kHubBlock) {
+            const int j = j0 + threadIdx.x;
+            const bool in = j < deg;
+            const int x = in ? col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] : (int)(0x80000000u | lane);
+            // One insert per distinct label of the warp's neighbours.
+            const unsigned peers = __match_any_sync(kFull, x);
+            if (in && (peers & ((1u << lane) - 1u)) == 0) {
+                uint32_t h = hash_slot(x, hbits);
+                for (int probe = 0; probe < HS; ++probe) {  // (at most HS / 2 distinct labels: a slot is found)
+                    const int prev = atomicCAS(hkey + h, -1, x);
+                    if (prev == -1 || prev == x) {
+                        atomicAdd(hcnt + h, __popc(peers));
+                        break;
+                    }
+                    h = (h + 1) & (uint32_t)(HS - 1);
+                }
+            }
+        }
+        __syncthreads();
+        unsigned my = 0;
+        for (int s = threadIdx.x; s < HS; s += kHubBlock) my = max(my, (unsigned)hcnt[s]);
+        const unsigned mx = hub_reduce<true>(my, s_red);
+        // The tied labels, compacted to hcnt[0, tied) once every thread has
+        // read its slots' counts.
+        for (int s = threadIdx.x; s < HS; s += kHubBlock)
+            if ((unsigned)hcnt[s] != mx) hkey[s] = -1;
+        __syncthreads();
+        for (int s = threadIdx.x; s < HS; s += kHubBlock) {  // (HS is a multiple of the block: warps stay whole)
+            const int key = hkey[s];
+            const unsigned who = __ballot_sync(kFull, key >= 0);
+            int at = 0;
+            if (lane == 0 && who) at = atomicAdd(&s_tied, __popc(who));
+            at = __shfl_sync(kFull, at, 0);
+            if (key >= 0) hcnt[at + __popc(who & ((1u << lane) - 1u))] = key;
+        }
+        __syncthreads();
+        const int tied = s_tied;
+        if (tied == 1) {
+            if (threadIdx.x == 0) s_res = hcnt[0];
+        } else {
+            // Bit by bit from the top, as in warp_mode_table.
+            unsigned prefix = 0, rank = pick_index(tie_word(gp, v, i, g), (uint32_t)tied);
+            for (int b = gp.label_bits - 1; b >= 0; --b) {
+                const unsigned above = ~((2u << b) - 1u);  // the bits above b
+                unsigned c = 0;
+                for (int s = threadIdx.x; s < tied; s += kHubBlock) {
+                    const unsigned key = (unsigned)hcnt[s];
+                    c += ((key & above) == prefix && ((key >> b) & 1u) == 0u) ? 1u : 0u;
+                }
+                const unsigned cnt = hub_reduce<false>(c, s_red);
+                if (rank >= cnt) {
+                    rank -= cnt;
+                    prefix |= 1u << b;
+                }
+            }
+            if (threadIdx.x == 0) s_res = (int)prefix;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int lab = s_res;
+            q[cell] = lab;
+            add_degree(gp, hist, lab, i, deg);
+            if (lab == own && 2 * (int)mx > deg) atomicAdd(hint + idx, 1u);
+        }
+        __syncthreads();
     }
 }
 
@@ -1370,7 +1348,7 @@ cudaError_t launch_vote_multi(const BatchMember *members, const int *starts, int
 {
     if (blocks <= 0) return cudaSuccess;
     if (cls == 0)
-        mutation_vote_multi_kernel<2 * kTileRows><<<blocks, kMutBlock, 0, s>>>(members, starts, count, 0);
+        mutation_vote_multi_kernel<2 * kLaneMax><<<blocks, kMutBlock, 0, s>>>(members, starts, count, 0);
     else
         mutation_vote_multi_kernel<kDeferMax><<<blocks, kMutBlock, 0, s>>>(members, starts, count, 1);
     return cudaGetLastError();
@@ -1378,7 +1356,7 @@ cudaError_t launch_vote_multi(const BatchMember *members, const int *starts, int
 
 int mutation_smem(int hash_size)
 {
-    return (kMutBlock / 32) * (2 * kMaxPop + kTileRows * kTileStride + 2 * hash_size) * (int)sizeof(int);
+    return (kMutBlock / 32) * 2 * hash_size * (int)sizeof(int);
 }
 
 int mutation_warps_per_block()
@@ -1386,16 +1364,27 @@ int mutation_warps_per_block()
     return kMutBlock / 32;
 }
 
-int grid_for_mutation(int sms, int hash_size, int *smem_bytes)
+int grid_for_mutation(int sms, int hash_size)
 {
     const int smem = mutation_smem(hash_size);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(mutation_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_kernel, kMutBlock, smem);
-    if (per_sm < 1) per_sm = 1;
-    *smem_bytes = smem;
-    return sms * per_sm;
+    if (hash_size > 0) {
+        cudaFuncSetAttribute(mutation_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_kernel<true>, kMutBlock, smem);
+    } else {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_kernel<false>, kMutBlock, 0);
+    }
+    return sms * (per_sm < 1 ? 1 : per_sm);
+}
+
+// Blocks of the hub kernel: as many as its shared table lets be resident.
+int grid_for_hubs(int sms, int smem_hs)
+{
+    const int smem = 2 * smem_hs * (int)sizeof(int);
+    cudaFuncSetAttribute(mutation_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_hub_kernel, kHubBlock, smem);
+    return sms * (per_sm < 1 ? 1 : per_sm);
 }
 
 void grid_for_votes(int sms, int vote_n0, int *grid64, int *grid128)
@@ -1406,54 +1395,55 @@ void grid_for_votes(int sms, int vote_n0, int *grid64, int *grid128)
     case 48: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<48>, kMutBlock, 0); break;
     case 56: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<56>, kMutBlock, 0); break;
     default:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<2 * kTileRows>, kMutBlock, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<2 * kLaneMax>, kMutBlock, 0);
     }
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, mutation_vote_kernel<kDeferMax>, kMutBlock, 0);
     *grid64 = sms * (a < 1 ? 1 : a);
     *grid128 = sms * (b < 1 ? 1 : b);
 }
 
-cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int32_t *row_ptr,
-                            const int32_t *col_idx, const int32_t *order, int grid, int grid64, int grid128,
-                            cudaStream_t s, bool with_votes)
+namespace {
+
+template <int N>
+void launch_vote(const GenParams &gp, const PopState &ps, int cls, const int4 *nodes, const int4 *adj, int grid,
+                 cudaStream_t s)
 {
-    mutation_kernel<<<grid, kMutBlock, mutation_smem(gp.hash_size), s>>>(gp, row_ptr, col_idx, order, ps.c, ps.q,
-                                                                       ps.gen, ps.hist, ps.acc, ps.hint, ps.dlist,
-                                                                       ps.dcount);
+    mutation_vote_kernel<N><<<grid, kMutBlock, 0, s>>>(gp, cls, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint,
+                                                       ps.dlist, ps.dcount);
+}
+
+}  // namespace
+
+cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj, int batch,
+                            int grid, int grid64, int grid128, cudaStream_t s, bool with_votes)
+{
+    if (gp.hash_size > 0)
+        mutation_kernel<true><<<grid, kMutBlock, mutation_smem(gp.hash_size), s>>>(
+            gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.acc, ps.hint, ps.dlist, ps.dcount, batch);
+    else
+        mutation_kernel<false><<<grid, kMutBlock, 0, s>>>(gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.acc, ps.hint,
+                                                          ps.dlist, ps.dcount, batch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (with_votes && gp.defer_cap[0] > 0) {
         // The class's network holds the graph's largest degree in it.
         switch (gp.vote_n0) {
-        case 40:
-            mutation_vote_kernel<40><<<grid64, kMutBlock, 0, s>>>(gp, 0, row_ptr, col_idx, ps.c, ps.q, ps.gen,
-                                                                  ps.hist, ps.hint, ps.dlist, ps.dcount);
-            break;
-        case 48:
-            mutation_vote_kernel<48><<<grid64, kMutBlock, 0, s>>>(gp, 0, row_ptr, col_idx, ps.c, ps.q, ps.gen,
-                                                                  ps.hist, ps.hint, ps.dlist, ps.dcount);
-            break;
-        case 56:
-            mutation_vote_kernel<56><<<grid64, kMutBlock, 0, s>>>(gp, 0, row_ptr, col_idx, ps.c, ps.q, ps.gen,
-                                                                  ps.hist, ps.hint, ps.dlist, ps.dcount);
-            break;
-        default:
-            mutation_vote_kernel<2 * kTileRows><<<grid64, kMutBlock, 0, s>>>(gp, 0, row_ptr, col_idx, ps.c, ps.q,
-                                                                               ps.gen, ps.hist, ps.hint, ps.dlist,
-                                                                               ps.dcount);
+        case 40: launch_vote<40>(gp, ps, 0, nodes, adj, grid64, s); break;
+        case 48: launch_vote<48>(gp, ps, 0, nodes, adj, grid64, s); break;
+        case 56: launch_vote<56>(gp, ps, 0, nodes, adj, grid64, s); break;
+        default: launch_vote<2 * kLaneMax>(gp, ps, 0, nodes, adj, grid64, s);
         }
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (with_votes && gp.defer_cap[1] > 0) {
-        mutation_vote_kernel<kDeferMax><<<grid128, kMutBlock, 0, s>>>(gp, 1, row_ptr, col_idx, ps.c, ps.q, ps.gen,
-                                                                        ps.hist, ps.hint, ps.dlist, ps.dcount);
+        launch_vote<kDeferMax>(gp, ps, 1, nodes, adj, grid128, s);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     if (gp.defer_cap[2] > 0) {
-        mutation_hub_kernel<<<gp.hub_warps / (kMutBlock / 32), kMutBlock, 0, s>>>(
-            gp, row_ptr, col_idx, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist, ps.dcount, ps.hub_table);
+        mutation_hub_kernel<<<gp.hub_blocks, kHubBlock, 2 * gp.hub_smem_hs * sizeof(int), s>>>(
+            gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist, ps.dcount, ps.hub_table);
         e = cudaGetLastError();
     }
     return e;

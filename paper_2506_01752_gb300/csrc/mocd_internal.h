@@ -36,14 +36,27 @@ bool inject_failure(int site, int *status);
 constexpr int kMaxPop = 128;      // N_p limit: one int4 of labels per lane per row
 constexpr int kMaxParents = 16;   // E_S limit
 constexpr int kBlock = 256;       // threads per block of the node-parallel kernels
-// Mutation votes of nodes with degree 33..kDeferMax that the Misra-Gries
-// pass leaves open run one pair per thread in a second kernel (degree
-// classes 33..64 and 65..128); higher degrees use a per-warp count table.
+// Mutation votes of nodes with degree 33..kDeferMax that the own label's count
+// leaves open run one pair per thread in a second kernel (degree classes
+// 33..64 and 65..128).
 constexpr int kDeferMax = 128;
-// Above this degree a node's count table no longer fits in shared memory:
-// its open pairs are listed for mutation_hub_kernel, which keeps the table of
-// each pair in a per-warp slice of global scratch.
+// Up to this degree a pair's vote is a warp's, with a count table in shared
+// memory; above it a block's (mutation_hub_kernel).
 constexpr int kSharedTableMax = 512;
+// Warps that share the pairs of a node of degree kDeferMax + 1 ..
+// kSharedTableMax (label quads q with q % kWideParts equal).
+constexpr int kWideParts = 8;
+// Largest count table of the hub kernel in shared memory (slots of 8 bytes).
+constexpr int kHubSmemSlots = 16384;
+// Set in the node of a listed hub pair when the own label's count is to be
+// tried first (node positions are below 2^30).
+constexpr int kHubFast = 1 << 30;
+// Words of PopState::dcount: [0, 3) deferred pairs per class, then the sampled
+// pairs of degree <= 32, those of them whose own label was on more than half
+// of the neighbours, and whether the next generation counts it first.
+constexpr int kDcountPairs = 3;
+constexpr int kDcountOk = 4;
+constexpr int kDcountFast = 5;
 
 // Random stream stages (third word of the Philox counter is the generation).
 constexpr uint32_t kStageInit = 1;
@@ -69,11 +82,12 @@ struct PopState {
     int32_t *front;           // [2 + kMaxPop]: count, best, members (P positions)
     int64_t *fint;            // [2][kMaxPop]: intra, S of each front member
     double *fval;             // [2][kMaxPop]: f1, f2 of each front member
-    uint32_t *hint;           // [n]: (mutating pairs << 16) | pairs the Misra-Gries pass settles (a label above
-                              // deg / (K + 1), K its counters), last generation; nodes of degree > 32
-    int2 *dlist;              // deferred mutation votes (node, child): class 0 then class 1
-    int *dcount;              // [3]: deferred votes appended this generation: degree 33..64, 65..128, hubs
-    int *hub_table;           // hub_warps x 2 hub_hs: per-warp count tables of the hub votes
+    uint32_t *hint;           // (mutating pairs << 16) | pairs whose own label is on more than half of the
+                              // neighbours, last generation: [n] by position in the order (degree > 32), then
+                              // kWideParts per node of degree kDeferMax + 1 .. kSharedTableMax
+    int2 *dlist;              // deferred mutation votes (node position, child): class 0, 1, then hubs
+    int *dcount;              // [6]: see kDcountPairs
+    int *hub_table;           // hub_blocks x 2 hub_hs: count tables of hubs too large for shared memory
 };
 
 struct GenParams {
@@ -83,9 +97,11 @@ struct GenParams {
     int es;                   // E_S
     int label_bits;           // bits needed for a label in [0, n)
     int hash_size;            // per-warp hash entries for degree > kDeferMax (0: none)
+    int n_hub, n_wide;        // nodes of degree > kSharedTableMax, and of kDeferMax + 1 .. kSharedTableMax
     int defer_cap[3];         // deferred-vote capacity per class: N_p x nodes of the class
-    int hub_hs;               // slots of a hub count table (power of two >= 2 dmax; 0: no hubs)
-    int hub_warps;            // warps of mutation_hub_kernel (one table slice each)
+    int hub_hs;               // slots of the largest hub's count table (power of two >= 2 dmax; 0: no hubs)
+    int hub_smem_hs;          // slots of the hub kernel's shared table (<= kHubSmemSlots)
+    int hub_blocks;           // blocks of mutation_hub_kernel
     int vote_n0;              // entries of the degree 33..64 vote's sorting network: the smallest multiple
                               // of 8 that holds the graph's largest degree in that class (40, 48, 56 or 64)
     int64_t m;                // edges
@@ -102,6 +118,8 @@ struct BatchMember {
     const int32_t *row_ptr;
     const int32_t *col_idx;
     const int32_t *order;
+    const int4 *nodes;    // the mutation's node records and adjacency (mocd_ctx::d_nodes / d_adj)
+    const int4 *adj;
     const int32_t *eptr;  // the offspring evaluation's oriented adjacency (mocd_ctx::d_eptr / d_eidx)
     const int32_t *eidx;
 };
@@ -116,9 +134,9 @@ cudaError_t launch_crossover(const GenParams &gp, const PopState &ps, int grid, 
 // (degree descending), or NULL for 0..n-1 (evaluation only).
 // with_votes false: the per-pair votes of the deferred classes are left to
 // launch_vote_multi (a batch launches them for all members at once).
-cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int32_t *row_ptr,
-                            const int32_t *col_idx, const int32_t *order, int grid, int grid64, int grid128,
-                            cudaStream_t s, bool with_votes = true);
+// nodes / adj: see mocd_ctx::d_nodes; batch: nodes a warp takes at a time.
+cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj, int batch,
+                            int grid, int grid64, int grid128, cudaStream_t s, bool with_votes = true);
 // Multi-member launches of a batch: member k owns blocks starts[k] ..
 // starts[k + 1] - 1 of the launch's `blocks` (each member's own grid for
 // the stage; zero for a member with nothing to do).
@@ -164,6 +182,11 @@ cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, in
 // each undirected edge listed once, at its endpoint of lower (degree, id).
 cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx, int32_t *eptr, int32_t *eidx,
                           int cap, int sms, cudaStream_t s);
+// The mutation's node records and adjacency (mocd_ctx::d_nodes / d_adj).
+// by_degree[d] = (first position, first group of four entries) of the nodes
+// of degree d in the order.
+cudaError_t launch_mutation_adjacency(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
+                                      const int2 *by_degree, int4 *nodes, int4 *adj, int sms, cudaStream_t s);
 // *bad = 1 if some stored entry (v, u) has no mirror (u, v); rows must be
 // sorted, in range and free of self loops (checked on the host first).
 cudaError_t launch_symmetry_check(int n, const int32_t *row_ptr, const int32_t *col_idx, int *bad, int sms,
@@ -186,7 +209,8 @@ cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *ep
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order);
 int grid_for_crossover(int sms, int es);
-int grid_for_mutation(int sms, int hash_size, int *smem_bytes);
+int grid_for_mutation(int sms, int hash_size);
+int grid_for_hubs(int sms, int smem_hs);
 int mutation_warps_per_block();
 
 }  // namespace mocd

@@ -30,6 +30,8 @@ using namespace mocd;
 namespace {
 
 constexpr int kStages = 4;
+constexpr long long kMutWaves = 2;      // batches per resident warp of the mutation
+constexpr long long kMutBatchMax = 8;   // and the most nodes of a batch
 
 }  // namespace
 
@@ -42,9 +44,15 @@ struct mocd_ctx {
     int64_t n = 0, m = 0;
     int dmax = 0;
     int64_t n_defer[3] = {0, 0, 0};  // nodes of degree 33..64, 65..128 and > 512 (deferred mutation votes)
+    int64_t n_wide = 0;              // nodes of degree 129..512
     int32_t *d_row_ptr = nullptr;
     int32_t *d_col_idx = nullptr;
-    int32_t *d_order = nullptr;   // nodes by degree, descending
+    int32_t *d_order = nullptr;   // nodes by degree, descending; the two arrays below follow in its allocation
+    // The mutation's view of the graph: per position of the order (id, first
+    // group, degree, 0), and the rows in that order, padded to groups of four
+    // entries with the id n.
+    int4 *d_nodes = nullptr;
+    int4 *d_adj = nullptr;
     // The offspring evaluation's adjacency: each undirected edge once, listed
     // at its endpoint of lower (degree, id), so that the label rows it reads
     // are those of the higher-degree endpoints (fewer, each read more often:
@@ -68,6 +76,7 @@ struct mocd_ctx {
     int grid_eval_intra = 0, grid_vote64 = 0, grid_vote128 = 0;
     int occ_eval = 0, occ_cross = 0, occ_mut = 0;  // occupancy-limited grids
     int occ_eval_intra = 0;
+    int mut_batch = 1;                              // nodes a warp of the mutation takes at a time
     int nodes_per_warp = 1;                         // launch shape (autotuned for batches)
     int32_t host_gen = 0;   // generations run since init
     int32_t version = 0;    // bumped whenever the population is (re)built
@@ -239,7 +248,24 @@ void size_grids(mocd_ctx *c)
     c->grid_eval = shape(c->occ_eval, kBlock / 32);
     c->grid_eval_intra = shape(c->occ_eval_intra, kBlock / 32);
     c->grid_cross = shape(c->occ_cross, kBlock / 32);
-    c->grid_mut = shape(c->occ_mut, mutation_warps_per_block());
+    // The mutation: batches of nodes fill its lanes (see mutation_kernel), but
+    // a graph too small to give every resident warp kMutWaves batches gets
+    // smaller ones.
+    {
+        const long long wide = (long long)c->n_defer[2] + (long long)c->n_wide * kWideParts;
+        const long long normal = n - c->n_defer[2] - c->n_wide;
+        const long long warps = (long long)c->occ_mut * mutation_warps_per_block();
+        c->mut_batch = (int)std::max<long long>(1, std::min<long long>(kMutBatchMax, normal / (kMutWaves * warps)));
+        const long long items = wide + (normal + c->mut_batch - 1) / c->mut_batch;
+        const long long per_block = (long long)mutation_warps_per_block() * c->nodes_per_warp;
+        c->grid_mut = (int)std::max<long long>(1, std::min<long long>(c->occ_mut, (items + per_block - 1) / per_block));
+    }
+}
+
+// Words of PopState::hint.
+size_t hint_words(const mocd_ctx *c)
+{
+    return (size_t)c->n + (size_t)kWideParts * (size_t)c->n_wide;
 }
 
 // Allocate (or reuse) the population buffers for params and fill gp / ps.
@@ -253,7 +279,10 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         int32_t *b[4] = {};
         for (int k = 0; k < 4; ++k) {
             void *q = nullptr;
-            cudaError_t e = dev_alloc(&q, cells * sizeof(int32_t), c->stream);
+            // The children have one more row, n: the padding of the mutation's
+            // adjacency, above every label.
+            const size_t rows = cells + (k == 3 ? (size_t)W : 0);
+            cudaError_t e = dev_alloc(&q, rows * sizeof(int32_t), c->stream);
             if (e != cudaSuccess) {
                 for (int j = 0; j < k; ++j) dev_free(b[j], c->stream);
                 return cuda_status(e);
@@ -297,10 +326,11 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         c->ps.fint = reinterpret_cast<int64_t *>(q); q += sizeof(int64_t) * 2 * kMaxPop;
         c->ps.fval = reinterpret_cast<double *>(q); q += sizeof(double) * 2 * kMaxPop;
         c->ps.gen = reinterpret_cast<uint32_t *>(q);
-        c->ps.dcount = reinterpret_cast<int *>(q + 16);  // [3], within the 64-byte tail
+        c->ps.dcount = reinterpret_cast<int *>(q + 16);  // [6], within the 64-byte tail
         CK(cudaMemsetAsync(s, 0, bytes, c->stream));
         CK(cudaMemsetAsync(c->ps.q, 0, cells * sizeof(int32_t), c->stream));
         CK(cudaMemsetAsync(c->ps.buf[0], 0, cells * sizeof(int32_t), c->stream));
+        CK(cudaMemsetAsync(c->ps.c + cells, 0x7f, (size_t)W * sizeof(int32_t), c->stream));
     }
     const size_t hist_need = (size_t)W * (size_t)c->n;
     // The deferred-vote list holds every pair a generation can defer; its
@@ -308,24 +338,29 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     if ((int64_t)p->pop_size * (c->n_defer[0] + c->n_defer[1] + c->n_defer[2]) > INT_MAX)
         return MOCD_ERR_INVALID_ARG;
     const size_t defer_need = (size_t)p->pop_size * (size_t)(c->n_defer[0] + c->n_defer[1] + c->n_defer[2]);
-    // Hubs above the shared table's degree: one count table of hub_hs slots
-    // (keys and counts) per warp of the hub kernel, at most 1 GiB in all.
-    int hub_hs = 0, hub_warps = 0;
+    // Hubs: the hub kernel's count table is in shared memory if the largest
+    // hub's fits there, else (for the pairs that do not fit) a table of hub_hs
+    // slots (keys and counts) per block in global memory, at most 1 GiB in all.
+    int hub_hs = 0, hub_smem_hs = 0, hub_blocks = 0;
+    size_t hub_need = 0;
     if (c->dmax > kSharedTableMax) {
-        hub_hs = 1024;
+        hub_hs = 2048;
         while (hub_hs < 2 * c->dmax) hub_hs <<= 1;
-        const int64_t per_warp = 2 * (int64_t)hub_hs * (int64_t)sizeof(int);
-        const int64_t fit = ((int64_t)1 << 30) / per_warp;
-        hub_warps = (int)std::max<int64_t>(4, std::min<int64_t>((int64_t)c->sms * 4, fit)) & ~3;
+        hub_smem_hs = std::min(hub_hs, kHubSmemSlots);
+        hub_blocks = grid_for_hubs(c->sms, hub_smem_hs);
+        if (hub_hs > hub_smem_hs) {
+            const int64_t per_block = 2 * (int64_t)hub_hs * (int64_t)sizeof(int);
+            const int64_t fit = ((int64_t)1 << 30) / per_block;
+            hub_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(hub_blocks, fit));
+            hub_need = (size_t)hub_blocks * 2 * (size_t)hub_hs;
+        }
     }
     {
         int rc = grow(c->stream, &c->ps.hist, &c->hist_cap, hist_need);
         if (rc) return rc;
-        if ((rc = grow(c->stream, &c->ps.hint, &c->hint_cap, (size_t)c->n))) return rc;
+        if ((rc = grow(c->stream, &c->ps.hint, &c->hint_cap, hint_words(c)))) return rc;
         if ((rc = grow(c->stream, &c->ps.dlist, &c->dlist_cap, defer_need))) return rc;
-        if (hub_hs > 0 &&
-            (rc = grow(c->stream, &c->ps.hub_table, &c->hub_cap, (size_t)hub_warps * 2 * (size_t)hub_hs)))
-            return rc;
+        if (hub_need > 0 && (rc = grow(c->stream, &c->ps.hub_table, &c->hub_cap, hub_need))) return rc;
     }
     c->W = W;
     c->params = *p;
@@ -345,8 +380,11 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.defer_cap[0] = (int)((int64_t)p->pop_size * c->n_defer[0]);
     gp.defer_cap[1] = (int)((int64_t)p->pop_size * c->n_defer[1]);
     gp.defer_cap[2] = (int)((int64_t)p->pop_size * c->n_defer[2]);
+    gp.n_hub = (int)c->n_defer[2];
+    gp.n_wide = (int)c->n_wide;
     gp.hub_hs = hub_hs;
-    gp.hub_warps = hub_warps;
+    gp.hub_smem_hs = hub_smem_hs;
+    gp.hub_blocks = hub_blocks;
     {
         // The degree 33..64 vote's network holds the largest degree of that
         // class in the graph: 40, 48, 56 or 64 entries.
@@ -362,8 +400,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     c->occ_eval_intra = grid_for_eval_intra(c->sms);
     grid_for_votes(c->sms, gp.vote_n0, &c->grid_vote64, &c->grid_vote128);
     c->occ_cross = grid_for_crossover(c->sms, gp.es);
-    int smem = 0;
-    c->occ_mut = grid_for_mutation(c->sms, gp.hash_size, &smem);
+    c->occ_mut = grid_for_mutation(c->sms, gp.hash_size);
     size_grids(c);
     return MOCD_OK;
 }
@@ -391,8 +428,7 @@ int issue_generation(mocd_ctx *c, cudaStream_t st, bool events, bool with_select
     if (events) CK(mark(c, 0, st));
     CK(launch_crossover(gp, ps, c->grid_cross, st));
     if (events) CK(mark(c, 1, st));
-    CK(launch_mutation(gp, ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->grid_mut, c->grid_vote64,
-                       c->grid_vote128, st));
+    CK(launch_mutation(gp, ps, c->d_nodes, c->d_adj, c->mut_batch, c->grid_mut, c->grid_vote64, c->grid_vote128, st));
     if (events) CK(mark(c, 2, st));
     CK(launch_evaluate_offspring(gp.n, gp.W, gp.np, c->d_eptr, c->d_eidx, ps.q, ps.hist, ps.acc,
                                  c->grid_eval_intra, st, c->d_order));
@@ -431,8 +467,8 @@ int start_population(mocd_ctx *c, uint32_t base_gen)
     int32_t *phalf = ps.buf[(base_gen + 1u) & 1u];
     int rc = clear_eval_state(c, ps.hist, (size_t)gp.W * (size_t)gp.n, ps.acc);
     if (rc) return rc;
-    // No mutation history yet: every node starts with the Misra-Gries pass.
-    CK(cudaMemsetAsync(ps.hint, 0, sizeof(uint32_t) * (size_t)gp.n, c->stream));
+    // No mutation history yet.
+    CK(cudaMemsetAsync(ps.hint, 0, sizeof(uint32_t) * hint_words(c), c->stream));
     CK(launch_evaluate(gp.n, gp.W, gp.np, c->d_row_ptr, c->d_col_idx, phalf, ps.hist, ps.acc,
                        c->grid_eval, c->stream));
     // Generations expect a zero histogram (the mutation kernel adds into it).
@@ -917,6 +953,7 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
         if (d > 32 && d <= 64) c->n_defer[0] += 1;
         else if (d > 64 && d <= kDeferMax) c->n_defer[1] += 1;
         else if (d > kSharedTableMax) c->n_defer[2] += 1;
+        else if (d > kDeferMax) c->n_wide += 1;
     }
     std::vector<int32_t> rp32(n + 1);
     for (int64_t v = 0; v <= n; ++v) rp32[v] = (int32_t)row_ptr[v];
@@ -931,17 +968,34 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
     // by node id), so that the costliest nodes are spread over all warps. A
     // counting sort on the degree.
     std::vector<int32_t> order(n);
+    // Per degree: the first position of its nodes, and the first group of four
+    // entries of their rows in the mutation's adjacency.
+    std::vector<int2> by_degree((size_t)dmax + 1, make_int2(0, 0));
+    int64_t groups = 0;
     {
         std::vector<int64_t> at((size_t)dmax + 2, 0);
         for (int64_t v = 0; v < n; ++v) at[(size_t)(dmax - (row_ptr[v + 1] - row_ptr[v])) + 1] += 1;
         for (size_t d = 1; d < at.size(); ++d) at[d] += at[d - 1];
+        for (int d = dmax; d >= 0; --d) {
+            const size_t k = (size_t)(dmax - d);
+            by_degree[(size_t)d] = make_int2((int)at[k], (int)groups);
+            groups += (at[k + 1] - at[k]) * ((d + 3) / 4);
+        }
         for (int64_t v = 0; v < n; ++v) order[at[(size_t)(dmax - (row_ptr[v + 1] - row_ptr[v]))]++] = (int32_t)v;
     }
-    e = dev_alloc(&p, sizeof(int32_t) * n, c->stream);
+    // One allocation: the order, the node records, the padded rows and the
+    // table per degree (read once, below).
+    const size_t order_bytes = (sizeof(int32_t) * (size_t)n + 15) & ~(size_t)15;
+    e = dev_alloc(&p, order_bytes + sizeof(int4) * (size_t)(n + groups) + sizeof(int2) * by_degree.size(), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_order = static_cast<int32_t *>(p);
+    c->d_nodes = reinterpret_cast<int4 *>(static_cast<char *>(p) + order_bytes);
+    c->d_adj = c->d_nodes + n;
+    int2 *d_by_degree = reinterpret_cast<int2 *>(c->d_adj + groups);
     if (cudaMemcpyAsync(c->d_order, order.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream) !=
-        cudaSuccess)
+            cudaSuccess ||
+        cudaMemcpyAsync(d_by_degree, by_degree.data(), sizeof(int2) * by_degree.size(), cudaMemcpyHostToDevice,
+                        c->stream) != cudaSuccess)
         return fail(MOCD_ERR_CUDA);
     e = dev_alloc(&p, sizeof(int32_t) * (n + 1), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
@@ -962,6 +1016,8 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
         launch_symmetry_check((int)n, c->d_row_ptr, c->d_col_idx, d_bad, c->sms, c->stream) == cudaSuccess &&
         launch_orient((int)n, c->d_row_ptr, c->d_col_idx, c->d_eptr, c->d_eidx, (int)(nnz / 2), c->sms,
                       c->stream) == cudaSuccess &&
+        launch_mutation_adjacency((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, d_by_degree, c->d_nodes, c->d_adj,
+                                  c->sms, c->stream) == cudaSuccess &&
         cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream) == cudaSuccess;
     cudaFreeAsync(d_bad, c->stream);
     if (!copied || cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(MOCD_ERR_CUDA);
@@ -1285,7 +1341,8 @@ static int batch_build(mocd_batch *b)
             mocd_ctx *c = b->ctx[(size_t)i];
             gps.push_back(c->gp);
             pss.push_back(c->ps);
-            mbs.push_back(BatchMember{c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_eptr, c->d_eidx});
+            mbs.push_back(BatchMember{c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_nodes, c->d_adj,
+                                      c->d_eptr, c->d_eidx});
             b->es_max = std::max(b->es_max, c->gp.es);
             // Per member and stage: its own grid (a deferred class's votes get
             // about one thread per four listed pairs at full capacity, at most
@@ -1319,7 +1376,7 @@ static int batch_build(mocd_batch *b)
         e = cudaStreamWaitEvent(b->branch[(size_t)i], b->fork, 0);
         if (e != cudaSuccess) break;
         if (b->form == 2)
-            e = launch_mutation(c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->grid_mut, c->grid_vote64,
+            e = launch_mutation(c->gp, c->ps, c->d_nodes, c->d_adj, c->mut_batch, c->grid_mut, c->grid_vote64,
                                 c->grid_vote128, b->branch[(size_t)i], false);
         else
             rc = issue_generation(c, b->branch[(size_t)i], false, b->form == 0);
