@@ -346,9 +346,6 @@ __device__ __forceinline__ void select_body(const GenParams &gp, const PopState 
     const uint32_t gn = g + 1u;
     const unsigned long long *acc = ps.acc;
     const int N = mode == 0 ? np : 2 * np;
-    // A fresh population has no mutation history.
-    if (mode == 0 && p >= kDcountPairs && p <= kDcountFast) ps.dcount[p] = 0;
-
     // Keys by point: P's (mode 1), then those of the evaluated labellings.
     if (p < N) {
         const int i = mode == 0 ? p : p - np;

@@ -161,17 +161,8 @@ __device__ __forceinline__ void crossover_body(const GenParams gp, const int32_t
                                                int32_t *out0, int32_t *out1, const int32_t *__restrict__ q,
                                                int32_t *__restrict__ child, const int32_t *__restrict__ keep,
                                                const int32_t *__restrict__ par_r, const int32_t *__restrict__ copy_r,
-                                               const uint32_t *__restrict__ gen_ptr, int *__restrict__ dcount,
-                                               int vblock, int vgrid)
+                                               const uint32_t *__restrict__ gen_ptr, int vblock, int vgrid)
 {
-    // The mutation kernel that follows appends deferred pairs from zero, and
-    // counts the own label first if that settled at least half of the last
-    // generation's sampled pairs.
-    if (vblock == 0 && threadIdx.x == 0) {
-        const int pairs = dcount[kDcountPairs], ok = dcount[kDcountOk];
-        dcount[kDcountFast] = pairs > 0 && 2 * ok >= pairs ? 1 : 0;
-        for (int k = 0; k <= kDcountOk; ++k) dcount[k] = 0;
-    }
     extern __shared__ int smem[];
     const int W = gp.W, np = gp.np, E = gp.es;
     const int nq = W >> 2;
@@ -338,11 +329,9 @@ __global__ void __launch_bounds__(kBlock)
 crossover_kernel(GenParams gp, const int32_t *buf0, const int32_t *buf1, int32_t *out0, int32_t *out1,
                  const int32_t *__restrict__ q, int32_t *__restrict__ child,
                  const int32_t *__restrict__ keep, const int32_t *__restrict__ par_r,
-                 const int32_t *__restrict__ copy_r, const uint32_t *__restrict__ gen_ptr,
-                 int *__restrict__ dcount)
+                 const int32_t *__restrict__ copy_r, const uint32_t *__restrict__ gen_ptr)
 {
-    crossover_body<EMAX>(gp, buf0, buf1, out0, out1, q, child, keep, par_r, copy_r, gen_ptr, dcount, blockIdx.x,
-                         gridDim.x);
+    crossover_body<EMAX>(gp, buf0, buf1, out0, out1, q, child, keep, par_r, copy_r, gen_ptr, blockIdx.x, gridDim.x);
 }
 
 // The member of a multi-member launch that block blockIdx.x belongs to:
@@ -370,7 +359,7 @@ crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__res
     const PopState &ps = mb.ps;
     const int b0 = __ldg(starts + k);
     crossover_body<EMAX>(mb.gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r,
-                         ps.copy_r, ps.gen, ps.dcount, (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
+                         ps.copy_r, ps.gen, (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
 }
 
 // ---------------------------------------------------------------------------
@@ -383,22 +372,31 @@ crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__res
 // A pair is a (node, selected child). A warp takes a batch of nodes, copies
 // their rows to Q, and lists the batch's pairs; then every lane works on a
 // pair of its own, so that the lanes stay full whatever number of children a
-// node has selected (about 20 of 100 at M_P 0.2). In a settled population the
-// result is nearly always the label the node already has, and counting the
-// neighbours that hold it proves that: when it is on more than half of them
-// it is the unique mode. The pairs this leaves open take the exact vote, by
-// degree:
-//   up to 32     in the same warp, a pair per lane: the labels are gathered
-//                into registers, sorted by a merge-exchange network of 8, 12,
-//                .., 28 or 32 entries (the smallest that holds the degree) and
-//                the tied labels read off the runs
-//   33..128      listed for mutation_vote_kernel, a pair per thread
+// node has selected (about 20 of 100 at M_P 0.2). By degree:
+//   up to 128    mutation_kernel, a pair per lane: the labels are gathered into
+//                registers, sorted by a merge-exchange network and the tied
+//                labels read off the runs. One launch for degrees up to 32
+//                (networks of 8, 12, .., 28 or 32 entries, the smallest that
+//                holds the lanes' degrees), one each for 33..64 (40, 48, 56 or
+//                64 entries, the smallest that holds the graph's largest
+//                degree there) and 65..128, so that no launch pays for the
+//                registers of a larger network than its own
 //   129..512     a warp per pair: count table in shared memory (the node's
-//                pairs are split over kWideParts warps)
-//   above 512    listed for mutation_hub_kernel, a block per pair
-// Whether the count of the own label is worth its pass over the neighbours is
-// read from the last generation: the share of the pairs it settled (or would
-// have settled), for degree <= 32 over a sample of all pairs, above per node.
+//                pairs are split over kWideParts warps), in the first launch
+//   above 512    mutation_hub_kernel, a block per pair
+// The launches touch different rows of Q and only add to the histogram, so
+// they run side by side.
+//
+// A count table costs several passes over the neighbours' labels, and in a
+// settled population the result is often the label the node already has:
+// counting the neighbours that hold it proves that when it is on more than
+// half of them (it is then the unique mode). Above degree 128 that count goes
+// first when the node's last generation says it pays (own_label_pays). The
+// vote in registers needs one pass, and a front keeps so many fragmented
+// members that the count settles at most 0.45 of the pairs (n = 40,000 and
+// 10^6, mu 0.3): trying it first there was slower at every threshold (n =
+// 10^6: 2.59 ms a generation's mutation with it from half settled on, 2.50
+// without).
 //
 // The neighbours come from the mutation's own adjacency: rows in processing
 // order (degree descending), padded to four entries with the id n, whose
@@ -426,21 +424,10 @@ __device__ __forceinline__ uint32_t hash_slot(int x, int hbits)
     return ((uint32_t)x * 2654435761u) >> (32 - hbits);
 }
 
-// Start of deferred-vote class c in the list: the classes are stored one
-// after the other (written with selects: indexing the kernel parameter array
-// at run time would copy it to local memory).
-__device__ __forceinline__ int defer_offset(const GenParams &gp, int c)
-{
-    return c == 0 ? 0 : c == 1 ? gp.defer_cap[0] : gp.defer_cap[0] + gp.defer_cap[1];
-}
-__device__ __forceinline__ int defer_capacity(const GenParams &gp, int c)
-{
-    return c == 0 ? gp.defer_cap[0] : c == 1 ? gp.defer_cap[1] : gp.defer_cap[2];
-}
 constexpr int kLaneMax = 32;     // largest degree of the per-lane vote
 constexpr int kMutBlock = 128;   // mutation threads per block
 constexpr int kHubBlock = 256;   // threads per block of the hub kernel
-constexpr int kBatch = 8;        // most nodes of a warp's batch
+static_assert(kMutBatchMax * kMaxPop <= 65536, "a pair is listed in 16 bits");
 
 // Sorting networks for any N: Batcher's merge exchange in the form of
 // Knuth, TAOCP vol. 3, Sec. 5.2.2, Algorithm M (for a power of two it is
@@ -538,24 +525,6 @@ __device__ __forceinline__ int select_at(const int (&x)[N], int pos)
     return y[0];
 }
 
-// The first entries of the longest runs of equal values among the deg sorted
-// entries behind e (bit j of e: entries j and j + 1 are equal, both < deg):
-// a run of L values is L - 1 consecutive set bits; each step m &= m >> 1
-// shortens every run of set bits by one, and the last non-zero m has one bit
-// per longest run, at its first entry (all entries when no two are equal).
-// best: the length of those runs.
-__device__ __forceinline__ unsigned longest_runs(unsigned e, int deg, int &best)
-{
-    e &= deg >= 2 ? 0xffffffffu >> (33 - deg) : 0u;  // pairs (j, j + 1) with j + 1 < deg
-    unsigned starts = deg >= 32 ? 0xffffffffu : (1u << deg) - 1u;
-    best = 1;
-    for (unsigned m = e; m != 0u; m &= m >> 1) {
-        starts = m;
-        ++best;
-    }
-    return starts;
-}
-
 // Position of the k-th set bit of m (k < popc(m)), halving the window.
 __device__ __forceinline__ int kth_bit(unsigned m, unsigned k)
 {
@@ -575,15 +544,20 @@ __device__ __forceinline__ int kth_bit(unsigned m, unsigned k)
     return pos;
 }
 
-// Exact neighbour-majority of one pair by its own lane (deg <= N <= 32; 0
-// for a lane without a pair): the labels are gathered into registers (the
-// padding and the entries past it sort last), sorted, and the tied labels are
-// the longest runs in ascending order. All lanes of the warp call together.
+// Exact neighbour-majority of one pair by its own lane (deg <= N; 0 for a
+// lane without a pair). The labels are gathered into registers (the padding
+// and the entries past it sort last) and sorted; equal labels then form runs,
+// the longest runs are the tied labels in ascending order, and the
+// pick(u, t)-th of them is the result. Bit j of eq is set when entries j and
+// j + 1 (< deg) are equal, so a run of L labels is L - 1 consecutive set bits;
+// each step m &= m >> 1 (across words) shortens every run of set bits by one,
+// and the last non-zero m has one bit per longest run, at its first entry (all
+// entries when no two are equal). All lanes of the warp call together.
 template <int N>
 __device__ __forceinline__ int lane_vote(const GenParams &gp, const int4 *__restrict__ adj,
-                                         const int32_t *__restrict__ child, int v, int i, int beg, int deg, uint32_t g,
-                                         int &best)
+                                         const int32_t *__restrict__ child, int v, int i, int beg, int deg, uint32_t g)
 {
+    constexpr int NW = (N + 31) / 32;
     const int32_t *col = child + i;
     int x[N];
 #pragma unroll
@@ -596,14 +570,46 @@ __device__ __forceinline__ int lane_vote(const GenParams &gp, const int4 *__rest
         x[j + 3] = in ? col[(size_t)checked_node(u.w, gp.n) * gp.W] : INT_MAX;
     }
     sort_network<N>(x);
-    unsigned e = 0;
+    unsigned m[NW], starts[NW];
 #pragma unroll
-    for (int j = 0; j + 1 < N; ++j) e |= (x[j] == x[j + 1] ? 1u : 0u) << j;
-    const unsigned starts = longest_runs(e, deg, best);
-    const int t = __popc(starts);
-    unsigned kk = 0;
-    if (__any_sync(kFull, t > 1)) kk = t > 1 ? pick_index(tie_word(gp, v, i, g), (uint32_t)t) : 0u;
-    return select_at<N>(x, kth_bit(starts, kk));
+    for (int w = 0; w < NW; ++w) m[w] = 0u;
+#pragma unroll
+    for (int j = 0; j + 1 < N; ++j) m[j >> 5] |= (x[j] == x[j + 1] ? 1u : 0u) << (j & 31);
+    bool any = false;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const int pairs = deg - 1 - 32 * w, ents = deg - 32 * w;  // valid bits of the word
+        m[w] &= pairs >= 32 ? ~0u : pairs <= 0 ? 0u : (1u << pairs) - 1u;
+        starts[w] = ents >= 32 ? ~0u : ents <= 0 ? 0u : (1u << ents) - 1u;
+        any |= m[w] != 0u;
+    }
+    while (any) {
+        any = false;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            starts[w] = m[w];
+            m[w] &= __funnelshift_r(m[w], w + 1 < NW ? m[w + 1 < NW ? w + 1 : w] : 0u, 1);
+            any |= m[w] != 0u;
+        }
+    }
+    int t = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) t += __popc(starts[w]);
+    unsigned k = 0;
+    if (__any_sync(kFull, t > 1)) k = t > 1 ? pick_index(tie_word(gp, v, i, g), (uint32_t)t) : 0u;
+    // The word that holds the k-th start, then its position there.
+    int base = 0;
+    unsigned word = starts[0];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) {
+        const unsigned c = (unsigned)__popc(word);
+        if (base == 32 * (w - 1) && k >= c) {
+            k -= c;
+            word = starts[w];
+            base = 32 * w;
+        }
+    }
+    return select_at<N>(x, base + kth_bit(word, k));
 }
 
 // Exact neighbour-majority of one pair of a node with degree kDeferMax + 1 ..
@@ -732,91 +738,68 @@ __device__ __forceinline__ unsigned selected(const GenParams &gp, int v, int lan
            ((i0 + 3 < gp.np && (unsigned long long)r.w < gp.thr_m) ? 8u : 0u);
 }
 
-// Node row of a warp: Q gets the children's own labels, the histogram the
-// unselected ones (mutating pairs add theirs once decided), and the selected
-// children go to list[total ..] tagged with `tag`. Returns their number.
-__device__ __forceinline__ int take_row(const GenParams &gp, int v, int deg, bool active, const int4 &out, int lane,
-                                        uint32_t g, int4 *__restrict__ Q4, uint32_t *__restrict__ hist,
-                                        unsigned short *list, int total, int tag)
+// Quad `lane_quad` of node v's row: Q gets the children's own labels and the
+// histogram the unselected ones (mutating pairs add theirs once decided).
+// Returns the selected children of the quad.
+__device__ __forceinline__ unsigned take_quad(const GenParams &gp, int v, int deg, int quad, const int4 &out,
+                                              uint32_t g, int4 *__restrict__ Q4, uint32_t *__restrict__ hist)
 {
-    unsigned sel = 0;
-    if (active && deg > 0) sel = selected(gp, v, lane, g);
-    if (active) {
-        Q4[(size_t)v * (gp.W >> 2) + lane] = out;
-        if (deg > 0) {
-            const int i0 = 4 * lane;
-            if (i0 + 0 < gp.np && !(sel & 1u)) add_degree(gp, hist, out.x, i0 + 0, deg);
-            if (i0 + 1 < gp.np && !(sel & 2u)) add_degree(gp, hist, out.y, i0 + 1, deg);
-            if (i0 + 2 < gp.np && !(sel & 4u)) add_degree(gp, hist, out.z, i0 + 2, deg);
-            if (i0 + 3 < gp.np && !(sel & 8u)) add_degree(gp, hist, out.w, i0 + 3, deg);
-        }
+    const unsigned sel = deg > 0 ? selected(gp, v, quad, g) : 0u;
+    Q4[(size_t)v * (gp.W >> 2) + quad] = out;
+    if (deg > 0) {
+        const int i0 = 4 * quad;
+        if (i0 + 0 < gp.np && !(sel & 1u)) add_degree(gp, hist, out.x, i0 + 0, deg);
+        if (i0 + 1 < gp.np && !(sel & 2u)) add_degree(gp, hist, out.y, i0 + 1, deg);
+        if (i0 + 2 < gp.np && !(sel & 4u)) add_degree(gp, hist, out.z, i0 + 2, deg);
+        if (i0 + 3 < gp.np && !(sel & 8u)) add_degree(gp, hist, out.w, i0 + 3, deg);
     }
-    // Place of the lane's selected children: its count (0 .. 4) by bits.
-    const unsigned lt = (1u << lane) - 1u;
+    return sel;
+}
+
+// Appends each lane's selected children (bits of sel), tagged, to list[total
+// ..]; returns their number. A lane's place: its count (0 .. 4) by bits.
+__device__ __forceinline__ int list_selected(unsigned short *list, int total, unsigned sel, int tag)
+{
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     const int mine = __popc(sel);
     const unsigned b0 = __ballot_sync(kFull, mine & 1), b1 = __ballot_sync(kFull, mine & 2),
                    b2 = __ballot_sync(kFull, mine & 4);
     int at = total + __popc(b0 & lt) + 2 * __popc(b1 & lt) + 4 * __popc(b2 & lt);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-        if ((sel >> k) & 1u) list[at++] = (unsigned short)(tag | (4 * lane + k));
+        if ((sel >> k) & 1u) list[at++] = (unsigned short)(tag + k);
     return __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
 }
 
-// Deferred pairs of one class, appended by the lanes of `who` (warp-uniform).
-// The capacity is the class's nodes x N_p, every pair a generation can defer:
-// the check only keeps a corrupted count in bounds.
-__device__ __forceinline__ void defer_pairs(const GenParams &gp, int cls, unsigned who, int node, int i, int lane,
-                                            int2 *__restrict__ dlist, int *__restrict__ dcount)
-{
-    int first = 0;
-    if (lane == 0) first = atomicAdd(dcount + cls, __popc(who));
-    first = __shfl_sync(kFull, first, 0);
-    if ((who >> lane) & 1u) {
-        const int at = first + __popc(who & ((1u << lane) - 1u));
-        if (at < defer_capacity(gp, cls)) dlist[defer_offset(gp, cls) + at] = make_int2(node, i);
-    }
-}
-
-// hint of a node (or part): (pairs << 16) | pairs whose own label was on more
-// than half of the neighbours, last generation; 0: no history.
+// hint of a part of a node (or of a hub's quad): (pairs << 16) | pairs whose
+// own label was on more than half of the neighbours, last generation; 0: no
+// history. A quarter settled pays for the count.
 __device__ __forceinline__ bool own_label_pays(uint32_t h)
 {
-    return h != 0u && 2u * (h & 0xffffu) >= (h >> 16);
+    return h != 0u && 4u * (h & 0xffffu) >= (h >> 16);
 }
 
-// One item of the nodes above kDeferMax: a hub (idx < gp.n_hub), whose pairs
-// are all listed for mutation_hub_kernel, or part `part` of a node of degree
-// kDeferMax + 1 .. kSharedTableMax: the quads q with q % kWideParts == part.
-__device__ __noinline__ void wide_item(const GenParams &gp, int item, const int4 *__restrict__ nodes,
+// Part `part` of a node of degree kDeferMax + 1 .. kSharedTableMax (position
+// idx): the quads q with q % kWideParts == part, a warp per pair.
+__device__ __noinline__ void wide_item(const GenParams &gp, int idx, int part, const int4 *__restrict__ nodes,
                                        const int4 *__restrict__ adj, const int32_t *__restrict__ child,
                                        int32_t *__restrict__ q, uint32_t *__restrict__ hist,
-                                       uint32_t *__restrict__ hint, int2 *__restrict__ dlist, int *__restrict__ dcount,
-                                       unsigned short *list, int *hkey, int *hcnt, uint32_t g)
+                                       uint32_t *__restrict__ hint, unsigned short *list, int *hkey, int *hcnt,
+                                       uint32_t g)
 {
     const int lane = threadIdx.x & 31;
     const int nq = gp.W >> 2;
-    const bool hub = item < gp.n_hub;
-    const int idx = hub ? item : gp.n_hub + (item - gp.n_hub) / kWideParts;
-    const int part = hub ? 0 : (item - gp.n_hub) % kWideParts;
     const int4 rec = __ldg(nodes + idx);
     const int v = rec.x, deg = rec.z;
-    const bool active = lane < nq && (hub || lane % kWideParts == part);
-    const int4 out = active ? reinterpret_cast<const int4 *>(child)[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
-    const int total = take_row(gp, v, deg, active, out, lane, g, reinterpret_cast<int4 *>(q), hist, list, 0, 0);
-    uint32_t *h = hint + (hub ? idx : gp.n + (idx - gp.n_hub) * kWideParts + part);
+    unsigned sel = 0;
+    if (lane < nq && lane % kWideParts == part) {
+        const int4 out = reinterpret_cast<const int4 *>(child)[(size_t)v * nq + lane];
+        sel = take_quad(gp, v, deg, lane, out, g, reinterpret_cast<int4 *>(q), hist);
+    }
+    const int total = list_selected(list, 0, sel, 4 * lane);
+    uint32_t *h = hint + (idx - gp.n_hub) * kWideParts + part;
     const bool fast = own_label_pays(*h);
     __syncwarp();
-    if (hub) {
-        // The flag travels with the pair: the hub kernel rewrites the hint.
-        for (int base = 0; base < total; base += 32) {
-            const bool has = base + lane < total;
-            defer_pairs(gp, 2, __ballot_sync(kFull, has), idx | (fast ? kHubFast : 0), has ? list[base + lane] : 0, lane,
-                        dlist, dcount);
-        }
-        if (lane == 0) *h = (uint32_t)total << 16;
-        return;
-    }
     int ok = 0;
     const int *nbr = reinterpret_cast<const int *>(adj + rec.y);
     for (int k = 0; k < total; ++k) {
@@ -842,301 +825,121 @@ __device__ __noinline__ void wide_item(const GenParams &gp, int item, const int4
     if (lane == 0) *h = ((uint32_t)total << 16) | (uint32_t)ok;
 }
 
-// WIDE: the graph has degrees above kDeferMax. batch: nodes a warp takes at a
-// time (<= kBatch).
-template <bool WIDE>
-__global__ void __launch_bounds__(kMutBlock, 6)
-mutation_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict__ nodes, const int4 *__restrict__ adj,
-                const int32_t *__restrict__ child, int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr,
-                uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc, uint32_t *__restrict__ hint,
-                int2 *__restrict__ dlist, int *__restrict__ dcount, int batch)
+// 16-byte words of a warp's shared memory in mutation_kernel.
+__host__ __device__ __forceinline__ int mutation_warp_words(int np, int batch, int hash_size)
 {
-    __shared__ unsigned short s_list[kMutBlock / 32][kBatch * kMaxPop];
-    __shared__ int4 s_rec[kMutBlock / 32][kBatch];
-    __shared__ int s_ok[kMutBlock / 32][kBatch];
-    extern __shared__ int s_table[];  // WIDE: per warp, keys and counts
+    return batch + (batch * np * 2 + 15) / 16 + hash_size / 2;
+}
+
+// The nodes at positions [first, last) of the order, of degree <= N
+// (N > kLaneMax: also above the next smaller class, see launch_mutation).
+// WIDE: the launch also takes the nodes of degree kDeferMax + 1 ..
+// kSharedTableMax (positions n_hub .. n_hub + n_wide - 1). batch: nodes a warp
+// takes at a time (<= kMutBatchMax).
+template <int N, bool WIDE>
+__global__ void __launch_bounds__(kMutBlock, N <= kLaneMax ? (WIDE ? 8 : 7) : N <= 40 ? 6 : N <= 64 ? 5 : 3)
+mutation_kernel(const __grid_constant__ GenParams gp, int first, int last, const int4 *__restrict__ nodes,
+                const int4 *__restrict__ adj, const int32_t *__restrict__ child, int32_t *__restrict__ q,
+                const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc,
+                uint32_t *__restrict__ hint, int batch)
+{
+    // Per warp: the batch's node records, the pair list (two bytes a pair; sized
+    // to the batch, so that the rest of the memory is L1 cache) and, WIDE, a
+    // count table.
+    extern __shared__ int4 s_warp[];
     const int W = gp.W;
     const int nq = W >> 2;
     const uint32_t g = *gen_ptr;
-    const bool lane_fast = dcount[kDcountFast] != 0;
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
-    unsigned short *list = s_list[wib];
-    int4 *recs = s_rec[wib];
-    int *oks = s_ok[wib];
+    int4 *recs = s_warp + wib * mutation_warp_words(gp.np, batch, WIDE ? gp.hash_size : 0);
+    unsigned short *list = reinterpret_cast<unsigned short *>(recs + batch);
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const bool active = lane < nq;
-    const unsigned lt = (1u << lane) - 1u;
     const int4 *__restrict__ C4 = reinterpret_cast<const int4 *>(child);
     int4 *__restrict__ Q4 = reinterpret_cast<int4 *>(q);
 
     // The evaluation that follows accumulates into acc: clear it here. The
     // histogram is zero on entry (the previous evaluation's square sweep
     // cleared it) and receives D below.
-    if (blockIdx.x == 0)
+    if (N <= kLaneMax && blockIdx.x == 0)
         for (int t = threadIdx.x; t < 2 * kMaxPop; t += blockDim.x) acc[t] = 0;
 
     // Nodes in degree-descending order: every warp starts with one of the
     // costliest batches, which balances the grid-stride loop.
-    const int wide = WIDE ? gp.n_hub + gp.n_wide * kWideParts : 0;
-    const int first = WIDE ? gp.n_hub + gp.n_wide : 0;
-    const int items = wide + (gp.n - first + batch - 1) / batch;
+    const int wide = WIDE ? gp.n_wide * kWideParts : 0;
+    const int items = wide + (last - first + batch - 1) / batch;
+    const unsigned inv_nq = (65536u + (unsigned)nq - 1u) / (unsigned)nq;  // t / nq = t * inv_nq >> 16, t < 2^10
     for (int item = warp; item < items; item += nwarps) {
         if (WIDE && item < wide) {
-            wide_item(gp, item, nodes, adj, child, q, hist, hint, dlist, dcount, list,
-                      s_table + wib * 2 * gp.hash_size, s_table + wib * 2 * gp.hash_size + gp.hash_size, g);
+            int *table = reinterpret_cast<int *>(recs + mutation_warp_words(gp.np, batch, 0));
+            wide_item(gp, gp.n_hub + item / kWideParts, item % kWideParts, nodes, adj, child, q, hist, hint, list, table,
+                      table + gp.hash_size, g);
             __syncwarp();
             continue;
         }
         const int idx0 = first + (item - wide) * batch;
-        const int nb = min(batch, gp.n - idx0);
-        int4 rec = make_int4(0, 0, 0, 0);
-        if (lane < nb) {
-            rec = __ldg(nodes + idx0 + lane);
-            const bool fast = rec.z <= kLaneMax ? lane_fast : own_label_pays(hint[idx0 + lane]);
-            recs[lane] = make_int4(rec.x, rec.y, rec.z, fast ? rec.z : 0);  // .w: degree if the count pays
-            oks[lane] = 0;
+        const int nb = min(batch, last - idx0);
+        if (lane < nb) recs[lane] = __ldg(nodes + idx0 + lane);
+        __syncwarp();
+        // The batch's rows, a quad per lane; the next quad is requested before
+        // this one is processed.
+        const int quads = nb * nq;
+        auto quad_of = [&](int t, int &k) {
+            k = (int)(((unsigned)t * inv_nq) >> 16);
+            return t - k * nq;
+        };
+        int total = 0;
+        int k = 0, quad = 0, v = 0, deg = 0;
+        int4 row = make_int4(0, 0, 0, 0);
+        if (lane < quads) {
+            quad = quad_of(lane, k);
+            v = recs[k].x;
+            deg = recs[k].z;
+            row = C4[(size_t)v * nq + quad];
         }
-        int total = 0, nsel = 0;
-        int v = __shfl_sync(kFull, rec.x, 0);
-        int4 nxt = active ? C4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
-        for (int k = 0; k < nb; ++k) {
-            const int deg = __shfl_sync(kFull, rec.z, k);
-            const int4 out = nxt;
-            const int cur = v;
-            if (k + 1 < nb) {  // the next row is requested before this one is processed
-                v = __shfl_sync(kFull, rec.x, k + 1);
-                if (active) nxt = C4[(size_t)v * nq + lane];
+        for (int t = lane; t - lane < quads; t += 32) {
+            const int4 out = row;
+            const int cur_k = k, cur_quad = quad, cur_v = v, cur_deg = deg;
+            if (t + 32 < quads) {
+                quad = quad_of(t + 32, k);
+                v = recs[k].x;
+                deg = recs[k].z;
+                row = C4[(size_t)v * nq + quad];
             }
-            const int c = take_row(gp, cur, deg, active, out, lane, g, Q4, hist, list, total, k << 7);
-            nsel = lane == k ? c : nsel;
-            total += c;
+            unsigned sel = 0;
+            if (t < quads) sel = take_quad(gp, cur_v, cur_deg, cur_quad, out, g, Q4, hist);
+            total += list_selected(list, total, sel, cur_k * kMaxPop + 4 * cur_quad);
         }
         __syncwarp();
 
-        // The own label's count; open pairs are compacted to the list's front.
-        int open = 0, settled32 = 0;
-        const bool any_fast = __any_sync(kFull, lane < nb && recs[lane < nb ? lane : 0].w != 0);
-        if (!any_fast) open = total;
-        for (int base = 0; any_fast && base < total; base += 32) {
+        // The votes (the list's degrees descend).
+        for (int base = 0; base < total; base += 32) {
             const bool has = base + lane < total;
             const int e = has ? list[base + lane] : 0;
-            const int i = e & 127;
-            const int4 r = recs[e >> 7];
-            const int32_t *col = child + i;
-            const int own = has ? col[(size_t)r.x * W] : 0;
-            const int n4 = has ? (r.w + 3) >> 2 : 0;  // groups of four neighbours to count
-            const int n4_max = __reduce_max_sync(kFull, n4);
-            int c = 0;
-            for (int j = 0; j < n4_max; j += 2) {
-                const bool p0 = j < n4, p1 = j + 1 < n4;
-                const int4 u0 = p0 ? __ldg(adj + r.y + j) : make_int4(0, 0, 0, 0);
-                const int4 u1 = p1 ? __ldg(adj + r.y + j + 1) : make_int4(0, 0, 0, 0);
-                int x[8];
-                x[0] = p0 ? col[(size_t)checked_node(u0.x, gp.n) * W] : -1;
-                x[1] = p0 ? col[(size_t)checked_node(u0.y, gp.n) * W] : -1;
-                x[2] = p0 ? col[(size_t)checked_node(u0.z, gp.n) * W] : -1;
-                x[3] = p0 ? col[(size_t)checked_node(u0.w, gp.n) * W] : -1;
-                x[4] = p1 ? col[(size_t)checked_node(u1.x, gp.n) * W] : -1;
-                x[5] = p1 ? col[(size_t)checked_node(u1.y, gp.n) * W] : -1;
-                x[6] = p1 ? col[(size_t)checked_node(u1.z, gp.n) * W] : -1;
-                x[7] = p1 ? col[(size_t)checked_node(u1.w, gp.n) * W] : -1;
-#pragma unroll
-                for (int t = 0; t < 8; ++t) c += x[t] == own;
+            const int i = e % kMaxPop;
+            const int4 r = recs[e / kMaxPop];
+            const int deg = has ? r.z : 0;
+            int res;
+            if constexpr (N > kLaneMax) {
+                res = lane_vote<N>(gp, adj, child, r.x, i, r.y, deg, g);
+            } else {
+                const int top = __reduce_max_sync(kFull, deg);
+                if (top <= 8) res = lane_vote<8>(gp, adj, child, r.x, i, r.y, deg, g);
+                else if (top <= 12) res = lane_vote<12>(gp, adj, child, r.x, i, r.y, deg, g);
+                else if (top <= 16) res = lane_vote<16>(gp, adj, child, r.x, i, r.y, deg, g);
+                else if (top <= 20) res = lane_vote<20>(gp, adj, child, r.x, i, r.y, deg, g);
+                else if (top <= 24) res = lane_vote<24>(gp, adj, child, r.x, i, r.y, deg, g);
+                else if (top <= 28) res = lane_vote<28>(gp, adj, child, r.x, i, r.y, deg, g);
+                else res = lane_vote<32>(gp, adj, child, r.x, i, r.y, deg, g);
             }
-            const bool ok = has && 2 * c > r.z;
-            if (ok) {
-                add_degree(gp, hist, own, i, r.z);
-                if (r.z > kLaneMax) atomicAdd(oks + (e >> 7), 1);
-            }
-            settled32 += __popc(__ballot_sync(kFull, ok && r.z <= kLaneMax));
-            const unsigned rest = __ballot_sync(kFull, has && !ok);
-            __syncwarp();
-            if (has && !ok) list[open + __popc(rest & lt)] = (unsigned short)e;
-            open += __popc(rest);
-        }
-        __syncwarp();
-
-        // The exact votes of the open pairs (degrees still descending).
-        int pairs32 = settled32;
-        for (int base = 0; base < open; base += 32) {
-            const bool has = base + lane < open;
-            const int e = has ? list[base + lane] : 0;
-            const int i = e & 127;
-            int4 r = recs[e >> 7];
-            const unsigned big = __ballot_sync(kFull, has && r.z > kLaneMax);
-            if (big) {
-                const unsigned far = __ballot_sync(kFull, has && r.z > 2 * kLaneMax);
-                if (far) defer_pairs(gp, 1, far, idx0 + (e >> 7), i, lane, dlist, dcount);
-                if (big & ~far) defer_pairs(gp, 0, big & ~far, idx0 + (e >> 7), i, lane, dlist, dcount);
-            }
-            const bool mine = has && r.z <= kLaneMax;
-            const int deg = mine ? r.z : 0;
-            const int top = __reduce_max_sync(kFull, deg);
-            if (top == 0) continue;
-            int res, best;
-            if (top <= 8) res = lane_vote<8>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else if (top <= 12) res = lane_vote<12>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else if (top <= 16) res = lane_vote<16>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else if (top <= 20) res = lane_vote<20>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else if (top <= 24) res = lane_vote<24>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else if (top <= 28) res = lane_vote<28>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            else res = lane_vote<32>(gp, adj, child, r.x, i, r.y, deg, g, best);
-            bool same = false;
-            if (mine) {
-                const size_t cell = (size_t)r.x * W + i;
-                same = res == child[cell];
-                if (!same) q[cell] = res;
+            if (has) {
+                q[(size_t)r.x * W + i] = res;
                 add_degree(gp, hist, res, i, deg);
             }
-            pairs32 += __popc(__ballot_sync(kFull, mine));
-            settled32 += __popc(__ballot_sync(kFull, mine && same && r.w == 0 && 2 * best > deg));
-        }
-        // The history: per node above kLaneMax, a sample of the batches below
-        // (the deferred pairs add theirs in mutation_vote_kernel).
-        if (lane < nb && rec.z > kLaneMax) hint[idx0 + lane] = ((uint32_t)nsel << 16) | (uint32_t)oks[lane];
-        if (((item - wide) & 7) == 0 && lane == 0 && pairs32 > 0) {
-            atomicAdd(dcount + kDcountPairs, pairs32);
-            atomicAdd(dcount + kDcountOk, settled32);
         }
         __syncwarp();
     }
-}
-
-// The exact neighbour-majority of one deferred pair (node of degree
-// kLaneMax + 1 .. N) per thread: the pair's labels are gathered into
-// registers, sorted by the merge-exchange network, and the pick(u, t)-th of
-// the t longest runs is the result, u the MTIE word. The thread writes the
-// label into Q, adds deg(v) to the degree histogram and, when the own label is
-// on more than half of the neighbours, counts the pair in the node's hint.
-template <int N>
-__device__ __forceinline__ void mutation_vote_body(const GenParams &gp, int cls, const int4 *__restrict__ nodes,
-                                                   const int4 *__restrict__ adj, const int32_t *__restrict__ child,
-                                                   int32_t *__restrict__ q, const uint32_t *__restrict__ gen_ptr,
-                                                   uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
-                                                   const int2 *__restrict__ dlist, const int *__restrict__ dcount,
-                                                   int vblock, int vgrid)
-{
-    constexpr int NW = (N + 63) / 64;
-    const uint32_t g = *gen_ptr;
-    const int W = gp.W;
-    const int total = min(dcount[cls], defer_capacity(gp, cls));
-    const int2 *list = dlist + defer_offset(gp, cls);
-    for (int t = vblock * blockDim.x + threadIdx.x; t < total; t += vgrid * blockDim.x) {
-        const int2 e = list[t];
-        const int i = e.y;
-        if (!MOCD_CHECK(e.x >= 0 && e.x < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;
-        const int4 rec = __ldg(nodes + e.x);
-        const int v = rec.x, deg = min(rec.z, N);
-        const int32_t *col = child + i;
-        int x[N];
-#pragma unroll
-        for (int j = 0; j < N; j += 4) {
-            const bool in = j < deg;
-            const int4 u = in ? __ldg(adj + rec.y + j / 4) : make_int4(0, 0, 0, 0);
-            x[j + 0] = in ? col[(size_t)checked_node(u.x, gp.n) * W] : INT_MAX;
-            x[j + 1] = in ? col[(size_t)checked_node(u.y, gp.n) * W] : INT_MAX;
-            x[j + 2] = in ? col[(size_t)checked_node(u.z, gp.n) * W] : INT_MAX;
-            x[j + 3] = in ? col[(size_t)checked_node(u.w, gp.n) * W] : INT_MAX;
-        }
-        sort_network<N>(x);
-        // Runs of equal labels as in longest_runs, over NW 64-bit words: bit j
-        // of eq is set when entries j and j + 1 (< deg) are equal; each step
-        // m &= m >> 1 (across words) shortens every run of set bits by one,
-        // and the last non-zero m marks the first entry of each longest run.
-        unsigned long long eq[NW], starts[NW], m[NW];
-#pragma unroll
-        for (int w = 0; w < NW; ++w) eq[w] = 0ull;
-#pragma unroll
-        for (int j = 0; j + 1 < N; ++j) eq[j >> 6] |= (x[j] == x[j + 1] ? 1ull : 0ull) << (j & 63);
-        bool any = false;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const int pairs = deg - 1 - 64 * w;  // valid bits of word w
-            const int ents = deg - 64 * w;
-            eq[w] &= pairs >= 64 ? ~0ull : pairs <= 0 ? 0ull : (1ull << pairs) - 1ull;
-            starts[w] = ents >= 64 ? ~0ull : ents <= 0 ? 0ull : (1ull << ents) - 1ull;
-            m[w] = eq[w];
-            any |= eq[w] != 0ull;
-        }
-        int best = 1;
-        while (any) {
-            any = false;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                starts[w] = m[w];
-                const unsigned long long carry = w + 1 < NW ? m[w + 1 < NW ? w + 1 : w] << 63 : 0ull;
-                m[w] &= (m[w] >> 1) | carry;
-                any |= m[w] != 0ull;
-            }
-            ++best;
-        }
-        int tcount = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) tcount += __popcll(starts[w]);
-        unsigned kk = 0;
-        if (tcount > 1) kk = pick_index(tie_word(gp, v, i, g), (uint32_t)tcount);
-        // Position of the kk-th set bit of the starts mask.
-        int pos = 0;
-        unsigned k = kk;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const unsigned c = (unsigned)__popcll(starts[w]);
-            if (k >= c) {
-                k -= c;
-                continue;
-            }
-            unsigned long long mm = starts[w];
-            int p = 64 * w;
-#pragma unroll
-            for (int width = 32; width >= 1; width >>= 1) {
-                const unsigned long long low = mm & ((1ull << width) - 1ull);
-                const unsigned lc = (unsigned)__popcll(low);
-                if (k >= lc) {
-                    k -= lc;
-                    mm >>= width;
-                    p += width;
-                } else {
-                    mm = low;
-                }
-            }
-            pos = p;
-            break;
-        }
-        const int res = select_at<N>(x, pos);
-        const size_t cell = (size_t)v * W + i;
-        q[cell] = res;
-        add_degree(gp, hist, res, i, deg);
-        if (2 * best > deg && res == child[cell]) atomicAdd(hint + e.x, 1u);
-    }
-}
-
-template <int N>
-__global__ void __launch_bounds__(kMutBlock)
-mutation_vote_kernel(const __grid_constant__ GenParams gp, int cls, const int4 *__restrict__ nodes,
-                     const int4 *__restrict__ adj, const int32_t *__restrict__ child, int32_t *__restrict__ q,
-                     const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
-                     const int2 *__restrict__ dlist, const int *__restrict__ dcount)
-{
-    mutation_vote_body<N>(gp, cls, nodes, adj, child, q, gen_ptr, hist, hint, dlist, dcount, blockIdx.x, gridDim.x);
-}
-
-// The deferred votes of one degree class of every member of a batch.
-// (Register cap: the single-member kernel's occupancy, 5 blocks of 128
-// threads for 64 entries; 2 for 128, whose registers do not fit 3 here.)
-template <int N>
-__global__ void __launch_bounds__(kMutBlock, N <= 64 ? 5 : 2)
-mutation_vote_multi_kernel(const BatchMember *__restrict__ members, const int *__restrict__ starts, int count,
-                           int cls)
-{
-    const int k = member_of_block(starts, count);
-    const BatchMember &mb = members[k];
-    const PopState &ps = mb.ps;
-    const GenParams gp = mb.gp;
-    const int b0 = __ldg(starts + k);
-    mutation_vote_body<N>(gp, cls, mb.nodes, mb.adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist, ps.dcount,
-                          (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
 }
 
 // Sum (or maximum) over the hub block; every thread gets it. s_red holds one
@@ -1154,127 +957,146 @@ __device__ __forceinline__ unsigned hub_reduce(unsigned x, unsigned *s_red)
     return r;
 }
 
-// The listed pairs of hubs above kSharedTableMax, a block each: the own
-// label's count if the node's history says it pays, else (or if it leaves the
-// pair open) the exact vote with a count table of the smallest power of two
-// >= 2 deg slots, in shared memory if it fits there (gp.hub_smem_hs), else in
-// the block's slice of global scratch (2 gp.hub_hs ints). Writes the label
-// into Q, adds deg(v) to the histogram and counts the pair in the hub's hint
-// when its own label is on more than half of the neighbours. A block per pair
-// keeps a hub of thousands of neighbours off the critical path: one warp per
-// pair is a chain of deg / 32 dependent table inserts.
+// Exact neighbour-majority of one pair by the whole block: a count table of
+// the smallest power of two >= 2 deg slots (at least 2048). Returns the label
+// to every thread; the tables are free on return.
+__device__ __forceinline__ int block_mode_table(const GenParams &gp, const int32_t *__restrict__ col,
+                                                const int *__restrict__ nbr, int deg, int v, int i, int *hkey,
+                                                int hbits, unsigned *s_red, int *s_tied, uint32_t g, unsigned &mx)
+{
+    const int lane = threadIdx.x & 31;
+    const int HS = 1 << hbits;
+    int *hcnt = hkey + HS;
+    for (int s = threadIdx.x; s < HS; s += kHubBlock) {
+        hkey[s] = -1;
+        hcnt[s] = 0;
+    }
+    if (threadIdx.x == 0) *s_tied = 0;
+    __syncthreads();
+    for (int j0 = 0; j0 < deg; j0 += kHubBlock) {
+        const int j = j0 + threadIdx.x;
+        const bool in = j < deg;
+        const int x = in ? col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] : (int)(0x80000000u | lane);
+        // One insert per distinct label of the warp's neighbours.
+        const unsigned peers = __match_any_sync(kFull, x);
+        if (in && (peers & ((1u << lane) - 1u)) == 0) {
+            uint32_t h = hash_slot(x, hbits);
+            for (int probe = 0; probe < HS; ++probe) {  // (at most HS / 2 distinct labels: a slot is found)
+                const int prev = atomicCAS(hkey + h, -1, x);
+                if (prev == -1 || prev == x) {
+                    atomicAdd(hcnt + h, __popc(peers));
+                    break;
+                }
+                h = (h + 1) & (uint32_t)(HS - 1);
+            }
+        }
+    }
+    __syncthreads();
+    unsigned my = 0;
+    for (int s = threadIdx.x; s < HS; s += kHubBlock) my = max(my, (unsigned)hcnt[s]);
+    mx = hub_reduce<true>(my, s_red);
+    // The tied labels, compacted to hcnt[0, tied) once every thread has read
+    // its slots' counts.
+    for (int s = threadIdx.x; s < HS; s += kHubBlock)
+        if ((unsigned)hcnt[s] != mx) hkey[s] = -1;
+    __syncthreads();
+    for (int s = threadIdx.x; s < HS; s += kHubBlock) {  // (HS is a multiple of the block: warps stay whole)
+        const int key = hkey[s];
+        const unsigned who = __ballot_sync(kFull, key >= 0);
+        int at = 0;
+        if (lane == 0 && who) at = atomicAdd(s_tied, __popc(who));
+        at = __shfl_sync(kFull, at, 0);
+        if (key >= 0) hcnt[at + __popc(who & ((1u << lane) - 1u))] = key;
+    }
+    __syncthreads();
+    const int tied = *s_tied;
+    int res = hcnt[0];
+    if (tied > 1) {
+        // Bit by bit from the top, as in warp_mode_table.
+        unsigned prefix = 0, rank = pick_index(tie_word(gp, v, i, g), (uint32_t)tied);
+        for (int b = gp.label_bits - 1; b >= 0; --b) {
+            const unsigned above = ~((2u << b) - 1u);  // the bits above b
+            unsigned c = 0;
+            for (int s = threadIdx.x; s < tied; s += kHubBlock) {
+                const unsigned key = (unsigned)hcnt[s];
+                c += ((key & above) == prefix && ((key >> b) & 1u) == 0u) ? 1u : 0u;
+            }
+            const unsigned cnt = hub_reduce<false>(c, s_red);
+            if (rank >= cnt) {
+                rank -= cnt;
+                prefix |= 1u << b;
+            }
+        }
+        res = (int)prefix;
+    }
+    __syncthreads();
+    return res;
+}
+
+// The hubs, degree above kSharedTableMax (positions 0 .. n_hub - 1): a block
+// per hub and quad of children, about one pair. The own label's count if the
+// last generation says it pays, else (or if it leaves the pair open) the exact
+// vote with a count table in shared memory if it fits there
+// (gp.hub_smem_hs), else in the block's slice of global scratch (2 gp.hub_hs
+// ints). A block per pair keeps a hub of thousands of neighbours off the
+// critical path: one warp per pair is a chain of deg / 32 dependent inserts.
+// The hint slot of (hub, quad) is that block's alone.
 __global__ void __launch_bounds__(kHubBlock)
 mutation_hub_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict__ nodes,
                     const int4 *__restrict__ adj, const int32_t *__restrict__ child, int32_t *__restrict__ q,
                     const uint32_t *__restrict__ gen_ptr, uint32_t *__restrict__ hist, uint32_t *__restrict__ hint,
-                    const int2 *__restrict__ dlist, const int *__restrict__ dcount, int *__restrict__ hub_table)
+                    int *__restrict__ hub_table)
 {
     extern __shared__ int s_table[];  // [2 gp.hub_smem_hs]
     __shared__ unsigned s_red[kHubBlock / 32];
-    __shared__ int s_tied, s_res;
+    __shared__ int s_tied;
     const uint32_t g = *gen_ptr;
-    const int lane = threadIdx.x & 31;
-    const int total = min(dcount[2], defer_capacity(gp, 2));
-    const int2 *list = dlist + defer_offset(gp, 2);
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const int2 e = list[t];
-        const int idx = e.x & ~kHubFast, i = e.y;
-        if (!MOCD_CHECK(idx >= 0 && idx < gp.n && i >= 0 && i < gp.np, kCheckNode, t)) continue;  // (block-uniform)
+    const int nq = gp.W >> 2;
+    for (int t = blockIdx.x; t < gp.n_hub * nq; t += gridDim.x) {
+        const int idx = t / nq, quad = t % nq;
         const int4 rec = __ldg(nodes + idx);
         const int v = rec.x, deg = min(rec.z, gp.hub_hs / 2);
         const int *nbr = reinterpret_cast<const int *>(adj + rec.y);
-        const int32_t *col = child + i;
-        const size_t cell = (size_t)v * gp.W + i;
-        const int own = child[cell];
-        if (e.x & kHubFast) {
-            unsigned c = 0;
-#pragma unroll 4
-            for (int j = threadIdx.x; j < deg; j += kHubBlock)
-                c += col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] == own ? 1u : 0u;
-            if (2 * (int)hub_reduce<false>(c, s_red) > deg) {  // (Q holds the own label already)
-                if (threadIdx.x == 0) {
-                    add_degree(gp, hist, own, i, deg);
-                    atomicAdd(hint + idx, 1u);
-                }
-                continue;
-            }
-        }
+        uint32_t *h = hint + gp.n_wide * kWideParts + t;
+        const bool fast = own_label_pays(*h);
+        const int4 own4 = reinterpret_cast<const int4 *>(child)[(size_t)v * nq + quad];
+        unsigned sel;
+        if (threadIdx.x == 0)
+            sel = take_quad(gp, v, deg, quad, own4, g, reinterpret_cast<int4 *>(q), hist);
+        else
+            sel = selected(gp, v, quad, g);
         int hbits = 11;
         while ((1 << hbits) < 2 * deg) ++hbits;
-        const int HS = 1 << hbits;
-        int *hkey = HS <= gp.hub_smem_hs ? s_table : hub_table + (size_t)blockIdx.x * 2 * gp.hub_hs;
-        int *hcnt = hkey + HS;
-        for (int s = threadIdx.x; s < HS; s += kHubBlock) {
-            hkey[s] = -1;
-            hcnt[s] = 0;
-        }
-        if (threadIdx.x == 0) s_tied = 0;
-        __syncthreads();
-        for (int j0 = 0; j0 < deg; j0 += kHubBlock) {
-            const int j = j0 + threadIdx.x;
-            const bool in = j < deg;
-            const int x = in ? col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] : (int)(0x80000000u | lane);
-            // One insert per distinct label of the warp's neighbours.
-            const unsigned peers = __match_any_sync(kFull, x);
-            if (in && (peers & ((1u << lane) - 1u)) == 0) {
-                uint32_t h = hash_slot(x, hbits);
-                for (int probe = 0; probe < HS; ++probe) {  // (at most HS / 2 distinct labels: a slot is found)
-                    const int prev = atomicCAS(hkey + h, -1, x);
-                    if (prev == -1 || prev == x) {
-                        atomicAdd(hcnt + h, __popc(peers));
-                        break;
-                    }
-                    h = (h + 1) & (uint32_t)(HS - 1);
-                }
-            }
-        }
-        __syncthreads();
-        unsigned my = 0;
-        for (int s = threadIdx.x; s < HS; s += kHubBlock) my = max(my, (unsigned)hcnt[s]);
-        const unsigned mx = hub_reduce<true>(my, s_red);
-        // The tied labels, compacted to hcnt[0, tied) once every thread has
-        // read its slots' counts.
-        for (int s = threadIdx.x; s < HS; s += kHubBlock)
-            if ((unsigned)hcnt[s] != mx) hkey[s] = -1;
-        __syncthreads();
-        for (int s = threadIdx.x; s < HS; s += kHubBlock) {  // (HS is a multiple of the block: warps stay whole)
-            const int key = hkey[s];
-            const unsigned who = __ballot_sync(kFull, key >= 0);
-            int at = 0;
-            if (lane == 0 && who) at = atomicAdd(&s_tied, __popc(who));
-            at = __shfl_sync(kFull, at, 0);
-            if (key >= 0) hcnt[at + __popc(who & ((1u << lane) - 1u))] = key;
-        }
-        __syncthreads();
-        const int tied = s_tied;
-        if (tied == 1) {
-            if (threadIdx.x == 0) s_res = hcnt[0];
-        } else {
-            // Bit by bit from the top, as in warp_mode_table.
-            unsigned prefix = 0, rank = pick_index(tie_word(gp, v, i, g), (uint32_t)tied);
-            for (int b = gp.label_bits - 1; b >= 0; --b) {
-                const unsigned above = ~((2u << b) - 1u);  // the bits above b
+        int *hkey = (1 << hbits) <= gp.hub_smem_hs ? s_table : hub_table + (size_t)blockIdx.x * 2 * gp.hub_hs;
+        const int pairs = __popc(sel);
+        int ok = 0;
+        __syncthreads();  // (every thread has read the hint)
+        for (int k = 0; k < 4; ++k) {
+            if (!((sel >> k) & 1u)) continue;  // (block-uniform)
+            const int i = 4 * quad + k;
+            const int own = k == 0 ? own4.x : k == 1 ? own4.y : k == 2 ? own4.z : own4.w;
+            const int32_t *col = child + i;
+            bool settled = false;
+            if (fast) {
                 unsigned c = 0;
-                for (int s = threadIdx.x; s < tied; s += kHubBlock) {
-                    const unsigned key = (unsigned)hcnt[s];
-                    c += ((key & above) == prefix && ((key >> b) & 1u) == 0u) ? 1u : 0u;
-                }
-                const unsigned cnt = hub_reduce<false>(c, s_red);
-                if (rank >= cnt) {
-                    rank -= cnt;
-                    prefix |= 1u << b;
-                }
+#pragma unroll 4
+                for (int j = threadIdx.x; j < deg; j += kHubBlock)
+                    c += col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] == own ? 1u : 0u;
+                settled = 2 * (int)hub_reduce<false>(c, s_red) > deg;
             }
-            if (threadIdx.x == 0) s_res = (int)prefix;
+            int lab = own;
+            if (!settled) {
+                unsigned mx = 0;
+                lab = block_mode_table(gp, col, nbr, deg, v, i, hkey, hbits, s_red, &s_tied, g, mx);
+                settled = !fast && lab == own && 2 * (int)mx > deg;
+            }
+            ok += settled ? 1 : 0;
+            if (threadIdx.x == 0) {
+                if (lab != own) q[(size_t)v * gp.W + i] = lab;
+                add_degree(gp, hist, lab, i, deg);
+            }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int lab = s_res;
-            q[cell] = lab;
-            add_degree(gp, hist, lab, i, deg);
-            if (lab == own && 2 * (int)mx > deg) atomicAdd(hint + idx, 1u);
-        }
-        __syncthreads();
+        if (threadIdx.x == 0) *h = ((uint32_t)pairs << 16) | (uint32_t)ok;
     }
 }
 
@@ -1317,16 +1139,13 @@ cudaError_t launch_crossover(const GenParams &gp, const PopState &ps, int grid, 
 {
     if (gp.es <= 4)
         crossover_kernel<4><<<grid, kBlock, crossover_smem<4>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen,
-            ps.dcount);
+            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
     else if (gp.es <= 8)
         crossover_kernel<8><<<grid, kBlock, crossover_smem<8>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen,
-            ps.dcount);
+            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
     else
         crossover_kernel<16><<<grid, kBlock, crossover_smem<16>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen,
-            ps.dcount);
+            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
     return cudaGetLastError();
 }
 
@@ -1343,37 +1162,48 @@ cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts
     return cudaGetLastError();
 }
 
-cudaError_t launch_vote_multi(const BatchMember *members, const int *starts, int count, int blocks, int cls,
-                              cudaStream_t s)
-{
-    if (blocks <= 0) return cudaSuccess;
-    if (cls == 0)
-        mutation_vote_multi_kernel<2 * kLaneMax><<<blocks, kMutBlock, 0, s>>>(members, starts, count, 0);
-    else
-        mutation_vote_multi_kernel<kDeferMax><<<blocks, kMutBlock, 0, s>>>(members, starts, count, 1);
-    return cudaGetLastError();
-}
-
-int mutation_smem(int hash_size)
-{
-    return (kMutBlock / 32) * 2 * hash_size * (int)sizeof(int);
-}
-
 int mutation_warps_per_block()
 {
     return kMutBlock / 32;
 }
 
-int grid_for_mutation(int sms, int hash_size)
+namespace {
+
+// Class c: 0: degree <= 32 (and the wide nodes), 1: 33..64, 2: 65..128.
+using MutationFn = void (*)(GenParams, int, int, const int4 *, const int4 *, const int32_t *, int32_t *,
+                            const uint32_t *, uint32_t *, unsigned long long *, uint32_t *, int);
+
+MutationFn mutation_fn(int cls, int vote_n0, bool wide)
 {
-    const int smem = mutation_smem(hash_size);
-    int per_sm = 0;
-    if (hash_size > 0) {
-        cudaFuncSetAttribute(mutation_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_kernel<true>, kMutBlock, smem);
-    } else {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_kernel<false>, kMutBlock, 0);
+    if (cls == 0) return wide ? mutation_kernel<kLaneMax, true> : mutation_kernel<kLaneMax, false>;
+    if (cls == 2) return mutation_kernel<kDeferMax, false>;
+    // The class's network holds the graph's largest degree in it.
+    switch (vote_n0) {
+    case 40: return mutation_kernel<40, false>;
+    case 48: return mutation_kernel<48, false>;
+    case 56: return mutation_kernel<56, false>;
+    default: return mutation_kernel<2 * kLaneMax, false>;
     }
+}
+
+}  // namespace
+
+namespace {
+
+size_t mutation_smem(int np, int batch, int cls, int hash_size)
+{
+    return (size_t)(kMutBlock / 32) * mutation_warp_words(np, batch, cls == 0 ? hash_size : 0) * sizeof(int4);
+}
+
+}  // namespace
+
+int grid_for_mutation(int sms, int cls, int vote_n0, int hash_size, int np, int batch)
+{
+    const MutationFn fn = mutation_fn(cls, vote_n0, hash_size > 0);
+    const size_t smem = mutation_smem(np, batch, cls, hash_size);
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kMutBlock, smem);
     return sms * (per_sm < 1 ? 1 : per_sm);
 }
 
@@ -1387,66 +1217,31 @@ int grid_for_hubs(int sms, int smem_hs)
     return sms * (per_sm < 1 ? 1 : per_sm);
 }
 
-void grid_for_votes(int sms, int vote_n0, int *grid64, int *grid128)
+cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj,
+                            const MutationShape &shape, cudaStream_t s)
 {
-    int a = 0, b = 0;
-    switch (vote_n0) {
-    case 40: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<40>, kMutBlock, 0); break;
-    case 48: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<48>, kMutBlock, 0); break;
-    case 56: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<56>, kMutBlock, 0); break;
-    default:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, mutation_vote_kernel<2 * kLaneMax>, kMutBlock, 0);
+    // The launches are independent of each other: on a capturing stream they
+    // become parallel branches, the longest votes first.
+    Branches br(s);
+    if (gp.n_hub > 0) {
+        mutation_hub_kernel<<<shape.hub_blocks, kHubBlock, 2 * gp.hub_smem_hs * sizeof(int), s>>>(
+            gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.hub_table);
+        br.next();
     }
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, mutation_vote_kernel<kDeferMax>, kMutBlock, 0);
-    *grid64 = sms * (a < 1 ? 1 : a);
-    *grid128 = sms * (b < 1 ? 1 : b);
-}
-
-namespace {
-
-template <int N>
-void launch_vote(const GenParams &gp, const PopState &ps, int cls, const int4 *nodes, const int4 *adj, int grid,
-                 cudaStream_t s)
-{
-    mutation_vote_kernel<N><<<grid, kMutBlock, 0, s>>>(gp, cls, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint,
-                                                       ps.dlist, ps.dcount);
-}
-
-}  // namespace
-
-cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj, int batch,
-                            int grid, int grid64, int grid128, cudaStream_t s, bool with_votes)
-{
-    if (gp.hash_size > 0)
-        mutation_kernel<true><<<grid, kMutBlock, mutation_smem(gp.hash_size), s>>>(
-            gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.acc, ps.hint, ps.dlist, ps.dcount, batch);
-    else
-        mutation_kernel<false><<<grid, kMutBlock, 0, s>>>(gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.acc, ps.hint,
-                                                          ps.dlist, ps.dcount, batch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (with_votes && gp.defer_cap[0] > 0) {
-        // The class's network holds the graph's largest degree in it.
-        switch (gp.vote_n0) {
-        case 40: launch_vote<40>(gp, ps, 0, nodes, adj, grid64, s); break;
-        case 48: launch_vote<48>(gp, ps, 0, nodes, adj, grid64, s); break;
-        case 56: launch_vote<56>(gp, ps, 0, nodes, adj, grid64, s); break;
-        default: launch_vote<2 * kLaneMax>(gp, ps, 0, nodes, adj, grid64, s);
+    int first = gp.n_hub + gp.n_wide;
+    for (int cls = 2; cls >= 0; --cls) {
+        const int last = cls == 0 ? gp.n : first + gp.n_vote[cls - 1];
+        if (cls == 0 || last > first) {
+            mutation_fn(cls, gp.vote_n0, gp.hash_size > 0)<<<shape.grid[cls], kMutBlock,
+                                                             mutation_smem(gp.np, shape.batch[cls], cls, gp.hash_size),
+                                                             s>>>(
+                gp, first, last, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.acc, ps.hint, shape.batch[cls]);
+            br.next();
         }
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+        first = last;
     }
-    if (with_votes && gp.defer_cap[1] > 0) {
-        launch_vote<kDeferMax>(gp, ps, 1, nodes, adj, grid128, s);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    if (gp.defer_cap[2] > 0) {
-        mutation_hub_kernel<<<gp.hub_blocks, kHubBlock, 2 * gp.hub_smem_hs * sizeof(int), s>>>(
-            gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.dlist, ps.dcount, ps.hub_table);
-        e = cudaGetLastError();
-    }
-    return e;
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : br.join();
 }
 
 }  // namespace mocd

@@ -16,6 +16,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 struct mocd_ctx;
 
 namespace mocd {
@@ -36,10 +38,10 @@ bool inject_failure(int site, int *status);
 constexpr int kMaxPop = 128;      // N_p limit: one int4 of labels per lane per row
 constexpr int kMaxParents = 16;   // E_S limit
 constexpr int kBlock = 256;       // threads per block of the node-parallel kernels
-// Mutation votes of nodes with degree 33..kDeferMax that the own label's count
-// leaves open run one pair per thread in a second kernel (degree classes
-// 33..64 and 65..128).
+// Mutation: up to this degree a pair's vote is one thread's, its labels sorted
+// in registers (launches for degrees up to 32, 33..64 and 65..128).
 constexpr int kDeferMax = 128;
+constexpr int kMutBatchMax = 16;  // most nodes a warp of the mutation takes at a time
 // Up to this degree a pair's vote is a warp's, with a count table in shared
 // memory; above it a block's (mutation_hub_kernel).
 constexpr int kSharedTableMax = 512;
@@ -48,16 +50,6 @@ constexpr int kSharedTableMax = 512;
 constexpr int kWideParts = 8;
 // Largest count table of the hub kernel in shared memory (slots of 8 bytes).
 constexpr int kHubSmemSlots = 16384;
-// Set in the node of a listed hub pair when the own label's count is to be
-// tried first (node positions are below 2^30).
-constexpr int kHubFast = 1 << 30;
-// Words of PopState::dcount: [0, 3) deferred pairs per class, then the sampled
-// pairs of degree <= 32, those of them whose own label was on more than half
-// of the neighbours, and whether the next generation counts it first.
-constexpr int kDcountPairs = 3;
-constexpr int kDcountOk = 4;
-constexpr int kDcountFast = 5;
-
 // Random stream stages (third word of the Philox counter is the generation).
 constexpr uint32_t kStageInit = 1;
 constexpr uint32_t kStageSelect = 2;
@@ -83,10 +75,8 @@ struct PopState {
     int64_t *fint;            // [2][kMaxPop]: intra, S of each front member
     double *fval;             // [2][kMaxPop]: f1, f2 of each front member
     uint32_t *hint;           // (mutating pairs << 16) | pairs whose own label is on more than half of the
-                              // neighbours, last generation: [n] by position in the order (degree > 32), then
-                              // kWideParts per node of degree kDeferMax + 1 .. kSharedTableMax
-    int2 *dlist;              // deferred mutation votes (node position, child): class 0, 1, then hubs
-    int *dcount;              // [6]: see kDcountPairs
+                              // neighbours, last generation: kWideParts per node of degree kDeferMax + 1 ..
+                              // kSharedTableMax, then one per hub and quad of children
     int *hub_table;           // hub_blocks x 2 hub_hs: count tables of hubs too large for shared memory
 };
 
@@ -98,10 +88,9 @@ struct GenParams {
     int label_bits;           // bits needed for a label in [0, n)
     int hash_size;            // per-warp hash entries for degree > kDeferMax (0: none)
     int n_hub, n_wide;        // nodes of degree > kSharedTableMax, and of kDeferMax + 1 .. kSharedTableMax
-    int defer_cap[3];         // deferred-vote capacity per class: N_p x nodes of the class
+    int n_vote[2];            // nodes of degree 33..64 and 65..128
     int hub_hs;               // slots of the largest hub's count table (power of two >= 2 dmax; 0: no hubs)
     int hub_smem_hs;          // slots of the hub kernel's shared table (<= kHubSmemSlots)
-    int hub_blocks;           // blocks of mutation_hub_kernel
     int vote_n0;              // entries of the degree 33..64 vote's sorting network: the smallest multiple
                               // of 8 that holds the graph's largest degree in that class (40, 48, 56 or 64)
     int64_t m;                // edges
@@ -132,23 +121,38 @@ cudaError_t launch_init_population(const GenParams &gp, int init_mode, const int
 cudaError_t launch_crossover(const GenParams &gp, const PopState &ps, int grid, cudaStream_t s);
 // order: the nodes in the sequence the grid-stride loop visits them
 // (degree descending), or NULL for 0..n-1 (evaluation only).
-// with_votes false: the per-pair votes of the deferred classes are left to
-// launch_vote_multi (a batch launches them for all members at once).
-// nodes / adj: see mocd_ctx::d_nodes; batch: nodes a warp takes at a time.
-cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj, int batch,
-                            int grid, int grid64, int grid128, cudaStream_t s, bool with_votes = true);
+// nodes / adj: see mocd_ctx::d_nodes.
+struct MutationShape {
+    int batch[3];    // nodes a warp takes at a time, by class (degree <= 32, 33..64, 65..128)
+    int grid[3];     // blocks
+    int hub_blocks;  // blocks of the hub kernel
+};
+cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj,
+                            const MutationShape &shape, cudaStream_t s);
+
+// Launches on one capturing stream as parallel branches of the graph: each
+// next() ends a branch and puts the stream back to where the object was made;
+// join() makes what follows depend on every branch. On a stream that does not
+// capture, the launches simply follow each other.
+class Branches {
+  public:
+    explicit Branches(cudaStream_t s);
+    void next();
+    cudaError_t join();
+
+  private:
+    cudaStream_t s_;
+    bool capturing_ = false;
+    cudaError_t status_ = cudaSuccess;
+    std::vector<cudaGraphNode_t> root_, ends_;
+};
 // Multi-member launches of a batch: member k owns blocks starts[k] ..
 // starts[k + 1] - 1 of the launch's `blocks` (each member's own grid for
 // the stage; zero for a member with nothing to do).
 cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts, int count, int blocks, int es_max,
                                    cudaStream_t s);
-cudaError_t launch_vote_multi(const BatchMember *members, const int *starts, int count, int blocks, int cls,
-                              cudaStream_t s);
 cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts, int count, int blocks,
                                   cudaStream_t s);
-// Resident-block grids of the two per-pair vote kernels (degree classes
-// 33..64 and 65..128).
-void grid_for_votes(int sms, int vote_n0, int *grid64, int *grid128);
 // hist: label-major [n][W] (label_major) or individual-major [count][n],
 // zeroed by the caller.
 cudaError_t launch_evaluate(int n, int W, int count, const int32_t *row_ptr, const int32_t *col_idx,
@@ -209,7 +213,7 @@ cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *ep
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order);
 int grid_for_crossover(int sms, int es);
-int grid_for_mutation(int sms, int hash_size);
+int grid_for_mutation(int sms, int cls, int vote_n0, int hash_size, int np, int batch);
 int grid_for_hubs(int sms, int smem_hs);
 int mutation_warps_per_block();
 

@@ -30,8 +30,8 @@ using namespace mocd;
 namespace {
 
 constexpr int kStages = 4;
-constexpr long long kMutWaves = 2;      // batches per resident warp of the mutation
-constexpr long long kMutBatchMax = 8;   // and the most nodes of a batch
+constexpr long long kMutWaves = 2;    // batches per resident warp of the mutation
+constexpr double kMutPairs = 160.0;   // and the pairs a batch aims at
 
 }  // namespace
 
@@ -43,7 +43,8 @@ struct mocd_ctx {
 
     int64_t n = 0, m = 0;
     int dmax = 0;
-    int64_t n_defer[3] = {0, 0, 0};  // nodes of degree 33..64, 65..128 and > 512 (deferred mutation votes)
+    int64_t n_vote[2] = {0, 0};      // nodes of degree 33..64 and 65..128
+    int64_t n_hub = 0;               // nodes of degree > 512
     int64_t n_wide = 0;              // nodes of degree 129..512
     int32_t *d_row_ptr = nullptr;
     int32_t *d_col_idx = nullptr;
@@ -69,14 +70,13 @@ struct mocd_ctx {
     size_t pop_cells = 0;   // n * W of the allocated label buffers
     size_t hist_cap = 0;    // entries of ps.hist
     size_t hint_cap = 0;    // entries of ps.hint
-    size_t dlist_cap = 0;   // entries of ps.dlist
     size_t hub_cap = 0;     // entries of ps.hub_table
     void *d_small = nullptr;
-    int grid_eval = 0, grid_cross = 0, grid_mut = 0;
-    int grid_eval_intra = 0, grid_vote64 = 0, grid_vote128 = 0;
-    int occ_eval = 0, occ_cross = 0, occ_mut = 0;  // occupancy-limited grids
+    int grid_eval = 0, grid_cross = 0;
+    int grid_eval_intra = 0;
+    MutationShape mut{};
+    int occ_eval = 0, occ_cross = 0;  // occupancy-limited grids
     int occ_eval_intra = 0;
-    int mut_batch = 1;                              // nodes a warp of the mutation takes at a time
     int nodes_per_warp = 1;                         // launch shape (autotuned for batches)
     int32_t host_gen = 0;   // generations run since init
     int32_t version = 0;    // bumped whenever the population is (re)built
@@ -202,7 +202,6 @@ void free_population(mocd_ctx *c)
     dev_free(c->ps.c, c->stream);
     dev_free(c->ps.hist, c->stream);
     dev_free(c->ps.hint, c->stream);
-    dev_free(c->ps.dlist, c->stream);
     dev_free(c->ps.hub_table, c->stream);
     dev_free(c->d_small, c->stream);
     c->ps = PopState{};
@@ -210,7 +209,6 @@ void free_population(mocd_ctx *c)
     c->pop_cells = 0;
     c->hist_cap = 0;
     c->hint_cap = 0;
-    c->dlist_cap = 0;
     c->hub_cap = 0;
     c->ready = false;
 }
@@ -248,24 +246,28 @@ void size_grids(mocd_ctx *c)
     c->grid_eval = shape(c->occ_eval, kBlock / 32);
     c->grid_eval_intra = shape(c->occ_eval_intra, kBlock / 32);
     c->grid_cross = shape(c->occ_cross, kBlock / 32);
-    // The mutation: batches of nodes fill its lanes (see mutation_kernel), but
-    // a graph too small to give every resident warp kMutWaves batches gets
-    // smaller ones.
-    {
-        const long long wide = (long long)c->n_defer[2] + (long long)c->n_wide * kWideParts;
-        const long long normal = n - c->n_defer[2] - c->n_wide;
-        const long long warps = (long long)c->occ_mut * mutation_warps_per_block();
-        c->mut_batch = (int)std::max<long long>(1, std::min<long long>(kMutBatchMax, normal / (kMutWaves * warps)));
-        const long long items = wide + (normal + c->mut_batch - 1) / c->mut_batch;
+    // The mutation: a batch of nodes fills a warp's lanes with pairs (about
+    // kMutPairs of them: five full rounds), but a class too small to give
+    // every resident warp kMutWaves batches gets smaller ones.
+    const double pairs = std::max(0.5, c->params.p_mutation * c->params.pop_size);
+    for (int cls = 0; cls < 3; ++cls) {
+        const long long nodes = cls > 0 ? c->n_vote[cls - 1] : n - c->n_vote[0] - c->n_vote[1] - c->n_wide - c->n_hub;
+        const long long wide = cls == 0 ? (long long)c->n_wide * kWideParts : 0;
+        const int most = (int)std::max<long long>(1, std::min<long long>(kMutBatchMax, (long long)(kMutPairs / pairs)));
+        const int occ = grid_for_mutation(c->sms, cls, c->gp.vote_n0, c->gp.hash_size, c->gp.np, most);
+        const long long warps = (long long)occ * mutation_warps_per_block();
+        c->mut.batch[cls] = (int)std::max<long long>(1, std::min<long long>(most, nodes / (kMutWaves * warps)));
+        const long long items = wide + (nodes + c->mut.batch[cls] - 1) / c->mut.batch[cls];
         const long long per_block = (long long)mutation_warps_per_block() * c->nodes_per_warp;
-        c->grid_mut = (int)std::max<long long>(1, std::min<long long>(c->occ_mut, (items + per_block - 1) / per_block));
+        c->mut.grid[cls] =
+            (int)std::max<long long>(1, std::min<long long>(occ, (items + per_block - 1) / per_block));
     }
 }
 
 // Words of PopState::hint.
 size_t hint_words(const mocd_ctx *c)
 {
-    return (size_t)c->n + (size_t)kWideParts * (size_t)c->n_wide;
+    return (size_t)kWideParts * (size_t)c->n_wide + (size_t)(kMaxPop / 4) * (size_t)c->n_hub;
 }
 
 // Allocate (or reuse) the population buffers for params and fill gp / ps.
@@ -326,18 +328,12 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         c->ps.fint = reinterpret_cast<int64_t *>(q); q += sizeof(int64_t) * 2 * kMaxPop;
         c->ps.fval = reinterpret_cast<double *>(q); q += sizeof(double) * 2 * kMaxPop;
         c->ps.gen = reinterpret_cast<uint32_t *>(q);
-        c->ps.dcount = reinterpret_cast<int *>(q + 16);  // [6], within the 64-byte tail
         CK(cudaMemsetAsync(s, 0, bytes, c->stream));
         CK(cudaMemsetAsync(c->ps.q, 0, cells * sizeof(int32_t), c->stream));
         CK(cudaMemsetAsync(c->ps.buf[0], 0, cells * sizeof(int32_t), c->stream));
         CK(cudaMemsetAsync(c->ps.c + cells, 0x7f, (size_t)W * sizeof(int32_t), c->stream));
     }
     const size_t hist_need = (size_t)W * (size_t)c->n;
-    // The deferred-vote list holds every pair a generation can defer; its
-    // per-class counts are 32-bit.
-    if ((int64_t)p->pop_size * (c->n_defer[0] + c->n_defer[1] + c->n_defer[2]) > INT_MAX)
-        return MOCD_ERR_INVALID_ARG;
-    const size_t defer_need = (size_t)p->pop_size * (size_t)(c->n_defer[0] + c->n_defer[1] + c->n_defer[2]);
     // Hubs: the hub kernel's count table is in shared memory if the largest
     // hub's fits there, else (for the pairs that do not fit) a table of hub_hs
     // slots (keys and counts) per block in global memory, at most 1 GiB in all.
@@ -347,7 +343,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         hub_hs = 2048;
         while (hub_hs < 2 * c->dmax) hub_hs <<= 1;
         hub_smem_hs = std::min(hub_hs, kHubSmemSlots);
-        hub_blocks = grid_for_hubs(c->sms, hub_smem_hs);
+        hub_blocks = (int)std::min<int64_t>(grid_for_hubs(c->sms, hub_smem_hs), c->n_hub * (W / 4));
         if (hub_hs > hub_smem_hs) {
             const int64_t per_block = 2 * (int64_t)hub_hs * (int64_t)sizeof(int);
             const int64_t fit = ((int64_t)1 << 30) / per_block;
@@ -359,7 +355,6 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         int rc = grow(c->stream, &c->ps.hist, &c->hist_cap, hist_need);
         if (rc) return rc;
         if ((rc = grow(c->stream, &c->ps.hint, &c->hint_cap, hint_words(c)))) return rc;
-        if ((rc = grow(c->stream, &c->ps.dlist, &c->dlist_cap, defer_need))) return rc;
         if (hub_need > 0 && (rc = grow(c->stream, &c->ps.hub_table, &c->hub_cap, hub_need))) return rc;
     }
     c->W = W;
@@ -377,14 +372,13 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         while (hs < 2 * std::min(c->dmax, kSharedTableMax)) hs <<= 1;
     }
     gp.hash_size = hs;
-    gp.defer_cap[0] = (int)((int64_t)p->pop_size * c->n_defer[0]);
-    gp.defer_cap[1] = (int)((int64_t)p->pop_size * c->n_defer[1]);
-    gp.defer_cap[2] = (int)((int64_t)p->pop_size * c->n_defer[2]);
-    gp.n_hub = (int)c->n_defer[2];
+    gp.n_vote[0] = (int)c->n_vote[0];
+    gp.n_vote[1] = (int)c->n_vote[1];
+    gp.n_hub = (int)c->n_hub;
     gp.n_wide = (int)c->n_wide;
     gp.hub_hs = hub_hs;
     gp.hub_smem_hs = hub_smem_hs;
-    gp.hub_blocks = hub_blocks;
+    c->mut.hub_blocks = hub_blocks;
     {
         // The degree 33..64 vote's network holds the largest degree of that
         // class in the graph: 40, 48, 56 or 64 entries.
@@ -398,9 +392,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.thr_m = (unsigned long long)floor(p->p_mutation * 4294967296.0);
     c->occ_eval = grid_for_eval(c->sms);
     c->occ_eval_intra = grid_for_eval_intra(c->sms);
-    grid_for_votes(c->sms, gp.vote_n0, &c->grid_vote64, &c->grid_vote128);
     c->occ_cross = grid_for_crossover(c->sms, gp.es);
-    c->occ_mut = grid_for_mutation(c->sms, gp.hash_size);
     size_grids(c);
     return MOCD_OK;
 }
@@ -428,7 +420,7 @@ int issue_generation(mocd_ctx *c, cudaStream_t st, bool events, bool with_select
     if (events) CK(mark(c, 0, st));
     CK(launch_crossover(gp, ps, c->grid_cross, st));
     if (events) CK(mark(c, 1, st));
-    CK(launch_mutation(gp, ps, c->d_nodes, c->d_adj, c->mut_batch, c->grid_mut, c->grid_vote64, c->grid_vote128, st));
+    CK(launch_mutation(gp, ps, c->d_nodes, c->d_adj, c->mut, st));
     if (events) CK(mark(c, 2, st));
     CK(launch_evaluate_offspring(gp.n, gp.W, gp.np, c->d_eptr, c->d_eidx, ps.q, ps.hist, ps.acc,
                                  c->grid_eval_intra, st, c->d_order));
@@ -836,6 +828,38 @@ cudaError_t mocd::dev_alloc(void **p, size_t bytes, cudaStream_t st)
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+mocd::Branches::Branches(cudaStream_t s) : s_(s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t count = 0;
+    status_ = cudaStreamGetCaptureInfo(s_, &st, nullptr, nullptr, &deps, nullptr, &count);
+    if (status_ != cudaSuccess || st != cudaStreamCaptureStatusActive) return;
+    capturing_ = true;
+    root_.assign(deps, deps + count);
+}
+
+void mocd::Branches::next()
+{
+    if (!capturing_ || status_ != cudaSuccess) return;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t count = 0;
+    status_ = cudaStreamGetCaptureInfo(s_, &st, nullptr, nullptr, &deps, nullptr, &count);
+    if (status_ != cudaSuccess) return;
+    ends_.insert(ends_.end(), deps, deps + count);
+    status_ = cudaStreamUpdateCaptureDependencies(s_, root_.data(), nullptr, root_.size(),
+                                                  cudaStreamSetCaptureDependencies);
+}
+
+cudaError_t mocd::Branches::join()
+{
+    if (capturing_ && status_ == cudaSuccess && !ends_.empty())
+        status_ = cudaStreamUpdateCaptureDependencies(s_, ends_.data(), nullptr, ends_.size(),
+                                                      cudaStreamSetCaptureDependencies);
+    return status_;
+}
+
 int mocd::record_on_stream(mocd_ctx *c, cudaEvent_t ev)
 {
     if (!c || !ev) return MOCD_ERR_INVALID_ARG;
@@ -950,10 +974,10 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
     c->dmax = dmax;
     for (int64_t v = 0; v < n; ++v) {
         const int64_t d = row_ptr[v + 1] - row_ptr[v];
-        if (d > 32 && d <= 64) c->n_defer[0] += 1;
-        else if (d > 64 && d <= kDeferMax) c->n_defer[1] += 1;
-        else if (d > kSharedTableMax) c->n_defer[2] += 1;
+        if (d > kSharedTableMax) c->n_hub += 1;
         else if (d > kDeferMax) c->n_wide += 1;
+        else if (d > 64) c->n_vote[1] += 1;
+        else if (d > 32) c->n_vote[0] += 1;
     }
     std::vector<int32_t> rp32(n + 1);
     for (int64_t v = 0; v <= n; ++v) rp32[v] = (int32_t)row_ptr[v];
@@ -1304,15 +1328,15 @@ struct mocd_batch {
     bool own_stream = false;
     // Form 0: each member's kernel chain, selection included, on its own
     // graph branch. Form 1: the selections of all members in one
-    // multi-population launch after the chains. Form 2: also crossover, the
-    // deferred mutation votes and the evaluation of all members in one
-    // multi-member launch each; only the mutation kernels stay per member.
+    // multi-population launch after the chains. Form 2: also crossover and the
+    // evaluation of all members in one multi-member launch each; only the
+    // mutation kernels stay per member.
     int form = 0;
     GenParams *d_gp = nullptr;  // [count], for the merged selection
     PopState *d_ps = nullptr;
     BatchMember *d_members = nullptr;  // [count], for the multi-member launches
-    int *d_starts = nullptr;           // [4][count + 1] block ranges: crossover, votes 33..64, 65..128, evaluation
-    int blocks[4] = {0, 0, 0, 0};      // blocks of each multi-member launch
+    int *d_starts = nullptr;           // [2][count + 1] block ranges: crossover, evaluation
+    int blocks[2] = {0, 0};            // blocks of each multi-member launch
     int es_max = 0;
     std::vector<mocd_ctx *> ctx;
     std::vector<int32_t> version;
@@ -1335,7 +1359,7 @@ static int batch_build(mocd_batch *b)
         std::vector<GenParams> gps;
         std::vector<PopState> pss;
         std::vector<BatchMember> mbs;
-        std::vector<int> starts(4 * (size_t)(count + 1), 0);
+        std::vector<int> starts(2 * (size_t)(count + 1), 0);
         b->es_max = 0;
         for (int i = 0; i < count; ++i) {
             mocd_ctx *c = b->ctx[(size_t)i];
@@ -1344,18 +1368,12 @@ static int batch_build(mocd_batch *b)
             mbs.push_back(BatchMember{c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_nodes, c->d_adj,
                                       c->d_eptr, c->d_eidx});
             b->es_max = std::max(b->es_max, c->gp.es);
-            // Per member and stage: its own grid (a deferred class's votes get
-            // about one thread per four listed pairs at full capacity, at most
-            // its single-member grid).
-            const int g[4] = {
-                c->grid_cross,
-                c->gp.defer_cap[0] > 0 ? std::min(c->grid_vote64, (c->gp.defer_cap[0] + 4 * 128 - 1) / (4 * 128)) : 0,
-                c->gp.defer_cap[1] > 0 ? std::min(c->grid_vote128, (c->gp.defer_cap[1] + 4 * 128 - 1) / (4 * 128)) : 0,
-                c->grid_eval_intra};
-            for (int st = 0; st < 4; ++st)
+            // Per member and stage: its own grid.
+            const int g[2] = {c->grid_cross, c->grid_eval_intra};
+            for (int st = 0; st < 2; ++st)
                 starts[(size_t)st * (count + 1) + i + 1] = starts[(size_t)st * (count + 1) + i] + g[st];
         }
-        for (int st = 0; st < 4; ++st) b->blocks[st] = starts[(size_t)st * (count + 1) + count];
+        for (int st = 0; st < 2; ++st) b->blocks[st] = starts[(size_t)st * (count + 1) + count];
         CK(cudaMemcpyAsync(b->d_gp, gps.data(), sizeof(GenParams) * gps.size(), cudaMemcpyHostToDevice, b->stream));
         CK(cudaMemcpyAsync(b->d_ps, pss.data(), sizeof(PopState) * pss.size(), cudaMemcpyHostToDevice, b->stream));
         CK(cudaMemcpyAsync(b->d_members, mbs.data(), sizeof(BatchMember) * mbs.size(), cudaMemcpyHostToDevice,
@@ -1364,8 +1382,7 @@ static int batch_build(mocd_batch *b)
                            b->stream));
         CK(cudaStreamSynchronize(b->stream));
     }
-    const int *st_cross = b->d_starts, *st_v64 = b->d_starts + (count + 1), *st_v128 = b->d_starts + 2 * (count + 1),
-              *st_eval = b->d_starts + 3 * (count + 1);
+    const int *st_cross = b->d_starts, *st_eval = b->d_starts + (count + 1);
     CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     int rc = MOCD_OK;
     cudaError_t e = cudaSuccess;
@@ -1376,18 +1393,14 @@ static int batch_build(mocd_batch *b)
         e = cudaStreamWaitEvent(b->branch[(size_t)i], b->fork, 0);
         if (e != cudaSuccess) break;
         if (b->form == 2)
-            e = launch_mutation(c->gp, c->ps, c->d_nodes, c->d_adj, c->mut_batch, c->grid_mut, c->grid_vote64,
-                                c->grid_vote128, b->branch[(size_t)i], false);
+            e = launch_mutation(c->gp, c->ps, c->d_nodes, c->d_adj, c->mut, b->branch[(size_t)i]);
         else
             rc = issue_generation(c, b->branch[(size_t)i], false, b->form == 0);
         if (rc == MOCD_OK && e == cudaSuccess) e = cudaEventRecord(b->join[(size_t)i], b->branch[(size_t)i]);
         if (rc == MOCD_OK && e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->join[(size_t)i], 0);
     }
-    if (rc == MOCD_OK && e == cudaSuccess && b->form == 2) {
-        e = launch_vote_multi(b->d_members, st_v64, count, b->blocks[1], 0, b->stream);
-        if (e == cudaSuccess) e = launch_vote_multi(b->d_members, st_v128, count, b->blocks[2], 1, b->stream);
-        if (e == cudaSuccess) e = launch_evaluate_multi(b->d_members, st_eval, count, b->blocks[3], b->stream);
-    }
+    if (rc == MOCD_OK && e == cudaSuccess && b->form == 2)
+        e = launch_evaluate_multi(b->d_members, st_eval, count, b->blocks[1], b->stream);
     if (rc == MOCD_OK && e == cudaSuccess && b->form >= 1)
         e = launch_select_multi(b->d_gp, b->d_ps, count, 1, b->stream);
     cudaGraph_t g = nullptr;
@@ -1438,7 +1451,7 @@ int mocd_batch_create(mocd_batch **out, int32_t count, mocd_ctx *const *ctxs, vo
         if (dev_alloc(&p, sizeof(BatchMember) * (size_t)count, b->stream) != cudaSuccess)
             return fail(MOCD_ERR_OUT_OF_MEMORY);
         b->d_members = static_cast<BatchMember *>(p);
-        if (dev_alloc(&p, sizeof(int) * 4 * (size_t)(count + 1), b->stream) != cudaSuccess)
+        if (dev_alloc(&p, sizeof(int) * 2 * (size_t)(count + 1), b->stream) != cudaSuccess)
             return fail(MOCD_ERR_OUT_OF_MEMORY);
         b->d_starts = static_cast<int *>(p);
     }

@@ -292,14 +292,12 @@ int mocd_job_footprint(int64_t n, const int64_t *row_ptr, int32_t pop_size, int6
 {
     if (!bytes || !row_ptr || n < 1 || pop_size < 1 || pop_size > mocd::kMaxPop) return MOCD_ERR_INVALID_ARG;
     const int64_t nnz = row_ptr[n];
-    int64_t deferred_nodes = 0;  // degree 33 .. kDeferMax and hubs: deferred mutation votes
-    int64_t wide_nodes = 0;      // degree kDeferMax + 1 .. kSharedTableMax: a hint per part
-    int64_t groups = 0;          // of four entries of the mutation's adjacency
+    int64_t hints = 0;   // one per part or quad of children of the nodes above kDeferMax
+    int64_t groups = 0;  // of four entries of the mutation's adjacency
     int64_t dmax = 0;
     for (int64_t v = 0; v < n; ++v) {
         const int64_t d = row_ptr[v + 1] - row_ptr[v];
-        deferred_nodes += ((d > 32 && d <= mocd::kDeferMax) || d > mocd::kSharedTableMax) ? 1 : 0;
-        wide_nodes += (d > mocd::kDeferMax && d <= mocd::kSharedTableMax) ? 1 : 0;
+        hints += d > mocd::kSharedTableMax ? mocd::kMaxPop / 4 : d > mocd::kDeferMax ? mocd::kWideParts : 0;
         groups += (d + 3) / 4;
         dmax = d > dmax ? d : dmax;
     }
@@ -324,7 +322,7 @@ int mocd_job_footprint(int64_t n, const int64_t *row_ptr, int32_t pop_size, int6
     const int64_t W = (pop_size + 3) & ~3;
     const int64_t labels = (4 * n + 1) * W * 4;   // P halves, Q, post-crossover children and their padding row
     const int64_t hist = W * n * 4;               // degree histogram
-    const int64_t mutation = (n + mocd::kWideParts * wide_nodes) * 4 + deferred_nodes * pop_size * 8 + hub_tables;  // hints, deferred votes
+    const int64_t mutation = hints * 4 + hub_tables;
     // CSR, oriented CSR, flag; order, node records, the mutation's rows, the table per degree
     const int64_t graph = 2 * (n + 1) * 4 + (nnz + nnz / 2) * 4 + 4 + n * 4 + 16 + (n + groups) * 16 + (dmax + 1) * 8;
     const int64_t front = (int64_t)pop_size * n * 4 + 2 * mocd::kMaxPop * 4;  // front download
