@@ -18,15 +18,11 @@
 // gathers, and the CSR is streamed once per population, not once per
 // individual.
 //
-// S without a sweep over the histogram: when node v adds deg(v) to D_c, the
-// atomic returns the old total o, and (o + d)^2 - o^2 = 2 o d + d^2. Summed
-// over every addition these increments telescope to D_c^2 whatever the order
-// of the atomics, so S is exact and deterministic.
-//
-// Histogram layout: label-major, D of (individual i, label c) at c * W + i,
-// so that one atomic instruction of a warp (25 individuals of node v) lands
-// in few cache lines whenever individuals share v's label; or
-// individual-major, i * n + c (count * n cells, for fixed-size scratch).
+// S comes from the histogram D, built by reductions (atomics whose old value
+// is not needed, so nothing waits for them) and then squared in a coalesced
+// sweep. Histogram layout: label-major, D of (individual i, label c) at
+// c * stride + i, so that one atomic instruction of a warp (25 individuals of
+// node v) lands in few cache lines whenever individuals share v's label.
 //
 // Inside a generation the D histogram is not built here: the mutation kernel,
 // which writes every child's final label of node v, adds deg(v) to the
@@ -39,6 +35,8 @@
 // histogram) cost a DRAM read and write-back each; done by the mutation
 // kernel, that traffic overlaps with its own work instead of stalling the
 // evaluation's row stream.
+#include <algorithm>
+
 #include "mocd_check.cuh"
 #include "mocd_internal.h"
 
@@ -46,8 +44,9 @@ namespace mocd {
 
 namespace {
 
-template <bool LABEL_MAJOR, bool COUNT_D>
-__device__ __forceinline__ void evaluate_body(int n, int W, int count, const int32_t *__restrict__ row_ptr,
+template <bool COUNT_D>
+__device__ __forceinline__ void evaluate_body(int n, int W, int count, int stride,
+                                              const int32_t *__restrict__ row_ptr,
                                               const int32_t *__restrict__ col_idx,
                                               const int32_t *__restrict__ labels, uint32_t *__restrict__ hist,
                                               unsigned long long *__restrict__ acc,
@@ -72,9 +71,6 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, const int
     int *nb = s_nb + (threadIdx.x & ~31);
     const unsigned lt = (1u << lane) - 1u;
 
-    auto cell = [&](int i, int c) -> size_t {
-        return LABEL_MAJOR ? (size_t)c * W + i : (size_t)i * n + c;
-    };
     uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
     unsigned long long q0 = 0, q1 = 0, q2 = 0, q3 = 0;
 
@@ -112,29 +108,21 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, const int
             }
             __syncwarp();
         }
-        const unsigned long long d = (unsigned long long)(end - beg);
-        if (COUNT_D && active && d > 0) {
-            const unsigned dd = (unsigned)d;
-            if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v)) {
-                const unsigned long long o = atomicAdd(hist + cell(i0 + 0, own.x), dd);
-                q0 += 2ull * o * d + d * d;
-            }
-            if (i0 + 1 < count && MOCD_CHECK((unsigned)own.y < (unsigned)n, kCheckLabel, v)) {
-                const unsigned long long o = atomicAdd(hist + cell(i0 + 1, own.y), dd);
-                q1 += 2ull * o * d + d * d;
-            }
-            if (i0 + 2 < count && MOCD_CHECK((unsigned)own.z < (unsigned)n, kCheckLabel, v)) {
-                const unsigned long long o = atomicAdd(hist + cell(i0 + 2, own.z), dd);
-                q2 += 2ull * o * d + d * d;
-            }
-            if (i0 + 3 < count && MOCD_CHECK((unsigned)own.w < (unsigned)n, kCheckLabel, v)) {
-                const unsigned long long o = atomicAdd(hist + cell(i0 + 3, own.w), dd);
-                q3 += 2ull * o * d + d * d;
-            }
+        if (COUNT_D && active && end > beg) {
+            const unsigned d = (unsigned)(end - beg);
+            uint32_t *cell = hist + i0;
+            if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v))
+                atomicAdd(cell + (size_t)own.x * stride + 0, d);
+            if (i0 + 1 < count && MOCD_CHECK((unsigned)own.y < (unsigned)n, kCheckLabel, v))
+                atomicAdd(cell + (size_t)own.y * stride + 1, d);
+            if (i0 + 2 < count && MOCD_CHECK((unsigned)own.z < (unsigned)n, kCheckLabel, v))
+                atomicAdd(cell + (size_t)own.z * stride + 2, d);
+            if (i0 + 3 < count && MOCD_CHECK((unsigned)own.w < (unsigned)n, kCheckLabel, v))
+                atomicAdd(cell + (size_t)own.w * stride + 3, d);
         }
     }
 
-    if (!COUNT_D && LABEL_MAJOR && active) {
+    if (!COUNT_D && active) {
         // S from the histogram [n][W] that the mutation kernel built: a warp
         // per row, lane q the int4 of individuals 4q..4q+3; every non-zero
         // cell is squared and cleared. D_c^2 < 2^62 and S <= (2m)^2, so the
@@ -161,7 +149,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, const int
             }
         }
     }
-    if (active) {
+    if (active) {  // (S is the square sweep's when COUNT_D)
         if (i0 + 0 < count) { atomicAdd(&s_intra[i0 + 0], (unsigned long long)c0); atomicAdd(&s_sq[i0 + 0], q0); }
         if (i0 + 1 < count) { atomicAdd(&s_intra[i0 + 1], (unsigned long long)c1); atomicAdd(&s_sq[i0 + 1], q1); }
         if (i0 + 2 < count) { atomicAdd(&s_intra[i0 + 2], (unsigned long long)c2); atomicAdd(&s_sq[i0 + 2], q2); }
@@ -174,15 +162,86 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, const int
     }
 }
 
-template <bool LABEL_MAJOR, bool COUNT_D>
+template <bool COUNT_D>
 __global__ void __launch_bounds__(kBlock)
-evaluate_kernel(int n, int W, int count, const int32_t *__restrict__ row_ptr,
+evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col_idx, const int32_t *__restrict__ labels,
                 uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc,
                 const int32_t *__restrict__ order)
 {
-    evaluate_body<LABEL_MAJOR, COUNT_D>(n, W, count, row_ptr, col_idx, labels, hist, acc, order, blockIdx.x,
-                                        gridDim.x);
+    evaluate_body<COUNT_D>(n, W, count, stride, row_ptr, col_idx, labels, hist, acc, order, blockIdx.x, gridDim.x);
+}
+
+// S of `count` individuals from the histogram [n][stride] that evaluate_kernel
+// built, squared and cleared; a thread keeps one column group of VEC cells
+// (stride is a multiple of VEC), four rows in flight. With `out_intra`, the
+// last block to finish writes both results (acc[2 kMaxPop] counts the blocks,
+// zero on entry).
+template <int VEC>
+__global__ void __launch_bounds__(kBlock)
+square_kernel(int n, int stride, int count, uint32_t *__restrict__ hist, unsigned long long *acc,
+              int64_t *__restrict__ out_intra, int64_t *__restrict__ out_sumsq)
+{
+    __shared__ unsigned long long s_sq[kMaxPop];
+    __shared__ bool s_last;
+    for (int t = threadIdx.x; t < kMaxPop; t += blockDim.x) s_sq[t] = 0;
+    __syncthreads();
+    const int groups = stride / VEC;             // per row
+    const int rows = blockDim.x / groups;        // a block takes at a time
+    const int group = threadIdx.x % groups;
+    unsigned long long q[VEC];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) q[k] = 0;
+    if ((int)threadIdx.x < rows * groups) {
+        const long long step = (long long)gridDim.x * rows;
+        for (long long c0 = (long long)blockIdx.x * rows + threadIdx.x / groups; c0 < n; c0 += 4 * step) {
+            uint32_t x[4][VEC];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const long long c = c0 + u * step;
+                const uint32_t *p = hist + (size_t)(c < n ? c : 0) * stride + (size_t)group * VEC;
+                if (VEC == 4) {
+                    const uint4 y = c < n ? *reinterpret_cast<const uint4 *>(p) : make_uint4(0, 0, 0, 0);
+                    x[u][0] = y.x;
+                    x[u][VEC > 1 ? 1 : 0] = y.y;
+                    x[u][VEC > 2 ? 2 : 0] = y.z;
+                    x[u][VEC > 3 ? 3 : 0] = y.w;
+                } else {
+                    x[u][0] = c < n ? *p : 0u;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                uint32_t any = 0;
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) {
+                    q[k] += (unsigned long long)x[u][k] * x[u][k];
+                    any |= x[u][k];
+                }
+                if (!any) continue;
+                uint32_t *p = hist + (size_t)(c0 + u * step) * stride + (size_t)group * VEC;
+                if (VEC == 4) *reinterpret_cast<uint4 *>(p) = make_uint4(0, 0, 0, 0);
+                else *p = 0u;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < VEC; ++k)
+            if (group * VEC + k < count) atomicAdd(&s_sq[group * VEC + k], q[k]);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < count; t += blockDim.x)
+        if (s_sq[t]) atomicAdd(acc + kMaxPop + t, s_sq[t]);
+    if (!out_intra) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(acc + 2 * kMaxPop, 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int t = threadIdx.x; t < count; t += blockDim.x) {
+        out_intra[t] = (int64_t)__ldcg(acc + t);
+        out_sumsq[t] = (int64_t)__ldcg(acc + kMaxPop + t);
+    }
 }
 
 // The offspring evaluation of every member of a batch in one launch: members
@@ -199,19 +258,16 @@ evaluate_multi_kernel(const BatchMember *__restrict__ members, const int *__rest
     }
     const BatchMember &mb = members[lo];
     const int b0 = __ldg(starts + lo);
-    evaluate_body<true, false>(mb.gp.n, mb.gp.W, mb.gp.np, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
-                               mb.order, bk - b0, __ldg(starts + lo + 1) - b0);
+    evaluate_body<false>(mb.gp.n, mb.gp.W, mb.gp.np, mb.gp.W, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
+                         mb.order, bk - b0, __ldg(starts + lo + 1) - b0);
 }
 
 }  // namespace
 
-int grid_for_eval(int sms, bool label_major)
+int grid_for_eval(int sms)
 {
     int per_sm = 0;
-    if (label_major)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<true, true>, kBlock, 0);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<false, true>, kBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<true>, kBlock, 0);
     if (per_sm < 1) per_sm = 1;
     return sms * per_sm;
 }
@@ -219,21 +275,27 @@ int grid_for_eval(int sms, bool label_major)
 int grid_for_eval_intra(int sms)
 {
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<true, false>, kBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<false>, kBlock, 0);
     if (per_sm < 1) per_sm = 1;
     return sms * per_sm;
 }
 
-cudaError_t launch_evaluate(int n, int W, int count, const int32_t *row_ptr, const int32_t *col_idx,
-                            const int32_t *labels, uint32_t *hist, unsigned long long *acc,
-                            int grid, cudaStream_t s, const int32_t *order, bool label_major)
+cudaError_t launch_evaluate(int n, int W, int count, int stride, const int32_t *row_ptr, const int32_t *col_idx,
+                            const int32_t *labels, uint32_t *hist, unsigned long long *acc, int grid, int sms,
+                            cudaStream_t s, const int32_t *order, int64_t *out_intra, int64_t *out_sumsq)
 {
-    if (label_major)
-        evaluate_kernel<true, true><<<grid, kBlock, 0, s>>>(n, W, count, row_ptr, col_idx, labels, hist, acc,
-                                                            order);
+    const long long blocks = std::min<long long>(grid, ((long long)n + kBlock / 32 - 1) / (kBlock / 32));
+    evaluate_kernel<true><<<(int)blocks, kBlock, 0, s>>>(n, W, count, stride, row_ptr, col_idx, labels, hist, acc,
+                                                         order);
+    // Four blocks per SM keep enough rows in flight to stream the histogram;
+    // fewer where that leaves a thread less than one round of rows.
+    const int vec = stride % 4 == 0 ? 4 : 1;
+    const int rows = kBlock / (stride / vec);
+    const int sq = (int)std::min<long long>(4 * sms, ((long long)n + 4 * rows - 1) / (4 * rows));
+    if (vec == 4)
+        square_kernel<4><<<sq, kBlock, 0, s>>>(n, stride, count, hist, acc, out_intra, out_sumsq);
     else
-        evaluate_kernel<false, true><<<grid, kBlock, 0, s>>>(n, W, count, row_ptr, col_idx, labels, hist, acc,
-                                                             order);
+        square_kernel<1><<<sq, kBlock, 0, s>>>(n, stride, count, hist, acc, out_intra, out_sumsq);
     return cudaGetLastError();
 }
 
@@ -248,7 +310,7 @@ cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *ep
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order)
 {
-    evaluate_kernel<true, false><<<grid, kBlock, 0, s>>>(n, W, count, eptr, eidx, labels, hist, acc, order);
+    evaluate_kernel<false><<<grid, kBlock, 0, s>>>(n, W, count, W, eptr, eidx, labels, hist, acc, order);
     return cudaGetLastError();
 }
 

@@ -15,6 +15,8 @@
 #include <limits.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "mocd_internal.h"
 #include "philox.cuh"
 #include "ratio.cuh"
@@ -499,40 +501,71 @@ __global__ void __launch_bounds__(kMaxPop) front_kernel(GenParams gp, PopState p
     ps.front[1] = count ? best : -1;
 }
 
-__global__ void gather_individuals_kernel(int n, int W, int np, const int32_t *__restrict__ phalf,
-                                          const int32_t *__restrict__ q, const int32_t *__restrict__ idx,
-                                          int count, int32_t *__restrict__ out)
+// The layout conversions of the host API go through a shared tile of 32 nodes
+// x 32 individuals, so that both sides are read and written in whole rows
+// (individual-major: 128 bytes of consecutive nodes; node-major: 128 bytes of
+// one node's individuals). A thread per node striding over the individuals
+// touched 32 rows per load instead.
+constexpr int kTile = 32;
+constexpr int kTileThreads = 256;
+constexpr int kTileStep = kTileThreads / 32;
+
+// out[k][v] = R_v[idx[k]] for k < count (idx NULL: identity on P).
+__global__ void __launch_bounds__(kTileThreads)
+gather_individuals_kernel(int n, int W, int np, const int32_t *__restrict__ phalf, const int32_t *__restrict__ q,
+                          const int32_t *__restrict__ idx, int count, int32_t *__restrict__ out)
 {
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        for (int k = 0; k < count; ++k) {
-            const int r = idx ? idx[k] : k;
-            const int32_t val = r < np ? phalf[(size_t)v * W + r] : q[(size_t)v * W + (r - np)];
-            out[(size_t)k * n + v] = val;
-        }
+    __shared__ int32_t tile[kTile][kTile + 1];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int k0 = blockIdx.y * kTile, k = k0 + lane;
+    const int r = k < count ? (idx ? idx[k] : k) : 0;
+    const int32_t *src = r < np ? phalf + r : q + (r - np);
+    for (int v0 = blockIdx.x * kTile; v0 < n; v0 += gridDim.x * kTile) {
+#pragma unroll
+        for (int j = row; j < kTile; j += kTileStep)
+            if (v0 + j < n && k < count) tile[j][lane] = src[(size_t)(v0 + j) * W];
+        __syncthreads();
+#pragma unroll
+        for (int j = row; j < kTile; j += kTileStep)
+            if (k0 + j < count && v0 + lane < n) out[(size_t)(k0 + j) * n + v0 + lane] = tile[lane][j];
+        __syncthreads();
     }
 }
 
-__global__ void to_node_major_kernel(int n, int W, int count, const int32_t *__restrict__ src,
-                                     int32_t *__restrict__ dst)
+// dst[v][k] = src[k][v] for k < count, zero for count <= k < W. A label
+// outside [0, n) sets *bad and becomes 0, so that whatever follows stays in
+// bounds (dst NULL: only the check).
+__global__ void __launch_bounds__(kTileThreads)
+to_node_major_kernel(int n, int W, int count, const int32_t *__restrict__ src, int32_t *__restrict__ dst,
+                     int *__restrict__ bad)
 {
-    const int nq = W >> 2;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        for (int qd = 0; qd < nq; ++qd) {
-            int4 o;
-            const int k = 4 * qd;
-            o.x = k + 0 < count ? src[(size_t)(k + 0) * n + v] : 0;
-            o.y = k + 1 < count ? src[(size_t)(k + 1) * n + v] : 0;
-            o.z = k + 2 < count ? src[(size_t)(k + 2) * n + v] : 0;
-            o.w = k + 3 < count ? src[(size_t)(k + 3) * n + v] : 0;
-            reinterpret_cast<int4 *>(dst)[(size_t)v * nq + qd] = o;
+    __shared__ int32_t tile[kTile][kTile + 1];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int k0 = blockIdx.y * kTile;
+    bool wrong = false;
+    for (int v0 = blockIdx.x * kTile; v0 < n; v0 += gridDim.x * kTile) {
+#pragma unroll
+        for (int j = row; j < kTile; j += kTileStep) {
+            int32_t x = k0 + j < count && v0 + lane < n ? src[(size_t)(k0 + j) * n + v0 + lane] : 0;
+            if ((uint32_t)x >= (uint32_t)n) {
+                wrong = true;
+                x = 0;
+            }
+            tile[j][lane] = x;
         }
+        if (!dst) continue;
+        __syncthreads();
+#pragma unroll
+        for (int j = row; j < kTile; j += kTileStep)
+            if (v0 + j < n && k0 + lane < W) dst[(size_t)(v0 + j) * W + k0 + lane] = tile[lane][j];
+        __syncthreads();
     }
+    if (wrong) *bad = 1;
 }
 
-int blocks_for(int n)
+dim3 tiles_for(int n, int width)
 {
-    int b = (n + 255) / 256;
-    return b < 1 ? 1 : (b > 4096 ? 4096 : b);
+    return dim3((unsigned)std::min((n + kTile - 1) / kTile, 4096), (unsigned)((width + kTile - 1) / kTile));
 }
 
 }  // namespace
@@ -559,14 +592,13 @@ cudaError_t launch_gather_individuals(int n, int W, int np, const int32_t *phalf
                                       const int32_t *idx, int count, int32_t *out, cudaStream_t s)
 {
     if (count <= 0) return cudaSuccess;
-    gather_individuals_kernel<<<blocks_for(n), 256, 0, s>>>(n, W, np, phalf, q, idx, count, out);
+    gather_individuals_kernel<<<tiles_for(n, count), kTileThreads, 0, s>>>(n, W, np, phalf, q, idx, count, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, int32_t *dst,
-                                 cudaStream_t s)
+cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, int32_t *dst, int *bad, cudaStream_t s)
 {
-    to_node_major_kernel<<<blocks_for(n), 256, 0, s>>>(n, W, count, src, dst);
+    to_node_major_kernel<<<tiles_for(n, W), kTileThreads, 0, s>>>(n, W, count, src, dst, bad);
     return cudaGetLastError();
 }
 

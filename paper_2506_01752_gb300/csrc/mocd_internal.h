@@ -153,12 +153,15 @@ cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts
                                    cudaStream_t s);
 cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts, int count, int blocks,
                                   cudaStream_t s);
-// hist: label-major [n][W] (label_major) or individual-major [count][n],
-// zeroed by the caller.
-cudaError_t launch_evaluate(int n, int W, int count, const int32_t *row_ptr, const int32_t *col_idx,
-                            const int32_t *labels, uint32_t *hist, unsigned long long *acc,
-                            int grid, cudaStream_t s, const int32_t *order = nullptr,
-                            bool label_major = true);
+// Objectives of `count` labellings (node-major rows of W) into acc (intra, S;
+// cleared by the caller): edge count and histogram, then the square sweep.
+// hist: [n][stride], stride >= count, zero on entry and again afterwards.
+// out_intra / out_sumsq (optional): the results, written by the sweep (acc
+// then has one more word, zero on entry). grid: grid_for_eval.
+cudaError_t launch_evaluate(int n, int W, int count, int stride, const int32_t *row_ptr, const int32_t *col_idx,
+                            const int32_t *labels, uint32_t *hist, unsigned long long *acc, int grid, int sms,
+                            cudaStream_t s, const int32_t *order = nullptr, int64_t *out_intra = nullptr,
+                            int64_t *out_sumsq = nullptr);
 // mode 0: keys of a fresh P from acc, keep = identity; mode 1: R = P u Q,
 // environmental selection. Both then rank P and draw the next tournament.
 cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s);
@@ -178,8 +181,9 @@ cudaError_t launch_front_stats(const GenParams &gp, const PopState &ps, const in
 // out[k][v] = R_v[idx[k]] for k < count, R_v = (phalf row v | q row v); idx NULL: identity on phalf.
 cudaError_t launch_gather_individuals(int n, int W, int np, const int32_t *phalf, const int32_t *q,
                                       const int32_t *idx, int count, int32_t *out, cudaStream_t s);
-// dst[v][k] = src[k][v] for k < count, zero for count <= k < W.
-cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, int32_t *dst,
+// dst[v][k] = src[k][v] for k < count, zero for count <= k < W; labels outside
+// [0, n) set *bad and become 0. dst NULL: only the check.
+cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, int32_t *dst, int *bad,
                                  cudaStream_t s);
 // The offspring evaluation's oriented adjacency of a host-checked CSR: eptr
 // [n + 1] row pointers, eidx [cap] entries (cap = m for a symmetric graph),
@@ -201,8 +205,7 @@ cudaError_t check_record_eval(unsigned long long *out, bool reset);
 cudaError_t check_record_variation(unsigned long long *out, bool reset);
 
 // Occupancy-derived grid sizes.
-// Resident blocks of the evaluation kernel in the given histogram layout.
-int grid_for_eval(int sms, bool label_major = true);
+int grid_for_eval(int sms);
 int grid_for_eval_intra(int sms);
 // Objectives of the offspring inside a generation: the mutation kernel has
 // already added every child's degrees to the label-major histogram (and

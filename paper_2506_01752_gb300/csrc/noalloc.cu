@@ -27,25 +27,15 @@ using namespace mocd;
 
 namespace {
 
-constexpr size_t kAccWords = 4 * kMaxPop;  // 2 x kMaxPop unsigned long long
+constexpr size_t kAccWords = 4 * kMaxPop + 8;  // 2 x kMaxPop unsigned long long, the sweep's block count, padding
 constexpr size_t kScratchWords = kAccWords + (size_t)MOCD_NOALLOC_MAX_CELLS;
 constexpr int kMaxDevices = 64;
 
-// [0, kAccWords): intra / S accumulators; then the histogram [count][n].
+// [0, kAccWords): intra / S accumulators; then the histogram [n][count].
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 
 uint32_t *g_scratch_addr[kMaxDevices];
 std::mutex g_setup_mutex;
-
-__global__ void finish_keys_kernel(int count, const unsigned long long *__restrict__ acc,
-                                   int64_t *__restrict__ intra, int64_t *__restrict__ sumsq)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) {
-        intra[i] = (int64_t)acc[i];
-        sumsq[i] = (int64_t)acc[kMaxPop + i];
-    }
-}
 
 // Address of the scratch on the current device, set up on first use.
 int scratch_on_current_device(uint32_t **out, int *device)
@@ -89,10 +79,8 @@ extern "C" int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_
         return MOCD_ERR_CUDA;
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MOCD_ERR_CUDA;
-    if (launch_evaluate((int)n, W, count, row_ptr, col_idx, labels, hist, acc, grid_for_eval(sms, false), s,
-                        nullptr, false) != cudaSuccess)
+    if (launch_evaluate((int)n, W, count, count, row_ptr, col_idx, labels, hist, acc, grid_for_eval(sms), sms, s, nullptr,
+                        intra, sumsq) != cudaSuccess)
         return MOCD_ERR_CUDA;
-    finish_keys_kernel<<<1, kMaxPop, 0, s>>>(count, acc, intra, sumsq);
-    if (cudaGetLastError() != cudaSuccess) return MOCD_ERR_CUDA;
     return MOCD_OK;
 }
