@@ -80,355 +80,6 @@ __global__ void init_sweep_kernel(int n, int W, int np, uint32_t k0, uint32_t k1
     }
 }
 
-// ---------------------------------------------------------------------------
-// Crossover. Row v of R = (P half | Q) is staged in shared memory; the next P
-// (environmental selection's keep list) is compacted into the other P half,
-// and child i of the generation gets
-//   copy_r[i] >= 0 : R_v[copy_r[i]]                    (x > C_P: random parent)
-//   otherwise      : majority of R_v[par_r[i][j]], j < E_S, the tie among the t
-//                    most frequent labels broken by the XTIE word: the
-//                    pick(u, t)-th smallest of them (Eq. arg_max).
-// ---------------------------------------------------------------------------
-
-// Count of the maximal label and number t of distinct labels reaching it.
-template <int EMAX>
-__device__ __forceinline__ int mode_ties(const int (&x)[EMAX], int E, int &best)
-{
-    int cnt[EMAX];
-#pragma unroll
-    for (int a = 0; a < EMAX; ++a) {
-        cnt[a] = 0;
-#pragma unroll
-        for (int b = 0; b < EMAX; ++b)
-            if (a < E && b < E && x[b] == x[a]) cnt[a] += 1;
-    }
-    best = 0;
-#pragma unroll
-    for (int a = 0; a < EMAX; ++a)
-        if (a < E && cnt[a] > best) best = cnt[a];
-    int t = 0;
-#pragma unroll
-    for (int a = 0; a < EMAX; ++a) {
-        bool first = a < E && cnt[a] == best;
-#pragma unroll
-        for (int b = 0; b < EMAX; ++b)
-            if (b < a && x[b] == x[a]) first = false;
-        t += first ? 1 : 0;
-    }
-    // Distinct maximal labels: a label's first occurrence is counted once.
-    return t;
-}
-
-// The k-th smallest distinct label among those of count `best`.
-template <int EMAX>
-__device__ __forceinline__ int kth_tied(const int (&x)[EMAX], int E, int best, int k)
-{
-    int res = x[0];
-#pragma unroll
-    for (int a = 0; a < EMAX; ++a) {
-        if (a >= E) continue;
-        int c = 0;
-        bool first = true;
-#pragma unroll
-        for (int b = 0; b < EMAX; ++b) {
-            if (b >= E) continue;
-            c += x[b] == x[a];
-            if (b < a && x[b] == x[a]) first = false;
-        }
-        if (!first || c != best) continue;
-        // rank of x[a] among the distinct tied labels
-        int rank = 0;
-#pragma unroll
-        for (int b = 0; b < EMAX; ++b) {
-            if (b >= E) continue;
-            int cb = 0;
-            bool fb = true;
-#pragma unroll
-            for (int e = 0; e < EMAX; ++e) {
-                if (e >= E) continue;
-                cb += x[e] == x[b];
-                if (e < b && x[e] == x[b]) fb = false;
-            }
-            if (fb && cb == best && x[b] < x[a]) rank += 1;
-        }
-        if (rank == k) res = x[a];
-    }
-    return res;
-}
-
-template <int EMAX>
-__device__ __forceinline__ void crossover_body(const GenParams gp, const int32_t *buf0, const int32_t *buf1,
-                                               int32_t *out0, int32_t *out1, const int32_t *__restrict__ q,
-                                               int32_t *__restrict__ child, const int32_t *__restrict__ keep,
-                                               const int32_t *__restrict__ par_r, const int32_t *__restrict__ copy_r,
-                                               const uint32_t *__restrict__ gen_ptr, int vblock, int vgrid)
-{
-    extern __shared__ int smem[];
-    const int W = gp.W, np = gp.np, E = gp.es;
-    const int nq = W >> 2;
-    // Per-child tables, stored so that lane q reading child 4q + k hits bank q:
-    // entry (k, q) of a table lives at [k * 32 + q] (and [(j * 4 + k) * 32 + q]
-    // for parent j).
-    int *s_keep = smem;                    // row position of P position i
-    int *s_copy = s_keep + kMaxPop;        // row position copied, or -1
-    int *s_par = s_copy + kMaxPop;         // row positions of parents
-    int *s_rows = s_par + kMaxPop * EMAX;  // per warp: [2W] staged row of R
-
-    const uint32_t g = *gen_ptr;
-    // R index r -> position in the staged row (P half at [0, W), Q at [W, 2W)).
-    for (int t = threadIdx.x; t < np; t += blockDim.x) {
-        const int slot = (t & 3) * 32 + (t >> 2);
-        int r = keep[t];
-        if (!MOCD_CHECK(r >= 0 && r < 2 * np, kCheckRIndex, t)) r = 0;
-        s_keep[slot] = r < np ? r : W + (r - np);
-        int c = copy_r[t];
-        if (!MOCD_CHECK(c >= -1 && c < 2 * np, kCheckRIndex, t)) c = 0;
-        s_copy[slot] = c < 0 ? -1 : (c < np ? c : W + (c - np));
-        for (int j = 0; j < E; ++j) {
-            int p = par_r[t * kMaxParents + j];
-            if (!MOCD_CHECK(p >= 0 && p < 2 * np, kCheckRIndex, t)) p = 0;
-            s_par[(j * 4 + (t & 3)) * 32 + (t >> 2)] = p < np ? p : W + (p - np);
-        }
-    }
-    __syncthreads();
-
-    // Generation g reads the P half buf[g & 1] and writes the compacted P
-    // into the other half (the two never alias within one launch).
-    const int4 *P4 = reinterpret_cast<const int4 *>((g & 1u) ? buf1 : buf0);
-    int4 *D4 = reinterpret_cast<int4 *>((g & 1u) ? out0 : out1);
-    const int4 *__restrict__ Q4 = reinterpret_cast<const int4 *>(q);
-    int4 *__restrict__ C4 = reinterpret_cast<int4 *>(child);
-
-    const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    int *row = s_rows + wib * 2 * W;
-    const int warp = (vblock * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (vgrid * blockDim.x) >> 5;
-    const bool active = lane < nq;
-
-    // Software pipeline: the next node's rows are requested before the
-    // current node is processed.
-    int4 cur_p = make_int4(0, 0, 0, 0), cur_q = make_int4(0, 0, 0, 0);
-    if (active && warp < gp.n) {
-        cur_p = P4[(size_t)warp * nq + lane];
-        cur_q = Q4[(size_t)warp * nq + lane];
-    }
-    for (int v = warp; v < gp.n; v += nwarps) {
-        const int vn = v + nwarps;
-        int4 nxt_p = make_int4(0, 0, 0, 0), nxt_q = make_int4(0, 0, 0, 0);
-        if (active && vn < gp.n) {
-            nxt_p = P4[(size_t)vn * nq + lane];
-            nxt_q = Q4[(size_t)vn * nq + lane];
-        }
-        if (active) {
-            reinterpret_cast<int4 *>(row)[lane] = cur_p;
-            reinterpret_cast<int4 *>(row + W)[lane] = cur_q;
-        }
-        cur_p = nxt_p;
-        cur_q = nxt_q;
-        __syncwarp();
-        if (active && EMAX == 4 && E == 4) {
-            // Sort each child's four votes (5 comparators); the run pattern of
-            // the sorted values gives the maximal labels in ascending order:
-            // t = 4 (all distinct), t = 2 (two pairs) or a unique maximum. All
-            // four children are classified first so that the lane's tie word
-            // (one Philox call for its four children) is computed at most once.
-            int o[4], srt[4][4], tk[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = 4 * lane + k;
-                o[k] = i < np ? row[s_keep[k * 32 + lane]] : 0;
-                const int cp = i < np ? s_copy[k * 32 + lane] : 0;
-                // Children past N_p (padding of the last quad) have no parent table.
-                const bool real = i < np;
-                int s0 = row[real ? s_par[(0 * 4 + k) * 32 + lane] : 0];
-                int s1 = row[real ? s_par[(1 * 4 + k) * 32 + lane] : 0];
-                int s2 = row[real ? s_par[(2 * 4 + k) * 32 + lane] : 0];
-                int s3 = row[real ? s_par[(3 * 4 + k) * 32 + lane] : 0];
-                int lo, hi;
-                lo = min(s0, s1); hi = max(s0, s1); s0 = lo; s1 = hi;
-                lo = min(s2, s3); hi = max(s2, s3); s2 = lo; s3 = hi;
-                lo = min(s0, s2); hi = max(s0, s2); s0 = lo; s2 = hi;
-                lo = min(s1, s3); hi = max(s1, s3); s1 = lo; s3 = hi;
-                lo = min(s1, s2); hi = max(s1, s2); s1 = lo; s2 = hi;
-                const bool e01 = s0 == s1, e12 = s1 == s2, e23 = s2 == s3;
-                int t = (!e01 && !e12 && !e23) ? 4 : ((e01 && e23 && !e12) ? 2 : 1);
-                int uniq = e01 ? s0 : (e12 ? s1 : s2);
-                if (i >= np) {
-                    t = 1;
-                    uniq = 0;
-                } else if (cp >= 0) {
-                    t = 1;
-                    uniq = row[cp];
-                }
-                srt[k][0] = t == 1 ? uniq : s0;
-                srt[k][1] = s1;
-                srt[k][2] = s2;
-                srt[k][3] = s3;
-                tk[k] = t;
-            }
-            uint4 u = make_uint4(0, 0, 0, 0);
-            if (tk[0] > 1 || tk[1] > 1 || tk[2] > 1 || tk[3] > 1)
-                u = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)lane, g, kStageCrossTie), gp.key0, gp.key1);
-            int r[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t w = word_of(u, k);
-                if (tk[k] == 4) {
-                    const uint32_t kk = pick_index(w, 4u);
-                    r[k] = kk == 0 ? srt[k][0] : kk == 1 ? srt[k][1] : kk == 2 ? srt[k][2] : srt[k][3];
-                } else if (tk[k] == 2) {
-                    r[k] = pick_index(w, 2u) == 0 ? srt[k][0] : srt[k][2];
-                } else {
-                    r[k] = srt[k][0];
-                }
-            }
-            D4[(size_t)v * nq + lane] = make_int4(o[0], o[1], o[2], o[3]);
-            C4[(size_t)v * nq + lane] = make_int4(r[0], r[1], r[2], r[3]);
-        } else if (active) {
-            int o[4];
-            int r[4];
-            bool have_u = false;
-            uint4 u = make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = 4 * lane + k;
-                o[k] = i < np ? row[s_keep[k * 32 + lane]] : 0;
-                r[k] = 0;
-                if (i >= np) continue;
-                const int cp = s_copy[k * 32 + lane];
-                if (cp >= 0) {
-                    r[k] = row[cp];
-                    continue;
-                }
-                int x[EMAX];
-#pragma unroll
-                for (int j = 0; j < EMAX; ++j) x[j] = j < E ? row[s_par[(j * 4 + k) * 32 + lane]] : 0;
-                int best;
-                const int t = mode_ties<EMAX>(x, E, best);
-                int kk = 0;
-                if (t > 1) {
-                    if (!have_u) {
-                        u = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)lane, g, kStageCrossTie),
-                                          gp.key0, gp.key1);
-                        have_u = true;
-                    }
-                    kk = (int)pick_index(word_of(u, k), (uint32_t)t);
-                }
-                r[k] = kth_tied<EMAX>(x, E, best, kk);
-            }
-            D4[(size_t)v * nq + lane] = make_int4(o[0], o[1], o[2], o[3]);
-            C4[(size_t)v * nq + lane] = make_int4(r[0], r[1], r[2], r[3]);
-        }
-        __syncwarp();
-    }
-}
-
-template <int EMAX>
-__global__ void __launch_bounds__(kBlock)
-crossover_kernel(GenParams gp, const int32_t *buf0, const int32_t *buf1, int32_t *out0, int32_t *out1,
-                 const int32_t *__restrict__ q, int32_t *__restrict__ child,
-                 const int32_t *__restrict__ keep, const int32_t *__restrict__ par_r,
-                 const int32_t *__restrict__ copy_r, const uint32_t *__restrict__ gen_ptr)
-{
-    crossover_body<EMAX>(gp, buf0, buf1, out0, out1, q, child, keep, par_r, copy_r, gen_ptr, blockIdx.x, gridDim.x);
-}
-
-// The member of a multi-member launch that block blockIdx.x belongs to:
-// members own consecutive block ranges, starts[k] .. starts[k + 1] - 1
-// (empty for a member with nothing to do).
-__device__ __forceinline__ int member_of_block(const int *__restrict__ starts, int count)
-{
-    const int b = (int)blockIdx.x;
-    int lo = 0, hi = count;  // starts[lo] <= b < starts[hi]
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(starts + mid) <= b) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// Crossover of every member of a batch in one launch.
-template <int EMAX>
-__global__ void __launch_bounds__(kBlock)
-crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__restrict__ starts, int count)
-{
-    const int k = member_of_block(starts, count);
-    const BatchMember &mb = members[k];
-    const PopState &ps = mb.ps;
-    const int b0 = __ldg(starts + k);
-    crossover_body<EMAX>(mb.gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r,
-                         ps.copy_r, ps.gen, (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
-}
-
-// ---------------------------------------------------------------------------
-// Mutation (Sec. 4.3.2). Node v of child i mutates iff its MCOIN word is
-// below thr_m and deg(v) > 0; it then takes the most frequent label among its
-// neighbours in the post-crossover child (synchronous: all reads come from
-// `child`), the tie among the t most frequent labels broken by the MTIE word
-// (the pick(u, t)-th smallest).
-//
-// A pair is a (node, selected child). A warp takes a batch of nodes, copies
-// their rows to Q, and lists the batch's pairs; then every lane works on a
-// pair of its own, so that the lanes stay full whatever number of children a
-// node has selected (about 20 of 100 at M_P 0.2). By degree:
-//   up to 128    mutation_kernel, a pair per lane: the labels are gathered into
-//                registers, sorted by a merge-exchange network and the tied
-//                labels read off the runs. One launch for degrees up to 32
-//                (networks of 8, 12, .., 28 or 32 entries, the smallest that
-//                holds the lanes' degrees), one each for 33..64 (40, 48, 56 or
-//                64 entries, the smallest that holds the graph's largest
-//                degree there) and 65..128, so that no launch pays for the
-//                registers of a larger network than its own
-//   129..512     a warp per pair: count table in shared memory (the node's
-//                pairs are split over kWideParts warps), in the first launch
-//   above 512    mutation_hub_kernel, a block per pair
-// The launches touch different rows of Q and only add to the histogram, so
-// they run side by side.
-//
-// A count table costs several passes over the neighbours' labels, and in a
-// settled population the result is often the label the node already has:
-// counting the neighbours that hold it proves that when it is on more than
-// half of them (it is then the unique mode). Above degree 128 that count goes
-// first when the node's last generation says it pays (own_label_pays). The
-// vote in registers needs one pass, and a front keeps so many fragmented
-// members that the count settles at most 0.45 of the pairs (n = 40,000 and
-// 10^6, mu 0.3): trying it first there was slower at every threshold (n =
-// 10^6: 2.59 ms a generation's mutation with it from half settled on, 2.50
-// without).
-//
-// The neighbours come from the mutation's own adjacency: rows in processing
-// order (degree descending), padded to four entries with the id n, whose
-// child row holds a value above every label, so that four neighbours are one
-// 16-byte load and padding needs no test.
-// ---------------------------------------------------------------------------
-
-// MTIE word of child i at node v.
-__device__ __forceinline__ uint32_t tie_word(const GenParams &gp, int v, int i, uint32_t g)
-{
-    const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)(i >> 2), g, kStageMutTie), gp.key0, gp.key1);
-    return word_of(r, i & 3);
-}
-
-// A neighbour id read from the adjacency; in the debug build an id outside
-// [0, n] is recorded and replaced by n (the padding row), so that the access
-// it feeds stays in bounds.
-__device__ __forceinline__ int checked_node(int u, int n)
-{
-    return MOCD_CHECK(u >= 0 && u <= n, kCheckNode, u) ? u : n;
-}
-
-__device__ __forceinline__ uint32_t hash_slot(int x, int hbits)
-{
-    return ((uint32_t)x * 2654435761u) >> (32 - hbits);
-}
-
-constexpr int kLaneMax = 32;     // largest degree of the per-lane vote
-constexpr int kMutBlock = 128;   // mutation threads per block
-constexpr int kHubBlock = 256;   // threads per block of the hub kernel
-static_assert(kMutBatchMax * kMaxPop <= 65536, "a pair is listed in 16 bits");
-
 // Sorting networks for any N: Batcher's merge exchange in the form of
 // Knuth, TAOCP vol. 3, Sec. 5.2.2, Algorithm M (for a power of two it is
 // Batcher's odd-even merge sort: 19, 63, 191, 543 comparators for 8, 16, 32,
@@ -543,6 +194,330 @@ __device__ __forceinline__ int kth_bit(unsigned m, unsigned k)
     }
     return pos;
 }
+
+// ---------------------------------------------------------------------------
+// Crossover. Row v of R = (P half | Q) is staged in shared memory; the next P
+// (environmental selection's keep list) is compacted into the other P half,
+// and child i of the generation gets
+//   copy_r[i] >= 0 : R_v[copy_r[i]]                    (x > C_P: random parent)
+//   otherwise      : majority of R_v[par_r[i][j]], j < E_S, the tie among the t
+//                    most frequent labels broken by the XTIE word: the
+//                    pick(u, t)-th smallest of them (Eq. arg_max).
+// A lane owns a quad of children; a warp takes as many nodes at a time as its
+// lanes hold quads. The parents of a copied child are E_S times the copied
+// member, those of a child past N_p (padding of the last quad) a cell that
+// holds 0, so neither needs a case of its own.
+// Up to four parents (the default), a lane keeps the row positions of its four
+// children's parents and kept members in registers for the whole kernel: per
+// node it loads 20 labels from shared memory and sorts four of them per child
+// (5 comparators). Bound by the half-rate integer pipe and by the bank
+// conflicts of the label reads. More parents: the positions stay in shared
+// memory and a network of 8 or 16 entries sorts the labels. Measured a launch,
+// N_p 100, E_S 4: n = 40,000 25.0 -> 21.4 us, n = 10^6 478 -> 388 us; E_S 3,
+// N_p 50, n = 30,011 42 -> 11.8 us; E_S 6, N_p 128, n = 4,001 34 -> 10.1 us (against
+// positions in shared memory, a node a warp, and pairwise counts of the votes
+// for every E_S but 4).
+// ---------------------------------------------------------------------------
+
+constexpr int kRowPad = 4;  // cells after a staged row: two above every label, one 0
+
+// Row position of member r of R.
+__device__ __forceinline__ int row_position(const GenParams &gp, int r, int t)
+{
+    if (!MOCD_CHECK(r >= 0 && r < 2 * gp.np, kCheckRIndex, t)) r = 0;
+    return r < gp.np ? r : gp.W + (r - gp.np);
+}
+
+// The pick(u, t)-th of the t most frequent of the E sorted values x (entries
+// at E and above sort last): the longest runs, from a bit mask of equal
+// neighbours (see lane_vote). word() is called only when t > 1.
+template <int N, class F>
+__device__ __forceinline__ int sorted_mode(const int (&x)[N], int E, F word)
+{
+    unsigned m = 0;
+#pragma unroll
+    for (int j = 0; j + 1 < N; ++j) m |= (x[j] == x[j + 1] ? 1u : 0u) << j;
+    m &= (1u << (E - 1)) - 1u;
+    unsigned starts = (1u << E) - 1u;
+    while (m) {
+        starts = m;
+        m &= m >> 1;
+    }
+    const int t = __popc(starts);
+    const unsigned k = t > 1 ? pick_index(word(), (uint32_t)t) : 0u;
+    return select_at<N>(x, kth_bit(starts, k));
+}
+
+template <int EMAX>
+__device__ __forceinline__ void crossover_body(const GenParams gp, const int32_t *buf0, const int32_t *buf1,
+                                               int32_t *out0, int32_t *out1, const int32_t *__restrict__ q,
+                                               int32_t *__restrict__ child, const int32_t *__restrict__ keep,
+                                               const int32_t *__restrict__ par_r, const int32_t *__restrict__ copy_r,
+                                               const uint32_t *__restrict__ gen_ptr, int vblock, int vgrid)
+{
+    extern __shared__ int smem[];
+    const int W = gp.W, np = gp.np, E = gp.es;
+    const int nq = W >> 2;
+    const int lane = threadIdx.x & 31;
+    const int wib = threadIdx.x >> 5;
+    const int per_warp = 32 / nq;  // nodes a warp takes at a time (nq <= 32)
+    const int sub = lane / nq, quad = lane - sub * nq;
+    const bool active = sub < per_warp;
+    const int row_words = 2 * W + kRowPad;
+    // EMAX > 4: the parents' row positions, [EMAX][4][32], then the rows.
+    constexpr int kTable = EMAX > 4 ? EMAX * kMaxPop : 0;
+    int *row = smem + kTable + (wib * per_warp + (active ? sub : 0)) * row_words;
+    const uint32_t g = *gen_ptr;
+
+    // Row positions of child 4 quad + k's kept member and parents.
+    const int zero = 2 * W + 2;
+    int kept[4], par[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = 4 * quad + k;
+        const bool real = active && i < np;
+        kept[k] = real ? row_position(gp, keep[i], i) : zero;
+        if (EMAX == 4) {
+            const int c = real ? copy_r[i] : -1;
+            if (!real || c >= 0) {
+                const int at = real ? row_position(gp, c, i) : zero;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) par[k][j] = at;
+            } else {
+                const int4 p = *reinterpret_cast<const int4 *>(par_r + i * kMaxParents);
+                par[k][0] = row_position(gp, p.x, i);
+                // Fewer than four: values above every label, which sort last
+                // and differ; one parent: four times the same.
+                par[k][1] = E > 1 ? row_position(gp, p.y, i) : par[k][0];
+                par[k][2] = E > 2 ? row_position(gp, p.z, i) : E == 2 ? 2 * W : par[k][0];
+                par[k][3] = E > 3 ? row_position(gp, p.w, i) : E > 1 ? 2 * W + 1 : par[k][0];
+            }
+        }
+    }
+    if (EMAX > 4) {
+        for (int t = threadIdx.x; t < kMaxPop; t += blockDim.x) {
+            const int c = t < np ? copy_r[t] : -1;
+            for (int j = 0; j < EMAX; ++j) {
+                int at = zero;
+                if (t < np) at = j >= E ? 2 * W + 1 : row_position(gp, c >= 0 ? c : par_r[t * kMaxParents + j], t);
+                else if (j >= E) at = 2 * W + 1;
+                smem[(j * 4 + (t & 3)) * 32 + (t >> 2)] = at;
+            }
+        }
+        __syncthreads();
+    }
+    if (active && quad == 0) {
+        row[2 * W] = INT_MAX - 1;
+        row[2 * W + 1] = INT_MAX;
+        row[2 * W + 2] = 0;
+    }
+
+    // Generation g reads the P half buf[g & 1] and writes the compacted P
+    // into the other half (the two never alias within one launch).
+    const int4 *P4 = reinterpret_cast<const int4 *>((g & 1u) ? buf1 : buf0);
+    int4 *D4 = reinterpret_cast<int4 *>((g & 1u) ? out0 : out1);
+    const int4 *__restrict__ Q4 = reinterpret_cast<const int4 *>(q);
+    int4 *__restrict__ C4 = reinterpret_cast<int4 *>(child);
+
+    const int warp = (vblock * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (vgrid * blockDim.x) >> 5;
+
+    // Software pipeline: the next node's rows are requested before the
+    // current node is processed.
+    int4 cur_p = make_int4(0, 0, 0, 0), cur_q = make_int4(0, 0, 0, 0);
+    if (active && warp * per_warp + sub < gp.n) {
+        cur_p = P4[(size_t)(warp * per_warp + sub) * nq + quad];
+        cur_q = Q4[(size_t)(warp * per_warp + sub) * nq + quad];
+    }
+    for (long long v0 = (long long)warp * per_warp; v0 < gp.n; v0 += (long long)nwarps * per_warp) {
+        const long long v = v0 + sub, vn = v + (long long)nwarps * per_warp;
+        const bool mine = active && v < gp.n;
+        int4 nxt_p = make_int4(0, 0, 0, 0), nxt_q = make_int4(0, 0, 0, 0);
+        if (active && vn < gp.n) {
+            nxt_p = P4[(size_t)vn * nq + quad];
+            nxt_q = Q4[(size_t)vn * nq + quad];
+        }
+        if (mine) {
+            reinterpret_cast<int4 *>(row)[quad] = cur_p;
+            reinterpret_cast<int4 *>(row + W)[quad] = cur_q;
+        }
+        cur_p = nxt_p;
+        cur_q = nxt_q;
+        __syncwarp();
+        if (mine) {
+            int o[4], r[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o[k] = row[kept[k]];
+            if (EMAX == 4) {
+                // Sort each child's votes; the run pattern of the sorted values
+                // gives the maximal labels in ascending order: all distinct
+                // (t = E), two pairs (t = 2) or a unique maximum. All four
+                // children are classified first so that the lane's tie word
+                // (one Philox call for its four children) is computed at most
+                // once.
+                int srt[4][4];
+                bool none[4], two[4];
+                bool tie = false;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) srt[k][j] = row[par[k][j]];
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    sort_network<4>(srt[k]);
+                    const bool e01 = srt[k][0] == srt[k][1], e12 = srt[k][1] == srt[k][2], e23 = srt[k][2] == srt[k][3];
+                    none[k] = !e01 && !e12 && !e23;
+                    two[k] = e01 && e23 && !e12;
+                    r[k] = e01 ? srt[k][0] : e12 ? srt[k][1] : srt[k][2];
+                    tie |= none[k] || two[k];
+                }
+                if (tie) {
+                    const uint4 u =
+                        philox4x32_10(make_uint4((uint32_t)v, (uint32_t)quad, g, kStageCrossTie), gp.key0, gp.key1);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t w = word_of(u, k);
+                        const uint32_t kk = pick_index(w, (uint32_t)E);
+                        const int low = (kk & 1u) ? srt[k][1] : srt[k][0];
+                        const int high = (kk & 1u) ? srt[k][3] : srt[k][2];
+                        if (none[k]) r[k] = (kk & 2u) ? high : low;
+                        else if (two[k] && (w >> 31)) r[k] = srt[k][2];
+                    }
+                }
+            } else {
+                bool have_u = false;
+                uint4 u = make_uint4(0, 0, 0, 0);
+                for (int k = 0; k < 4; ++k) {
+                    int x[EMAX];
+#pragma unroll
+                    for (int j = 0; j < EMAX; ++j) x[j] = row[smem[(j * 4 + k) * 32 + quad]];
+                    sort_network<EMAX>(x);
+                    const int res = sorted_mode<EMAX>(x, E, [&]() {
+                        if (!have_u) {
+                            u = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)quad, g, kStageCrossTie), gp.key0,
+                                              gp.key1);
+                            have_u = true;
+                        }
+                        return word_of(u, k);
+                    });
+                    r[0] = k == 0 ? res : r[0];
+                    r[1] = k == 1 ? res : r[1];
+                    r[2] = k == 2 ? res : r[2];
+                    r[3] = k == 3 ? res : r[3];
+                }
+            }
+            D4[(size_t)v * nq + quad] = make_int4(o[0], o[1], o[2], o[3]);
+            C4[(size_t)v * nq + quad] = make_int4(r[0], r[1], r[2], r[3]);
+        }
+        __syncwarp();
+    }
+}
+
+template <int EMAX>
+__global__ void __launch_bounds__(kBlock, 2)
+crossover_kernel(const __grid_constant__ GenParams gp, const int32_t *buf0, const int32_t *buf1, int32_t *out0,
+                 int32_t *out1, const int32_t *__restrict__ q, int32_t *__restrict__ child,
+                 const int32_t *__restrict__ keep, const int32_t *__restrict__ par_r,
+                 const int32_t *__restrict__ copy_r, const uint32_t *__restrict__ gen_ptr)
+{
+    crossover_body<EMAX>(gp, buf0, buf1, out0, out1, q, child, keep, par_r, copy_r, gen_ptr, blockIdx.x, gridDim.x);
+}
+
+// The member of a multi-member launch that block blockIdx.x belongs to:
+// members own consecutive block ranges, starts[k] .. starts[k + 1] - 1
+// (empty for a member with nothing to do).
+__device__ __forceinline__ int member_of_block(const int *__restrict__ starts, int count)
+{
+    const int b = (int)blockIdx.x;
+    int lo = 0, hi = count;  // starts[lo] <= b < starts[hi]
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(starts + mid) <= b) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Crossover of every member of a batch in one launch.
+template <int EMAX>
+__global__ void __launch_bounds__(kBlock, 2)
+crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__restrict__ starts, int count)
+{
+    const int k = member_of_block(starts, count);
+    const BatchMember &mb = members[k];
+    const PopState &ps = mb.ps;
+    const int b0 = __ldg(starts + k);
+    crossover_body<EMAX>(mb.gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r,
+                         ps.copy_r, ps.gen, (int)blockIdx.x - b0, __ldg(starts + k + 1) - b0);
+}
+
+// ---------------------------------------------------------------------------
+// Mutation (Sec. 4.3.2). Node v of child i mutates iff its MCOIN word is
+// below thr_m and deg(v) > 0; it then takes the most frequent label among its
+// neighbours in the post-crossover child (synchronous: all reads come from
+// `child`), the tie among the t most frequent labels broken by the MTIE word
+// (the pick(u, t)-th smallest).
+//
+// A pair is a (node, selected child). A warp takes a batch of nodes, copies
+// their rows to Q, and lists the batch's pairs; then every lane works on a
+// pair of its own, so that the lanes stay full whatever number of children a
+// node has selected (about 20 of 100 at M_P 0.2). By degree:
+//   up to 128    mutation_kernel, a pair per lane: the labels are gathered into
+//                registers, sorted by a merge-exchange network and the tied
+//                labels read off the runs. One launch for degrees up to 32
+//                (networks of 8, 12, .., 28 or 32 entries, the smallest that
+//                holds the lanes' degrees), one each for 33..64 (40, 48, 56 or
+//                64 entries, the smallest that holds the graph's largest
+//                degree there) and 65..128, so that no launch pays for the
+//                registers of a larger network than its own
+//   129..512     a warp per pair: count table in shared memory (the node's
+//                pairs are split over kWideParts warps), in the first launch
+//   above 512    mutation_hub_kernel, a block per pair
+// The launches touch different rows of Q and only add to the histogram, so
+// they run side by side.
+//
+// A count table costs several passes over the neighbours' labels, and in a
+// settled population the result is often the label the node already has:
+// counting the neighbours that hold it proves that when it is on more than
+// half of them (it is then the unique mode). Above degree 128 that count goes
+// first when the node's last generation says it pays (own_label_pays). The
+// vote in registers needs one pass, and a front keeps so many fragmented
+// members that the count settles at most 0.45 of the pairs (n = 40,000 and
+// 10^6, mu 0.3): trying it first there was slower at every threshold (n =
+// 10^6: 2.59 ms a generation's mutation with it from half settled on, 2.50
+// without).
+//
+// The neighbours come from the mutation's own adjacency: rows in processing
+// order (degree descending), padded to four entries with the id n, whose
+// child row holds a value above every label, so that four neighbours are one
+// 16-byte load and padding needs no test.
+// ---------------------------------------------------------------------------
+
+// MTIE word of child i at node v.
+__device__ __forceinline__ uint32_t tie_word(const GenParams &gp, int v, int i, uint32_t g)
+{
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)v, (uint32_t)(i >> 2), g, kStageMutTie), gp.key0, gp.key1);
+    return word_of(r, i & 3);
+}
+
+// A neighbour id read from the adjacency; in the debug build an id outside
+// [0, n] is recorded and replaced by n (the padding row), so that the access
+// it feeds stays in bounds.
+__device__ __forceinline__ int checked_node(int u, int n)
+{
+    return MOCD_CHECK(u >= 0 && u <= n, kCheckNode, u) ? u : n;
+}
+
+__device__ __forceinline__ uint32_t hash_slot(int x, int hbits)
+{
+    return ((uint32_t)x * 2654435761u) >> (32 - hbits);
+}
+
+constexpr int kLaneMax = 32;     // largest degree of the per-lane vote
+constexpr int kMutBlock = 128;   // mutation threads per block
+constexpr int kHubBlock = 256;   // threads per block of the hub kernel
+static_assert(kMutBatchMax * kMaxPop <= 65536, "a pair is listed in 16 bits");
 
 // Exact neighbour-majority of one pair by its own lane (deg <= N; 0 for a
 // lane without a pair). The labels are gathered into registers (the padding
@@ -1101,9 +1076,10 @@ mutation_hub_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict
 }
 
 template <int EMAX>
-size_t crossover_smem()
+size_t crossover_smem(int W)
 {
-    return sizeof(int) * (2 * kMaxPop + kMaxPop * EMAX + (kBlock / 32) * 2 * kMaxPop);
+    const int per_warp = 32 / (W >> 2);
+    return sizeof(int) * ((EMAX > 4 ? EMAX * kMaxPop : 0) + (kBlock / 32) * per_warp * (2 * W + kRowPad));
 }
 
 }  // namespace
@@ -1122,44 +1098,56 @@ cudaError_t launch_init_population(const GenParams &gp, int init_mode, const int
     return cudaGetLastError();
 }
 
-int grid_for_crossover(int sms, int es)
+namespace {
+
+template <int EMAX>
+int crossover_occupancy(int W)
 {
     int per_sm = 0;
-    if (es <= 4)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crossover_kernel<4>, kBlock, crossover_smem<4>());
-    else if (es <= 8)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crossover_kernel<8>, kBlock, crossover_smem<8>());
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crossover_kernel<16>, kBlock, crossover_smem<16>());
-    if (per_sm < 1) per_sm = 1;
-    return sms * per_sm;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crossover_kernel<EMAX>, kBlock, crossover_smem<EMAX>(W));
+    return per_sm < 1 ? 1 : per_sm;
+}
+
+template <int EMAX>
+void crossover_launch(const GenParams &gp, const PopState &ps, int grid, cudaStream_t s)
+{
+    crossover_kernel<EMAX><<<grid, kBlock, crossover_smem<EMAX>(gp.W), s>>>(
+        gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
+}
+
+}  // namespace
+
+int grid_for_crossover(int sms, int es, int W)
+{
+    return sms * (es <= 4 ? crossover_occupancy<4>(W) : es <= 8 ? crossover_occupancy<8>(W) : crossover_occupancy<16>(W));
 }
 
 cudaError_t launch_crossover(const GenParams &gp, const PopState &ps, int grid, cudaStream_t s)
 {
-    if (gp.es <= 4)
-        crossover_kernel<4><<<grid, kBlock, crossover_smem<4>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
-    else if (gp.es <= 8)
-        crossover_kernel<8><<<grid, kBlock, crossover_smem<8>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
-    else
-        crossover_kernel<16><<<grid, kBlock, crossover_smem<16>(), s>>>(
-            gp, ps.buf[0], ps.buf[1], ps.buf[0], ps.buf[1], ps.q, ps.c, ps.keep, ps.par_r, ps.copy_r, ps.gen);
+    if (gp.es <= 4) crossover_launch<4>(gp, ps, grid, s);
+    else if (gp.es <= 8) crossover_launch<8>(gp, ps, grid, s);
+    else crossover_launch<16>(gp, ps, grid, s);
     return cudaGetLastError();
 }
 
 cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts, int count, int blocks, int es_max,
-                                   cudaStream_t s)
+                                   int rows_max, cudaStream_t s)
 {
     if (blocks <= 0) return cudaSuccess;
+    // rows_max: the largest member's words of staged rows per warp.
+    const size_t rows = sizeof(int) * (kBlock / 32) * (size_t)rows_max;
     if (es_max <= 4)
-        crossover_multi_kernel<4><<<blocks, kBlock, crossover_smem<4>(), s>>>(members, starts, count);
+        crossover_multi_kernel<4><<<blocks, kBlock, rows, s>>>(members, starts, count);
     else if (es_max <= 8)
-        crossover_multi_kernel<8><<<blocks, kBlock, crossover_smem<8>(), s>>>(members, starts, count);
+        crossover_multi_kernel<8><<<blocks, kBlock, rows + sizeof(int) * 8 * kMaxPop, s>>>(members, starts, count);
     else
-        crossover_multi_kernel<16><<<blocks, kBlock, crossover_smem<16>(), s>>>(members, starts, count);
+        crossover_multi_kernel<16><<<blocks, kBlock, rows + sizeof(int) * 16 * kMaxPop, s>>>(members, starts, count);
     return cudaGetLastError();
+}
+
+int crossover_row_words(int W)
+{
+    return 32 / (W >> 2) * (2 * W + kRowPad);
 }
 
 int mutation_warps_per_block()

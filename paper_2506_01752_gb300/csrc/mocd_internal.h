@@ -150,7 +150,8 @@ class Branches {
 // starts[k + 1] - 1 of the launch's `blocks` (each member's own grid for
 // the stage; zero for a member with nothing to do).
 cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts, int count, int blocks, int es_max,
-                                   cudaStream_t s);
+                                   int rows_max, cudaStream_t s);
+int crossover_row_words(int W);  // rows_max: the largest over the members
 cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts, int count, int blocks,
                                   cudaStream_t s);
 // Objectives of `count` labellings (node-major rows of W) into acc (intra, S;
@@ -215,7 +216,7 @@ int grid_for_eval_intra(int sms);
 cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *eptr, const int32_t *eidx,
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order);
-int grid_for_crossover(int sms, int es);
+int grid_for_crossover(int sms, int es, int W);
 int grid_for_mutation(int sms, int cls, int vote_n0, int hash_size, int np, int batch);
 int grid_for_hubs(int sms, int smem_hs);
 int mutation_warps_per_block();

@@ -245,7 +245,7 @@ void size_grids(mocd_ctx *c)
     };
     c->grid_eval = shape(c->occ_eval, kBlock / 32);
     c->grid_eval_intra = shape(c->occ_eval_intra, kBlock / 32);
-    c->grid_cross = shape(c->occ_cross, kBlock / 32);
+    c->grid_cross = shape(c->occ_cross, kBlock / 32 * (32 / (c->W >> 2)));
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
     // kMutPairs of them: five full rounds), but a class too small to give
     // every resident warp kMutWaves batches gets smaller ones.
@@ -392,7 +392,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.thr_m = (unsigned long long)floor(p->p_mutation * 4294967296.0);
     c->occ_eval = grid_for_eval(c->sms);
     c->occ_eval_intra = grid_for_eval_intra(c->sms);
-    c->occ_cross = grid_for_crossover(c->sms, gp.es);
+    c->occ_cross = grid_for_crossover(c->sms, gp.es, gp.W);
     size_grids(c);
     return MOCD_OK;
 }
@@ -1358,7 +1358,7 @@ struct mocd_batch {
     BatchMember *d_members = nullptr;  // [count], for the multi-member launches
     int *d_starts = nullptr;           // [2][count + 1] block ranges: crossover, evaluation
     int blocks[2] = {0, 0};            // blocks of each multi-member launch
-    int es_max = 0;
+    int es_max = 0, rows_max = 0;
     std::vector<mocd_ctx *> ctx;
     std::vector<int32_t> version;
     std::vector<cudaStream_t> branch;
@@ -1381,7 +1381,7 @@ static int batch_build(mocd_batch *b)
         std::vector<PopState> pss;
         std::vector<BatchMember> mbs;
         std::vector<int> starts(2 * (size_t)(count + 1), 0);
-        b->es_max = 0;
+        b->es_max = b->rows_max = 0;
         for (int i = 0; i < count; ++i) {
             mocd_ctx *c = b->ctx[(size_t)i];
             gps.push_back(c->gp);
@@ -1389,6 +1389,7 @@ static int batch_build(mocd_batch *b)
             mbs.push_back(BatchMember{c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_nodes, c->d_adj,
                                       c->d_eptr, c->d_eidx});
             b->es_max = std::max(b->es_max, c->gp.es);
+            b->rows_max = std::max(b->rows_max, crossover_row_words(c->gp.W));
             // Per member and stage: its own grid.
             const int g[2] = {c->grid_cross, c->grid_eval_intra};
             for (int st = 0; st < 2; ++st)
@@ -1407,7 +1408,8 @@ static int batch_build(mocd_batch *b)
     CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     int rc = MOCD_OK;
     cudaError_t e = cudaSuccess;
-    if (b->form == 2) e = launch_crossover_multi(b->d_members, st_cross, count, b->blocks[0], b->es_max, b->stream);
+    if (b->form == 2) e = launch_crossover_multi(b->d_members, st_cross, count, b->blocks[0], b->es_max, b->rows_max,
+                                                     b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(b->fork, b->stream);
     for (int i = 0; i < count && rc == MOCD_OK && e == cudaSuccess; ++i) {
         mocd_ctx *c = b->ctx[(size_t)i];
