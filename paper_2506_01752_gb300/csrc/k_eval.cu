@@ -169,6 +169,10 @@ evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__
                 uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc,
                 const int32_t *__restrict__ order)
 {
+    // (see overlap_next) The selection that follows is one block: it may come in
+    // as soon as every block here runs.
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
     evaluate_body<COUNT_D>(n, W, count, stride, row_ptr, col_idx, labels, hist, acc, order, blockIdx.x, gridDim.x);
 }
 

@@ -429,6 +429,7 @@ __global__ void __launch_bounds__(kSelThreads)
 select_kernel(GenParams gp, PopState ps, int mode)
 {
     __shared__ SelShared S;
+    cudaGridDependencySynchronize();  // (see overlap_next)
     select_body(gp, ps, mode, S);
 }
 

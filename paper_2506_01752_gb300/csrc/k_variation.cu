@@ -822,6 +822,7 @@ mutation_kernel(const __grid_constant__ GenParams gp, int first, int last, const
     // to the batch, so that the rest of the memory is L1 cache) and, WIDE, a
     // count table.
     extern __shared__ int4 s_warp[];
+    cudaGridDependencySynchronize();  // (see overlap_next)
     const int W = gp.W;
     const int nq = W >> 2;
     const uint32_t g = *gen_ptr;
@@ -1025,6 +1026,7 @@ mutation_hub_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict
     extern __shared__ int s_table[];  // [2 gp.hub_smem_hs]
     __shared__ unsigned s_red[kHubBlock / 32];
     __shared__ int s_tied;
+    cudaGridDependencySynchronize();  // (see overlap_next)
     const uint32_t g = *gen_ptr;
     const int nq = gp.W >> 2;
     for (int t = blockIdx.x; t < gp.n_hub * nq; t += gridDim.x) {
@@ -1211,7 +1213,9 @@ cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 
     // The launches are independent of each other: on a capturing stream they
     // become parallel branches, the longest votes first.
     Branches br(s);
+    cudaError_t o = cudaSuccess;
     if (gp.n_hub > 0) {
+        o = overlap_next(s);
         mutation_hub_kernel<<<shape.hub_blocks, kHubBlock, 2 * gp.hub_smem_hs * sizeof(int), s>>>(
             gp, nodes, adj, ps.c, ps.q, ps.gen, ps.hist, ps.hint, ps.hub_table);
         br.next();
@@ -1220,6 +1224,7 @@ cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 
     for (int cls = 2; cls >= 0; --cls) {
         const int last = cls == 0 ? gp.n : first + gp.n_vote[cls - 1];
         if (cls == 0 || last > first) {
+            if (o == cudaSuccess) o = overlap_next(s);
             mutation_fn(cls, gp.vote_n0, gp.hash_size > 0)<<<shape.grid[cls], kMutBlock,
                                                              mutation_smem(gp.np, shape.batch[cls], cls, gp.hash_size),
                                                              s>>>(
@@ -1229,7 +1234,7 @@ cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 
         first = last;
     }
     const cudaError_t e = cudaGetLastError();
-    return e != cudaSuccess ? e : br.join();
+    return e != cudaSuccess ? e : o != cudaSuccess ? o : br.join();
 }
 
 }  // namespace mocd

@@ -130,6 +130,13 @@ struct MutationShape {
 cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 *nodes, const int4 *adj,
                             const MutationShape &shape, cudaStream_t s);
 
+// Makes the next kernel captured on the stream a programmatic dependent of the
+// kernels it follows: its blocks may become resident while theirs drain, and
+// it waits (cudaGridDependencySynchronize, first thing in the kernel) before it
+// touches anything they write. No effect outside a capture, or when it follows
+// anything but kernels. Only for kernels that do wait.
+cudaError_t overlap_next(cudaStream_t s);
+
 // Launches on one capturing stream as parallel branches of the graph: each
 // next() ends a branch and puts the stream back to where the object was made;
 // join() makes what follows depend on every branch. On a stream that does not
