@@ -44,8 +44,12 @@ namespace mocd {
 
 namespace {
 
-template <bool COUNT_D>
+// FULL: row_ptr / col_idx hold both directions of every edge, else each edge
+// once (the oriented adjacency). ADD: the degrees (from deg_ptr) go into the
+// histogram; otherwise a histogram (if given) is complete: square and clear it.
+template <bool FULL, bool ADD>
 __device__ __forceinline__ void evaluate_body(int n, int W, int count, int stride,
+                                              const int32_t *__restrict__ deg_ptr,
                                               const int32_t *__restrict__ row_ptr,
                                               const int32_t *__restrict__ col_idx,
                                               const int32_t *__restrict__ labels, uint32_t *__restrict__ hist,
@@ -85,7 +89,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
             const int my_u = lane < cnt ? __ldg(col_idx + e0 + lane) : 0;
             // Keep the neighbours whose rows v reads, compacted: u > v of the
             // full adjacency, or every entry of the oriented one.
-            const bool up = lane < cnt && (!COUNT_D || my_u > v) && MOCD_CHECK(my_u < n, kCheckNode, v);
+            const bool up = lane < cnt && (!FULL || my_u > v) && MOCD_CHECK(my_u < n, kCheckNode, v);
             const unsigned upm = __ballot_sync(0xffffffffu, up);
             const int cu = __popc(upm);
             if (up) nb[__popc(upm & lt)] = my_u;
@@ -108,8 +112,8 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
             }
             __syncwarp();
         }
-        if (COUNT_D && active && end > beg) {
-            const unsigned d = (unsigned)(end - beg);
+        const unsigned d = ADD ? (unsigned)(__ldg(deg_ptr + v + 1) - __ldg(deg_ptr + v)) : 0u;
+        if (ADD && active && d > 0) {
             uint32_t *cell = hist + i0;
             if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v))
                 atomicAdd(cell + (size_t)own.x * stride + 0, d);
@@ -122,7 +126,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
         }
     }
 
-    if (!COUNT_D && active) {
+    if (!ADD && active && hist) {
         // S from the histogram [n][W] that the mutation kernel built: a warp
         // per row, lane q the int4 of individuals 4q..4q+3; every non-zero
         // cell is squared and cleared. D_c^2 < 2^62 and S <= (2m)^2, so the
@@ -149,7 +153,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
             }
         }
     }
-    if (active) {  // (S is the square sweep's when COUNT_D)
+    if (active) {  // (S is the square sweep's when ADD)
         if (i0 + 0 < count) { atomicAdd(&s_intra[i0 + 0], (unsigned long long)c0); atomicAdd(&s_sq[i0 + 0], q0); }
         if (i0 + 1 < count) { atomicAdd(&s_intra[i0 + 1], (unsigned long long)c1); atomicAdd(&s_sq[i0 + 1], q1); }
         if (i0 + 2 < count) { atomicAdd(&s_intra[i0 + 2], (unsigned long long)c2); atomicAdd(&s_sq[i0 + 2], q2); }
@@ -158,36 +162,78 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
     __syncthreads();
     for (int t = threadIdx.x; t < count; t += blockDim.x) {
         if (s_intra[t]) atomicAdd(acc + t, s_intra[t]);
-        if (s_sq[t]) atomicAdd(acc + kMaxPop + t, s_sq[t]);
+        if (!ADD && s_sq[t]) atomicAdd(acc + kMaxPop + t, s_sq[t]);
     }
 }
 
-template <bool COUNT_D>
+// beside: the launch before this one on the stream (hist_block_kernel) only
+// runs beside it: nothing here depends on it, but this launch ends after it.
+template <bool FULL, bool ADD>
 __global__ void __launch_bounds__(kBlock)
-evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__ row_ptr,
+evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__ deg_ptr,
+                const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col_idx, const int32_t *__restrict__ labels,
                 uint32_t *__restrict__ hist, unsigned long long *__restrict__ acc,
-                const int32_t *__restrict__ order)
+                const int32_t *__restrict__ order, bool beside)
 {
     // (see overlap_next) The selection that follows is one block: it may come in
     // as soon as every block here runs.
-    cudaGridDependencySynchronize();
+    if (!beside) cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
-    evaluate_body<COUNT_D>(n, W, count, stride, row_ptr, col_idx, labels, hist, acc, order, blockIdx.x, gridDim.x);
+    evaluate_body<FULL, ADD>(n, W, count, stride, deg_ptr, row_ptr, col_idx, labels, hist, acc, order, blockIdx.x,
+                             gridDim.x);
+    if (beside) cudaGridDependencySynchronize();
+}
+
+// S of individual blockIdx.x with its histogram in shared memory (n words): no
+// global atomics, nothing to clear. The block reads one label a row, an eighth
+// of each sector, which costs less than n additions at the L2's atomic rate
+// do. out: S of each individual.
+constexpr int kHistThreads = 1024;
+__global__ void __launch_bounds__(kHistThreads)
+hist_block_kernel(int n, int W, const int32_t *__restrict__ deg_ptr, const int32_t *__restrict__ labels,
+                  unsigned long long *__restrict__ out)
+{
+    cudaTriggerProgrammaticLaunchCompletion();  // the edge count runs beside this
+    extern __shared__ uint32_t s_hist[];
+    __shared__ unsigned long long s_sum[kHistThreads / 32];
+    for (int c = threadIdx.x; c < n; c += kHistThreads) s_hist[c] = 0;
+    __syncthreads();
+    const int32_t *col = labels + blockIdx.x;
+    for (int v0 = threadIdx.x; v0 < n; v0 += 8 * kHistThreads) {
+        int lab[8], d[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int v = v0 + u * kHistThreads;
+            lab[u] = v < n ? col[(size_t)v * W] : 0;
+            d[u] = v < n ? __ldg(deg_ptr + v + 1) - __ldg(deg_ptr + v) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (d[u] > 0 && MOCD_CHECK((unsigned)lab[u] < (unsigned)n, kCheckLabel, v0)) atomicAdd(s_hist + lab[u], (unsigned)d[u]);
+    }
+    __syncthreads();
+    unsigned long long q = 0;
+    for (int c = threadIdx.x; c < n; c += kHistThreads) q += (unsigned long long)s_hist[c] * s_hist[c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = q;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    q = s_sum[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
+    if (threadIdx.x == 0) out[blockIdx.x] = q;
 }
 
 // S of `count` individuals from the histogram [n][stride] that evaluate_kernel
 // built, squared and cleared; a thread keeps one column group of VEC cells
-// (stride is a multiple of VEC), four rows in flight. With `out_intra`, the
-// last block to finish writes both results (acc[2 kMaxPop] counts the blocks,
-// zero on entry).
+// (stride is a multiple of VEC), four rows in flight. Adds into out.
 template <int VEC>
 __global__ void __launch_bounds__(kBlock)
-square_kernel(int n, int stride, int count, uint32_t *__restrict__ hist, unsigned long long *acc,
-              int64_t *__restrict__ out_intra, int64_t *__restrict__ out_sumsq)
+square_kernel(int n, int stride, int count, uint32_t *__restrict__ hist, unsigned long long *__restrict__ out)
 {
     __shared__ unsigned long long s_sq[kMaxPop];
-    __shared__ bool s_last;
     for (int t = threadIdx.x; t < kMaxPop; t += blockDim.x) s_sq[t] = 0;
     __syncthreads();
     const int groups = stride / VEC;             // per row
@@ -234,18 +280,7 @@ square_kernel(int n, int stride, int count, uint32_t *__restrict__ hist, unsigne
     }
     __syncthreads();
     for (int t = threadIdx.x; t < count; t += blockDim.x)
-        if (s_sq[t]) atomicAdd(acc + kMaxPop + t, s_sq[t]);
-    if (!out_intra) return;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(acc + 2 * kMaxPop, 1ull) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    for (int t = threadIdx.x; t < count; t += blockDim.x) {
-        out_intra[t] = (int64_t)__ldcg(acc + t);
-        out_sumsq[t] = (int64_t)__ldcg(acc + kMaxPop + t);
-    }
+        if (s_sq[t]) atomicAdd(out + t, s_sq[t]);
 }
 
 // The offspring evaluation of every member of a batch in one launch: members
@@ -262,44 +297,62 @@ evaluate_multi_kernel(const BatchMember *__restrict__ members, const int *__rest
     }
     const BatchMember &mb = members[lo];
     const int b0 = __ldg(starts + lo);
-    evaluate_body<false>(mb.gp.n, mb.gp.W, mb.gp.np, mb.gp.W, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
+    evaluate_body<false, false>(mb.gp.n, mb.gp.W, mb.gp.np, mb.gp.W, nullptr, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
                          mb.order, bk - b0, __ldg(starts + lo + 1) - b0);
 }
 
 }  // namespace
 
-int grid_for_eval(int sms)
-{
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<true>, kBlock, 0);
-    if (per_sm < 1) per_sm = 1;
-    return sms * per_sm;
-}
-
 int grid_for_eval_intra(int sms)
 {
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<false>, kBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, evaluate_kernel<false, false>, kBlock, 0);
     if (per_sm < 1) per_sm = 1;
     return sms * per_sm;
 }
 
-cudaError_t launch_evaluate(int n, int W, int count, int stride, const int32_t *row_ptr, const int32_t *col_idx,
-                            const int32_t *labels, uint32_t *hist, unsigned long long *acc, int grid, int sms,
-                            cudaStream_t s, const int32_t *order, int64_t *out_intra, int64_t *out_sumsq)
+bool evaluate_needs_histogram(int64_t n) { return n * (int64_t)sizeof(uint32_t) > kHistBlockBytes; }
+
+cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, const int32_t *deg_ptr,
+                            const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,
+                            unsigned long long *intra, unsigned long long *sumsq, int sms, cudaStream_t s,
+                            const int32_t *order)
 {
-    const long long blocks = std::min<long long>(grid, ((long long)n + kBlock / 32 - 1) / (kBlock / 32));
-    evaluate_kernel<true><<<(int)blocks, kBlock, 0, s>>>(n, W, count, stride, row_ptr, col_idx, labels, hist, acc,
-                                                         order);
+    const bool add = evaluate_needs_histogram(n);
+    const auto kernel = full ? (add ? evaluate_kernel<true, true> : evaluate_kernel<true, false>)
+                             : (add ? evaluate_kernel<false, true> : evaluate_kernel<false, false>);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, 0);
+    const long long blocks =
+        std::min<long long>((long long)sms * std::max(per_sm, 1), ((long long)n + kBlock / 32 - 1) / (kBlock / 32));
+    if (!add) {
+        // A histogram block fills one SM's shared memory on `count` of them; the
+        // edge count takes the rest of the GPU at the same time.
+        cudaFuncSetAttribute(hist_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistBlockBytes);
+        hist_block_kernel<<<count, kHistThreads, n * sizeof(uint32_t), s>>>(n, W, deg_ptr, labels, sumsq);
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)blocks);
+        cfg.blockDim = dim3(kBlock);
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel, n, W, count, stride, deg_ptr, row_ptr, col_idx, labels,
+                                  static_cast<uint32_t *>(nullptr), intra, order, true);
+    }
+    kernel<<<(int)blocks, kBlock, 0, s>>>(n, W, count, stride, deg_ptr, row_ptr, col_idx, labels, hist, intra, order,
+                                          false);
     // Four blocks per SM keep enough rows in flight to stream the histogram;
     // fewer where that leaves a thread less than one round of rows.
     const int vec = stride % 4 == 0 ? 4 : 1;
     const int rows = kBlock / (stride / vec);
     const int sq = (int)std::min<long long>(4 * sms, ((long long)n + 4 * rows - 1) / (4 * rows));
     if (vec == 4)
-        square_kernel<4><<<sq, kBlock, 0, s>>>(n, stride, count, hist, acc, out_intra, out_sumsq);
+        square_kernel<4><<<sq, kBlock, 0, s>>>(n, stride, count, hist, sumsq);
     else
-        square_kernel<1><<<sq, kBlock, 0, s>>>(n, stride, count, hist, acc, out_intra, out_sumsq);
+        square_kernel<1><<<sq, kBlock, 0, s>>>(n, stride, count, hist, sumsq);
     return cudaGetLastError();
 }
 
@@ -314,7 +367,7 @@ cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *ep
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order)
 {
-    evaluate_kernel<false><<<grid, kBlock, 0, s>>>(n, W, count, W, eptr, eidx, labels, hist, acc, order);
+    evaluate_kernel<false, false><<<grid, kBlock, 0, s>>>(n, W, count, W, nullptr, eptr, eidx, labels, hist, acc, order, false);
     return cudaGetLastError();
 }
 

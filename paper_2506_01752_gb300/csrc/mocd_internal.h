@@ -161,15 +161,18 @@ cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts
 int crossover_row_words(int W);  // rows_max: the largest over the members
 cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts, int count, int blocks,
                                   cudaStream_t s);
-// Objectives of `count` labellings (node-major rows of W) into acc (intra, S;
-// cleared by the caller): edge count and histogram, then the square sweep.
-// hist: [n][stride], stride >= count, zero on entry and again afterwards.
-// out_intra / out_sumsq (optional): the results, written by the sweep (acc
-// then has one more word, zero on entry). grid: grid_for_eval.
-cudaError_t launch_evaluate(int n, int W, int count, int stride, const int32_t *row_ptr, const int32_t *col_idx,
-                            const int32_t *labels, uint32_t *hist, unsigned long long *acc, int grid, int sms,
-                            cudaStream_t s, const int32_t *order = nullptr, int64_t *out_intra = nullptr,
-                            int64_t *out_sumsq = nullptr);
+// Objectives of `count` labellings (node-major rows of W): adds the edge counts
+// into intra and S into sumsq (both zero on entry). row_ptr / col_idx: both
+// directions of every edge (full), or the oriented adjacency; deg_ptr: row
+// pointers whose differences are the degrees. Up to kHistBlockBytes of labels
+// the histogram of each labelling is one block's shared memory; above, it is
+// hist [n][stride] (stride >= count), zero on entry and again afterwards.
+constexpr int64_t kHistBlockBytes = 200 * 1024;
+bool evaluate_needs_histogram(int64_t n);
+cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, const int32_t *deg_ptr,
+                            const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,
+                            unsigned long long *intra, unsigned long long *sumsq, int sms, cudaStream_t s,
+                            const int32_t *order = nullptr);
 // mode 0: keys of a fresh P from acc, keep = identity; mode 1: R = P u Q,
 // environmental selection. Both then rank P and draw the next tournament.
 cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s);
@@ -213,7 +216,6 @@ cudaError_t check_record_eval(unsigned long long *out, bool reset);
 cudaError_t check_record_variation(unsigned long long *out, bool reset);
 
 // Occupancy-derived grid sizes.
-int grid_for_eval(int sms);
 int grid_for_eval_intra(int sms);
 // Objectives of the offspring inside a generation: the mutation kernel has
 // already added every child's degrees to the label-major histogram (and

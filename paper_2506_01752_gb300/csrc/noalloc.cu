@@ -12,7 +12,7 @@
 // and outputs.
 //
 // The scratch below is a device symbol: every GPU that loads this library
-// holds it (16 MiB + 2 KiB) until the process exits. On the host its name is
+// holds it (16 MiB) until the process exits. On the host its name is
 // only a stand-in, never a device address, so the address is fetched once per
 // device with cudaGetSymbolAddress (the first call on each device does that)
 // and then passed to the kernels. The cached address belongs to the device's
@@ -27,11 +27,11 @@ using namespace mocd;
 
 namespace {
 
-constexpr size_t kAccWords = 4 * kMaxPop + 8;  // 2 x kMaxPop unsigned long long, the sweep's block count, padding
-constexpr size_t kScratchWords = kAccWords + (size_t)MOCD_NOALLOC_MAX_CELLS;
+constexpr size_t kScratchWords = (size_t)MOCD_NOALLOC_MAX_CELLS;
 constexpr int kMaxDevices = 64;
 
-// [0, kAccWords): intra / S accumulators; then the histogram [n][count].
+// The histogram [n][count] of a graph whose labels do not fit a block's shared
+// memory.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 
 uint32_t *g_scratch_addr[kMaxDevices];
@@ -71,16 +71,19 @@ extern "C" int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_
     int rc = scratch_on_current_device(&scratch, &dev);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    unsigned long long *acc = reinterpret_cast<unsigned long long *>(scratch);
-    uint32_t *hist = scratch + kAccWords;
     const int W = (count + 3) & ~3;
-    // The scratch keeps the previous call's contents: clear what must start at 0.
-    if (cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kAccWords + (size_t)count * (size_t)n), s) != cudaSuccess)
+    // The results are accumulated in place; the scratch keeps the previous
+    // call's contents: clear what must start at 0.
+    const size_t bytes = sizeof(int64_t) * (size_t)count;
+    if (cudaMemsetAsync(intra, 0, bytes, s) != cudaSuccess || cudaMemsetAsync(sumsq, 0, bytes, s) != cudaSuccess ||
+        (evaluate_needs_histogram(n) &&
+         cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (size_t)count * (size_t)n, s) != cudaSuccess))
         return MOCD_ERR_CUDA;
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MOCD_ERR_CUDA;
-    if (launch_evaluate((int)n, W, count, count, row_ptr, col_idx, labels, hist, acc, grid_for_eval(sms), sms, s, nullptr,
-                        intra, sumsq) != cudaSuccess)
+    if (launch_evaluate((int)n, W, count, count, true, row_ptr, row_ptr, col_idx, labels, scratch,
+                        reinterpret_cast<unsigned long long *>(intra), reinterpret_cast<unsigned long long *>(sumsq), sms,
+                        s) != cudaSuccess)
         return MOCD_ERR_CUDA;
     return MOCD_OK;
 }

@@ -77,10 +77,10 @@ struct mocd_ctx {
     size_t hint_cap = 0;    // entries of ps.hint
     size_t hub_cap = 0;     // entries of ps.hub_table
     void *d_small = nullptr;
-    int grid_eval = 0, grid_cross = 0;
+    int grid_cross = 0;
     int grid_eval_intra = 0;
     MutationShape mut{};
-    int occ_eval = 0, occ_cross = 0;  // occupancy-limited grids
+    int occ_cross = 0;  // occupancy-limited grids
     int occ_eval_intra = 0;
     int nodes_per_warp = 1;                         // launch shape (autotuned for batches)
     int32_t host_gen = 0;   // generations run since init
@@ -249,7 +249,6 @@ void size_grids(mocd_ctx *c)
         const long long want = (n + per_block - 1) / per_block;
         return (int)std::max<long long>(1, std::min<long long>(occ, want));
     };
-    c->grid_eval = shape(c->occ_eval, kBlock / 32);
     c->grid_eval_intra = shape(c->occ_eval_intra, kBlock / 32);
     c->grid_cross = shape(c->occ_cross, kBlock / 32 * (32 / (c->W >> 2)));
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
@@ -396,7 +395,6 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.key1 = (uint32_t)(p->seed >> 32);
     gp.thr_c = (unsigned long long)floor(p->p_crossover * 4294967296.0);
     gp.thr_m = (unsigned long long)floor(p->p_mutation * 4294967296.0);
-    c->occ_eval = grid_for_eval(c->sms);
     c->occ_eval_intra = grid_for_eval_intra(c->sms);
     c->occ_cross = grid_for_crossover(c->sms, gp.es, gp.W);
     size_grids(c);
@@ -491,8 +489,8 @@ int start_population(mocd_ctx *c, uint32_t base_gen)
     CK(cudaMemsetAsync(ps.hint, 0, sizeof(uint32_t) * hint_words(c), c->stream));
     // (The sweep leaves the histogram zero, as generations expect it: the
     // mutation adds into it.)
-    CK(launch_evaluate(gp.n, gp.W, gp.np, gp.W, c->d_row_ptr, c->d_col_idx, phalf, ps.hist, ps.acc, c->grid_eval,
-                       c->sms, c->stream, c->d_order));
+    CK(launch_evaluate(gp.n, gp.W, gp.np, gp.W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, phalf, ps.hist, ps.acc,
+                       ps.acc + kMaxPop, c->sms, c->stream, c->d_order));
     c->gen_host_value = base_gen;
     CK(cudaMemcpyAsync(ps.gen, &c->gen_host_value, sizeof(uint32_t), cudaMemcpyHostToDevice, c->stream));
     CK(launch_select(gp, ps, 0, c->stream));
@@ -1315,9 +1313,9 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
     const size_t n = (size_t)c->n;
     if ((rc = grow(c->stream, &c->d_im, &c->im_cap, (size_t)batch * n))) return rc;
     if ((rc = grow(c->stream, &c->d_nm, &c->nm_cap, (size_t)kMaxPop * n))) return rc;
-    if ((rc = grow(c->stream, &c->d_eval_hist, &c->eval_hist_cap, (size_t)((batch + 3) & ~3) * n))) return rc;
+    const bool apart = evaluate_needs_histogram(c->n);
+    if (apart && (rc = grow(c->stream, &c->d_eval_hist, &c->eval_hist_cap, (size_t)((batch + 3) & ~3) * n))) return rc;
     if ((rc = eval_scratch(c))) return rc;
-    const int grid = grid_for_eval(c->sms);
     // The labels are checked on the device, as they are rearranged; results
     // are handed out once all batches have passed.
     std::vector<unsigned long long> acc(kEvalWords);
@@ -1329,9 +1327,9 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
         CK(cudaMemcpyAsync(c->d_im, labels + (size_t)b0 * n, sizeof(int32_t) * (size_t)b * n,
                            cudaMemcpyHostToDevice, c->stream));
         CK(launch_to_node_major((int)n, W, b, c->d_im, c->d_nm, eval_bad(c), c->stream));
-        CK(cudaMemsetAsync(c->d_eval_hist, 0, sizeof(uint32_t) * (size_t)W * n, c->stream));
-        CK(launch_evaluate((int)n, W, b, W, c->d_row_ptr, c->d_col_idx, c->d_nm, c->d_eval_hist, c->d_eval_acc, grid,
-                           c->sms, c->stream, c->d_order));
+        if (apart) CK(cudaMemsetAsync(c->d_eval_hist, 0, sizeof(uint32_t) * (size_t)W * n, c->stream));
+        CK(launch_evaluate((int)n, W, b, W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, c->d_nm, c->d_eval_hist,
+                           c->d_eval_acc, c->d_eval_acc + kMaxPop, c->sms, c->stream, c->d_order));
         CK(cudaMemcpyAsync(acc.data(), c->d_eval_acc, sizeof(unsigned long long) * kEvalWords,
                            cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
