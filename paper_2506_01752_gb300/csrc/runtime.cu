@@ -35,8 +35,22 @@ constexpr int kStages = 4;
 // generation one at a time, 25.4 in eights; n = 40,000: 106.8 and 104.5).
 constexpr int kChunk = 8;
 constexpr int kChunkGraph = 2;
-constexpr long long kMutWaves = 2;    // batches per resident warp of the mutation
-constexpr double kMutPairs = 160.0;   // and the pairs a batch aims at
+// Launch shape of the mutation: a warp's batch aims at kMutPairs pairs (three
+// rounds of its lanes), smaller where that leaves fewer than kMutWaves batches
+// per resident warp; the grid holds every batch up to kMutRounds full GPUs of
+// blocks. More blocks than fit at once let a block that ends early make room
+// for the next batches, and keep the batches in flight close together in the
+// order, whose rows they share. A generation, against 160 pairs and as many
+// blocks as fit: n = 170,001 488 -> 430 us, n = 10^6 3.44 -> 2.85 ms, hubs 124
+// -> 114 us, n = 40,000 105.7 -> 104.2 us. (40 pairs, or 4 and 64 rounds, are
+// slower at n = 10^6.)
+constexpr double kMutPairs = 96.0;
+constexpr long long kMutWaves = 2;
+constexpr long long kMutRounds = 24;
+// The edge count: up to four full GPUs of blocks, as long as a warp keeps this
+// many nodes (n = 170,001 464 -> 454 us a generation, n = 10^6 3.33 -> 3.26 ms;
+// two rounds at n = 40,000 are 2 us slower).
+constexpr long long kEvalNodes = 12;
 
 }  // namespace
 
@@ -249,7 +263,11 @@ void size_grids(mocd_ctx *c)
         const long long want = (n + per_block - 1) / per_block;
         return (int)std::max<long long>(1, std::min<long long>(occ, want));
     };
-    c->grid_eval_intra = shape(c->occ_eval_intra, kBlock / 32);
+    // The edge count: several rounds of blocks where each warp keeps kEvalNodes
+    // nodes (a block that ends early makes room for the next).
+    const long long rounds = n / ((long long)c->occ_eval_intra * (kBlock / 32) * kEvalNodes);
+    c->grid_eval_intra =
+        shape((int)std::max<long long>(1, std::min<long long>(4, rounds)) * c->occ_eval_intra, kBlock / 32);
     c->grid_cross = shape(c->occ_cross, kBlock / 32 * (32 / (c->W >> 2)));
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
     // kMutPairs of them: five full rounds), but a class too small to give
@@ -264,8 +282,10 @@ void size_grids(mocd_ctx *c)
         c->mut.batch[cls] = (int)std::max<long long>(1, std::min<long long>(most, nodes / (kMutWaves * warps)));
         const long long items = wide + (nodes + c->mut.batch[cls] - 1) / c->mut.batch[cls];
         const long long per_block = (long long)mutation_warps_per_block() * c->nodes_per_warp;
-        c->mut.grid[cls] =
-            (int)std::max<long long>(1, std::min<long long>(occ, (items + per_block - 1) / per_block));
+        // Up to kMutRounds times the resident blocks: a block that ends early
+        // makes room for the next batches (degrees descend, the last are short).
+        c->mut.grid[cls] = (int)std::max<long long>(
+            1, std::min<long long>(kMutRounds * occ, (items + per_block - 1) / per_block));
     }
 }
 
