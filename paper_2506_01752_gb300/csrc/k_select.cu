@@ -48,7 +48,8 @@ constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;  // +inf
 // us for four unrolled bitonic sorts with block-wide scans.
 struct SelShared {
     uint4 key[kMaxPoints];             // by point: k1, low and high word of k2
-    unsigned ck[kMaxPoints];           // by point: rank of k1 << 16 | rank of k2 << 8 | point
+    float4 keyf[kMaxPoints];           // m < 2^23: k1, high and low 24 bits of k2 (exact)
+    float ck[kMaxPoints];              // by point: rank of k1 << 16 | rank of k2 << 8 | point (exact)
     uint4 row[kMaxPoints];             // by place: tie index, inverted crowding distance (low, high), front
     int q[kMaxPoints];                 // by point: rank of k2 << 8 | rank of k1 (equal iff the keys are)
     int rank[kMaxPoints];              // by point: front, 1-based
@@ -62,7 +63,7 @@ struct SelShared {
     int placed;                        // places taken (the fronts that hold the next population)
     int order[kMaxPoints];             // (rank, crowding desc, index) order
     int keep[kMaxPop];
-    unsigned pkey[kMaxPop];            // by P position: gs << 8 | position
+    float pkey[kMaxPop];               // by P position: gs << 8 | position (exact)
     unsigned char minpos[kMaxPop * kMaxParents];  // tournament winners: places of P's order
     unsigned char skip[kMaxPop];       // parent copied when crossover is skipped, else 255
 };
@@ -91,6 +92,21 @@ __device__ __forceinline__ void count_below(unsigned &c, const uint4 &x, const u
         : "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w), "r"(y.x), "r"(y.y), "r"(y.z), "r"(y.w));
 }
 
+// c += 1 if x < y, for integers of at most 24 bits held in floats: the
+// difference is exact and saturates to 0 or 1. This and the next run in the FMA
+// pipe, at twice the rate of the integer pipe's subtractions.
+__device__ __forceinline__ void count_below(float &c, float x, float y)
+{
+    c = __fadd_rn(c, __saturatef(__fsub_rn(y, x)));
+}
+// The same for (xh, xl) < (yh, yl), integers of at most 24 bits each: a
+// difference of the high parts outweighs any of the low parts, and the fused
+// multiply-add keeps the sign and a magnitude of at least 1.
+__device__ __forceinline__ void count_below(float &c, float xh, float xl, float yh, float yl)
+{
+    c = __fadd_rn(c, __saturatef(__fmaf_rn(__fsub_rn(yh, xh), 33554432.0f, __fsub_rn(yl, xl))));
+}
+
 // The four (negative) counts of a thread summed over the SUBS lanes that
 // share its points; lane sub returns the count of point sub % 4. Counts stay
 // below 2^16, so two travel in one word.
@@ -107,19 +123,28 @@ __device__ __forceinline__ int sum_shared(const unsigned (&c)[kOwn], int sub)
     return (int)((sub & 1) ? w >> 16 : w & 0xffffu);
 }
 
-// The place of each of n distinct one-word keys: lane sub < 4 of a group
-// returns that of its group's point sub.
 template <int SUBS>
-__device__ __forceinline__ int place_of(const unsigned *keys, int n)
+__device__ __forceinline__ int sum_shared(const float (&c)[kOwn], int sub)
+{
+    unsigned w[kOwn];
+#pragma unroll
+    for (int k = 0; k < kOwn; ++k) w[k] = 0u - (unsigned)c[k];
+    return sum_shared<SUBS>(w, sub);
+}
+
+// The place of each of n distinct keys below 2^24, held in floats: lane sub <
+// 4 of a group returns that of its group's point sub.
+template <int SUBS>
+__device__ __forceinline__ int place_of(const float *keys, int n)
 {
     const int i0 = threadIdx.x / SUBS * kOwn, sub = threadIdx.x % SUBS;
-    unsigned mine[kOwn], c[kOwn] = {0, 0, 0, 0};
+    float mine[kOwn], c[kOwn] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < kOwn; ++k) mine[k] = keys[i0 + k];
     if (i0 < n) {
 #pragma unroll 2
         for (int j = sub; j < n; j += SUBS) {
-            const unsigned x = keys[j];
+            const float x = keys[j];
 #pragma unroll
             for (int k = 0; k < kOwn; ++k) count_below(c[k], x, mine[k]);
         }
@@ -129,31 +154,53 @@ __device__ __forceinline__ int place_of(const unsigned *keys, int n)
 
 // Fronts of the N points of S.key, first to last, until they hold `want`
 // points: q, rank, fstart and the places cid of the fronts-contiguous
-// (rank, k1, k2, index) order of those points.
-__device__ void rank_points(SelShared &S, int N, int want)
+// (rank, k1, k2, index) order of those points. small: S.keyf is set (k1 below
+// 2^24, k2 below 2^48).
+__device__ void rank_points(SelShared &S, int N, int want, bool small)
 {
     const int i0 = threadIdx.x / kSubR * kOwn, sub = threadIdx.x % kSubR;
     const int i = i0 + sub;  // the point whose sums this lane takes (sub < 4)
     {
         // Ranks of k1 and of k2 among the points.
-        uint4 mine[kOwn];
-        unsigned c1[kOwn] = {0, 0, 0, 0}, c2[kOwn] = {0, 0, 0, 0};
+        int r1, r2;
+        if (small) {
+            float4 mine[kOwn];
+            float c1[kOwn] = {0.0f, 0.0f, 0.0f, 0.0f}, c2[kOwn] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int k = 0; k < kOwn; ++k) mine[k] = S.key[i0 + k];
-        if (i0 < N) {
-            for (int j = sub; j < N; j += kSubR) {
-                const uint4 x = S.key[j];
+            for (int k = 0; k < kOwn; ++k) mine[k] = S.keyf[i0 + k];
+            if (i0 < N) {
+                for (int j = sub; j < N; j += kSubR) {
+                    const float4 x = S.keyf[j];
 #pragma unroll
-                for (int k = 0; k < kOwn; ++k) {
-                    count_below(c1[k], x.x, mine[k].x);
-                    count_below(c2[k], x.y, x.z, mine[k].y, mine[k].z);
+                    for (int k = 0; k < kOwn; ++k) {
+                        count_below(c1[k], x.x, mine[k].x);
+                        count_below(c2[k], x.y, x.z, mine[k].y, mine[k].z);
+                    }
                 }
             }
+            r1 = sum_shared<kSubR>(c1, sub);
+            r2 = sum_shared<kSubR>(c2, sub);
+        } else {
+            uint4 mine[kOwn];
+            unsigned c1[kOwn] = {0, 0, 0, 0}, c2[kOwn] = {0, 0, 0, 0};
+#pragma unroll
+            for (int k = 0; k < kOwn; ++k) mine[k] = S.key[i0 + k];
+            if (i0 < N) {
+                for (int j = sub; j < N; j += kSubR) {
+                    const uint4 x = S.key[j];
+#pragma unroll
+                    for (int k = 0; k < kOwn; ++k) {
+                        count_below(c1[k], x.x, mine[k].x);
+                        count_below(c2[k], x.y, x.z, mine[k].y, mine[k].z);
+                    }
+                }
+            }
+            r1 = sum_shared<kSubR>(c1, sub);
+            r2 = sum_shared<kSubR>(c2, sub);
         }
-        const int r1 = sum_shared<kSubR>(c1, sub), r2 = sum_shared<kSubR>(c2, sub);
         if (sub < kOwn && i < N) {
             S.q[i] = (r2 << 8) | r1;
-            S.ck[i] = ((unsigned)r1 << 16) | ((unsigned)r2 << 8) | (unsigned)i;
+            S.ck[i] = (float)((r1 << 16) | (r2 << 8) | i);
         }
     }
     __syncthreads();
@@ -348,19 +395,12 @@ __device__ __forceinline__ void select_body(const GenParams &gp, const PopState 
     const uint32_t gn = g + 1u;
     const unsigned long long *acc = ps.acc;
     const int N = mode == 0 ? np : 2 * np;
-    // Keys by point: P's (mode 1), then those of the evaluated labellings.
-    if (p < N) {
-        const int i = mode == 0 ? p : p - np;
-        const long long k1 = i < 0 ? ps.pk[p] : m - (long long)acc[i];
-        const long long k2 = i < 0 ? ps.pk[kMaxPop + p] : (long long)acc[kMaxPop + i];
-        S.key[p] = make_uint4((unsigned)k1, (unsigned)k2, (unsigned)((unsigned long long)k2 >> 32), 0u);
-        if (mode == 1) {
-            ps.rk[p] = k1;
-            ps.rk[2 * kMaxPop + p] = k2;
-        }
-    }
+    const bool small = m < (1ll << 23);  // k1 <= m, k2 <= (2 m)^2
+
     // TournamentSelection's draws for generation gn = g + 1 do not depend on
-    // the keys: parent j of child i is the better of sorted positions a, b,
+    // the keys, and the generation number is the last selection's, which every
+    // launch since then followed: they come before the wait for the evaluation
+    // (see overlap_next). Parent j of child i is the better of sorted positions a, b,
     // i.e. position min(a, b). A thread takes a Philox block (two parents).
     const int blocks = E / 2 + 1;  // (2 E + 2 words) / 4, rounded up
     for (int t = threadIdx.x; t < np * blocks; t += kSelThreads) {
@@ -379,8 +419,22 @@ __device__ __forceinline__ void select_body(const GenParams &gp, const PopState 
             }
         }
     }
+    cudaGridDependencySynchronize();
+    // Keys by point: P's (mode 1), then those of the evaluated labellings.
+    if (p < N) {
+        const int i = mode == 0 ? p : p - np;
+        const long long k1 = i < 0 ? ps.pk[p] : m - (long long)acc[i];
+        const long long k2 = i < 0 ? ps.pk[kMaxPop + p] : (long long)acc[kMaxPop + i];
+        S.key[p] = make_uint4((unsigned)k1, (unsigned)k2, (unsigned)((unsigned long long)k2 >> 32), 0u);
+        S.keyf[p] = make_float4((float)(unsigned)k1, (float)(unsigned)((unsigned long long)k2 >> 24),
+                                (float)((unsigned)k2 & 0xffffffu), 0.0f);
+        if (mode == 1) {
+            ps.rk[p] = k1;
+            ps.rk[2 * kMaxPop + p] = k2;
+        }
+    }
     __syncthreads();
-    rank_points(S, N, np);
+    rank_points(S, N, np, small);
     crowd_places(S, S.placed);
     if (mode == 1) {
         order_places<kSubR>(S, S.placed);
@@ -400,7 +454,7 @@ __device__ __forceinline__ void select_body(const GenParams &gp, const PopState 
         ps.pk[kMaxPop + p] = (int64_t)(((unsigned long long)x.z << 32) | x.y);
         ps.keep[p] = id;
         ps.prank[p] = S.rank[id];
-        S.pkey[p] = ((unsigned)S.gs[id] << 8) | (unsigned)p;
+        S.pkey[p] = (float)((S.gs[id] << 8) | p);
     }
     __syncthreads();
     {
@@ -429,7 +483,6 @@ __global__ void __launch_bounds__(kSelThreads)
 select_kernel(GenParams gp, PopState ps, int mode)
 {
     __shared__ SelShared S;
-    cudaGridDependencySynchronize();  // (see overlap_next)
     select_body(gp, ps, mode, S);
 }
 
