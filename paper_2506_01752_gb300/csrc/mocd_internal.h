@@ -25,6 +25,9 @@ namespace mocd {
 // Record `ev` on the context's stream (after all work issued so far).
 int record_on_stream(mocd_ctx *c, cudaEvent_t ev);
 
+// Copies between host buffers, large ones on the library's worker threads.
+void parallel_copy(void *dst, const void *src, size_t bytes);
+
 // Every device allocation of the library (stream-ordered cudaMallocAsync);
 // fails with cudaErrorMemoryAllocation when a test injects a failure there.
 cudaError_t dev_alloc(void **p, size_t bytes, cudaStream_t st);

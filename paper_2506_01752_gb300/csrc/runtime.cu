@@ -866,6 +866,22 @@ cudaError_t mocd::dev_alloc(void **p, size_t bytes, cudaStream_t st)
     return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
+void mocd::parallel_copy(void *dst, const void *src, size_t bytes)
+{
+    // A chunk per MiB at least; the destination's pages are usually fresh, and
+    // mapping them is what takes the time.
+    WorkerPool &pool = WorkerPool::get();
+    const size_t T = std::min<size_t>((size_t)pool.width(), bytes >> 20);
+    if (T <= 1) {
+        std::memcpy(dst, src, bytes);
+        return;
+    }
+    pool.run((int)T, [&](int t) {
+        const size_t b = bytes * (size_t)t / T, e = bytes * ((size_t)t + 1) / T;
+        std::memcpy(static_cast<char *>(dst) + b, static_cast<const char *>(src) + b, e - b);
+    });
+}
+
 cudaError_t mocd::overlap_next(cudaStream_t s)
 {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;

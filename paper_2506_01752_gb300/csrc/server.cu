@@ -18,6 +18,7 @@
 #include <condition_variable>
 #include <deque>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <thread>
@@ -53,7 +54,7 @@ struct Job {
     cudaEvent_t done = nullptr;
     // result
     int32_t count = 0, best = -1;
-    std::vector<int32_t> labels;
+    std::unique_ptr<int32_t[]> labels;  // [count][n], written by the download alone
     std::vector<double> f1, f2;
     std::vector<int64_t> intra, sumsq;
 };
@@ -182,14 +183,16 @@ void round_locked(mocd_server *s, std::unique_lock<std::mutex> &lock)
             finish(s, j, kCancelled, MOCD_ERR_CANCELLED);
         } else {
             const int64_t cap = j->params.pop_size;
-            j->labels.resize((size_t)cap * (size_t)j->n);
+            // Not zeroed: the download maps the pages it needs on several threads
+            // (filling 40 MB here took longer than a job's generations).
+            j->labels.reset(new (std::nothrow) int32_t[(size_t)cap * (size_t)j->n]);
             j->f1.resize(cap);
             j->f2.resize(cap);
             j->intra.resize(cap);
             j->sumsq.resize(cap);
-            const int rc = mocd_pareto_front(j->ctx, (int32_t)cap, &j->count, j->labels.data(), j->f1.data(),
-                                             j->f2.data(), j->intra.data(), j->sumsq.data(), &j->best);
-            if (rc == MOCD_OK) j->labels.resize((size_t)j->count * (size_t)j->n);
+            const int rc = j->labels ? mocd_pareto_front(j->ctx, (int32_t)cap, &j->count, j->labels.get(), j->f1.data(),
+                                                         j->f2.data(), j->intra.data(), j->sumsq.data(), &j->best)
+                                     : MOCD_ERR_OUT_OF_MEMORY;
             if (rc == MOCD_OK && j->work > 0.0) {
                 const double took = std::chrono::duration<double>(Clock::now() - j->started).count();
                 s->sec_per_work = 0.8 * s->sec_per_work + 0.2 * (took / j->work);
@@ -452,7 +455,7 @@ int mocd_server_result(mocd_server *s, int64_t job_id, int32_t cap, int32_t *cou
         if (sumsq) sumsq[k] = j->sumsq[k];
     }
     if (labels)
-        for (size_t k = 0; k < j->labels.size(); ++k) labels[k] = j->labels[k];
+        mocd::parallel_copy(labels, j->labels.get(), sizeof(int32_t) * (size_t)j->count * (size_t)j->n);
     if (best) *best = j->best;
     return MOCD_OK;
 }
