@@ -384,14 +384,15 @@ __device__ void order_places(SelShared &S, int N)
 }
 
 // One block: selection of one population (mode 0: keys of a fresh P from
-// acc; mode 1: R = P u Q), then rank, crowding and order of P and the next
+// acc, `base` generations run so far; mode 1: R = P u Q), then rank, crowding and order of P and the next
 // tournament.
-__device__ __forceinline__ void select_body(const GenParams &gp, const PopState &ps, int mode, SelShared &S)
+__device__ __forceinline__ void select_body(const GenParams &gp, const PopState &ps, int mode, uint32_t base,
+                                            SelShared &S)
 {
     const int p = threadIdx.x;
     const int np = gp.np, E = gp.es;
     const long long m = gp.m;
-    const uint32_t g = *ps.gen;
+    const uint32_t g = mode == 0 ? base : *ps.gen;
     const uint32_t gn = g + 1u;
     const unsigned long long *acc = ps.acc;
     const int N = mode == 0 ? np : 2 * np;
@@ -480,10 +481,10 @@ __device__ __forceinline__ void select_body(const GenParams &gp, const PopState 
 }
 
 __global__ void __launch_bounds__(kSelThreads)
-select_kernel(GenParams gp, PopState ps, int mode)
+select_kernel(GenParams gp, PopState ps, int mode, uint32_t base)
 {
     __shared__ SelShared S;
-    select_body(gp, ps, mode, S);
+    select_body(gp, ps, mode, base, S);
 }
 
 // The selections of several populations in one launch (a batch of
@@ -494,7 +495,7 @@ select_multi_kernel(const GenParams *__restrict__ gps, const PopState *__restric
     __shared__ SelShared S;
     const GenParams gp = gps[blockIdx.x];
     const PopState ps = pss[blockIdx.x];
-    select_body(gp, ps, mode, S);
+    select_body(gp, ps, mode, 0u, S);
 }
 
 // F_1 of P in P order and SelectSolution: argmin of 4 m k1 + k2 (= argmax of
@@ -624,9 +625,9 @@ dim3 tiles_for(int n, int width)
 
 }  // namespace
 
-cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s)
+cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s, uint32_t base)
 {
-    select_kernel<<<1, kSelThreads, 0, s>>>(gp, ps, mode);
+    select_kernel<<<1, kSelThreads, 0, s>>>(gp, ps, mode, base);
     return cudaGetLastError();
 }
 

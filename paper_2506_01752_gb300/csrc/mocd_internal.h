@@ -176,9 +176,10 @@ cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, cons
                             const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,
                             unsigned long long *intra, unsigned long long *sumsq, int sms, cudaStream_t s,
                             const int32_t *order = nullptr);
-// mode 0: keys of a fresh P from acc, keep = identity; mode 1: R = P u Q,
-// environmental selection. Both then rank P and draw the next tournament.
-cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s);
+// mode 0: keys of a fresh P from acc, keep = identity, `base` generations run
+// so far; mode 1: R = P u Q, environmental selection. Both then rank P and draw
+// the next tournament.
+cudaError_t launch_select(const GenParams &gp, const PopState &ps, int mode, cudaStream_t s, uint32_t base = 0);
 // The selections of `count` populations (device arrays of their parameters
 // and states) in one launch, a block each.
 cudaError_t launch_select_multi(const GenParams *gps, const PopState *pss, int count, int mode, cudaStream_t s);

@@ -99,7 +99,6 @@ struct mocd_ctx {
     int nodes_per_warp = 1;                         // launch shape (autotuned for batches)
     int32_t host_gen = 0;   // generations run since init
     int32_t version = 0;    // bumped whenever the population is (re)built
-    uint32_t gen_host_value = 0;
 
     // Generation graphs: [0] plain, [1] with stage events (timing); each is
     // captured on first use and both stay valid until the population or the
@@ -511,14 +510,13 @@ int start_population(mocd_ctx *c, uint32_t base_gen)
     // mutation adds into it.)
     CK(launch_evaluate(gp.n, gp.W, gp.np, gp.W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, phalf, ps.hist, ps.acc,
                        ps.acc + kMaxPop, c->sms, c->stream, c->d_order));
-    c->gen_host_value = base_gen;
-    CK(cudaMemcpyAsync(ps.gen, &c->gen_host_value, sizeof(uint32_t), cudaMemcpyHostToDevice, c->stream));
-    CK(launch_select(gp, ps, 0, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    c->host_gen = (int32_t)base_gen;
+    CK(launch_select(gp, ps, 0, c->stream, base_gen));
+    // The generation graph is captured while the GPU works on the above.
     drop_graphs(c);
     rc = build_graph(c, c->timing ? 1 : 0);
+    CK(cudaStreamSynchronize(c->stream));
     if (rc) return rc;
+    c->host_gen = (int32_t)base_gen;
     c->ready = true;
     c->timing_valid = false;
     return MOCD_OK;
@@ -1663,13 +1661,12 @@ int mocd_batch_configure(mocd_batch *b, int32_t nodes_per_warp, int32_t form)
         return MOCD_ERR_INVALID_ARG;
     for (size_t i = 0; i < b->ctx.size(); ++i)
         if (!b->ctx[i]->ready || b->ctx[i]->version != b->version[i]) return MOCD_ERR_NOT_READY;
-    int rc;
     for (mocd_ctx *c : b->ctx) {
         c->nodes_per_warp = nodes_per_warp;
         size_grids(c);
-        // Keep each member's own generation graph in the same launch shape.
+        // A member's own generation graph gets the same launch shape when it is
+        // next used.
         drop_graphs(c);
-        if ((rc = build_graph(c, c->timing ? 1 : 0))) return rc;
     }
     b->form = form;
     return batch_build(b);
