@@ -472,7 +472,7 @@ crossover_multi_kernel(const BatchMember *__restrict__ members, const int *__res
 //                degree there) and 65..128, so that no launch pays for the
 //                registers of a larger network than its own
 //   129..512     a warp per pair: count table in shared memory (the node's
-//                pairs are split over kWideParts warps), in the first launch
+//                pairs are split over gp.wide_parts warps), in the first launch
 //   above 512    mutation_hub_kernel, a block per pair
 // The launches touch different rows of Q and only add to the histogram, so
 // they run side by side.
@@ -587,6 +587,40 @@ __device__ __forceinline__ int lane_vote(const GenParams &gp, const int4 *__rest
     return select_at<N>(x, base + kth_bit(word, k));
 }
 
+// Adds the labels of the first 32 CHUNKS of the deg neighbours nbr to the
+// warp's count table.
+template <int CHUNKS>
+__device__ __forceinline__ void table_insert(const GenParams &gp, const int32_t *__restrict__ col,
+                                             const int *__restrict__ nbr, int deg, int *hkey, int *hcnt, int hbits)
+{
+    const int lane = threadIdx.x & 31;
+    int x[CHUNKS];
+#pragma unroll
+    for (int k = 0; k < CHUNKS; ++k) {
+        const int e = 32 * k + lane;
+        x[k] = e < deg ? col[(size_t)checked_node(__ldg(nbr + e), gp.n) * gp.W] : (int)(0x80000000u | lane);
+    }
+#pragma unroll
+    for (int k = 0; k < CHUNKS; ++k) {
+        if (32 * k >= deg) break;  // (warp-uniform)
+        // One insert per distinct label of the chunk, with its multiplicity.
+        const unsigned peers = __match_any_sync(kFull, x[k]);
+        if (x[k] >= 0 && (peers & ((1u << lane) - 1u)) == 0) {
+            uint32_t h = hash_slot(x[k], hbits);
+            // The table holds at most deg <= HS / 2 distinct labels, so an empty
+            // or matching slot is always found.
+            for (int probe = 0; probe < (1 << hbits); ++probe) {
+                const int prev = atomicCAS(hkey + h, -1, x[k]);
+                if (prev == -1 || prev == x[k]) {
+                    atomicAdd(hcnt + h, __popc(peers));
+                    break;
+                }
+                h = (h + 1) & (uint32_t)((1 << hbits) - 1);
+            }
+        }
+    }
+}
+
 // Exact neighbour-majority of one pair of a node with degree kDeferMax + 1 ..
 // kSharedTableMax by the whole warp: an open-addressing count table in shared
 // memory, sized to the node (the smallest power of two with at least 2 deg
@@ -605,40 +639,31 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
     int hbits = 8;
     while ((1 << hbits) < 2 * deg) ++hbits;
     const int HS = 1 << hbits;
-    const int per_lane = HS >> 5;  // 8 .. 32
-    for (int e = lane; e < HS; e += 32) {
-        hkey[e] = -1;
-        hcnt[e] = 0;
+    int4 *key4 = reinterpret_cast<int4 *>(hkey), *cnt4 = reinterpret_cast<int4 *>(hcnt);
+    for (int e = lane; e < HS / 4; e += 32) {
+        key4[e] = make_int4(-1, -1, -1, -1);
+        cnt4[e] = make_int4(0, 0, 0, 0);
     }
     __syncwarp();
-    for (int e0 = 0; e0 < deg; e0 += 32) {
-        const bool in = e0 + lane < deg;
-        int x = (int)(0x80000000u | lane);
-        if (in) x = child[(size_t)checked_node(__ldg(nbr + e0 + lane), gp.n) * W + i];
-        // One insert per distinct label of the chunk, with its multiplicity.
-        const unsigned peers = __match_any_sync(kFull, x);
-        if (in && (peers & ((1u << lane) - 1u)) == 0) {
-            uint32_t h = hash_slot(x, hbits);
-            // The table holds at most deg <= HS / 2 distinct labels, so an empty
-            // or matching slot is always found.
-            for (int probe = 0; probe < HS; ++probe) {
-                const int prev = atomicCAS(hkey + h, -1, x);
-                if (prev == -1 || prev == x) {
-                    atomicAdd(hcnt + h, __popc(peers));
-                    break;
-                }
-                h = (h + 1) & (uint32_t)(HS - 1);
-            }
-        }
-    }
+    // Four labels a lane in flight, then their inserts (eight or sixteen spill
+    // under the kernel's register cap: n = 10^6 2.91 -> 3.00 ms a generation).
+    for (int e0 = 0; e0 < deg; e0 += 128) table_insert<4>(gp, child + i, nbr + e0, deg - e0, hkey, hcnt, hbits);
     __syncwarp();
+    // Lane's slots: 4 (lane + 32 s) .. + 3, s < HS / 128 (2 .. 8).
     unsigned mx_l = 0;
-    for (int s = 0; s < per_lane; ++s) mx_l = max(mx_l, (unsigned)hcnt[lane + 32 * s]);
+    for (int s = 0; s < HS / 128; ++s) {
+        const int4 c = cnt4[lane + 32 * s];
+        mx_l = max(mx_l, (unsigned)max(max(c.x, c.y), max(c.z, c.w)));
+    }
     const unsigned mx = __reduce_max_sync(kFull, mx_l);
     best_count = mx;
     unsigned act = 0;
-    for (int s = 0; s < per_lane; ++s)
-        if ((unsigned)hcnt[lane + 32 * s] == mx) act |= 1u << s;
+    for (int s = 0; s < HS / 128; ++s) {
+        const int4 c = cnt4[lane + 32 * s];
+        act |= (((unsigned)c.x == mx ? 1u : 0u) | ((unsigned)c.y == mx ? 2u : 0u) | ((unsigned)c.z == mx ? 4u : 0u) |
+                ((unsigned)c.w == mx ? 8u : 0u))
+               << (4 * s);
+    }
     // Compact the tied labels into hcnt[0, t) (the counts are no longer needed).
     const unsigned mine = (unsigned)__popc(act);
     unsigned incl = mine;
@@ -650,8 +675,10 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
     const int t = (int)__shfl_sync(kFull, incl, 31);
     int at = (int)(incl - mine);
     __syncwarp();
-    for (int s = 0; s < per_lane; ++s)
-        if ((act >> s) & 1u) hcnt[at++] = hkey[lane + 32 * s];
+    for (unsigned m = act; m != 0u; m &= m - 1u) {
+        const int s = __ffs((int)m) - 1;
+        hcnt[at++] = hkey[4 * (lane + 32 * (s >> 2)) + (s & 3)];
+    }
     __syncwarp();
     const unsigned kk = t > 1 ? pick_index(tie_word(gp, v, i, g), (uint32_t)t) : 0u;
     int res;
@@ -746,7 +773,7 @@ __device__ __forceinline__ int list_selected(unsigned short *list, int total, un
     return __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
 }
 
-// hint of a part of a node (or of a hub's quad): (pairs << 16) | pairs whose
+// hint of a part of a node above degree 128: (pairs << 16) | pairs whose
 // own label was on more than half of the neighbours, last generation; 0: no
 // history. A quarter settled pays for the count.
 __device__ __forceinline__ bool own_label_pays(uint32_t h)
@@ -755,7 +782,7 @@ __device__ __forceinline__ bool own_label_pays(uint32_t h)
 }
 
 // Part `part` of a node of degree kDeferMax + 1 .. kSharedTableMax (position
-// idx): the quads q with q % kWideParts == part, a warp per pair.
+// idx): the quads q with q % gp.wide_parts == part, a warp per pair.
 __device__ __noinline__ void wide_item(const GenParams &gp, int idx, int part, const int4 *__restrict__ nodes,
                                        const int4 *__restrict__ adj, const int32_t *__restrict__ child,
                                        int32_t *__restrict__ q, uint32_t *__restrict__ hist,
@@ -767,12 +794,12 @@ __device__ __noinline__ void wide_item(const GenParams &gp, int idx, int part, c
     const int4 rec = __ldg(nodes + idx);
     const int v = rec.x, deg = rec.z;
     unsigned sel = 0;
-    if (lane < nq && lane % kWideParts == part) {
+    if (lane < nq && lane % gp.wide_parts == part) {
         const int4 out = reinterpret_cast<const int4 *>(child)[(size_t)v * nq + lane];
         sel = take_quad(gp, v, deg, lane, out, g, reinterpret_cast<int4 *>(q), hist);
     }
     const int total = list_selected(list, 0, sel, 4 * lane);
-    uint32_t *h = hint + (idx - gp.n_hub) * kWideParts + part;
+    uint32_t *h = hint + (idx - gp.n_hub) * gp.wide_parts + part;
     const bool fast = own_label_pays(*h);
     __syncwarp();
     int ok = 0;
@@ -843,13 +870,13 @@ mutation_kernel(const __grid_constant__ GenParams gp, int first, int last, const
 
     // Nodes in degree-descending order: every warp starts with one of the
     // costliest batches, which balances the grid-stride loop.
-    const int wide = WIDE ? gp.n_wide * kWideParts : 0;
+    const int wide = WIDE ? gp.n_wide * gp.wide_parts : 0;
     const int items = wide + (last - first + batch - 1) / batch;
     const unsigned inv_nq = (65536u + (unsigned)nq - 1u) / (unsigned)nq;  // t / nq = t * inv_nq >> 16, t < 2^10
     for (int item = warp; item < items; item += nwarps) {
         if (WIDE && item < wide) {
             int *table = reinterpret_cast<int *>(recs + mutation_warp_words(gp.np, batch, 0));
-            wide_item(gp, gp.n_hub + item / kWideParts, item % kWideParts, nodes, adj, child, q, hist, hint, list, table,
+            wide_item(gp, gp.n_hub + item / gp.wide_parts, item % gp.wide_parts, nodes, adj, child, q, hist, hint, list, table,
                       table + gp.hash_size, g);
             __syncwarp();
             continue;
@@ -949,21 +976,27 @@ __device__ __forceinline__ int block_mode_table(const GenParams &gp, const int32
     }
     if (threadIdx.x == 0) *s_tied = 0;
     __syncthreads();
-    for (int j0 = 0; j0 < deg; j0 += kHubBlock) {
-        const int j = j0 + threadIdx.x;
-        const bool in = j < deg;
-        const int x = in ? col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] : (int)(0x80000000u | lane);
-        // One insert per distinct label of the warp's neighbours.
-        const unsigned peers = __match_any_sync(kFull, x);
-        if (in && (peers & ((1u << lane) - 1u)) == 0) {
-            uint32_t h = hash_slot(x, hbits);
-            for (int probe = 0; probe < HS; ++probe) {  // (at most HS / 2 distinct labels: a slot is found)
-                const int prev = atomicCAS(hkey + h, -1, x);
-                if (prev == -1 || prev == x) {
-                    atomicAdd(hcnt + h, __popc(peers));
-                    break;
+    for (int j0 = 0; j0 < deg; j0 += 4 * kHubBlock) {
+        int x[4];  // four labels in flight per thread
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = j0 + k * kHubBlock + (int)threadIdx.x;
+            x[k] = j < deg ? col[(size_t)checked_node(__ldg(nbr + j), gp.n) * gp.W] : (int)(0x80000000u | lane);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            // One insert per distinct label of the warp's neighbours.
+            const unsigned peers = __match_any_sync(kFull, x[k]);
+            if (x[k] >= 0 && (peers & ((1u << lane) - 1u)) == 0) {
+                uint32_t h = hash_slot(x[k], hbits);
+                for (int probe = 0; probe < HS; ++probe) {  // (at most HS / 2 distinct labels: a slot is found)
+                    const int prev = atomicCAS(hkey + h, -1, x[k]);
+                    if (prev == -1 || prev == x[k]) {
+                        atomicAdd(hcnt + h, __popc(peers));
+                        break;
+                    }
+                    h = (h + 1) & (uint32_t)(HS - 1);
                 }
-                h = (h + 1) & (uint32_t)(HS - 1);
             }
         }
     }
@@ -1034,7 +1067,7 @@ mutation_hub_kernel(const __grid_constant__ GenParams gp, const int4 *__restrict
         const int4 rec = __ldg(nodes + idx);
         const int v = rec.x, deg = min(rec.z, gp.hub_hs / 2);
         const int *nbr = reinterpret_cast<const int *>(adj + rec.y);
-        uint32_t *h = hint + gp.n_wide * kWideParts + t;
+        uint32_t *h = hint + gp.n_wide * gp.wide_parts + t;
         const bool fast = own_label_pays(*h);
         const int4 own4 = reinterpret_cast<const int4 *>(child)[(size_t)v * nq + quad];
         unsigned sel;

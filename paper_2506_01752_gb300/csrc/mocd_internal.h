@@ -48,9 +48,6 @@ constexpr int kMutBatchMax = 16;  // most nodes a warp of the mutation takes at 
 // Up to this degree a pair's vote is a warp's, with a count table in shared
 // memory; above it a block's (mutation_hub_kernel).
 constexpr int kSharedTableMax = 512;
-// Warps that share the pairs of a node of degree kDeferMax + 1 ..
-// kSharedTableMax (label quads q with q % kWideParts equal).
-constexpr int kWideParts = 8;
 // Largest count table of the hub kernel in shared memory (slots of 8 bytes).
 constexpr int kHubSmemSlots = 16384;
 // Random stream stages (third word of the Philox counter is the generation).
@@ -78,7 +75,7 @@ struct PopState {
     int64_t *fint;            // [2][kMaxPop]: intra, S of each front member
     double *fval;             // [2][kMaxPop]: f1, f2 of each front member
     uint32_t *hint;           // (mutating pairs << 16) | pairs whose own label is on more than half of the
-                              // neighbours, last generation: kWideParts per node of degree kDeferMax + 1 ..
+                              // neighbours, last generation: wide_parts per node of degree kDeferMax + 1 ..
                               // kSharedTableMax, then one per hub and quad of children
     int *hub_table;           // hub_blocks x 2 hub_hs: count tables of hubs too large for shared memory
 };
@@ -91,6 +88,7 @@ struct GenParams {
     int label_bits;           // bits needed for a label in [0, n)
     int hash_size;            // per-warp hash entries for degree > kDeferMax (0: none)
     int n_hub, n_wide;        // nodes of degree > kSharedTableMax, and of kDeferMax + 1 .. kSharedTableMax
+    int wide_parts;           // warps that share the pairs of a node of degree kDeferMax + 1 .. kSharedTableMax
     int n_vote[2];            // nodes of degree 33..64 and 65..128
     int hub_hs;               // slots of the largest hub's count table (power of two >= 2 dmax; 0: no hubs)
     int hub_smem_hs;          // slots of the hub kernel's shared table (<= kHubSmemSlots)

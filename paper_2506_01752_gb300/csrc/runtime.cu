@@ -47,6 +47,12 @@ constexpr int kChunkGraph = 2;
 constexpr double kMutPairs = 96.0;
 constexpr long long kMutWaves = 2;
 constexpr long long kMutRounds = 24;
+// Nodes of degree 129 .. 512: a warp per quad of children (about one pair, which
+// takes long: with eighths of a node the launch waits for a warp with six) up
+// to this many quads, above it eighths, whose rows and coins are cheaper. A
+// generation with quads: hubs 116 -> 89 us, dense 118 -> 105 us, n = 10^6 (275,000
+// quads) 2.93 -> 3.01 ms.
+constexpr int64_t kWideItems = 65536;
 // The edge count: up to four full GPUs of blocks, as long as a warp keeps this
 // many nodes (n = 170,001 464 -> 454 us a generation, n = 10^6 3.33 -> 3.26 ms;
 // two rounds at n = 40,000 are 2 us slower).
@@ -274,7 +280,7 @@ void size_grids(mocd_ctx *c)
     const double pairs = std::max(0.5, c->params.p_mutation * c->params.pop_size);
     for (int cls = 0; cls < 3; ++cls) {
         const long long nodes = cls > 0 ? c->n_vote[cls - 1] : n - c->n_vote[0] - c->n_vote[1] - c->n_wide - c->n_hub;
-        const long long wide = cls == 0 ? (long long)c->n_wide * kWideParts : 0;
+        const long long wide = cls == 0 ? (long long)c->n_wide * c->gp.wide_parts : 0;
         const int most = (int)std::max<long long>(1, std::min<long long>(kMutBatchMax, (long long)(kMutPairs / pairs)));
         const int occ = grid_for_mutation(c->sms, cls, c->gp.vote_n0, c->gp.hash_size, c->gp.np, most);
         const long long warps = (long long)occ * mutation_warps_per_block();
@@ -291,7 +297,7 @@ void size_grids(mocd_ctx *c)
 // Words of PopState::hint.
 size_t hint_words(const mocd_ctx *c)
 {
-    return (size_t)kWideParts * (size_t)c->n_wide + (size_t)(kMaxPop / 4) * (size_t)c->n_hub;
+    return (size_t)(kMaxPop / 4) * (size_t)(c->n_wide + c->n_hub);
 }
 
 // Allocate (or reuse) the population buffers for params and fill gp / ps.
@@ -400,6 +406,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.n_vote[1] = (int)c->n_vote[1];
     gp.n_hub = (int)c->n_hub;
     gp.n_wide = (int)c->n_wide;
+    gp.wide_parts = c->n_wide * (W >> 2) <= kWideItems ? W >> 2 : std::min(8, W >> 2);
     gp.hub_hs = hub_hs;
     gp.hub_smem_hs = hub_smem_hs;
     c->mut.hub_blocks = hub_blocks;

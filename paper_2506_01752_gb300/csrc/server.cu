@@ -295,12 +295,12 @@ int mocd_job_footprint(int64_t n, const int64_t *row_ptr, int32_t pop_size, int6
 {
     if (!bytes || !row_ptr || n < 1 || pop_size < 1 || pop_size > mocd::kMaxPop) return MOCD_ERR_INVALID_ARG;
     const int64_t nnz = row_ptr[n];
-    int64_t hints = 0;   // one per part or quad of children of the nodes above kDeferMax
+    int64_t hints = 0;   // one per quad of children of the nodes above kDeferMax
     int64_t groups = 0;  // of four entries of the mutation's adjacency
     int64_t dmax = 0;
     for (int64_t v = 0; v < n; ++v) {
         const int64_t d = row_ptr[v + 1] - row_ptr[v];
-        hints += d > mocd::kSharedTableMax ? mocd::kMaxPop / 4 : d > mocd::kDeferMax ? mocd::kWideParts : 0;
+        hints += d > mocd::kDeferMax ? mocd::kMaxPop / 4 : 0;
         groups += (d + 3) / 4;
         dmax = d > dmax ? d : dmax;
     }
