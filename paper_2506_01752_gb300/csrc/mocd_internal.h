@@ -167,8 +167,8 @@ cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts,
 // directions of every edge (full), or the oriented adjacency; deg_ptr: row
 // pointers whose differences are the degrees. Up to kHistBlockBytes of labels
 // the histogram of each labelling is one block's shared memory; above, it is
-// hist [n][stride] (stride >= count), zero on entry and again afterwards.
-constexpr int64_t kHistBlockBytes = 200 * 1024;
+// hist [n][stride] (stride >= count), zero on entry.
+constexpr int64_t kHistBlockBytes = 160 * 1024;
 bool evaluate_needs_histogram(int64_t n);
 cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, const int32_t *deg_ptr,
                             const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,

@@ -513,10 +513,11 @@ int start_population(mocd_ctx *c, uint32_t base_gen)
     if (rc) return rc;
     // No mutation history yet.
     CK(cudaMemsetAsync(ps.hint, 0, sizeof(uint32_t) * hint_words(c), c->stream));
-    // (The sweep leaves the histogram zero, as generations expect it: the
-    // mutation adds into it.)
     CK(launch_evaluate(gp.n, gp.W, gp.np, gp.W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, phalf, ps.hist, ps.acc,
                        ps.acc + kMaxPop, c->sms, c->stream, c->d_order));
+    // Generations expect a zero histogram (the mutation adds into it).
+    if (evaluate_needs_histogram(c->n))
+        CK(cudaMemsetAsync(ps.hist, 0, sizeof(uint32_t) * (size_t)gp.W * (size_t)gp.n, c->stream));
     CK(launch_select(gp, ps, 0, c->stream, base_gen));
     // The generation graph is captured while the GPU works on the above.
     drop_graphs(c);
