@@ -48,8 +48,8 @@ namespace mocd {
 
 namespace {
 
-// FULL: row_ptr / col_idx hold both directions of every edge, else each edge
-// once (the oriented adjacency). ADD: the degrees (from deg_ptr) go into the
+// FULL: row_ptr / col_idx hold both directions of every edge, rows by node id;
+// else each edge once, lists by position in the order (the oriented adjacency). ADD: the degrees (from deg_ptr) go into the
 // histogram; otherwise a histogram (if given) is complete: square and clear it.
 template <bool FULL, bool ADD>
 __device__ __forceinline__ void evaluate_body(int n, int W, int count, int stride,
@@ -63,73 +63,128 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
 {
     __shared__ unsigned long long s_intra[kMaxPop];
     __shared__ unsigned long long s_sq[kMaxPop];
-    __shared__ int s_nb[kBlock];  // per warp: the chunk's neighbours u > v
+    __shared__ int s_nb[FULL ? kBlock : 1];  // FULL, per warp: the chunk's neighbours u > v
     for (int t = threadIdx.x; t < kMaxPop; t += blockDim.x) {
         s_intra[t] = 0;
         s_sq[t] = 0;
     }
     __syncthreads();
 
-    const int lane = threadIdx.x & 31;
     const int nq = W >> 2;
-    const bool active = lane < nq;
-    const int warp = (vblock * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (vgrid * blockDim.x) >> 5;
+    const int wlane = threadIdx.x & 31;
+    // A warp takes as many nodes at a time as its lanes hold rows (FULL: one).
+    const int per_warp = FULL ? 1 : 32 / nq;
+    const int sub = FULL ? 0 : wlane / nq;
+    const int lane = wlane - sub * nq;  // the quad of individuals
+    const bool active = sub < per_warp && lane < nq;
+    const int first = ((vblock * blockDim.x + threadIdx.x) >> 5) * per_warp + sub;
+    const int nodes = ((vgrid * blockDim.x) >> 5) * per_warp;  // taken at a time by all warps
     const int4 *__restrict__ L4 = reinterpret_cast<const int4 *>(labels);
     const int i0 = 4 * lane;
-    int *nb = s_nb + (threadIdx.x & ~31);
-    const unsigned lt = (1u << lane) - 1u;
 
     uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0;
     unsigned long long q0 = 0, q1 = 0, q2 = 0, q3 = 0;
 
-    for (int idx = warp; idx < n; idx += nwarps) {
-        const int v = order ? __ldg(order + idx) : idx;
-        const int beg = __ldg(row_ptr + v);
-        const int end = __ldg(row_ptr + v + 1);
-        if (!MOCD_CHECK(end >= beg, kCheckRowPtr, v)) continue;  // (warp-uniform)
-        const int4 own = active ? L4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
-        for (int e0 = beg; e0 < end; e0 += 32) {
-            const int cnt = min(32, end - e0);
-            const int my_u = lane < cnt ? __ldg(col_idx + e0 + lane) : 0;
-            // Keep the neighbours whose rows v reads, compacted: u > v of the
-            // full adjacency, or every entry of the oriented one.
-            const bool up = lane < cnt && (!FULL || my_u > v) && MOCD_CHECK(my_u < n, kCheckNode, v);
-            const unsigned upm = __ballot_sync(0xffffffffu, up);
-            const int cu = __popc(upm);
-            if (up) nb[__popc(upm & lt)] = my_u;
-            __syncwarp();
-            // Four independent row loads in flight per lane.
-            for (int j0 = 0; j0 < cu; j0 += 4) {
-                int4 a[4];
+    // Counts, per individual, the rows u (-1: none) that agree with `own`: four
+    // independent row loads in flight per lane.
+    auto count4 = [&](const int (&u)[4], const int4 &own) {
+        int4 a[4];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int u = nb[min(j0 + t, cu - 1)];
-                    a[t] = (active && j0 + t < cu) ? L4[(size_t)u * nq + lane] : make_int4(-1, -1, -1, -1);
-                }
+        for (int t = 0; t < 4; ++t)
+            a[t] = active && u[t] >= 0 ? L4[(size_t)u[t] * nq + lane] : make_int4(-1, -1, -1, -1);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    c0 += a[t].x == own.x;
-                    c1 += a[t].y == own.y;
-                    c2 += a[t].z == own.z;
-                    c3 += a[t].w == own.w;
-                }
-            }
-            __syncwarp();
+        for (int t = 0; t < 4; ++t) {
+            c0 += a[t].x == own.x;
+            c1 += a[t].y == own.y;
+            c2 += a[t].z == own.z;
+            c3 += a[t].w == own.w;
         }
-        const unsigned d = !ADD ? 0u : FULL ? (unsigned)(end - beg)
-                                          : (unsigned)(__ldg(deg_ptr + v + 1) - __ldg(deg_ptr + v));
-        if (ADD && active && d > 0) {
-            const unsigned long long d2 = (unsigned long long)d * d, dd = 2ull * d;
-            uint32_t *cell = hist + i0;
-            if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v))
-                q0 += dd * atomicAdd(cell + (size_t)own.x * stride + 0, d) + d2;
-            if (i0 + 1 < count && MOCD_CHECK((unsigned)own.y < (unsigned)n, kCheckLabel, v))
-                q1 += dd * atomicAdd(cell + (size_t)own.y * stride + 1, d) + d2;
-            if (i0 + 2 < count && MOCD_CHECK((unsigned)own.z < (unsigned)n, kCheckLabel, v))
-                q2 += dd * atomicAdd(cell + (size_t)own.z * stride + 2, d) + d2;
-            if (i0 + 3 < count && MOCD_CHECK((unsigned)own.w < (unsigned)n, kCheckLabel, v))
-                q3 += dd * atomicAdd(cell + (size_t)own.w * stride + 3, d) + d2;
+    };
+    // Adds degree d of node v to the histogram cells of its labels.
+    auto add = [&](int v, const int4 &own, unsigned d) {
+        if (!active || d == 0) return;
+        const unsigned long long d2 = (unsigned long long)d * d, dd = 2ull * d;
+        uint32_t *cell = hist + i0;
+        if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v))
+            q0 += dd * atomicAdd(cell + (size_t)own.x * stride + 0, d) + d2;
+        if (i0 + 1 < count && MOCD_CHECK((unsigned)own.y < (unsigned)n, kCheckLabel, v))
+            q1 += dd * atomicAdd(cell + (size_t)own.y * stride + 1, d) + d2;
+        if (i0 + 2 < count && MOCD_CHECK((unsigned)own.z < (unsigned)n, kCheckLabel, v))
+            q2 += dd * atomicAdd(cell + (size_t)own.z * stride + 2, d) + d2;
+        if (i0 + 3 < count && MOCD_CHECK((unsigned)own.w < (unsigned)n, kCheckLabel, v))
+            q3 += dd * atomicAdd(cell + (size_t)own.w * stride + 3, d) + d2;
+    };
+    if constexpr (FULL) {
+        int *nb = s_nb + (threadIdx.x & ~31);
+        for (int v = first; v < n; v += nodes) {
+            const int beg = __ldg(row_ptr + v);
+            const int end = __ldg(row_ptr + v + 1);
+            if (!MOCD_CHECK(end >= beg, kCheckRowPtr, v)) continue;  // (warp-uniform)
+            const int4 own = active ? L4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
+            for (int e0 = beg; e0 < end; e0 += 32) {
+                const int cnt = min(32, end - e0);
+                const int my_u = wlane < cnt ? __ldg(col_idx + e0 + wlane) : 0;
+                // Keep the neighbours u > v, compacted.
+                const bool up = wlane < cnt && my_u > v && MOCD_CHECK(my_u < n, kCheckNode, v);
+                const unsigned upm = __ballot_sync(0xffffffffu, up);
+                const int cu = __popc(upm);
+                if (up) nb[__popc(upm & ((1u << wlane) - 1u))] = my_u;
+                __syncwarp();
+                for (int j0 = 0; j0 < cu; j0 += 4) {
+                    int u[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) u[t] = j0 + t < cu ? nb[j0 + t] : -1;
+                    count4(u, own);
+                }
+                __syncwarp();
+            }
+            if (ADD) add(v, own, (unsigned)(end - beg));
+        }
+    } else {
+        // A node takes four dependent loads (position -> id and list -> own row
+        // and entries -> rows) and has ten entries or so: the kernel is bound by
+        // that chain unless the next nodes' loads are under way. While a node's
+        // rows are compared, the next one's own row and first entries and the
+        // one after's id and list bounds are requested.
+        auto entries = [&](int e, int end, int (&u)[4]) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                u[t] = e + t < end ? __ldg(col_idx + e + t) : -1;
+                if (!MOCD_CHECK(u[t] < n, kCheckNode, e)) u[t] = -1;
+            }
+        };
+        auto head = [&](long long idx, int &v, int &beg, int &end) {
+            const bool in = active && idx < n;
+            v = in ? __ldg(order + idx) : 0;
+            beg = in ? __ldg(row_ptr + idx) : 0;
+            end = in ? __ldg(row_ptr + idx + 1) : 0;
+            if (!MOCD_CHECK(end >= beg, kCheckRowPtr, v)) end = beg;
+        };
+        int v, beg, end, v1, beg1, end1, u[4];
+        head(first, v, beg, end);
+        head((long long)first + nodes, v1, beg1, end1);
+        int4 own = active && first < n ? L4[(size_t)v * nq + lane] : make_int4(0, 0, 0, 0);
+        entries(beg, end, u);
+        for (long long idx = first; active && idx < n; idx += nodes) {
+            int v2, beg2, end2, u1[4];
+            const int4 own1 = L4[(size_t)v1 * nq + lane];
+            entries(beg1, end1, u1);
+            head(idx + 2ll * nodes, v2, beg2, end2);
+            for (int e = beg; e < end; e += 4) {
+                const int cur[4] = {u[0], u[1], u[2], u[3]};
+                entries(e + 4, end, u);
+                count4(cur, own);
+            }
+            if (ADD) add(v, own, (unsigned)(__ldg(deg_ptr + v + 1) - __ldg(deg_ptr + v)));
+            v = v1;
+            beg = beg1;
+            end = end1;
+            own = own1;
+            v1 = v2;
+            beg1 = beg2;
+            end1 = end2;
+#pragma unroll
+            for (int t = 0; t < 4; ++t) u[t] = u1[t];
         }
     }
 
@@ -140,16 +195,16 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
         // 64-bit sums are exact.
         uint4 *__restrict__ H4 = reinterpret_cast<uint4 *>(hist);
         // Four rows in flight per lane.
-        for (int c0 = warp; c0 < n; c0 += 4 * nwarps) {
+        for (long long c0 = first; c0 < n; c0 += 4ll * nodes) {
             uint4 x[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int c = c0 + k * nwarps;
+                const long long c = c0 + (long long)k * nodes;
                 x[k] = c < n ? H4[(size_t)c * nq + lane] : make_uint4(0, 0, 0, 0);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int c = c0 + k * nwarps;
+                const long long c = c0 + (long long)k * nodes;
                 if (x[k].x | x[k].y | x[k].z | x[k].w) {
                     q0 += (unsigned long long)x[k].x * x[k].x;
                     q1 += (unsigned long long)x[k].y * x[k].y;
@@ -176,7 +231,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
 // beside: the launch before this one on the stream (hist_block_kernel) only
 // runs beside it: nothing here depends on it, but this launch ends after it.
 template <bool FULL, bool ADD>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 4)
 evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__ deg_ptr,
                 const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col_idx, const int32_t *__restrict__ labels,

@@ -5,8 +5,8 @@
 //   warp takes a row v; each lane takes one of its neighbours u and binary
 //   searches v in the (sorted) row of u. A missing mirror sets *bad.
 // * the oriented adjacency of the offspring evaluation: every undirected
-//   edge listed once, at its endpoint of lower (degree, id). A warp per node
-//   counts the neighbours above it, one block scans the counts into row
+//   edge listed once, at its endpoint of lower (degree, id), the lists in
+//   processing order. A warp per node counts the neighbours above it, one block scans the counts into row
 //   pointers, and a warp per node writes the entries in row order.
 // * the mutation's adjacency: the rows in processing order (degree
 //   descending), padded to groups of four entries with the id n, so that a
@@ -56,23 +56,25 @@ __device__ __forceinline__ bool above(const int32_t *__restrict__ row_ptr, int v
     return du > dv || (du == dv && u > v);
 }
 
-// eptr[v + 1] = neighbours of v above v; eptr[0] = 0.
+// eptr[k + 1] = neighbours above v, v the node at position k of the order;
+// eptr[0] = 0.
 __global__ void __launch_bounds__(kBlock)
 orient_count_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                    int32_t *__restrict__ eptr)
+                    const int32_t *__restrict__ order, int32_t *__restrict__ eptr)
 {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     if (warp == 0 && lane == 0) eptr[0] = 0;
-    for (int v = warp; v < n; v += nwarps) {
+    for (int k = warp; k < n; k += nwarps) {
+        const int v = __ldg(order + k);
         const int beg = __ldg(row_ptr + v), end = __ldg(row_ptr + v + 1);
         int cnt = 0;
         for (int k0 = beg; k0 < end; k0 += 32) {
             const bool up = k0 + lane < end && above(row_ptr, v, end - beg, __ldg(col_idx + k0 + lane));
             cnt += __popc(__ballot_sync(0xffffffffu, up));
         }
-        if (lane == 0) eptr[v + 1] = cnt;
+        if (lane == 0) eptr[k + 1] = cnt;
     }
 }
 
@@ -105,19 +107,20 @@ __global__ void scan_kernel(int32_t *__restrict__ a, int len)
     }
 }
 
-// eidx[eptr[v] ..] = the neighbours of v above v, in row order; positions at
-// or past cap (possible only for an asymmetric graph) are skipped.
+// eidx[eptr[k] ..] = the neighbours above v (at position k), in row order;
+// entries at or past cap (possible only for an asymmetric graph) are skipped.
 __global__ void __launch_bounds__(kBlock)
 orient_fill_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                   const int32_t *__restrict__ eptr, int32_t *__restrict__ eidx, int cap)
+                   const int32_t *__restrict__ order, const int32_t *__restrict__ eptr, int32_t *__restrict__ eidx, int cap)
 {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    for (int v = warp; v < n; v += nwarps) {
+    for (int k = warp; k < n; k += nwarps) {
+        const int v = __ldg(order + k);
         const int beg = __ldg(row_ptr + v), end = __ldg(row_ptr + v + 1);
-        int at = eptr[v];
+        int at = eptr[k];
         for (int k0 = beg; k0 < end; k0 += 32) {
             const int u = k0 + lane < end ? __ldg(col_idx + k0 + lane) : 0;
             const bool up = k0 + lane < end && above(row_ptr, v, end - beg, u);
@@ -172,14 +175,14 @@ int warp_grid(const void *kernel, int n, int sms)
 
 }  // namespace
 
-cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx, int32_t *eptr, int32_t *eidx,
-                          int cap, int sms, cudaStream_t s)
+cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
+                          int32_t *eptr, int32_t *eidx, int cap, int sms, cudaStream_t s)
 {
     orient_count_kernel<<<warp_grid((const void *)orient_count_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr,
-                                                                                                col_idx, eptr);
+                                                                                                col_idx, order, eptr);
     scan_kernel<<<1, 1024, 0, s>>>(eptr, n + 1);
     orient_fill_kernel<<<warp_grid((const void *)orient_fill_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr, col_idx,
-                                                                                              eptr, eidx, cap);
+                                                                                              order, eptr, eidx, cap);
     return cudaGetLastError();
 }
 

@@ -1234,7 +1234,9 @@ int grid_for_mutation(int sms, int cls, int vote_n0, int hash_size, int np, int 
 int grid_for_hubs(int sms, int smem_hs)
 {
     const int smem = 2 * smem_hs * (int)sizeof(int);
-    cudaFuncSetAttribute(mutation_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // (The limit is the function's, for every context: always the largest table.)
+    cudaFuncSetAttribute(mutation_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         2 * kHubSmemSlots * (int)sizeof(int));
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mutation_hub_kernel, kHubBlock, smem);
     return sms * (per_sm < 1 ? 1 : per_sm);

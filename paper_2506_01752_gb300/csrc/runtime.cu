@@ -82,7 +82,7 @@ struct mocd_ctx {
     // The offspring evaluation's adjacency: each undirected edge once, listed
     // at its endpoint of lower (degree, id), so that the label rows it reads
     // are those of the higher-degree endpoints (fewer, each read more often:
-    // more of them stay in L2). eptr [n + 1], eidx [m].
+    // more of them stay in L2). eptr [n + 1] by position in the order, eidx [m].
     int32_t *d_eptr = nullptr;
     int32_t *d_eidx = nullptr;
 
@@ -270,10 +270,10 @@ void size_grids(mocd_ctx *c)
     };
     // The edge count: several rounds of blocks where each warp keeps kEvalNodes
     // nodes (a block that ends early makes room for the next).
-    const long long rounds = n / ((long long)c->occ_eval_intra * (kBlock / 32) * kEvalNodes);
-    c->grid_eval_intra =
-        shape((int)std::max<long long>(1, std::min<long long>(4, rounds)) * c->occ_eval_intra, kBlock / 32);
-    c->grid_cross = shape(c->occ_cross, kBlock / 32 * (32 / (c->W >> 2)));
+    const int rows = kBlock / 32 * (32 / (c->W >> 2));  // nodes a block of either kernel takes at a time
+    const long long rounds = n / ((long long)c->occ_eval_intra * rows * kEvalNodes);
+    c->grid_eval_intra = shape((int)std::max<long long>(1, std::min<long long>(4, rounds)) * c->occ_eval_intra, rows);
+    c->grid_cross = shape(c->occ_cross, rows);
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
     // kMutPairs of them: five full rounds), but a class too small to give
     // every resident warp kMutWaves batches gets smaller ones.
@@ -364,6 +364,9 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
         CK(cudaMemsetAsync(c->ps.c + cells, 0x7f, (size_t)W * sizeof(int32_t), c->stream));
     }
     const size_t hist_need = (size_t)W * (size_t)c->n;
+    // A limit of the interface: N_p times the nodes of degree 33 .. kDeferMax and
+    // the hubs fits 31 bits.
+    if ((int64_t)p->pop_size * (c->n_vote[0] + c->n_vote[1] + c->n_hub) > INT_MAX) return MOCD_ERR_INVALID_ARG;
     // Hubs: the hub kernel's count table is in shared memory if the largest
     // hub's fits there, else (for the pairs that do not fit) a table of hub_hs
     // slots (keys and counts) per block in global memory, at most 1 GiB in all.
@@ -1120,7 +1123,7 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
             cudaSuccess &&
         cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream) == cudaSuccess &&
         launch_symmetry_check((int)n, c->d_row_ptr, c->d_col_idx, d_bad, c->sms, c->stream) == cudaSuccess &&
-        launch_orient((int)n, c->d_row_ptr, c->d_col_idx, c->d_eptr, c->d_eidx, (int)(nnz / 2), c->sms,
+        launch_orient((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_eptr, c->d_eidx, (int)(nnz / 2), c->sms,
                       c->stream) == cudaSuccess &&
         launch_mutation_adjacency((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, d_by_degree, c->d_nodes, c->d_adj,
                                   c->sms, c->stream) == cudaSuccess &&
