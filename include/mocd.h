@@ -27,9 +27,10 @@
  *
  * Limits: 1 <= N_p <= 128, 1 <= E_S <= 16, n < 2^30, 2m < 2^31, and
  * N_p x (number of nodes of degree 33..128 or above 512) < 2^31. There is no
- * degree limit: the mutation's count tables of hubs above degree 512 live in
- * a global scratch of at most 1 GiB per context (one table per warp of the
- * hub kernel, each 2 x the smallest power of two >= 2 d_max ints).
+ * degree limit: the mutation's count tables of hubs above degree 512 are in
+ * shared memory up to degree 8192, above that in a global scratch of at most
+ * 1 GiB per context (one table per block of the hub kernel, each 2 x the
+ * smallest power of two >= 2 d_max ints).
  */
 #ifndef MOCD_H
 #define MOCD_H
@@ -108,7 +109,8 @@ int mocd_population_init(mocd_ctx *ctx, const mocd_params *params);
 
 /*
  * Run n_generations generations of Alg. 1 (the "for gen" loop body), issued
- * asynchronously on the context stream as one CUDA graph launch each.
+ * asynchronously on the context stream as CUDA graph launches: one per
+ * generation, or one per eight in a run of 24 or more without stage timing.
  * Errors: INVALID_ARG (n_generations < 0), NOT_READY, CUDA.
  */
 int mocd_generation(mocd_ctx *ctx, int32_t n_generations);
@@ -222,8 +224,8 @@ int mocd_evaluate(mocd_ctx *ctx, int32_t count, const int32_t *labels, int64_t *
  * plug-in whose process gives all free device memory to another allocator, a
  * component under a fixed device-memory budget, or a latency-critical loop
  * that cannot take cudaMalloc's implicit synchronisation). It computes the
- * same exact intra and S as mocd_evaluate, with the evaluation kernel's
- * per-individual histogram kept in a fixed 16 MiB array compiled into the
+ * same exact intra and S as mocd_evaluate, with each individual's histogram
+ * in shared memory (n <= 40,960) or in a fixed 16 MiB array compiled into the
  * library, which every GPU that loads the library holds until exit.
  *   row_ptr  device int32[n + 1], col_idx device int32[row_ptr[n]]: the
  *            symmetric CSR (no self loops, no repeats; not validated here)
@@ -284,11 +286,10 @@ int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_idx, int64_
  *                       its own graph branch (the chains proceed
  *                       independently); 1 runs the selections of all members
  *                       in one launch (a block per member) after every chain
- *                       has evaluated; 2 also runs the crossover, the
- *                       deferred per-pair mutation votes and the evaluation
- *                       of all members in one launch each (each member owns a
- *                       range of the launch's blocks), only the mutation
- *                       kernels staying per member.
+ *                       has evaluated; 2 also runs the crossover and the
+ *                       evaluation of all members in one launch each (each
+ *                       member owns a range of the launch's blocks), only the
+ *                       mutation kernels staying per member.
  *                       Errors: INVALID_ARG, NOT_READY, CUDA.
  *   mocd_batch_form     reports the current nodes per warp and form.
  */
@@ -349,11 +350,11 @@ void mocd_batch_destroy(mocd_batch *b);
  *                       runs (admission compares their sum with the budget):
  *                       the four label buffers and the degree histogram
  *                       (5 x 4 n W bytes, W = N_p rounded up to a multiple of
- *                       4), the CSR and node order, the mutation's per-node
- *                       hints (4 n), deferred-vote list (8 N_p per node of
- *                       degree 33..128 or above 512) and hub count tables
- *                       (graphs with a degree above 512), the individual-major
- *                       buffer of the
+ *                       4), the CSR and its oriented copy, the node order,
+ *                       the mutation's node records and padded rows (16 bytes
+ *                       a node and per four entries), its hints (128 bytes per
+ *                       node of degree above 128) and global hub count tables
+ *                       (a degree above 8192), the individual-major buffer of the
  *                       front download (4 n N_p) and 1 MiB of small state.
  *                       Errors: INVALID_ARG.
  */
@@ -430,9 +431,8 @@ int mocd_synchronize(mocd_ctx *ctx);
  * of the method): when enabled, the generation graph records CUDA events
  * between its kernels. mocd_kernel_times writes, for the most recent
  * generation, the duration in milliseconds of each stage, in this order:
- * crossover, mutation (its main kernel plus the per-pair vote kernels of
- * the graph's degree classes; it also builds the degree histogram of the
- * children), evaluation (which squares and clears that histogram),
+ * crossover, mutation (the kernels of the graph's degree classes, side by
+ * side; they also build the degree histogram of the children), evaluation (which squares and clears that histogram),
  * selection; returns the number of stages (4) or a negative status.
  * NOT_READY if timing is off or no generation ran since it was enabled.
  */
@@ -443,7 +443,7 @@ int mocd_kernel_times(mocd_ctx *ctx, float *ms, int32_t cap);
  * Number of kernel launches in one generation (measurement support): the
  * kernel nodes of the captured generation graph without timing events.
  * It depends on the graph: crossover, mutation, evaluation and selection,
- * plus one per-pair vote kernel for each degree class the graph has
+ * plus one more mutation kernel for each further degree class the graph has
  * (33..64, 65..128, above 512). Captures the graph if it does not exist
  * yet. NOT_READY before initialisation.
  */

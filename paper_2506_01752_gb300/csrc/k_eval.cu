@@ -32,8 +32,8 @@
 // which writes every child's final label of node v, adds deg(v) to the
 // label-major cell of that label as it goes (fire-and-forget reductions that
 // overlap its own latency-bound work). The evaluation of the offspring then
-// counts intra (COUNT_D = false) and, in the same launch once a warp's nodes
-// are done, forms S = sum_c D_c^2 in a coalesced sweep of the histogram rows,
+// counts intra (ADD = false) and, in the same launch once a warp's nodes are
+// done, forms S = sum_c D_c^2 in a coalesced sweep of the histogram rows,
 // zeroing them for the next generation. While the labels are still nearly all distinct, the N_p n
 // histogram additions land on different sectors, which at n = 10^6 (a 400 MB
 // histogram) cost a DRAM read and write-back each; done by the mutation
@@ -141,7 +141,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
             if (ADD) add(v, own, (unsigned)(end - beg));
         }
     } else {
-        // A node takes four dependent loads (position -> id and list -> own row
+        // A node takes a chain of dependent loads (position -> id and list -> own row
         // and entries -> rows) and has ten entries or so: the kernel is bound by
         // that chain unless the next nodes' loads are under way. While a node's
         // rows are compared, the next one's own row and first entries and the

@@ -2,8 +2,8 @@
 // topology-aware crossover (Sec. 4.3.1, Alg. 2) and topology-aware mutation
 // (Sec. 4.3.2), for all N_p children of a generation at once.
 //
-// Both kernels work on node-major rows: a warp owns node v; lane q owns the
-// four children 4q..4q+3, which share one Philox call per stage because the
+// Both kernels work on node-major rows, in quads: the four children 4q..4q+3
+// of a node are one lane's, and share one Philox call per stage because the
 // stream counter of (child i, node v) is (v, i / 4, g, stage), word i % 4.
 #include <limits.h>
 
@@ -833,8 +833,18 @@ __host__ __device__ __forceinline__ int mutation_warp_words(int np, int batch, i
     return batch + (batch * np * 2 + 15) / 16 + hash_size / 2;
 }
 
-// The nodes at positions [first, last) of the order, of degree <= N
-// (N > kLaneMax: also above the next smaller class, see launch_mutation).
+// The nodes at positions [first, last) of the order, of degree <= N.
+//
+// Bound by the half-rate integer pipe (58% of its peak at n = 40,000, the sorting
+// networks) with waits for gathered labels between, so four-node batches in many
+// blocks and 28 warps an SM; at n = 10^6 by DRAM and the L2's atomic rate (the
+// histogram additions are 0.7 of 2.4 ms). Sizes of networks in steps of two, or
+// 32 to 40 warps with fewer registers, are slower (instruction cache, spills).
+// The launch for degrees up to 32, against one node a warp, staged labels and
+// deferred votes of the higher degrees in launches behind it: n = 40,000 66.7 us
+// + 12.7 -> 44.6, n = 170,001 270 us + 86 -> 205, n = 10^6 (tenth generation)
+// 3.38 ms + 0.53 -> 2.0.
+//
 // WIDE: the launch also takes the nodes of degree kDeferMax + 1 ..
 // kSharedTableMax (positions n_hub .. n_hub + n_wide - 1). batch: nodes a warp
 // takes at a time (<= kMutBatchMax).

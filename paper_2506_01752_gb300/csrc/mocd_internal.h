@@ -6,8 +6,8 @@
 //                            of row v is individual i's label of node v, so a
 //                            warp reads a node's labels for every individual
 //                            as one contiguous 16-byte-per-lane row.
-//   hist     uint32 [Np][n] per-individual community degree totals D_c
-//                            (scratch, cleared before every evaluation)
+//   hist     uint32 [n][W]  label-major community degree totals D_c of every
+//                            individual (zero between evaluations)
 //   CSR      int32 row_ptr[n + 1], int32 col_idx[2m] (symmetric)
 //   order    int32[n] nodes by degree, descending (work order of the
 //            degree-proportional kernels; results do not depend on it)

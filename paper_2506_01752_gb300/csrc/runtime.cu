@@ -1,9 +1,9 @@
 // runtime.cu -- host side of the C ABI declared in include/mocd.h.
 //
 // A context owns the uploaded CSR, the population buffers (node-major label
-// rows, see mocd_internal.h) and one CUDA graph that runs a whole generation
-// of Alg. 1: crossover -> mutation (which also builds the degree histogram of
-// the offspring) -> evaluate -> select.
+// rows, see mocd_internal.h) and CUDA graphs that run a whole generation of
+// Alg. 1, or eight: crossover -> mutation (which also builds the degree
+// histogram of the offspring) -> evaluate -> select.
 // Every kernel reads the generation number from device memory, so the same
 // graph is replayed for every generation with no host work in between.
 #include <algorithm>
@@ -275,7 +275,7 @@ void size_grids(mocd_ctx *c)
     c->grid_eval_intra = shape((int)std::max<long long>(1, std::min<long long>(4, rounds)) * c->occ_eval_intra, rows);
     c->grid_cross = shape(c->occ_cross, rows);
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
-    // kMutPairs of them: five full rounds), but a class too small to give
+    // kMutPairs of them), but a class too small to give
     // every resident warp kMutWaves batches gets smaller ones.
     const double pairs = std::max(0.5, c->params.p_mutation * c->params.pop_size);
     for (int cls = 0; cls < 3; ++cls) {
