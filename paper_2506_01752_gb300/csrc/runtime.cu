@@ -15,6 +15,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <thread>
@@ -485,24 +486,48 @@ int issue_generation(mocd_ctx *c, cudaStream_t st, bool events, bool with_select
 }
 
 // Capture generation graph k (0 plain, 1 with stage events, kChunkGraph), if
-// missing.
+// missing. A caller's stream is not captured itself (another thread may be
+// issuing on it, or the caller capturing it): a stream of its priority is.
 int build_graph(mocd_ctx *c, int k)
 {
     if (c->graph_exec[k]) return MOCD_OK;
-    CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = MOCD_OK;
-    for (int u = 0; u < (k == kChunkGraph ? kChunk : 1) && rc == MOCD_OK; ++u)
-        rc = issue_generation(c, c->stream, k == 1);
+    cudaStream_t st = c->stream;
+    if (!c->own_stream) {
+        int priority = 0;
+        CK(cudaStreamGetPriority(c->stream, &priority));
+        CK(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, priority));
+    }
     cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+    cudaGraphExec_t x = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+    int rc = cuda_status(e);
+    if (e == cudaSuccess) {
+        for (int u = 0; u < (k == kChunkGraph ? kChunk : 1) && rc == MOCD_OK; ++u)
+            rc = issue_generation(c, st, k == 1);
+        e = cudaStreamEndCapture(st, &g);
+        if (rc == MOCD_OK) rc = cuda_status(e);
+    }
+    if (rc == MOCD_OK) rc = cuda_status(cudaGraphInstantiate(&x, g, 0));
+    if (st != c->stream) cudaStreamDestroy(st);
     if (rc) {
         if (g) cudaGraphDestroy(g);
         return rc;
     }
-    CK(e);
     c->graph[k] = g;
-    CK(cudaGraphInstantiate(&c->graph_exec[k], g, 0));
+    c->graph_exec[k] = x;
     return MOCD_OK;
+}
+
+// The graph of kChunk generations, if it can be had. The caller's thread may
+// be capturing a stream, which takes no notice in the relaxed mode.
+void build_chunk_graph(mocd_ctx *c)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess) {
+        build_graph(c, kChunkGraph);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    cudaGetLastError();
 }
 
 // Evaluate, rank and draw the first tournament of a population whose labels
@@ -1194,12 +1219,13 @@ int mocd_generation(mocd_ctx *c, int32_t n_generations)
     };
     if (g == 0 && (c->graph_exec[kChunkGraph] ? left >= kChunk : left >= 3 * kChunk)) {
         // The first long run of a population: its graph is captured while the
-        // GPU works on the generations launched one at a time.
+        // GPU works on the generations launched one at a time. Where it cannot be
+        // had, they all are.
         if (!c->graph_exec[kChunkGraph]) {
             if ((rc = launch(0, kChunk))) return rc;
-            if ((rc = build_graph(c, kChunkGraph))) return rc;
+            build_chunk_graph(c);
         }
-        if ((rc = launch(kChunkGraph, left / kChunk))) return rc;
+        if (c->graph_exec[kChunkGraph] && (rc = launch(kChunkGraph, left / kChunk))) return rc;
     }
     if ((rc = launch(g, left))) return rc;
     c->host_gen += n_generations;
@@ -1363,8 +1389,9 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
     if ((rc = eval_scratch(c))) return rc;
     // The labels are checked on the device, as they are rearranged; results
     // are handed out once all batches have passed.
-    std::vector<unsigned long long> acc(kEvalWords);
-    std::vector<int64_t> keys(2 * (size_t)count);
+    unsigned long long acc[kEvalWords];
+    std::unique_ptr<int64_t[]> keys(new (std::nothrow) int64_t[2 * (size_t)count]);
+    if (!keys) return MOCD_ERR_OUT_OF_MEMORY;
     for (int b0 = 0; b0 < count; b0 += batch) {
         const int b = std::min(batch, count - b0);
         const int W = (b + 3) & ~3;
@@ -1375,7 +1402,7 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
         if (apart) CK(cudaMemsetAsync(c->d_eval_hist, 0, sizeof(uint32_t) * (size_t)W * n, c->stream));
         CK(launch_evaluate((int)n, W, b, W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, c->d_nm, c->d_eval_hist,
                            c->d_eval_acc, c->d_eval_acc + kMaxPop, c->sms, c->stream, c->d_order));
-        CK(cudaMemcpyAsync(acc.data(), c->d_eval_acc, sizeof(unsigned long long) * kEvalWords,
+        CK(cudaMemcpyAsync(acc, c->d_eval_acc, sizeof(unsigned long long) * kEvalWords,
                            cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
         if (acc[2 * kMaxPop]) return MOCD_ERR_INVALID_ARG;
@@ -1384,8 +1411,8 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
             keys[(size_t)count + b0 + k] = (int64_t)acc[kMaxPop + k];
         }
     }
-    std::copy(keys.begin(), keys.begin() + count, intra);
-    std::copy(keys.begin() + count, keys.end(), sumsq);
+    std::copy_n(keys.get(), count, intra);
+    std::copy_n(keys.get() + count, count, sumsq);
     return MOCD_OK;
 }
 

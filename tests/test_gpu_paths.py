@@ -163,3 +163,65 @@ def test_server_result_above_a_copy_chunk():
         srv.close()
     assert ref.labels.nbytes > 2 << 20
     assert np.array_equal(got.labels, ref.labels) and np.array_equal(got.sumsq, ref.sumsq)
+
+
+# Eights are captured inside generation(): on a caller's stream, and while the
+# caller's thread captures another stream.
+@pytest.mark.parametrize("capturing", [False, True])
+def test_eights_on_a_callers_stream(capturing):
+    torch = pytest.importorskip("torch")
+    rp, ci, _ = synth.planted_partition(5, 30, 0.3, 0.02, seed=4)
+    op = oracle.Params(pop_size=20, seed=3)
+    ref = oracle.run(rp, ci, op, oracle.population_init(rp, ci, op), 41)
+    x = torch.zeros(8, device="cuda")
+    own, other, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    h = mocd.graph_upload(rp, ci, own)
+    try:
+        mocd.population_init(h, mocd.Params(pop_size=20, seed=3))
+        torch.cuda.synchronize()
+        if capturing:
+            with torch.cuda.stream(other):
+                graph.capture_begin()
+                x.add_(1)
+                mocd.generation(h, 41)
+                graph.capture_end()
+            graph.replay()
+        else:
+            mocd.generation(h, 41)
+        _state_equals(h, ref)
+    finally:
+        mocd.destroy(h)
+    torch.cuda.synchronize()
+    assert float(x.sum()) == (8 if capturing else 0)
+
+
+# Both forms of the scoring's histogram, captured once and replayed twice.
+@pytest.mark.parametrize("n", [1000, 40_964])
+def test_noalloc_scoring_in_a_callers_graph(n):
+    torch = pytest.importorskip("torch")
+    rp, ci = _regular(n, 6, seed=n)
+    count, graph, side = 8, torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    lab = synth.random_labels(n, count, seed=1, n_distinct=300)
+    rows = torch.from_numpy(lab.T.copy()).cuda()
+    out = torch.full((2, count), -1, dtype=torch.int64, device="cuda")
+    d_rp, d_ci = torch.from_numpy(rp.astype(np.int32)).cuda(), torch.from_numpy(ci).cuda()
+
+    def score(stream):
+        mocd.evaluate_noalloc(d_rp.data_ptr(), d_ci.data_ptr(), n, rows.data_ptr(), count, out[0].data_ptr(),
+                              out[1].data_ptr(), stream)
+
+    with torch.cuda.stream(side):
+        score(side)  # looks the scratch's address up
+        side.synchronize()
+        graph.capture_begin()
+        score(side)
+        graph.capture_end()
+    for seed in (2, 3):
+        lab = synth.random_labels(n, count, seed=seed, n_distinct=n if seed == 3 else 300)
+        rows.copy_(torch.from_numpy(lab.T.copy()))
+        out.fill_(-1)
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        ref = oracle.objectives(rp, ci, lab)
+        assert np.array_equal(out[0].cpu().numpy(), ref[0]) and np.array_equal(out[1].cpu().numpy(), ref[1])
