@@ -72,11 +72,12 @@ extern "C" int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const int W = (count + 3) & ~3;
-    // The results are accumulated in place; the scratch keeps the previous
-    // call's contents: clear what must start at 0.
+    // intra, and S with its histogram in the scratch (which keeps the previous
+    // call's contents), are accumulated in place: clear what must start at 0.
     const size_t bytes = sizeof(int64_t) * (size_t)count;
-    if (cudaMemsetAsync(intra, 0, bytes, s) != cudaSuccess || cudaMemsetAsync(sumsq, 0, bytes, s) != cudaSuccess ||
-        (evaluate_needs_histogram(n) &&
+    if (cudaMemsetAsync(intra, 0, bytes, s) != cudaSuccess) return MOCD_ERR_CUDA;
+    if (evaluate_needs_histogram(n) &&
+        (cudaMemsetAsync(sumsq, 0, bytes, s) != cudaSuccess ||
          cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (size_t)count * (size_t)n, s) != cudaSuccess))
         return MOCD_ERR_CUDA;
     int sms = 1;
