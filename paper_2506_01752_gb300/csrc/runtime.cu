@@ -485,12 +485,41 @@ int issue_generation(mocd_ctx *c, cudaStream_t st, bool events, bool with_select
     return MOCD_OK;
 }
 
+// Makes a device current for as long as the object lives, then the one before.
+class OnDevice {
+  public:
+    explicit OnDevice(int device)
+    {
+        status_ = cudaGetDevice(&before_);
+        if (status_ == cudaSuccess && before_ != device) {
+            status_ = cudaSetDevice(device);
+            changed_ = status_ == cudaSuccess;
+        }
+    }
+    ~OnDevice()
+    {
+        if (changed_) cudaSetDevice(before_);
+    }
+    OnDevice(const OnDevice &) = delete;
+    OnDevice &operator=(const OnDevice &) = delete;
+    cudaError_t status() const { return status_; }
+
+  private:
+    int before_ = 0;
+    bool changed_ = false;
+    cudaError_t status_ = cudaSuccess;
+};
+
 // Capture generation graph k (0 plain, 1 with stage events, kChunkGraph), if
 // missing. A caller's stream is not captured itself (another thread may be
-// issuing on it, or the caller capturing it): a stream of its priority is.
+// issuing on it, or the caller capturing it): a stream of its priority is. A
+// generation may be asked for while another device is current, but kernels are
+// captured for the current one.
 int build_graph(mocd_ctx *c, int k)
 {
     if (c->graph_exec[k]) return MOCD_OK;
+    const OnDevice here(c->device);
+    CK(here.status());
     cudaStream_t st = c->stream;
     if (!c->own_stream) {
         int priority = 0;
