@@ -333,8 +333,12 @@ cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, cons
     if (!add) {
         // A histogram block fills one SM's shared memory on `count` of them; the
         // edge count takes the rest of the GPU at the same time.
-        cudaFuncSetAttribute(hist_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistBlockBytes);
+        // (If it cannot be had, nothing would write sumsq.)
+        cudaError_t e = cudaFuncSetAttribute(hist_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kHistBlockBytes);
+        if (e != cudaSuccess) return e;
         hist_block_kernel<<<count, kHistThreads, n * sizeof(uint32_t), s>>>(n, W, deg_ptr, labels, sumsq);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         cudaLaunchAttribute attr = {};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
