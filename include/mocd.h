@@ -225,8 +225,8 @@ int mocd_evaluate(mocd_ctx *ctx, int32_t count, const int32_t *labels, int64_t *
  * component under a fixed device-memory budget, or a latency-critical loop
  * that cannot take cudaMalloc's implicit synchronisation). It computes the
  * same exact intra and S as mocd_evaluate, with each individual's histogram
- * in shared memory (n <= 40,960) or in a fixed 16 MiB array compiled into the
- * library, which every GPU that loads the library holds until exit.
+ * in shared memory (up to 40,960 nodes, where that is the faster one) or in a
+ * fixed 16 MiB array compiled into the library, which every GPU that loads the library holds until exit.
  *   row_ptr  device int32[n + 1], col_idx device int32[row_ptr[n]]: the
  *            symmetric CSR (no self loops, no repeats; not validated here)
  *   n        nodes, 1 <= n < 2^30

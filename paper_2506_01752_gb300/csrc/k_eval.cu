@@ -22,11 +22,14 @@
 // atomic returns the old total o, and (o + d)^2 - o^2 = 2 o d + d^2. Summed
 // over every addition these increments telescope to D_c^2 whatever the order
 // of the atomics, so S is exact and deterministic. (Reductions and a sweep
-// afterwards took 10 us more at n = 40,000, count 100, and 20 us more at n =
-// 51,300, count 81.) Histogram layout: label-major, D of (individual i, label
-// c) at c * stride + i, so that one atomic instruction of a warp (25
+// afterwards took 20 us more at n = 51,300, count 81.) Histogram layout: with
+// the oriented adjacency (contexts) label-major, D of (individual i, label c) at
+// c * W + i, as the generations have it: one atomic instruction of a warp (25
 // individuals of node v) lands in few cache lines whenever individuals share
-// v's label.
+// v's label. With the full adjacency (mocd_evaluate_noalloc) individual-major,
+// i * n + c: cells of different individuals then do not share sectors, which
+// additions take turns on (n = 60,000, 69 labellings: of one community each
+// 1,224 us label-major and 140 so, of some 500 communities 62 and 64).
 //
 // Inside a generation the D histogram is not built here: the mutation kernel,
 // which writes every child's final label of node v, adds deg(v) to the
@@ -48,11 +51,15 @@ namespace mocd {
 
 namespace {
 
+// Blocks of the edge count that an SM holds, by their registers (48 and 62).
+constexpr int kFullBlocks = 5;
+constexpr int kOrientedBlocks = 4;
+
 // FULL: row_ptr / col_idx hold both directions of every edge, rows by node id;
 // else each edge once, lists by position in the order (the oriented adjacency). ADD: the degrees (from deg_ptr) go into the
 // histogram; otherwise a histogram (if given) is complete: square and clear it.
 template <bool FULL, bool ADD>
-__device__ __forceinline__ void evaluate_body(int n, int W, int count, int stride,
+__device__ __forceinline__ void evaluate_body(int n, int W, int count,
                                               const int32_t *__restrict__ deg_ptr,
                                               const int32_t *__restrict__ row_ptr,
                                               const int32_t *__restrict__ col_idx,
@@ -107,15 +114,17 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
     auto add = [&](int v, const int4 &own, unsigned d) {
         if (!active || d == 0) return;
         const unsigned long long d2 = (unsigned long long)d * d, dd = 2ull * d;
-        uint32_t *cell = hist + i0;
+        auto cell = [&](int k, int c) {
+            return FULL ? hist + (size_t)(i0 + k) * n + c : hist + (size_t)c * W + i0 + k;
+        };
         if (i0 + 0 < count && MOCD_CHECK((unsigned)own.x < (unsigned)n, kCheckLabel, v))
-            q0 += dd * atomicAdd(cell + (size_t)own.x * stride + 0, d) + d2;
+            q0 += dd * atomicAdd(cell(0, own.x), d) + d2;
         if (i0 + 1 < count && MOCD_CHECK((unsigned)own.y < (unsigned)n, kCheckLabel, v))
-            q1 += dd * atomicAdd(cell + (size_t)own.y * stride + 1, d) + d2;
+            q1 += dd * atomicAdd(cell(1, own.y), d) + d2;
         if (i0 + 2 < count && MOCD_CHECK((unsigned)own.z < (unsigned)n, kCheckLabel, v))
-            q2 += dd * atomicAdd(cell + (size_t)own.z * stride + 2, d) + d2;
+            q2 += dd * atomicAdd(cell(2, own.z), d) + d2;
         if (i0 + 3 < count && MOCD_CHECK((unsigned)own.w < (unsigned)n, kCheckLabel, v))
-            q3 += dd * atomicAdd(cell + (size_t)own.w * stride + 3, d) + d2;
+            q3 += dd * atomicAdd(cell(3, own.w), d) + d2;
     };
     if constexpr (FULL) {
         int *nb = s_nb + (threadIdx.x & ~31);
@@ -245,8 +254,8 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count, int strid
 // beside: the launch before this one on the stream (hist_block_kernel) only
 // runs beside it: nothing here depends on it, but this launch ends after it.
 template <bool FULL, bool ADD>
-__global__ void __launch_bounds__(kBlock, 4)
-evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__ deg_ptr,
+__global__ void __launch_bounds__(kBlock, FULL ? kFullBlocks : kOrientedBlocks)
+evaluate_kernel(int n, int W, int count, const int32_t *__restrict__ deg_ptr,
                 const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col_idx, const int32_t *__restrict__ labels,
                 uint32_t *__restrict__ hist, unsigned long long *__restrict__ intra,
@@ -256,7 +265,7 @@ evaluate_kernel(int n, int W, int count, int stride, const int32_t *__restrict__
     // as soon as every block here runs.
     if (!beside) cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
-    evaluate_body<FULL, ADD>(n, W, count, stride, deg_ptr, row_ptr, col_idx, labels, hist, intra, sumsq, order,
+    evaluate_body<FULL, ADD>(n, W, count, deg_ptr, row_ptr, col_idx, labels, hist, intra, sumsq, order,
                              blockIdx.x, gridDim.x);
     if (beside) cudaGridDependencySynchronize();
 }
@@ -316,7 +325,7 @@ evaluate_multi_kernel(const BatchMember *__restrict__ members, const int *__rest
     }
     const BatchMember &mb = members[lo];
     const int b0 = __ldg(starts + lo);
-    evaluate_body<false, false>(mb.gp.n, mb.gp.W, mb.gp.np, mb.gp.W, nullptr, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
+    evaluate_body<false, false>(mb.gp.n, mb.gp.W, mb.gp.np, nullptr, mb.eptr, mb.eidx, mb.ps.q, mb.ps.hist, mb.ps.acc,
                          mb.ps.acc + kMaxPop, mb.order, bk - b0, __ldg(starts + lo + 1) - b0);
 }
 
@@ -330,20 +339,32 @@ int grid_for_eval_intra(int sms)
     return sms * per_sm;
 }
 
-bool evaluate_needs_histogram(int64_t n) { return n * (int64_t)sizeof(uint32_t) > kHistBlockBytes; }
+// A histogram block takes a time of its own, however few labellings there are
+// (it reads a sector a node), and longer where a row is 128 or 256 bytes; the
+// histogram in global memory takes longer the more there are. With the full
+// adjacency, whose launch has no other work to hide either, global memory is
+// the faster one in a band of few labellings of many nodes (us a call, full
+// adjacency of mean degree 16, blocks / global): n = 27,000, 32 labellings 35.7
+// / 35.2, 48 34.3 / 43.0; n = 34,000, 32 47.5 / 36.1, 56 41.7 / 48.6, 100 44.6 /
+// 61.1; n = 40,960, 20 39.1 / 39.4, 36 46.8 / 41.3, 64 56.2 / 54.4, 100 52.7 /
+// 71.9. With the oriented adjacency the blocks are no slower up to their limit,
+// and several times faster where the labels are few.
+bool evaluate_needs_histogram(int64_t n, int W, bool full)
+{
+    if (n * (int64_t)sizeof(uint32_t) > kHistBlockBytes) return true;
+    return full && ((n > 27000 && (W == 32 || W == 64)) || (n > 30000 && W > 24 && W <= 48));
+}
 
-cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, const int32_t *deg_ptr,
+cudaError_t launch_evaluate(int n, int W, int count, bool full, const int32_t *deg_ptr,
                             const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,
                             unsigned long long *intra, unsigned long long *sumsq, int sms, cudaStream_t s,
                             const int32_t *order)
 {
-    const bool add = evaluate_needs_histogram(n);
+    const bool add = evaluate_needs_histogram(n, W, full);
     const auto kernel = full ? (add ? evaluate_kernel<true, true> : evaluate_kernel<true, false>)
                              : (add ? evaluate_kernel<false, true> : evaluate_kernel<false, false>);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBlock, 0);
-    const long long blocks =
-        std::min<long long>((long long)sms * std::max(per_sm, 1), ((long long)n + kBlock / 32 - 1) / (kBlock / 32));
+    const long long blocks = std::min<long long>((long long)sms * (full ? kFullBlocks : kOrientedBlocks),
+                                                 ((long long)n + kBlock / 32 - 1) / (kBlock / 32));
     if (!add) {
         // A histogram block fills one SM's shared memory on `count` of them; the
         // edge count takes the rest of the GPU at the same time.
@@ -362,10 +383,10 @@ cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, cons
         cfg.stream = s;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, kernel, n, W, count, stride, deg_ptr, row_ptr, col_idx, labels,
+        return cudaLaunchKernelEx(&cfg, kernel, n, W, count, deg_ptr, row_ptr, col_idx, labels,
                                   static_cast<uint32_t *>(nullptr), intra, sumsq, order, true);
     }
-    kernel<<<(int)blocks, kBlock, 0, s>>>(n, W, count, stride, deg_ptr, row_ptr, col_idx, labels, hist, intra, sumsq,
+    kernel<<<(int)blocks, kBlock, 0, s>>>(n, W, count, deg_ptr, row_ptr, col_idx, labels, hist, intra, sumsq,
                                           order, false);
     return cudaGetLastError();
 }
@@ -381,7 +402,7 @@ cudaError_t launch_evaluate_offspring(int n, int W, int count, const int32_t *ep
                                       const int32_t *labels, uint32_t *hist, unsigned long long *acc,
                                       int grid, cudaStream_t s, const int32_t *order)
 {
-    evaluate_kernel<false, false><<<grid, kBlock, 0, s>>>(n, W, count, W, nullptr, eptr, eidx, labels, hist, acc,
+    evaluate_kernel<false, false><<<grid, kBlock, 0, s>>>(n, W, count, nullptr, eptr, eidx, labels, hist, acc,
                                                         acc + kMaxPop, order, false);
     return cudaGetLastError();
 }

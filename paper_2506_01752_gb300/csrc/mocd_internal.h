@@ -165,12 +165,13 @@ cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts,
 // Objectives of `count` labellings (node-major rows of W): adds the edge counts
 // into intra and S into sumsq (both zero on entry). row_ptr / col_idx: both
 // directions of every edge (full), or the oriented adjacency; deg_ptr: row
-// pointers whose differences are the degrees. Up to kHistBlockBytes of labels
-// the histogram of each labelling is one block's shared memory; above, it is
-// hist [n][stride] (stride >= count), zero on entry.
+// pointers whose differences are the degrees. The histogram of each labelling
+// is one block's shared memory (up to kHistBlockBytes), or, where
+// evaluate_needs_histogram says so, hist: [n][W], full: [count][n], zero on
+// entry.
 constexpr int64_t kHistBlockBytes = 160 * 1024;
-bool evaluate_needs_histogram(int64_t n);
-cudaError_t launch_evaluate(int n, int W, int count, int stride, bool full, const int32_t *deg_ptr,
+bool evaluate_needs_histogram(int64_t n, int W, bool full);
+cudaError_t launch_evaluate(int n, int W, int count, bool full, const int32_t *deg_ptr,
                             const int32_t *row_ptr, const int32_t *col_idx, const int32_t *labels, uint32_t *hist,
                             unsigned long long *intra, unsigned long long *sumsq, int sms, cudaStream_t s,
                             const int32_t *order = nullptr);

@@ -12,7 +12,7 @@
 // and outputs.
 //
 // The scratch below is a device symbol: every GPU that loads this library
-// holds it (16 MiB) until the process exits. On the host its name is
+// holds it (16 MiB + 2 KiB) until the process exits. On the host its name is
 // only a stand-in, never a device address, so the address is fetched once per
 // device with cudaGetSymbolAddress (the first call on each device does that)
 // and then passed to the kernels. The cached address belongs to the device's
@@ -27,15 +27,26 @@ using namespace mocd;
 
 namespace {
 
-constexpr size_t kScratchWords = (size_t)MOCD_NOALLOC_MAX_CELLS;
+constexpr size_t kAccWords = 4 * kMaxPop;  // 2 x kMaxPop unsigned long long
+constexpr size_t kScratchWords = kAccWords + (size_t)MOCD_NOALLOC_MAX_CELLS;
 constexpr int kMaxDevices = 64;
 
-// The histogram [n][count] of a graph whose labels do not fit a block's shared
-// memory.
+// [0, kAccWords): intra and S; then the histogram [count][n]. Used where the
+// histograms are not in shared memory.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[kScratchWords];
 
 uint32_t *g_scratch_addr[kMaxDevices];
 std::mutex g_setup_mutex;
+
+__global__ void finish_keys_kernel(int count, const unsigned long long *__restrict__ acc,
+                                   int64_t *__restrict__ intra, int64_t *__restrict__ sumsq)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < count) {
+        intra[i] = (int64_t)acc[i];
+        sumsq[i] = (int64_t)acc[kMaxPop + i];
+    }
+}
 
 // Address of the scratch on the current device, set up on first use.
 int scratch_on_current_device(uint32_t **out, int *device)
@@ -72,19 +83,24 @@ extern "C" int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const int W = (count + 3) & ~3;
-    // intra, and S with its histogram in the scratch (which keeps the previous
-    // call's contents), are accumulated in place: clear what must start at 0.
-    const size_t bytes = sizeof(int64_t) * (size_t)count;
-    if (cudaMemsetAsync(intra, 0, bytes, s) != cudaSuccess) return MOCD_ERR_CUDA;
-    if (evaluate_needs_histogram(n) &&
-        (cudaMemsetAsync(sumsq, 0, bytes, s) != cudaSuccess ||
-         cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (size_t)count * (size_t)n, s) != cudaSuccess))
-        return MOCD_ERR_CUDA;
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MOCD_ERR_CUDA;
-    if (launch_evaluate((int)n, W, count, count, true, row_ptr, row_ptr, col_idx, labels, scratch,
-                        reinterpret_cast<unsigned long long *>(intra), reinterpret_cast<unsigned long long *>(sumsq), sms,
-                        s) != cudaSuccess)
+    if (!evaluate_needs_histogram(n, W, true)) {
+        // S is written by the launch that has its histograms, intra accumulated in place.
+        unsigned long long *in = reinterpret_cast<unsigned long long *>(intra);
+        if (cudaMemsetAsync(in, 0, sizeof(int64_t) * (size_t)count, s) != cudaSuccess ||
+            launch_evaluate((int)n, W, count, true, row_ptr, row_ptr, col_idx, labels, nullptr, in,
+                            reinterpret_cast<unsigned long long *>(sumsq), sms, s) != cudaSuccess)
+            return MOCD_ERR_CUDA;
+        return MOCD_OK;
+    }
+    // The scratch keeps the previous call's contents: clear what must start at 0.
+    unsigned long long *acc = reinterpret_cast<unsigned long long *>(scratch);
+    if (cudaMemsetAsync(scratch, 0, sizeof(uint32_t) * (kAccWords + (size_t)count * (size_t)n), s) != cudaSuccess ||
+        launch_evaluate((int)n, W, count, true, row_ptr, row_ptr, col_idx, labels, scratch + kAccWords, acc,
+                        acc + kMaxPop, sms, s) != cudaSuccess)
         return MOCD_ERR_CUDA;
+    finish_keys_kernel<<<1, kMaxPop, 0, s>>>(count, acc, intra, sumsq);
+    if (cudaGetLastError() != cudaSuccess) return MOCD_ERR_CUDA;
     return MOCD_OK;
 }

@@ -570,10 +570,10 @@ int start_population(mocd_ctx *c, uint32_t base_gen)
     if (rc) return rc;
     // No mutation history yet.
     CK(cudaMemsetAsync(ps.hint, 0, sizeof(uint32_t) * hint_words(c), c->stream));
-    CK(launch_evaluate(gp.n, gp.W, gp.np, gp.W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, phalf, ps.hist, ps.acc,
+    CK(launch_evaluate(gp.n, gp.W, gp.np, false, c->d_row_ptr, c->d_eptr, c->d_eidx, phalf, ps.hist, ps.acc,
                        ps.acc + kMaxPop, c->sms, c->stream, c->d_order));
     // Generations expect a zero histogram (the mutation adds into it).
-    if (evaluate_needs_histogram(c->n))
+    if (evaluate_needs_histogram(c->n, gp.W, false))
         CK(cudaMemsetAsync(ps.hist, 0, sizeof(uint32_t) * (size_t)gp.W * (size_t)gp.n, c->stream));
     CK(launch_select(gp, ps, 0, c->stream, base_gen));
     // The generation graph is captured while the GPU works on the above.
@@ -1413,7 +1413,7 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
     const size_t n = (size_t)c->n;
     if ((rc = grow(c->stream, &c->d_im, &c->im_cap, (size_t)batch * n))) return rc;
     if ((rc = grow(c->stream, &c->d_nm, &c->nm_cap, (size_t)kMaxPop * n))) return rc;
-    const bool apart = evaluate_needs_histogram(c->n);
+    const bool apart = evaluate_needs_histogram(c->n, (batch + 3) & ~3, false);
     if (apart && (rc = grow(c->stream, &c->d_eval_hist, &c->eval_hist_cap, (size_t)((batch + 3) & ~3) * n))) return rc;
     if ((rc = eval_scratch(c))) return rc;
     // The labels are checked on the device, as they are rearranged; results
@@ -1429,7 +1429,7 @@ int mocd_evaluate(mocd_ctx *c, int32_t count, const int32_t *labels, int64_t *in
                            cudaMemcpyHostToDevice, c->stream));
         CK(launch_to_node_major((int)n, W, b, c->d_im, c->d_nm, eval_bad(c), c->stream));
         if (apart) CK(cudaMemsetAsync(c->d_eval_hist, 0, sizeof(uint32_t) * (size_t)W * n, c->stream));
-        CK(launch_evaluate((int)n, W, b, W, false, c->d_row_ptr, c->d_eptr, c->d_eidx, c->d_nm, c->d_eval_hist,
+        CK(launch_evaluate((int)n, W, b, false, c->d_row_ptr, c->d_eptr, c->d_eidx, c->d_nm, c->d_eval_hist,
                            c->d_eval_acc, c->d_eval_acc + kMaxPop, c->sms, c->stream, c->d_order));
         CK(cudaMemcpyAsync(acc, c->d_eval_acc, sizeof(unsigned long long) * kEvalWords,
                            cudaMemcpyDeviceToHost, c->stream));

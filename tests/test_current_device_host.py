@@ -84,7 +84,7 @@ cudaError_t launch_front(const GenParams &, const PopState &, cudaStream_t s) { 
 cudaError_t launch_orient(int, const int32_t *, const int32_t *, const int32_t *, int32_t *, int32_t *, int, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_select(const GenParams &, const PopState &, int, cudaStream_t s, uint32_t) { return launched(s); }
 cudaError_t launch_select_multi(const GenParams *, const PopState *, int, int, cudaStream_t s) { return launched(s); }
-cudaError_t launch_evaluate(int, int, int, int, bool, const int32_t *, const int32_t *, const int32_t *, const int32_t *, uint32_t *, unsigned long long *, unsigned long long *, int, cudaStream_t s, const int32_t *) { return launched(s); }
+cudaError_t launch_evaluate(int, int, int, bool, const int32_t *, const int32_t *, const int32_t *, const int32_t *, uint32_t *, unsigned long long *, unsigned long long *, int, cudaStream_t s, const int32_t *) { return launched(s); }
 cudaError_t launch_evaluate_multi(const BatchMember *, const int *, int, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_evaluate_offspring(int, int, int, const int32_t *, const int32_t *, const int32_t *, uint32_t *, unsigned long long *, int, cudaStream_t s, const int32_t *) { return launched(s); }
 cudaError_t launch_mutation(const GenParams &, const PopState &, const int4 *, const int4 *, const MutationShape &, cudaStream_t s) { return launched(s); }
@@ -105,7 +105,7 @@ int grid_for_crossover(int sms, int, int) { return sms; }
 int grid_for_eval_intra(int sms) { return sms; }
 int crossover_row_words(int) { return 1; }
 int mutation_warps_per_block() { return 4; }
-bool evaluate_needs_histogram(int64_t) { return false; }
+bool evaluate_needs_histogram(int64_t, int, bool) { return false; }
 }
 
 #define DO(call) if (const int rc = (call)) { printf("%s: %d\n", #call, rc); return 1; }

@@ -76,3 +76,67 @@ def test_scoring_of_collapsed_labellings(n, d, count):
                           out[1].data_ptr(), torch.cuda.current_stream())
     torch.cuda.synchronize()
     assert np.array_equal(out[0].cpu().numpy(), ref[0]) and np.array_equal(out[1].cpu().numpy(), ref[1])
+
+
+def _scoring(torch, rp, ci, lab):
+    count, n = lab.shape
+    rows = torch.zeros((n, (count + 3) // 4 * 4), dtype=torch.int32)
+    rows[:, :count] = torch.from_numpy(lab.T.copy())
+    rows, out = rows.cuda(), torch.full((2, count), -1, dtype=torch.int64, device="cuda")
+    d_rp, d_ci = torch.from_numpy(rp.astype(np.int32)).cuda(), torch.from_numpy(ci).cuda()
+
+    def run():
+        mocd.evaluate_noalloc(d_rp.data_ptr(), d_ci.data_ptr(), n, rows.data_ptr(), count, out[0].data_ptr(),
+                              out[1].data_ptr(), torch.cuda.current_stream())
+        return out
+    return run
+
+
+def _pass_us(torch, run, passes=50):
+    for _ in range(10):
+        run()
+    best = float("inf")
+    for _ in range(7):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        for _ in range(passes):
+            run()
+        torch.cuda.synchronize()
+        best = min(best, (time.perf_counter() - t) / passes * 1e6)
+    return best
+
+
+# Where the scoring's histograms move between shared and global memory, by the
+# nodes (27,000, 30,000, 40,960) and the row (32 and 64 labellings, 25 to 48).
+@pytest.mark.parametrize("n", [27_000, 27_001, 30_001, 40_961])
+@pytest.mark.parametrize("count", [24, 25, 29, 32, 33, 48, 49, 61, 64, 65])
+def test_scoring_in_either_histogram(n, count):
+    torch = pytest.importorskip("torch")
+    rp, ci = _regular(n, 6, seed=n)
+    lab = synth.random_labels(n, count, seed=count, n_distinct=200)
+    lab[:, -1] = n - 1
+    lab[-1] = n - 1  # the last labelling's last label, everywhere
+    ref = oracle.objectives_parallel(rp, ci, lab)
+    run = _scoring(torch, rp, ci, lab)
+    for _ in range(2):  # the second call finds what the first left
+        got = run().cpu().numpy()
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+
+
+# Few communities: the labellings' cells must not share sectors, where the
+# additions of all nodes would take turns.
+def test_scoring_of_few_communities_is_no_cliff():
+    torch = pytest.importorskip("torch")
+    rp, ci = _regular(60_000, 10, seed=2)
+    many = synth.random_labels(60_000, 64, seed=1, n_distinct=600)
+    few = np.broadcast_to(many[:1] % 2, many.shape)
+    assert _pass_us(torch, _scoring(torch, rp, ci, few)) < 3 * _pass_us(torch, _scoring(torch, rp, ci, many))
+
+
+# A row of 128 bytes, which a histogram block reads slowest.
+def test_scoring_of_32_labellings_costs_little_more_than_20():
+    torch = pytest.importorskip("torch")
+    rp, ci = _regular(40_000, 16, seed=2)
+    t = {c: _pass_us(torch, _scoring(torch, rp, ci, synth.random_labels(40_000, c, seed=1, n_distinct=400)))
+         for c in (20, 32)}
+    assert t[32] < 1.25 * t[20], t
