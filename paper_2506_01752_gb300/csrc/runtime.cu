@@ -58,6 +58,11 @@ constexpr int64_t kWideItems = 65536;
 // many nodes (n = 170,001 464 -> 454 us a generation, n = 10^6 3.33 -> 3.26 ms;
 // two rounds at n = 40,000 are 2 us slower).
 constexpr long long kEvalNodes = 12;
+// mocd_set_population: up to this many labels are checked on the host, 0.4 ns
+// each, more on the device, a launch and a synchronisation of 13 us (n = 200,
+// one member: 65 us a call with the host check, 78 with the device's; n = 40,000,
+// 100 members: 1,840 and 231).
+constexpr size_t kHostCheckLabels = 32768;
 
 }  // namespace
 
@@ -1209,21 +1214,24 @@ int mocd_set_population(mocd_ctx *c, const mocd_params *params, const int32_t *l
     int rc = check_params(c, params);
     if (rc) return rc;
     CK(cudaSetDevice(c->device));
-    // The labels are checked on the device (a pass over a host array of n N_p
-    // labels took longer than copying and evaluating it: 1.5 of 1.9 ms at n =
-    // 40,000, N_p = 100), before the population there was is touched.
-    rc = grow(c->stream, &c->d_im, &c->im_cap, (size_t)params->pop_size * (size_t)c->n);
+    // The labels are checked before the population there was is touched.
+    const size_t cells = (size_t)params->pop_size * (size_t)c->n;
+    if (cells <= kHostCheckLabels)
+        for (size_t k = 0; k < cells; ++k)
+            if ((uint32_t)labels[k] >= (uint32_t)c->n) return MOCD_ERR_INVALID_ARG;
+    rc = grow(c->stream, &c->d_im, &c->im_cap, cells);
     if (rc) return rc;
     if ((rc = eval_scratch(c))) return rc;
-    int bad = 0;
-    CK(cudaMemcpyAsync(c->d_im, labels, sizeof(int32_t) * (size_t)params->pop_size * (size_t)c->n,
-                       cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemsetAsync(eval_bad(c), 0, sizeof(int), c->stream));
-    CK(launch_to_node_major((int)c->n, (params->pop_size + 3) & ~3, params->pop_size, c->d_im, nullptr, eval_bad(c),
-                            c->stream));
-    CK(cudaMemcpyAsync(&bad, eval_bad(c), sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    if (bad) return MOCD_ERR_INVALID_ARG;
+    CK(cudaMemcpyAsync(c->d_im, labels, sizeof(int32_t) * cells, cudaMemcpyHostToDevice, c->stream));
+    if (cells > kHostCheckLabels) {
+        int bad = 0;
+        CK(cudaMemsetAsync(eval_bad(c), 0, sizeof(int), c->stream));
+        CK(launch_to_node_major((int)c->n, (params->pop_size + 3) & ~3, params->pop_size, c->d_im, nullptr,
+                                eval_bad(c), c->stream));
+        CK(cudaMemcpyAsync(&bad, eval_bad(c), sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        if (bad) return MOCD_ERR_INVALID_ARG;
+    }
     c->ready = false;
     rc = prepare_population(c, params);
     if (rc) return rc;

@@ -140,3 +140,43 @@ def test_scoring_of_32_labellings_costs_little_more_than_20():
     t = {c: _pass_us(torch, _scoring(torch, rp, ci, synth.random_labels(40_000, c, seed=1, n_distinct=400)))
          for c in (20, 32)}
     assert t[32] < 1.25 * t[20], t
+
+
+# mocd_set_population checks up to 32,768 labels on the host, more on the
+# device. Either way a label out of range is refused and the population that
+# was there stays.
+@pytest.mark.parametrize("n,np_", [(64, 1), (256, 128), (257, 128), (8191, 4), (8193, 4)])
+def test_set_population_refuses_labels_out_of_range(n, np_):
+    rp, ci = _regular(n, 6, seed=n)
+    good = synth.random_labels(n, np_, seed=1)
+    params = mocd.Params(pop_size=np_, n_parents=1, seed=3)
+    h = mocd.graph_upload(rp, ci)
+    try:
+        mocd.set_population(h, params, good, 5)
+        before = mocd.get_population(h)
+        assert np.array_equal(before[0], good)
+        for at, label in ((0, -1), (-1, n), (good.size // 2, -2**31), (-1, 2**31 - 1)):
+            bad = good.copy()
+            bad.reshape(-1)[at] = label
+            with pytest.raises(mocd.MocdError):
+                mocd.set_population(h, params, bad, 7)
+            after = mocd.get_population(h)
+            assert all(np.array_equal(x, y) for x, y in zip(before, after))
+        mocd.generation(h, 1)  # and it still runs
+        ref = oracle.run(rp, ci, oracle.Params(pop_size=np_, n_parents=1, seed=3),
+                         oracle.State(good, before[1], before[2], 5), 1)
+        assert np.array_equal(mocd.get_population(h)[0], ref.labels)
+    finally:
+        mocd.destroy(h)
+
+
+def test_set_population_of_few_labels_costs_little_more_than_an_init():
+    rp, ci = _regular(200, 6, seed=1)
+    params = mocd.Params(pop_size=1, n_parents=1, seed=3)
+    lab = synth.random_labels(200, 1, seed=1)
+    h = mocd.graph_upload(rp, ci)
+    try:
+        init = _best(lambda: mocd.population_init(h, params), times=60)
+        assert _best(lambda: mocd.set_population(h, params, lab, 0), times=60) < 1.35 * init
+    finally:
+        mocd.destroy(h)
