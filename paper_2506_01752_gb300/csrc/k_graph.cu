@@ -4,15 +4,17 @@
 // * the symmetry check (an undirected graph, Sec. 2.1: u ~ v iff v ~ u). A
 //   warp takes a row v; each lane takes one of its neighbours u and binary
 //   searches v in the (sorted) row of u. A missing mirror sets *bad.
-// * the oriented adjacency of the offspring evaluation: every undirected
-//   edge listed once, at its endpoint of lower (degree, id), the lists in
-//   processing order. A warp per node counts the neighbours above it, one block scans the counts into row
-//   pointers, and a warp per node writes the entries in row order.
+// * the oriented adjacency of the evaluation: every undirected edge listed
+//   once, at its endpoint of lower (degree, id), the lists in processing order.
+//   A warp per node counts the neighbours above it, one block scans the counts
+//   into row pointers, and a warp per node writes the entries in row order.
 // * the mutation's adjacency: the rows in processing order (degree
 //   descending), padded to groups of four entries with the id n, so that a
 //   thread reads four neighbours with one 16-byte load; and a record per node
 //   (id, first group, degree) in the same order, one load instead of the
-//   chain order -> row pointers.
+//   chain order -> row pointers. Written by the warps that write the oriented
+//   entries, which read the same rows (n = 400,000, mean degree 16: 61 + 47 us
+//   in launches of their own).
 //
 // Every index these kernels form is in range because the host checks ran
 // first; the oriented entries are also bounded by their buffer, so a graph
@@ -109,9 +111,13 @@ __global__ void scan_kernel(int32_t *__restrict__ a, int len)
 
 // eidx[eptr[k] ..] = the neighbours above v (at position k), in row order;
 // entries at or past cap (possible only for an asymmetric graph) are skipped.
+// And nodes[k] = (v, first group of four of its row in the mutation's adjacency,
+// deg v, 0) with that row, padded with n; its place follows from the degree
+// because the order is by degree. A warp a node.
 __global__ void __launch_bounds__(kBlock)
-orient_fill_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                   const int32_t *__restrict__ order, const int32_t *__restrict__ eptr, int32_t *__restrict__ eidx, int cap)
+rows_fill_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
+                 const int32_t *__restrict__ order, const int32_t *__restrict__ eptr, int32_t *__restrict__ eidx,
+                 int cap, const int2 *__restrict__ by_degree, int4 *__restrict__ nodes, int4 *__restrict__ adj)
 {
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -119,47 +125,22 @@ orient_fill_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__
     const unsigned lt = (1u << lane) - 1u;
     for (int k = warp; k < n; k += nwarps) {
         const int v = __ldg(order + k);
-        const int beg = __ldg(row_ptr + v), end = __ldg(row_ptr + v + 1);
+        const int beg = __ldg(row_ptr + v), d = __ldg(row_ptr + v + 1) - beg;
+        const int2 place = __ldg(by_degree + d);
+        const int first = place.y + (k - place.x) * ((d + 3) / 4);
+        if (lane == 0) nodes[k] = make_int4(v, first, d, 0);
+        int32_t *row = reinterpret_cast<int32_t *>(adj + first);
         int at = eptr[k];
-        for (int k0 = beg; k0 < end; k0 += 32) {
-            const int u = k0 + lane < end ? __ldg(col_idx + k0 + lane) : 0;
-            const bool up = k0 + lane < end && above(row_ptr, v, end - beg, u);
+        for (int e0 = 0; e0 < d; e0 += 32) {
+            const int e = e0 + lane;
+            const int u = e < d ? __ldg(col_idx + beg + e) : n;
+            if (e < ((d + 3) & ~3)) row[e] = u;
+            const bool up = e < d && above(row_ptr, v, d, u);
             const unsigned m = __ballot_sync(0xffffffffu, up);
-            const int pos = at + __popc(m & lt);
-            if (up && pos >= 0 && pos < cap) eidx[pos] = u;
+            const int w = at + __popc(m & lt);
+            if (up && w < cap) eidx[w] = u;
             at += __popc(m);
         }
-    }
-}
-
-// nodes[k] = (v, first group of four of its adjacency, deg v, 0) of the node
-// at position k of the order; its place follows from its degree because the
-// order is by degree.
-__global__ void __launch_bounds__(kBlock)
-node_records_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ order,
-                    const int2 *__restrict__ by_degree, int4 *__restrict__ nodes)
-{
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int v = order[k];
-        const int d = row_ptr[v + 1] - row_ptr[v];
-        const int2 at = by_degree[d];
-        nodes[k] = make_int4(v, at.y + (k - at.x) * ((d + 3) / 4), d, 0);
-    }
-}
-
-// The rows of the mutation's adjacency, a warp each, padded with n.
-__global__ void __launch_bounds__(kBlock)
-mutation_rows_kernel(int n, const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_idx,
-                     const int4 *__restrict__ nodes, int4 *__restrict__ adj)
-{
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int k = warp; k < n; k += nwarps) {
-        const int4 rec = nodes[k];
-        const int beg = __ldg(row_ptr + rec.x);
-        int32_t *row = reinterpret_cast<int32_t *>(adj + rec.y);
-        for (int e = lane; e < ((rec.z + 3) & ~3); e += 32) row[e] = e < rec.z ? __ldg(col_idx + beg + e) : n;
     }
 }
 
@@ -175,25 +156,15 @@ int warp_grid(const void *kernel, int n, int sms)
 
 }  // namespace
 
-cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
-                          int32_t *eptr, int32_t *eidx, int cap, int sms, cudaStream_t s)
+cudaError_t launch_rows(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
+                        int32_t *eptr, int32_t *eidx, int cap, const int2 *by_degree, int4 *nodes, int4 *adj,
+                        int sms, cudaStream_t s)
 {
     orient_count_kernel<<<warp_grid((const void *)orient_count_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr,
                                                                                                 col_idx, order, eptr);
     scan_kernel<<<1, 1024, 0, s>>>(eptr, n + 1);
-    orient_fill_kernel<<<warp_grid((const void *)orient_fill_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr, col_idx,
-                                                                                              order, eptr, eidx, cap);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_mutation_adjacency(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
-                                      const int2 *by_degree, int4 *nodes, int4 *adj, int sms, cudaStream_t s)
-{
-    long long blocks = ((long long)n + kBlock - 1) / kBlock;
-    if (blocks > 16ll * sms) blocks = 16ll * sms;
-    node_records_kernel<<<(int)blocks, kBlock, 0, s>>>(n, row_ptr, order, by_degree, nodes);
-    mutation_rows_kernel<<<warp_grid((const void *)mutation_rows_kernel, n, sms), kBlock, 0, s>>>(n, row_ptr, col_idx,
-                                                                                                  nodes, adj);
+    rows_fill_kernel<<<warp_grid((const void *)rows_fill_kernel, n, sms), kBlock, 0, s>>>(
+        n, row_ptr, col_idx, order, eptr, eidx, cap, by_degree, nodes, adj);
     return cudaGetLastError();
 }
 

@@ -199,17 +199,15 @@ cudaError_t launch_gather_individuals(int n, int W, int np, const int32_t *phalf
 // [0, n) set *bad and become 0. dst NULL: only the check.
 cudaError_t launch_to_node_major(int n, int W, int count, const int32_t *src, int32_t *dst, int *bad,
                                  cudaStream_t s);
-// The evaluation's oriented adjacency of a host-checked CSR: eptr [n + 1] list
-// pointers by position in the order, eidx [cap] entries (cap = m for a symmetric
-// graph), each undirected edge listed once, at its endpoint of lower (degree,
-// id).
-cudaError_t launch_orient(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
-                          int32_t *eptr, int32_t *eidx, int cap, int sms, cudaStream_t s);
-// The mutation's node records and adjacency (mocd_ctx::d_nodes / d_adj).
-// by_degree[d] = (first position, first group of four entries) of the nodes
-// of degree d in the order.
-cudaError_t launch_mutation_adjacency(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
-                                      const int2 *by_degree, int4 *nodes, int4 *adj, int sms, cudaStream_t s);
+// The adjacencies of a host-checked CSR in the order: the evaluation's oriented
+// one, eptr [n + 1] list pointers by position, eidx [cap] entries (cap = m for a
+// symmetric graph), each undirected edge listed once, at its endpoint of lower
+// (degree, id); and the mutation's node records and rows (mocd_ctx::d_nodes /
+// d_adj), by_degree[d] = (first position, first group of four entries) of the
+// nodes of degree d.
+cudaError_t launch_rows(int n, const int32_t *row_ptr, const int32_t *col_idx, const int32_t *order,
+                        int32_t *eptr, int32_t *eidx, int cap, const int2 *by_degree, int4 *nodes, int4 *adj,
+                        int sms, cudaStream_t s);
 // *bad = 1 if some stored entry (v, u) has no mirror (u, v); rows must be
 // sorted, in range and free of self loops (checked on the host first).
 cudaError_t launch_symmetry_check(int n, const int32_t *row_ptr, const int32_t *col_idx, int *bad, int sms,

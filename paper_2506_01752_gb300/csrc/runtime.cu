@@ -1098,8 +1098,10 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
 
     mocd_ctx *c = new (std::nothrow) mocd_ctx();
     if (!c) return MOCD_ERR_OUT_OF_MEMORY;
+    int *d_bad = nullptr;  // a missing mirror; freed below
     auto fail = [&](int rc) {
-        mocd_destroy(c);
+        dev_free(d_bad, c->stream);
+        mocd_destroy(c);  // (synchronises: copies from this function's vectors may be under way)
         return rc;
     };
     if (cudaGetDevice(&c->device) != cudaSuccess) return fail(MOCD_ERR_CUDA);
@@ -1116,15 +1118,21 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
     c->n = n;
     c->m = nnz / 2;
     c->dmax = dmax;
-    for (int64_t v = 0; v < n; ++v) {
-        const int64_t d = row_ptr[v + 1] - row_ptr[v];
-        if (d > kSharedTableMax) c->n_hub += 1;
-        else if (d > kDeferMax) c->n_wide += 1;
-        else if (d > 64) c->n_vote[1] += 1;
-        else if (d > 32) c->n_vote[0] += 1;
-    }
+    // One pass over the degrees: the row pointers in 32 bits, and the number of
+    // nodes of each degree, the largest first.
     std::vector<int32_t> rp32(n + 1);
-    for (int64_t v = 0; v <= n; ++v) rp32[v] = (int32_t)row_ptr[v];
+    std::vector<int64_t> at((size_t)dmax + 2, 0);
+    rp32[0] = 0;
+    for (int64_t v = 0; v < n; ++v) {
+        rp32[v + 1] = (int32_t)row_ptr[v + 1];
+        at[(size_t)(dmax - (row_ptr[v + 1] - row_ptr[v])) + 1] += 1;
+    }
+    for (int d = 33; d <= dmax; ++d) {
+        const int64_t nodes = at[(size_t)(dmax - d) + 1];
+        if (d > kSharedTableMax) c->n_hub += nodes;
+        else if (d > kDeferMax) c->n_wide += nodes;
+        else c->n_vote[d > 64] += nodes;
+    }
     void *p = nullptr;
     cudaError_t e = dev_alloc(&p, sizeof(int32_t) * (n + 1), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
@@ -1132,64 +1140,57 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
     e = dev_alloc(&p, sizeof(int32_t) * nnz, c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_col_idx = static_cast<int32_t *>(p);
+    e = dev_alloc(reinterpret_cast<void **>(&d_bad), sizeof(int), c->stream);
+    if (e != cudaSuccess) return fail(cuda_status(e));
+    // The rows are copied, and their symmetry checked, while the host finds the
+    // order of the nodes.
+    if (cudaMemcpyAsync(c->d_row_ptr, rp32.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, c->stream) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(c->d_col_idx, src, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+        cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream) != cudaSuccess ||
+        launch_symmetry_check((int)n, c->d_row_ptr, c->d_col_idx, d_bad, c->sms, c->stream) != cudaSuccess)
+        return fail(MOCD_ERR_CUDA);
     // Work order of the degree-proportional kernels: degree descending (ties
     // by node id), so that the costliest nodes are spread over all warps. A
-    // counting sort on the degree.
-    std::vector<int32_t> order(n);
-    // Per degree: the first position of its nodes, and the first group of four
-    // entries of their rows in the mutation's adjacency.
-    std::vector<int2> by_degree((size_t)dmax + 1, make_int2(0, 0));
+    // counting sort on the degree. Behind it, per degree: the first position of
+    // its nodes, and the first group of four entries of their rows in the
+    // mutation's adjacency.
+    const size_t head = ((size_t)n + 1) & ~(size_t)1;
+    std::vector<int32_t> order(head + 2 * ((size_t)dmax + 1));
     int64_t groups = 0;
-    {
-        std::vector<int64_t> at((size_t)dmax + 2, 0);
-        for (int64_t v = 0; v < n; ++v) at[(size_t)(dmax - (row_ptr[v + 1] - row_ptr[v])) + 1] += 1;
-        for (size_t d = 1; d < at.size(); ++d) at[d] += at[d - 1];
-        for (int d = dmax; d >= 0; --d) {
-            const size_t k = (size_t)(dmax - d);
-            by_degree[(size_t)d] = make_int2((int)at[k], (int)groups);
-            groups += (at[k + 1] - at[k]) * ((d + 3) / 4);
-        }
-        for (int64_t v = 0; v < n; ++v) order[at[(size_t)(dmax - (row_ptr[v + 1] - row_ptr[v]))]++] = (int32_t)v;
+    for (size_t d = 1; d < at.size(); ++d) at[d] += at[d - 1];
+    for (int d = dmax; d >= 0; --d) {
+        const size_t k = (size_t)(dmax - d);
+        order[head + 2 * (size_t)d] = (int32_t)at[k];
+        order[head + 2 * (size_t)d + 1] = (int32_t)groups;
+        groups += (at[k + 1] - at[k]) * ((d + 3) / 4);
     }
-    // One allocation: the order, the node records, the padded rows and the
-    // table per degree (read once, below).
-    const size_t order_bytes = (sizeof(int32_t) * (size_t)n + 15) & ~(size_t)15;
-    e = dev_alloc(&p, order_bytes + sizeof(int4) * (size_t)(n + groups) + sizeof(int2) * by_degree.size(), c->stream);
+    for (int64_t v = 0; v < n; ++v) order[at[(size_t)(dmax - (rp32[v + 1] - rp32[v]))]++] = (int32_t)v;
+    // One allocation: the order with its table per degree (read once, below),
+    // the node records and the padded rows.
+    const size_t order_bytes = (sizeof(int32_t) * order.size() + 15) & ~(size_t)15;
+    e = dev_alloc(&p, order_bytes + sizeof(int4) * (size_t)(n + groups), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_order = static_cast<int32_t *>(p);
     c->d_nodes = reinterpret_cast<int4 *>(static_cast<char *>(p) + order_bytes);
     c->d_adj = c->d_nodes + n;
-    int2 *d_by_degree = reinterpret_cast<int2 *>(c->d_adj + groups);
-    if (cudaMemcpyAsync(c->d_order, order.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, c->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(d_by_degree, by_degree.data(), sizeof(int2) * by_degree.size(), cudaMemcpyHostToDevice,
-                        c->stream) != cudaSuccess)
-        return fail(MOCD_ERR_CUDA);
+    const int2 *d_by_degree = reinterpret_cast<const int2 *>(c->d_order + head);
     e = dev_alloc(&p, sizeof(int32_t) * (n + 1), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_eptr = static_cast<int32_t *>(p);
     e = dev_alloc(&p, sizeof(int32_t) * (size_t)(nnz / 2), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_eidx = static_cast<int32_t *>(p);
-    int *d_bad = nullptr;
     int h_bad = 0;
-    e = dev_alloc(reinterpret_cast<void **>(&d_bad), sizeof(int), c->stream);
-    if (e != cudaSuccess) return fail(cuda_status(e));
-    const bool copied =
-        cudaMemcpyAsync(c->d_row_ptr, rp32.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice,
-                        c->stream) == cudaSuccess &&
-        cudaMemcpyAsync(c->d_col_idx, src, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, c->stream) ==
-            cudaSuccess &&
-        cudaMemsetAsync(d_bad, 0, sizeof(int), c->stream) == cudaSuccess &&
-        launch_symmetry_check((int)n, c->d_row_ptr, c->d_col_idx, d_bad, c->sms, c->stream) == cudaSuccess &&
-        launch_orient((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_eptr, c->d_eidx, (int)(nnz / 2), c->sms,
-                      c->stream) == cudaSuccess &&
-        launch_mutation_adjacency((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, d_by_degree, c->d_nodes, c->d_adj,
-                                  c->sms, c->stream) == cudaSuccess &&
-        cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream) == cudaSuccess;
-    cudaFreeAsync(d_bad, c->stream);
-    if (!copied || cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(MOCD_ERR_CUDA);
+    if (cudaMemcpyAsync(c->d_order, order.data(), sizeof(int32_t) * order.size(), cudaMemcpyHostToDevice, c->stream) !=
+            cudaSuccess ||
+        launch_rows((int)n, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_eptr, c->d_eidx, (int)(nnz / 2), d_by_degree,
+                    c->d_nodes, c->d_adj, c->sms, c->stream) != cudaSuccess ||
+        cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
+        cudaStreamSynchronize(c->stream) != cudaSuccess)
+        return fail(MOCD_ERR_CUDA);
     if (h_bad) return fail(MOCD_ERR_NOT_SYMMETRIC);
+    cudaFreeAsync(d_bad, c->stream);
     *out = c;
     return MOCD_OK;
 }

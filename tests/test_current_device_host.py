@@ -81,14 +81,13 @@ cudaError_t cudaGraphNodeGetType(cudaGraphNode_t, cudaGraphNodeType *t) { *t = c
 
 namespace mocd {
 cudaError_t launch_front(const GenParams &, const PopState &, cudaStream_t s) { return launched(s); }
-cudaError_t launch_orient(int, const int32_t *, const int32_t *, const int32_t *, int32_t *, int32_t *, int, int, cudaStream_t s) { return launched(s); }
+cudaError_t launch_rows(int, const int32_t *, const int32_t *, const int32_t *, int32_t *, int32_t *, int, const int2 *, int4 *, int4 *, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_select(const GenParams &, const PopState &, int, cudaStream_t s, uint32_t) { return launched(s); }
 cudaError_t launch_select_multi(const GenParams *, const PopState *, int, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_evaluate(int, int, int, bool, const int32_t *, const int32_t *, const int32_t *, const int32_t *, uint32_t *, unsigned long long *, unsigned long long *, int, cudaStream_t s, const int32_t *) { return launched(s); }
 cudaError_t launch_evaluate_multi(const BatchMember *, const int *, int, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_evaluate_offspring(int, int, int, const int32_t *, const int32_t *, const int32_t *, uint32_t *, unsigned long long *, int, cudaStream_t s, const int32_t *) { return launched(s); }
 cudaError_t launch_mutation(const GenParams &, const PopState &, const int4 *, const int4 *, const MutationShape &, cudaStream_t s) { return launched(s); }
-cudaError_t launch_mutation_adjacency(int, const int32_t *, const int32_t *, const int32_t *, const int2 *, int4 *, int4 *, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_crossover(const GenParams &, const PopState &, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_crossover_multi(const BatchMember *, const int *, int, int, int, int, cudaStream_t s) { return launched(s); }
 cudaError_t launch_front_stats(const GenParams &, const PopState &, const int32_t *, int, const int32_t *, const int32_t *, const int32_t *, int32_t *, unsigned long long *, uint32_t *, unsigned long long *, unsigned long long *, int, cudaStream_t s) { return launched(s); }
