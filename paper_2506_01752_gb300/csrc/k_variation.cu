@@ -1257,7 +1257,7 @@ cudaError_t launch_mutation(const GenParams &gp, const PopState &ps, const int4 
 {
     // The launches are independent of each other: on a capturing stream they
     // become parallel branches, the longest votes first.
-    Branches br(s);
+    Branches br(s, gp.n_hub > 0 || gp.n_vote[0] > 0 || gp.n_vote[1] > 0);
     cudaError_t o = cudaSuccess;
     if (gp.n_hub > 0) {
         o = overlap_next(s);

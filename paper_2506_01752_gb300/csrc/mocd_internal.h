@@ -141,10 +141,10 @@ cudaError_t overlap_next(cudaStream_t s);
 // Launches on one capturing stream as parallel branches of the graph: each
 // next() ends a branch and puts the stream back to where the object was made;
 // join() makes what follows depend on every branch. On a stream that does not
-// capture, the launches simply follow each other.
+// capture, or if there are not several, the launches simply follow each other.
 class Branches {
   public:
-    explicit Branches(cudaStream_t s);
+    Branches(cudaStream_t s, bool several);
     void next();
     cudaError_t join();
 

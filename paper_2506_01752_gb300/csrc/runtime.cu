@@ -970,8 +970,9 @@ cudaError_t mocd::overlap_next(cudaStream_t s)
     return cudaStreamUpdateCaptureDependencies(s, nodes.data(), edges.data(), count, cudaStreamSetCaptureDependencies);
 }
 
-mocd::Branches::Branches(cudaStream_t s) : s_(s)
+mocd::Branches::Branches(cudaStream_t s, bool several) : s_(s)
 {
+    if (!several) return;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     const cudaGraphNode_t *deps = nullptr;
     size_t count = 0;
