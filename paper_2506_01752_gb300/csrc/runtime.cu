@@ -289,10 +289,14 @@ void size_grids(mocd_ctx *c)
         const long long wide = cls == 0 ? (long long)c->n_wide * c->gp.wide_parts : 0;
         const int most = (int)std::max<long long>(1, std::min<long long>(kMutBatchMax, (long long)(kMutPairs / pairs)));
         const int occ = grid_for_mutation(c->sms, cls, c->gp.vote_n0, c->gp.hash_size, c->gp.np, most);
-        const long long warps = (long long)occ * mutation_warps_per_block();
+        const long long warps_per_block = mutation_warps_per_block();
+        const long long warps = (long long)occ * warps_per_block;
         c->mut.batch[cls] = (int)std::max<long long>(1, std::min<long long>(most, nodes / (kMutWaves * warps)));
         const long long items = wide + (nodes + c->mut.batch[cls] - 1) / c->mut.batch[cls];
-        const long long per_block = (long long)mutation_warps_per_block() * c->nodes_per_warp;
+        // nodes_per_warp leaves the votes of degrees 33 .. 128 alone: a warp that takes
+        // eight such batches in a row holds the launch up (eight members of 1,000 nodes of
+        // degree up to 100, 8 nodes a warp: 140 us a generation, 80 with a batch a warp).
+        const long long per_block = warps_per_block * (cls == 0 ? c->nodes_per_warp : 1);
         // Up to kMutRounds times the resident blocks: a block that ends early
         // makes room for the next batches (degrees descend, the last are short).
         c->mut.grid[cls] = (int)std::max<long long>(

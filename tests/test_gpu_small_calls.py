@@ -180,3 +180,34 @@ def test_set_population_of_few_labels_costs_little_more_than_an_init():
         assert _best(lambda: mocd.set_population(h, params, lab, 0), times=60) < 1.35 * init
     finally:
         mocd.destroy(h)
+
+
+# nodes_per_warp is for the many short items: the votes of degrees 33 to 128 must
+# not queue up behind each other on few warps. 60 nodes of degree about 100.
+def test_nodes_per_warp_leaves_long_votes_alone():
+    hs = []
+    try:
+        for seed in range(8):
+            rng = np.random.default_rng(seed)
+            u = np.concatenate([np.repeat(np.arange(1000), 10), np.repeat(np.arange(60), 80)])
+            rp, ci = synth.csr_from_edges(1000, u, rng.integers(0, 1000, u.size))
+            d = np.diff(rp)
+            assert ((d > 64) & (d <= 128)).sum() >= 50
+            hs.append(mocd.graph_upload(rp, ci))
+            mocd.population_init(hs[-1], mocd.Params(seed=seed))
+        batch = mocd.batch_create(hs)
+        t = {}
+        try:
+            for npw in (1, 8):
+                mocd.batch_configure(batch, npw, 0)
+
+                def run():
+                    mocd.batch_generation(batch, 10)
+                    mocd.batch_synchronize(batch)
+                t[npw] = _best(run)
+        finally:
+            mocd.batch_destroy(batch)
+        assert t[8] < 1.5 * t[1], t
+    finally:
+        for h in hs:
+            mocd.destroy(h)
