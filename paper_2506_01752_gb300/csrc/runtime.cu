@@ -50,10 +50,13 @@ constexpr long long kMutWaves = 2;
 constexpr long long kMutRounds = 24;
 // Nodes of degree 129 .. 512: a warp per quad of children (about one pair, which
 // takes long: with eighths of a node the launch waits for a warp with six) up
-// to this many quads, above it eighths, whose rows and coins are cheaper. A
-// generation with quads: hubs 116 -> 89 us, dense 118 -> 105 us, n = 10^6 (275,000
-// quads) 2.93 -> 3.01 ms.
+// to this many quads, above it a warp per kWideParts-th of a node, whose rows and
+// coins are cheaper. A generation with quads, against eighths: hubs 116 -> 89 us,
+// dense 118 -> 105 us, n = 10^6 (275,000 quads) 2.93 -> 3.01 ms. With quarters,
+// against eighths: n = 20,000 of degree 200, 100 members, settled, 523 -> 478 us
+// (halves 472), n = 8,000 of degree 400 592 -> 571 (586).
 constexpr int64_t kWideItems = 65536;
+constexpr int kWideParts = 4;
 // The edge count: up to four full GPUs of blocks, as long as a warp keeps this
 // many nodes (n = 170,001 464 -> 454 us a generation, n = 10^6 3.33 -> 3.26 ms;
 // two rounds at n = 40,000 are 2 us slower).
@@ -419,7 +422,7 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.n_vote[1] = (int)c->n_vote[1];
     gp.n_hub = (int)c->n_hub;
     gp.n_wide = (int)c->n_wide;
-    gp.wide_parts = c->n_wide * (W >> 2) <= kWideItems ? W >> 2 : std::min(8, W >> 2);
+    gp.wide_parts = c->n_wide * (W >> 2) <= kWideItems ? W >> 2 : std::min(kWideParts, W >> 2);
     gp.hub_hs = hub_hs;
     gp.hub_smem_hs = hub_smem_hs;
     c->mut.hub_blocks = hub_blocks;

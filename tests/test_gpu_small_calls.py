@@ -211,3 +211,32 @@ def test_nodes_per_warp_leaves_long_votes_alone():
     finally:
         for h in hs:
             mocd.destroy(h)
+
+
+# Nodes of degree 129..512 of a settled population, whose pairs are settled by
+# counting the own label first: by quads up to 65,536 quads, by quarters above.
+@pytest.mark.parametrize("n", [2600, 2660])
+def test_wide_nodes_of_a_settled_population(n):
+    rng = np.random.default_rng(n)
+    u = np.repeat(np.arange(n), 130)
+    v = np.where(rng.random(u.size) < 0.9, u // 400 * 400 + rng.integers(0, 400, u.size), rng.integers(0, n, u.size))
+    rp, ci = synth.csr_from_edges(n, u, np.minimum(v, n - 1))
+    deg = np.diff(rp)
+    wide = int(((deg > 128) & (deg <= 512)).sum())
+    assert (wide * 25 > 65536) == (n == 2660) and wide > 0.9 * n
+    lab = np.repeat((np.arange(n) // 400 * 400).astype(np.int32)[None], 100, 0)
+    stray = rng.random(lab.shape) < 0.05 * rng.random((100, 1))
+    lab[stray] = rng.integers(0, n, int(stray.sum()))
+    k1, k2 = oracle.objectives_parallel(rp, ci, lab)
+    op = oracle.Params(pop_size=100, seed=n)
+    ref = oracle.State(lab, int(rp[-1]) // 2 - k1, k2, 0)
+    h = mocd.graph_upload(rp, ci)
+    try:
+        mocd.set_population(h, mocd.Params(pop_size=100, seed=n), lab, 0)
+        for _ in range(3):  # the second and third know what the one before settled
+            mocd.generation(h, 1)
+            ref = oracle.run_parallel(rp, ci, op, ref, 1)
+            labels, g1, g2, gen = mocd.get_population(h)
+            assert np.array_equal(g1, ref.k1) and np.array_equal(g2, ref.k2) and np.array_equal(labels, ref.labels)
+    finally:
+        mocd.destroy(h)
