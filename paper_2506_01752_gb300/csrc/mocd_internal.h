@@ -101,15 +101,11 @@ struct GenParams {
 };
 
 // One member of a multi-member launch (a batch of contexts): its parameters,
-// state and graph.
+// state, and what the edge count reads of its graph.
 struct BatchMember {
     GenParams gp;
     PopState ps;
-    const int32_t *row_ptr;
-    const int32_t *col_idx;
     const int32_t *order;
-    const int4 *nodes;    // the mutation's node records and adjacency (mocd_ctx::d_nodes / d_adj)
-    const int4 *adj;
     const int32_t *eptr;  // the offspring evaluation's oriented adjacency (mocd_ctx::d_eptr / d_eidx)
     const int32_t *eidx;
 };

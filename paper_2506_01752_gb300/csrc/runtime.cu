@@ -1543,8 +1543,7 @@ static int batch_build(mocd_batch *b)
             mocd_ctx *c = b->ctx[(size_t)i];
             gps.push_back(c->gp);
             pss.push_back(c->ps);
-            mbs.push_back(BatchMember{c->gp, c->ps, c->d_row_ptr, c->d_col_idx, c->d_order, c->d_nodes, c->d_adj,
-                                      c->d_eptr, c->d_eidx});
+            mbs.push_back(BatchMember{c->gp, c->ps, c->d_order, c->d_eptr, c->d_eidx});
             b->es_max = std::max(b->es_max, c->gp.es);
             b->rows_max = std::max(b->rows_max, crossover_row_words(c->gp.W));
             // Per member and stage: its own grid.
