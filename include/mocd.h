@@ -90,9 +90,10 @@ typedef struct {
  * checks every row first (ids in range, self loops, repeats; the first
  * failing row decides the status), then symmetry is checked on the device.
  * The context keeps on the device the CSR (4(n + 1) + 8m bytes), the nodes
- * in degree order (4n) and, for the offspring evaluation, the adjacency with
- * each undirected edge listed once (4(n + 1) + 4m); mocd_job_footprint
- * counts them.
+ * in degree order (4n, and 8 bytes per degree up to the largest), for the
+ * evaluation the adjacency with each undirected edge listed once (4(n + 1) +
+ * 4m), and for the mutation a record per node and the rows padded to groups of
+ * four entries (16 bytes a node and a group); mocd_job_footprint counts them.
  * Errors: INVALID_ARG, NOT_SYMMETRIC, SELF_LOOP, DUPLICATE_EDGE, EMPTY_GRAPH,
  * OUT_OF_MEMORY, CUDA.
  */
@@ -110,7 +111,9 @@ int mocd_population_init(mocd_ctx *ctx, const mocd_params *params);
 /*
  * Run n_generations generations of Alg. 1 (the "for gen" loop body), issued
  * asynchronously on the context stream as CUDA graph launches: one per
- * generation, or one per eight in a run of 24 or more without stage timing.
+ * generation, or, without stage timing, one per eight: from the first call with
+ * 24 or more of a population on, in every call with eight or more. The context's
+ * device need not be the current one, and the current one stays.
  * Errors: INVALID_ARG (n_generations < 0), NOT_READY, CUDA.
  */
 int mocd_generation(mocd_ctx *ctx, int32_t n_generations);

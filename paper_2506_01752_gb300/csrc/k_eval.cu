@@ -5,18 +5,19 @@
 //   intra_i = #{{v, u} in E : L_i(v) = L_i(u)}   (= sum_c |E(c)|)
 //   S_i     = sum_c D_c^2,  D_c = sum_{v : L_i(v) = c} deg v
 // exactly in integers. Each undirected edge is counted once, from one
-// endpoint: with the full adjacency (the initial population, mocd_evaluate)
-// a warp reads the label rows of the neighbours u > v only; the offspring
-// evaluation inside a generation walks an oriented adjacency that lists
-// every edge once, at its endpoint of lower (degree, id), so the rows it
-// reads are the higher-degree endpoints' -- fewer distinct rows, each read
-// more often, which keeps more of them in L2.
+// endpoint. A context (its generations, its initial population, mocd_evaluate)
+// walks an oriented adjacency that lists every edge once, at its endpoint of
+// lower (degree, id), so the rows it reads are the higher-degree endpoints' --
+// fewer distinct rows, each read more often, which keeps more of them in L2.
+// mocd_evaluate_noalloc has only the caller's full adjacency, of which a warp
+// reads the label rows of the neighbours u > v.
 //
-// Layout is node-major: a warp owns node v and lane q holds the int4 of
-// labels of individuals 4q..4q+3, so each neighbour u costs one coalesced
-// row read of all individuals' labels instead of N_p scattered 4-byte
-// gathers, and the CSR is streamed once per population, not once per
-// individual.
+// Layout is node-major: lane q of the lanes that hold node v has the int4 of
+// labels of individuals 4q..4q+3, so each neighbour u costs one coalesced row
+// read of all individuals' labels instead of N_p scattered 4-byte gathers, and
+// the adjacency is streamed once per population, not once per individual. With
+// the oriented adjacency a warp takes as many nodes at a time as its lanes hold
+// rows, with the full one a node.
 //
 // S without a sweep over the histogram D: when node v adds deg(v) to D_c, the
 // atomic returns the old total o, and (o + d)^2 - o^2 = 2 o d + d^2. Summed
@@ -37,11 +38,14 @@
 // overlap its own latency-bound work). The evaluation of the offspring then
 // counts intra (ADD = false) and, in the same launch once a warp's nodes are
 // done, forms S = sum_c D_c^2 in a coalesced sweep of the histogram rows,
-// zeroing them for the next generation. While the labels are still nearly all distinct, the N_p n
-// histogram additions land on different sectors, which at n = 10^6 (a 400 MB
-// histogram) cost a DRAM read and write-back each; done by the mutation
-// kernel, that traffic overlaps with its own work instead of stalling the
-// evaluation's row stream.
+// zeroing them for the next generation. While the labels are still nearly all
+// distinct, the N_p n histogram additions land on different sectors, which at n
+// = 10^6 (a 400 MB histogram) cost a DRAM read and write-back each; done by the
+// mutation kernel, that traffic overlaps with its own work instead of stalling
+// the evaluation's row stream.
+//
+// Labellings given from outside, up to 40,960 nodes: the histogram of each is one
+// block's shared memory (hist_block_kernel), beside the edge count.
 #include <algorithm>
 
 #include "mocd_check.cuh"
@@ -56,8 +60,9 @@ constexpr int kFullBlocks = 5;
 constexpr int kOrientedBlocks = 4;
 
 // FULL: row_ptr / col_idx hold both directions of every edge, rows by node id;
-// else each edge once, lists by position in the order (the oriented adjacency). ADD: the degrees (from deg_ptr) go into the
-// histogram; otherwise a histogram (if given) is complete: square and clear it.
+// else each edge once, lists by position in the order (the oriented adjacency).
+// ADD: the degrees (from deg_ptr) go into the histogram; otherwise a histogram
+// (if given) is complete: square and clear it.
 template <bool FULL, bool ADD>
 __device__ __forceinline__ void evaluate_body(int n, int W, int count,
                                               const int32_t *__restrict__ deg_ptr,
@@ -295,7 +300,8 @@ hist_block_kernel(int n, int W, const int32_t *__restrict__ deg_ptr, const int32
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            if (d[u] > 0 && MOCD_CHECK((unsigned)lab[u] < (unsigned)n, kCheckLabel, v0)) atomicAdd(s_hist + lab[u], (unsigned)d[u]);
+            if (d[u] > 0 && MOCD_CHECK((unsigned)lab[u] < (unsigned)n, kCheckLabel, v0))
+                atomicAdd(s_hist + lab[u], (unsigned)d[u]);
     }
     __syncthreads();
     unsigned long long q = 0;

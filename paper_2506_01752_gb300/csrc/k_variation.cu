@@ -634,7 +634,6 @@ __device__ __forceinline__ int warp_mode_table(const GenParams &gp, const int32_
                                                int *hcnt, uint32_t g, unsigned &best_count)
 {
     const int lane = threadIdx.x & 31;
-    const int W = gp.W;
     // 2 deg <= the per-warp capacity (gp.hash_size), so the table fits.
     int hbits = 8;
     while ((1 << hbits) < 2 * deg) ++hbits;
@@ -811,7 +810,8 @@ __device__ __noinline__ void wide_item(const GenParams &gp, int idx, int part, c
         if (fast) {
             int c = 0;
 #pragma unroll 4
-            for (int e = lane; e < deg; e += 32) c += child[(size_t)checked_node(__ldg(nbr + e), gp.n) * gp.W + i] == own;
+            for (int e = lane; e < deg; e += 32)
+                c += child[(size_t)checked_node(__ldg(nbr + e), gp.n) * gp.W + i] == own;
             settled = 2 * __reduce_add_sync(kFull, c) > deg;
         }
         int lab = own;
@@ -844,6 +844,12 @@ __host__ __device__ __forceinline__ int mutation_warp_words(int np, int batch, i
 // deferred votes of the higher degrees in launches behind it: n = 40,000 66.7 us
 // + 12.7 -> 44.6, n = 170,001 270 us + 86 -> 205, n = 10^6 (tenth generation)
 // 3.38 ms + 0.53 -> 2.0.
+//
+// The 128-entry network (1,471 comparators, for every degree of 65..128) keeps
+// three blocks an SM at 168 registers and spills 268 bytes for it. Without the
+// spills it is two blocks of 239: n = 5,000 of degree 100 94 -> 101 us a
+// generation, n = 20,000 248 -> 245, n = 400,000 of degrees to 200 1.162 -> 1.152
+// ms; not better, and slower where few blocks run.
 //
 // WIDE: the launch also takes the nodes of degree kDeferMax + 1 ..
 // kSharedTableMax (positions n_hub .. n_hub + n_wide - 1). batch: nodes a warp
@@ -886,8 +892,8 @@ mutation_kernel(const __grid_constant__ GenParams gp, int first, int last, const
     for (int item = warp; item < items; item += nwarps) {
         if (WIDE && item < wide) {
             int *table = reinterpret_cast<int *>(recs + mutation_warp_words(gp.np, batch, 0));
-            wide_item(gp, gp.n_hub + item / gp.wide_parts, item % gp.wide_parts, nodes, adj, child, q, hist, hint, list, table,
-                      table + gp.hash_size, g);
+            wide_item(gp, gp.n_hub + item / gp.wide_parts, item % gp.wide_parts, nodes, adj, child, q, hist, hint, list,
+                      table, table + gp.hash_size, g);
             __syncwarp();
             continue;
         }
@@ -1164,7 +1170,10 @@ void crossover_launch(const GenParams &gp, const PopState &ps, int grid, cudaStr
 
 int grid_for_crossover(int sms, int es, int W)
 {
-    return sms * (es <= 4 ? crossover_occupancy<4>(W) : es <= 8 ? crossover_occupancy<8>(W) : crossover_occupancy<16>(W));
+    const int per_sm = es <= 4   ? crossover_occupancy<4>(W)
+                       : es <= 8 ? crossover_occupancy<8>(W)
+                                 : crossover_occupancy<16>(W);
+    return sms * per_sm;
 }
 
 cudaError_t launch_crossover(const GenParams &gp, const PopState &ps, int grid, cudaStream_t s)

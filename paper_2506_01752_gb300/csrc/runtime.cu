@@ -284,8 +284,8 @@ void size_grids(mocd_ctx *c)
     c->grid_eval_intra = shape((int)std::max<long long>(1, std::min<long long>(4, rounds)) * c->occ_eval_intra, rows);
     c->grid_cross = shape(c->occ_cross, rows);
     // The mutation: a batch of nodes fills a warp's lanes with pairs (about
-    // kMutPairs of them), but a class too small to give
-    // every resident warp kMutWaves batches gets smaller ones.
+    // kMutPairs of them), but a class too small to give every resident warp
+    // kMutWaves batches gets smaller ones.
     const double pairs = std::max(0.5, c->params.p_mutation * c->params.pop_size);
     for (int cls = 0; cls < 3; ++cls) {
         const long long nodes = cls > 0 ? c->n_vote[cls - 1] : n - c->n_vote[0] - c->n_vote[1] - c->n_wide - c->n_hub;
@@ -378,7 +378,8 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     }
     const size_t hist_need = (size_t)W * (size_t)c->n;
     // A limit of the interface: N_p times the nodes of degree 33 .. kDeferMax and
-    // the hubs fits 31 bits.
+    // the hubs fits 31 bits. (The kernels' own items are fewer: n_hub W / 4 and
+    // n_wide wide_parts. What was refused stays refused.)
     if ((int64_t)p->pop_size * (c->n_vote[0] + c->n_vote[1] + c->n_hub) > INT_MAX) return MOCD_ERR_INVALID_ARG;
     // Hubs: the hub kernel's count table is in shared memory if the largest
     // hub's fits there, else (for the pairs that do not fit) a table of hub_hs
@@ -1260,7 +1261,8 @@ int mocd_generation(mocd_ctx *c, int32_t n_generations)
     if (rc) return rc;
     int32_t left = n_generations;
     auto launch = [&](int k, int32_t times) -> int {
-        for (; times > 0; --times, left -= k == kChunkGraph ? kChunk : 1) CK(cudaGraphLaunch(c->graph_exec[k], c->stream));
+        for (; times > 0; --times, left -= k == kChunkGraph ? kChunk : 1)
+            CK(cudaGraphLaunch(c->graph_exec[k], c->stream));
         return MOCD_OK;
     };
     if (g == 0 && (c->graph_exec[kChunkGraph] ? left >= kChunk : left >= 3 * kChunk)) {
