@@ -50,13 +50,16 @@ constexpr long long kMutWaves = 2;
 constexpr long long kMutRounds = 24;
 // Nodes of degree 129 .. 512: a warp per quad of children (about one pair, which
 // takes long: with eighths of a node the launch waits for a warp with six) up
-// to this many quads, above it a warp per kWideParts-th of a node, whose rows and
-// coins are cheaper. A generation with quads, against eighths: hubs 116 -> 89 us,
-// dense 118 -> 105 us, n = 10^6 (275,000 quads) 2.93 -> 3.01 ms. With quarters,
-// against eighths: n = 20,000 of degree 200, 100 members, settled, 523 -> 478 us
-// (halves 472), n = 8,000 of degree 400 592 -> 571 (586).
+// to this many quads. A generation with quads, against eighths: hubs 116 -> 89 us,
+// dense 118 -> 105 us, n = 10^6 (275,000 quads) 2.93 -> 3.01 ms. Above it a warp per
+// quarter of a node, whose rows and coins are cheaper, or per eighth where such
+// nodes are fewer than one in kWideShare: among many short items a warp with a long
+// one keeps the other warps' places in its block. Quarters against eighths, settled:
+// n = 20,000 of degree 200 523 -> 478 us, n = 8,000 of degree 400 592 -> 571, n =
+// 400,000 with 1.5% of them 1,569 -> 1,541, n = 10^6 with 1.4% 3.52 -> 3.45 ms, with
+// 0.8% 2.55 -> 2.58 (settled) and 3.18 -> 3.24 (another graph's sixty generations).
 constexpr int64_t kWideItems = 65536;
-constexpr int kWideParts = 4;
+constexpr int64_t kWideShare = 100;
 // The edge count: up to four full GPUs of blocks, as long as a warp keeps this
 // many nodes (n = 170,001 464 -> 454 us a generation, n = 10^6 3.33 -> 3.26 ms;
 // two rounds at n = 40,000 are 2 us slower).
@@ -423,7 +426,8 @@ int prepare_population(mocd_ctx *c, const mocd_params *p)
     gp.n_vote[1] = (int)c->n_vote[1];
     gp.n_hub = (int)c->n_hub;
     gp.n_wide = (int)c->n_wide;
-    gp.wide_parts = c->n_wide * (W >> 2) <= kWideItems ? W >> 2 : std::min(kWideParts, W >> 2);
+    gp.wide_parts = W >> 2;
+    if (c->n_wide * (W >> 2) > kWideItems) gp.wide_parts = std::min(W >> 2, c->n_wide * kWideShare >= c->n ? 4 : 8);
     gp.hub_hs = hub_hs;
     gp.hub_smem_hs = hub_smem_hs;
     c->mut.hub_blocks = hub_blocks;
@@ -1176,13 +1180,14 @@ int mocd_graph_upload(mocd_ctx **out, int64_t n, const int64_t *row_ptr, const i
     }
     for (int64_t v = 0; v < n; ++v) order[at[(size_t)(dmax - (rp32[v + 1] - rp32[v]))]++] = (int32_t)v;
     // One allocation: the order with its table per degree (read once, below),
-    // the node records and the padded rows.
-    const size_t order_bytes = (sizeof(int32_t) * order.size() + 15) & ~(size_t)15;
-    e = dev_alloc(&p, order_bytes + sizeof(int4) * (size_t)(n + groups), c->stream);
+    // the node records and the padded rows, each on a cache line of its own.
+    const auto lines = [](size_t bytes) { return (bytes + 127) & ~(size_t)127; };
+    const size_t order_bytes = lines(sizeof(int32_t) * order.size()), node_bytes = lines(sizeof(int4) * (size_t)n);
+    e = dev_alloc(&p, order_bytes + node_bytes + sizeof(int4) * (size_t)groups, c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));
     c->d_order = static_cast<int32_t *>(p);
     c->d_nodes = reinterpret_cast<int4 *>(static_cast<char *>(p) + order_bytes);
-    c->d_adj = c->d_nodes + n;
+    c->d_adj = reinterpret_cast<int4 *>(static_cast<char *>(p) + order_bytes + node_bytes);
     const int2 *d_by_degree = reinterpret_cast<const int2 *>(c->d_order + head);
     e = dev_alloc(&p, sizeof(int32_t) * (n + 1), c->stream);
     if (e != cudaSuccess) return fail(cuda_status(e));

@@ -327,7 +327,7 @@ int mocd_job_footprint(int64_t n, const int64_t *row_ptr, int32_t pop_size, int6
     const int64_t hist = W * n * 4;               // degree histogram
     const int64_t mutation = hints * 4 + hub_tables;
     // CSR, oriented CSR, flag; order, node records, the mutation's rows, the table per degree
-    const int64_t graph = 2 * (n + 1) * 4 + (nnz + nnz / 2) * 4 + 4 + n * 4 + 16 + (n + groups) * 16 + (dmax + 1) * 8;
+    const int64_t graph = 2 * (n + 1) * 4 + (nnz + nnz / 2) * 4 + 4 + n * 4 + 260 + (n + groups) * 16 + (dmax + 1) * 8;
     const int64_t front = (int64_t)pop_size * n * 4 + 2 * mocd::kMaxPop * 4;  // front download
     const int64_t fixed = (int64_t)1 << 20;       // small state, graph executable, events
     *bytes = labels + hist + mutation + graph + front + fixed;
