@@ -71,7 +71,8 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count,
                                               const int32_t *__restrict__ labels, uint32_t *__restrict__ hist,
                                               unsigned long long *__restrict__ intra,
                                               unsigned long long *__restrict__ sumsq,
-                                              const int32_t *__restrict__ order, int vblock, int vgrid)
+                                              const int32_t *__restrict__ order, int vblock, int vgrid,
+                                              bool beside = false)
 {
     // The block's sums: the edge count (at most m < 2^30), then S in limbs of 22
     // bits, 256 of which fit a word. 64-bit additions in shared memory are loops
@@ -247,6 +248,7 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count,
         put(3, c3, q3);
     }
     __syncthreads();
+    if (beside) cudaGridDependencySynchronize();  // (it cleared intra)
     for (int t = threadIdx.x; t < count; t += blockDim.x) {
         const uint32_t *at = &s_sum[0][(t & 3) * (kMaxPop / 4) + (t >> 2)];
         const unsigned long long q = at[kMaxPop] + ((unsigned long long)at[2 * kMaxPop] << kLimbBits) +
@@ -256,8 +258,8 @@ __device__ __forceinline__ void evaluate_body(int n, int W, int count,
     }
 }
 
-// beside: the launch before this one on the stream (hist_block_kernel) only
-// runs beside it: nothing here depends on it, but this launch ends after it.
+// beside: the launch before this one on the stream (hist_block_kernel) runs
+// beside it, until the sums are added to intra, which that launch cleared.
 template <bool FULL, bool ADD>
 __global__ void __launch_bounds__(kBlock, FULL ? kFullBlocks : kOrientedBlocks)
 evaluate_kernel(int n, int W, int count, const int32_t *__restrict__ deg_ptr,
@@ -271,18 +273,18 @@ evaluate_kernel(int n, int W, int count, const int32_t *__restrict__ deg_ptr,
     if (!beside) cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
     evaluate_body<FULL, ADD>(n, W, count, deg_ptr, row_ptr, col_idx, labels, hist, intra, sumsq, order,
-                             blockIdx.x, gridDim.x);
-    if (beside) cudaGridDependencySynchronize();
+                             blockIdx.x, gridDim.x, beside);
 }
 
 // S of individual blockIdx.x with its histogram in shared memory (n words): no
 // global atomics, nothing to clear. The block reads one label a row, an eighth
 // of each sector, which costs less than n additions at the L2's atomic rate
-// do. out: S of each individual.
+// do. out: S of each individual; intra: 0 for each.
 constexpr int kHistThreads = 1024;
+constexpr size_t kPlainSharedBytes = 47 * 1024;  // dynamic shared memory a launch gets unasked, beside the static
 __global__ void __launch_bounds__(kHistThreads)
 hist_block_kernel(int n, int W, const int32_t *__restrict__ deg_ptr, const int32_t *__restrict__ labels,
-                  unsigned long long *__restrict__ out)
+                  unsigned long long *__restrict__ out, unsigned long long *__restrict__ intra)
 {
     cudaTriggerProgrammaticLaunchCompletion();  // the edge count runs beside this
     extern __shared__ uint32_t s_hist[];
@@ -314,7 +316,10 @@ hist_block_kernel(int n, int W, const int32_t *__restrict__ deg_ptr, const int32
     q = s_sum[threadIdx.x];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
-    if (threadIdx.x == 0) out[blockIdx.x] = q;
+    if (threadIdx.x == 0) {
+        out[blockIdx.x] = q;
+        intra[blockIdx.x] = 0;
+    }
 }
 
 // The offspring evaluation of every member of a batch in one launch: members
@@ -374,11 +379,14 @@ cudaError_t launch_evaluate(int n, int W, int count, bool full, const int32_t *d
     if (!add) {
         // A histogram block fills one SM's shared memory on `count` of them; the
         // edge count takes the rest of the GPU at the same time.
-        // (If it cannot be had, nothing would write sumsq.)
-        cudaError_t e = cudaFuncSetAttribute(hist_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kHistBlockBytes);
-        if (e != cudaSuccess) return e;
-        hist_block_kernel<<<count, kHistThreads, n * sizeof(uint32_t), s>>>(n, W, deg_ptr, labels, sumsq);
+        // (If it cannot be had, nothing would write sumsq and clear intra.)
+        const size_t bytes = n * sizeof(uint32_t);
+        cudaError_t e = cudaSuccess;
+        if (bytes > kPlainSharedBytes) {
+            e = cudaFuncSetAttribute(hist_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHistBlockBytes);
+            if (e != cudaSuccess) return e;
+        }
+        hist_block_kernel<<<count, kHistThreads, bytes, s>>>(n, W, deg_ptr, labels, sumsq, intra);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         cudaLaunchAttribute attr = {};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

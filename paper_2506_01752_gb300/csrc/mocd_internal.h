@@ -158,8 +158,8 @@ cudaError_t launch_crossover_multi(const BatchMember *members, const int *starts
 int crossover_row_words(int W);  // rows_max: the largest over the members
 cudaError_t launch_evaluate_multi(const BatchMember *members, const int *starts, int count, int blocks,
                                   cudaStream_t s);
-// Objectives of `count` labellings (node-major rows of W): adds the edge counts
-// into intra and S into sumsq (both zero on entry). row_ptr / col_idx: both
+// Objectives of `count` labellings (node-major rows of W): the edge counts into
+// intra and S into sumsq (both zero on entry where a histogram is needed). row_ptr / col_idx: both
 // directions of every edge (full), or the oriented adjacency; deg_ptr: row
 // pointers whose differences are the degrees. The histogram of each labelling
 // is one block's shared memory (up to kHistBlockBytes), or, where

@@ -86,10 +86,9 @@ extern "C" int mocd_evaluate_noalloc(const int32_t *row_ptr, const int32_t *col_
     int sms = 1;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MOCD_ERR_CUDA;
     if (!evaluate_needs_histogram(n, W, true)) {
-        // S is written by the launch that has its histograms, intra accumulated in place.
-        unsigned long long *in = reinterpret_cast<unsigned long long *>(intra);
-        if (cudaMemsetAsync(in, 0, sizeof(int64_t) * (size_t)count, s) != cudaSuccess ||
-            launch_evaluate((int)n, W, count, true, row_ptr, row_ptr, col_idx, labels, nullptr, in,
+        // Two launches that write the caller's arrays: nothing to clear here.
+        if (launch_evaluate((int)n, W, count, true, row_ptr, row_ptr, col_idx, labels, nullptr,
+                            reinterpret_cast<unsigned long long *>(intra),
                             reinterpret_cast<unsigned long long *>(sumsq), sms, s) != cudaSuccess)
             return MOCD_ERR_CUDA;
         return MOCD_OK;
